@@ -93,10 +93,9 @@ struct EncArgs {
   // below it, all of level below 3, may be sources)
   uint64_t c0, c1, ws;
   uint16_t* prev;     // per position of the chunk: distance to the previous one with the same 4-byte hash (0: none)
-  uint16_t* lens;     // per position: in-block candidate length (low byte), external (high byte), capped at kCap
-  uint64_t* q_in;     // per position: the in-block candidate's source
-  uint64_t* q_ex;     // per position: the external candidate's source
-  uint8_t* wave;      // per position: resolution wave of the byte (0: literal)
+  uint2* cand;        // per position: x = in-block candidate length (bits 0..7), external length (8..15), both
+                      // capped at kCap, and the in-block source as an offset in the block (16..31); y = the external
+                      // source (below kHead blocks, so below 2^24)
   uint32_t* tok;      // per chunk block: tok_cap x (lit_run, match_len, src lo, src hi)
   uint32_t tok_cap;
   uint32_t* ntok;     // per chunk block
@@ -212,116 +211,206 @@ __global__ void candidate_kernel(EncArgs a) {
     }
     if (li < a.min_match) li = 0;
     if (le < a.min_match) le = 0;
-    a.lens[p - base] = (uint16_t)(li | (le << 8));
-    a.q_in[p - base] = qi;
-    a.q_ex[p - base] = qe;
+    a.cand[p - base] = make_uint2(li | (le << 8) | ((uint32_t)(qi - bstart) << 16), (uint32_t)qe);
   }
 }
 
 // ----------------------------------------------------------- greedy parse
 
-// The resolution wave a match from q of len bytes at p would take: 1 + the
-// deepest wave among the bytes of its own block it reads (literals and
-// bytes of earlier blocks are wave 0).
-__device__ __forceinline__ uint32_t wave_of(const uint8_t* wv, uint64_t bstart, uint64_t q, uint64_t len,
-                                            uint64_t p) {
-  const uint64_t lo = max(q, bstart), hi = min(q + len, p);
-  uint32_t w = 0;
-  for (uint64_t k = lo; k < hi && w < kMaxWave; k++) w = max(w, (uint32_t)wv[k - bstart]);
-  return w + 1;
+// Eight bytes of the input at pos (pos + 8 <= n), from the aligned words
+// around them where those lie inside the input.
+__device__ __forceinline__ uint64_t ld64_in(const EncArgs& a, uint64_t pos) {
+  const uint8_t* p = a.in + pos;
+  const uintptr_t A = reinterpret_cast<uintptr_t>(p);
+  const uint32_t sh = 8 * (uint32_t)(A & 7);
+  if (!sh) return *reinterpret_cast<const uint64_t*>(p);
+  const uint8_t* al = p - (A & 7);
+  if (al < a.in || al + 16 > a.in + a.n) return ld64u(p);
+  const uint64_t* w = reinterpret_cast<const uint64_t*>(al);
+  return (w[0] >> sh) | (w[1] << (64 - sh));
 }
 
-// A thread per block: the greedy walk over its positions.  At each, both
-// candidates are extended past the measured cap, a candidate deeper than
-// kMaxWave is refused, and of the rest the longer one is taken -- except
-// that a shallower one within max(4, len / 8) bytes of the longer wins.
-__global__ void parse_kernel(EncArgs a) {
-  const uint64_t b = a.c0 + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (b >= a.c1) return;
-  const uint64_t base = a.c0 << a.log2B, bstart = b << a.log2B;
-  const uint64_t bend = min((uint64_t)a.n, (uint64_t)(bstart + (1ull << a.log2B)));
-  uint8_t* wv = a.wave + (bstart - base);
-  uint32_t* tk = a.tok + (b - a.c0) * (uint64_t)a.tok_cap * 4;
-  uint32_t nt = 0, lit = 0;
-  unsigned long long n_match = 0, mbytes = 0, msrc = 0, lbytes = 0;
-  uint64_t p = bstart;
-  while (p < bend) {
-    // eight positions without a candidate at once (16-byte loads of the
-    // candidate lengths; the wave bytes of eight literals as one word)
-    if (((p - base) & 7) == 0 && p + 8 <= bend) {
-      const uint4 v = *reinterpret_cast<const uint4*>(a.lens + (p - base));
-      if ((v.x | v.y | v.z | v.w) == 0) {
-        *reinterpret_cast<uint64_t*>(wv + (p - bstart)) = 0;
-        lit += 8;
-        lbytes += 8;
-        p += 8;
-        continue;
-      }
-    }
-    const uint32_t ll = a.lens[p - base];
-    uint32_t best_len = 0, best_w = 0;
-    uint64_t best_q = 0;
-    if (ll) {
-      const uint32_t room = (uint32_t)(bend - p);
-      auto consider = [&](uint64_t q, uint32_t l) {
-        if (l < a.min_match) return;
-        const uint32_t w = wave_of(wv, bstart, q, l, p);
-        if (w > kMaxWave) return;
-        const uint32_t slack = max(4u, max(l, best_len) / 8);
-        bool take;
-        if (!best_len) take = true;
-        else if (w < best_w) take = l + slack >= best_len;
-        else if (w > best_w) take = l > best_len + max(4u, l / 8);
-        else take = l > best_len || (l == best_len && q < best_q);
-        if (take) {
-          best_len = l;
-          best_q = q;
-          best_w = w;
-        }
-      };
-      const uint32_t li = ll & 0xff, le = ll >> 8;
-      if (li) {
-        const uint64_t q = a.q_in[p - base];
-        uint32_t l = li;
-        if (li == kCap && room > kCap) l = kCap + common(a.in + q + kCap, a.in + p + kCap, room - kCap);
-        consider(q, l);
-      }
-      if (le) {
-        const uint64_t q = a.q_ex[p - base];
-        uint32_t l = le;
-        if (le == kCap && room > kCap) l = span(a, q, b, kCap + common(a.in + q + kCap, a.in + p + kCap, room - kCap));
-        consider(q, l);
-      }
-    }
-    if (best_len >= a.min_match && nt + 1 < a.tok_cap) {
-      uint32_t* t = tk + 4 * nt++;
-      t[0] = lit;
-      t[1] = best_len;
-      t[2] = (uint32_t)best_q;
-      t[3] = (uint32_t)(best_q >> 32);
-      for (uint64_t k = p; k < p + best_len; k++) wv[k - bstart] = (uint8_t)best_w;
-      n_match++;
-      mbytes += best_len;
-      msrc += min((uint64_t)best_len, p - best_q);
-      lit = 0;
-      p += best_len;
+// Common prefix of the input at q and at p (q < p), at most limit bytes, by
+// the warp: eight bytes per lane, 256 a round.
+__device__ __forceinline__ uint32_t common_warp(const EncArgs& a, uint64_t q, uint64_t p, uint32_t limit,
+                                                uint32_t lane) {
+  for (uint32_t o = 0; o < limit; o += 256) {
+    const uint32_t at = o + 8 * lane;
+    uint32_t l = 8;  // equal bytes among this lane's
+    if (at + 8 <= limit) {
+      const uint64_t x = ld64_in(a, q + at) ^ ld64_in(a, p + at);
+      if (x) l = (__ffsll((long long)x) - 1) >> 3;
     } else {
-      wv[p - bstart] = 0;
-      lit++;
-      lbytes++;
-      p++;
+      l = 0;
+      while (at + l < limit && a.in[q + at + l] == a.in[p + at + l]) l++;  // at most 7
+    }
+    const uint32_t stop = __ballot_sync(kFull, l < 8);
+    if (stop) {
+      const uint32_t f = __ffs(stop) - 1;
+      return min(limit, o + 8 * f + __shfl_sync(kFull, l, f));
     }
   }
-  uint32_t* t = tk + 4 * nt++;  // the last token: literals only
-  t[0] = lit;
-  t[1] = 0;
-  t[2] = t[3] = 0;
-  a.ntok[b - a.c0] = nt;
-  atomicAdd(a.stats + 0, (unsigned long long)nt);
-  atomicAdd(a.stats + 1, n_match);
-  atomicAdd(a.stats + 2, lbytes);
-  atomicAdd(a.stats + 3, mbytes);
-  atomicAdd(a.stats + 4, msrc);
+  return limit;
+}
+
+// Bits [lo, hi) of word i of a bit map (those of them the word holds).
+__device__ __forceinline__ uint32_t word_mask(uint32_t i, uint32_t lo, uint32_t hi) {
+  uint32_t m = kFull;
+  if (i == lo >> 5) m <<= lo & 31;
+  if (i == (hi - 1) >> 5) m &= kFull >> (31 - ((hi - 1) & 31));
+  return m;
+}
+
+// Whether the external candidate (len 0: none) is taken over the in-block one
+// (len 0: none or refused): the longer one, but a shallower one within
+// max(4, len / 8) bytes of it; on a tie of both, the smaller source, which is
+// the external one.
+__device__ __forceinline__ bool external_wins(uint32_t li, uint32_t wi, uint32_t le, uint32_t we) {
+  if (!li || !le) return le != 0;
+  if (we < wi) return le + max(4u, max(le, li) / 8) >= li;
+  if (we > wi) return le > li + max(4u, le / 8);
+  return le >= li;
+}
+
+// The greedy walk over a block's positions, a warp per block: at the first
+// position with an acceptable candidate a match, literals before it.  A
+// match's resolution wave is 1 + the deepest wave among the bytes of its own
+// block it reads (literals and bytes of earlier blocks are wave 0); deeper
+// than kMaxWave is refused.
+//
+// The walk is a serial chain of decisions, so its latency bounds it.  The
+// warp therefore decides 32 positions at once, a lane each, as if every
+// position before them were a literal: true for the first that accepts, and
+// the others are decided again after it.  The waves are three bit maps in
+// shared memory (bit: wave at least 1, 2, 3), so the wave of a source of at
+// most kCap bytes is two words of each.  Only candidates that extend past the
+// cap, or external sources that run into the block, take the warp as a whole
+// (256 bytes compared a round).  The next 32 positions' candidates load ahead.
+// A thread per block with a byte per wave took 14.5 ms of the 64 MiB FASTQ
+// encode and 45.8 ms of the 11 MiB text one; a warp per block that decided one
+// position at a time 4.2 ms of the text one; this takes 0.93 and 2.1 ms.
+__global__ void __launch_bounds__(32) parse_kernel(EncArgs a) {
+  extern __shared__ uint32_t planes[];  // [3][B / 32 + 1]
+  const uint32_t lane = threadIdx.x;
+  const uint64_t b = a.c0 + blockIdx.x;
+  const uint64_t base = a.c0 << a.log2B, bstart = b << a.log2B;
+  const uint32_t blen = (uint32_t)min(a.n - bstart, (uint64_t)1 << a.log2B);
+  const uint32_t words = (1u << (a.log2B - 5)) + 1;  // one past the block, for two-word reads
+  uint32_t* const w1 = planes;
+  uint32_t* const w2 = w1 + words;
+  uint32_t* const w3 = w2 + words;
+  for (uint32_t i = lane; i < 3 * words; i += 32) planes[i] = 0;
+  __syncwarp();
+  const uint2* cd = a.cand + (bstart - base);
+  uint4* tk = reinterpret_cast<uint4*>(a.tok) + blockIdx.x * (uint64_t)a.tok_cap;
+  auto load = [&](uint32_t i) { return i < blen ? __ldcg(cd + i) : make_uint2(0u, 0u); };
+  uint32_t nt = 0, lit = 0, lbytes = 0, msrc = 0;
+  uint32_t p = 0, wb = 0;  // positions count from the block's start; the window is [wb, wb + 32)
+  uint2 cur = load(lane), nxt = load(32 + lane);
+  while (p < blen) {
+    if (p >= wb + 32) {
+      const uint32_t nb = p & ~31u;
+      cur = nb == wb + 32 ? nxt : load(nb + lane);
+      wb = nb;
+      nxt = load(nb + 32 + lane);
+    }
+    // this lane's position: 0 refused or no candidate, 1 decided, 2 left to the warp
+    const uint32_t pos = wb + lane;
+    const uint32_t li = cur.x & 0xffu, le = (cur.x >> 8) & 0xffu;
+    uint32_t state = 0, len = 0, wave = 1;
+    bool ext = false;
+    if (pos >= p && (li | le)) {
+      if ((max(li, le) == kCap && pos + kCap < blen) || (le && cur.y + le > bstart)) {
+        state = 2;
+      } else {
+        uint32_t l = li;
+        if (li) {
+          const uint32_t q = cur.x >> 16, i = q >> 5, sh = q & 31;
+          const uint32_t m = kFull >> (32 - min(li, pos - q));
+          if (__funnelshift_r(w1[i], w1[i + 1], sh) & m) wave = 2;
+          if (__funnelshift_r(w2[i], w2[i + 1], sh) & m) wave = 3;
+          if (__funnelshift_r(w3[i], w3[i + 1], sh) & m) l = 0;
+        }
+        ext = external_wins(l, wave, le, 1);
+        len = ext ? le : l;
+        if (ext) wave = 1;
+        state = len != 0;
+      }
+    }
+    uint32_t todo = __ballot_sync(kFull, state);
+    const uint32_t slow = __ballot_sync(kFull, state == 2);
+    while (todo) {
+      const uint32_t f = __ffs(todo) - 1, at = wb + f;
+      uint32_t mlen = __shfl_sync(kFull, len | wave << 8 | (uint32_t)ext << 16, f);
+      const uint32_t cx = __shfl_sync(kFull, cur.x, f), cy = __shfl_sync(kFull, cur.y, f);
+      uint32_t mw = (mlen >> 8) & 0xffu;
+      bool mext = mlen >> 16;
+      mlen &= 0xffu;
+      const uint64_t P = bstart + at, qi = bstart + (cx >> 16);
+      if (slow >> f & 1) {
+        const uint32_t room = blen - at;
+        uint32_t fi = cx & 0xffu, fe = (cx >> 8) & 0xffu;
+        if (fi == kCap && room > kCap) fi = kCap + common_warp(a, qi + kCap, P + kCap, room - kCap, lane);
+        if (fe == kCap && room > kCap)
+          fe = span(a, cy, b, kCap + common_warp(a, cy + kCap, P + kCap, room - kCap, lane));
+        // the waves of both sources: lanes 0..15 the in-block one's words, 16..31 the external one's
+        const uint64_t q = lane < 16 ? qi : cy;
+        const uint32_t l = lane < 16 ? fi : fe;
+        const uint32_t lo = q > bstart ? (uint32_t)(q - bstart) : 0u;
+        const uint32_t hi = q + l > bstart ? (uint32_t)min(q + l - bstart, (uint64_t)at) : 0u;
+        uint32_t d1 = 0, d2 = 0, d3 = 0;
+        if (l && lo < hi) {
+          for (uint32_t i = (lo >> 5) + (lane & 15); i <= (hi - 1) >> 5; i += 16) {
+            const uint32_t m = word_mask(i, lo, hi);
+            d1 |= w1[i] & m;
+            d2 |= w2[i] & m;
+            d3 |= w3[i] & m;
+          }
+        }
+        const uint32_t b1 = __ballot_sync(kFull, d1), b2 = __ballot_sync(kFull, d2), b3 = __ballot_sync(kFull, d3);
+        const uint32_t wi = 1 + ((b1 & 0xffffu) != 0) + ((b2 & 0xffffu) != 0), we = 1 + ((b1 >> 16) != 0) + ((b2 >> 16) != 0);
+        if (b3 & 0xffffu) fi = 0;
+        if ((b3 >> 16) || fe < a.min_match) fe = 0;
+        mext = external_wins(fi, wi, fe, we);
+        mlen = mext ? fe : fi;
+        mw = mext ? we : wi;
+        if (!mlen) {  // refused: a literal like the positions before it
+          todo &= todo - 1;
+          continue;
+        }
+      }
+      const uint64_t src = mext ? (uint64_t)cy : qi;
+      const uint32_t end = at + mlen, run = lit + (at - p);
+      if (lane == 0) tk[nt] = make_uint4(run, mlen, (uint32_t)src, (uint32_t)(src >> 32));
+      nt++;
+      __syncwarp();  // every lane has read the maps
+      for (uint32_t i = (at >> 5) + lane; i <= (end - 1) >> 5; i += 32) {
+        const uint32_t m = word_mask(i, at, end);
+        w1[i] |= m;
+        if (mw > 1) w2[i] |= m;
+        if (mw > 2) w3[i] |= m;
+      }
+      __syncwarp();
+      lbytes += run;
+      msrc += (uint32_t)min((uint64_t)mlen, P - src);
+      lit = 0;
+      p = end;
+      break;
+    }
+    if (!todo) {  // literals to the window's end
+      const uint32_t e = min(wb + 32, blen);
+      lit += e - p;
+      p = e;
+    }
+  }
+  if (lane) return;
+  tk[nt] = make_uint4(lit, 0u, 0u, 0u);  // the last token: literals only
+  a.ntok[blockIdx.x] = nt + 1;
+  atomicAdd(a.stats + 0, (unsigned long long)(nt + 1));
+  atomicAdd(a.stats + 1, (unsigned long long)nt);
+  atomicAdd(a.stats + 2, (unsigned long long)(lbytes + lit));
+  atomicAdd(a.stats + 3, (unsigned long long)(blen - lbytes - lit));
+  atomicAdd(a.stats + 4, (unsigned long long)msrc);
 }
 
 // ------------------------------------------------------------ block coder
@@ -775,7 +864,7 @@ __global__ void deps_write_kernel(AsmArgs a, const ace_block_dir* dir, uint8_t* 
 namespace {
 
 struct EncLayout {
-  uint64_t table, level, dir, iv, n_iv, dep_ptr, hdr, prev, lens, q_in, q_ex, wave, tok, ntok, syms, tmp, pay,
+  uint64_t table, level, dir, iv, n_iv, dep_ptr, hdr, prev, cand, tok, ntok, syms, tmp, pay,
       pay_bytes, pay_off, total;
   uint64_t nb, chunk, reserve, arc_bound;
   uint32_t bits, tok_cap, sym_cap, tmp_cap, pay_cap;
@@ -819,14 +908,8 @@ ace_status enc_layout(uint64_t n, const ace_encode_params* p, EncLayout* L) {
   o = a256(o + 4 * (nb + 1));
   L->prev = o;
   o = a256(o + 2 * cb);
-  L->lens = o;
-  o = a256(o + 2 * cb);
-  L->q_in = o;
+  L->cand = o;
   o = a256(o + 8 * cb);
-  L->q_ex = o;
-  o = a256(o + 8 * cb);
-  L->wave = o;
-  o = a256(o + cb);
   L->tok = o;
   o = a256(o + 16ull * L->tok_cap * C);
   L->ntok = o;
@@ -899,10 +982,7 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   e.table = reinterpret_cast<unsigned long long*>(base + L.table);
   e.level = reinterpret_cast<uint32_t*>(base + L.level);
   e.prev = reinterpret_cast<uint16_t*>(base + L.prev);
-  e.lens = reinterpret_cast<uint16_t*>(base + L.lens);
-  e.q_in = reinterpret_cast<uint64_t*>(base + L.q_in);
-  e.q_ex = reinterpret_cast<uint64_t*>(base + L.q_ex);
-  e.wave = base + L.wave;
+  e.cand = reinterpret_cast<uint2*>(base + L.cand);
   e.tok = reinterpret_cast<uint32_t*>(base + L.tok);
   e.tok_cap = L.tok_cap;
   e.ntok = reinterpret_cast<uint32_t*>(base + L.ntok);
@@ -954,7 +1034,7 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
                    kChainWarps * (4u << kHashBits4), s>>>(e);
     const uint64_t npos = std::min(n, pc.c1 * B) - pc.c0 * B;
     candidate_kernel<<<(uint32_t)std::min<uint64_t>((npos + 255) / 256, 152ull * 64), 256, 0, s>>>(e);
-    parse_kernel<<<(uint32_t)((cn + 31) / 32), 32, 0, s>>>(e);
+    parse_kernel<<<(uint32_t)cn, 32, 3 * (B / 8 + 4), s>>>(e);  // at most 24.1 KB of bit maps
     ca.e = e;
     code_kernel<<<(uint32_t)((cn + 7) / 8), 256, 0, s>>>(ca);
     pa.c0 = pc.c0;
