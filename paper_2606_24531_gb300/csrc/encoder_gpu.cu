@@ -5,10 +5,10 @@
 //
 // Match layer (Section 2: greedy parse with a global match search, absolute
 // back-references): candidates are found for every position at once, a
-// thread per position -- the earliest earlier occurrence of the 16-byte keys
+// CTA per block -- the earliest earlier occurrence of the 16-byte keys
 // around it (a table over the whole input, built with atomic minima) and
-// the most recent repeats inside its block (hash chains built a warp per
-// block) -- then one thread per block walks its positions greedily, taking
+// the most recent repeats inside its block (hash chains in shared memory)
+// -- then a warp per block walks its positions greedily, taking
 // at each the longest candidate allowed there.  Blocks are parsed in
 // windows of 64 that take no sources from each other; the first three
 // windows are parsed one after another, and every later block takes its
@@ -48,7 +48,6 @@ constexpr uint32_t kHead = kWin * kHeadWins;
 constexpr uint32_t kMaxWave = 3;     // deepest in-block resolution wave taken
 constexpr uint32_t kCap = 32;        // match lengths measured by the candidate search (extended later)
 constexpr uint32_t kHashBits4 = 12;  // in-block chains: hash of 4 bytes
-constexpr uint64_t kEmpty = ~0ull;
 constexpr uint32_t kMaxChain = 64;
 
 __host__ __device__ inline uint64_t align16(uint64_t v) { return (v + 15) & ~15ull; }
@@ -60,16 +59,11 @@ __device__ __forceinline__ uint64_t ld64u(const uint8_t* p) {
   return v;
 }
 
-__device__ __forceinline__ uint32_t ld32u(const uint8_t* p) {
-  return (uint32_t)p[0] | ((uint32_t)p[1] << 8) | ((uint32_t)p[2] << 16) | ((uint32_t)p[3] << 24);
-}
-
-__device__ __forceinline__ uint32_t hash_key(const uint8_t* p, uint32_t bits) {
-  const uint64_t a = ld64u(p) * 0x9E3779B97F4A7C15ull, b = ld64u(p + 8) * 0xC2B2AE3D27D4EB4Full;
+// The table's slot of a 16-byte key (its two halves, little endian).
+__device__ __forceinline__ uint32_t hash_words(uint64_t lo, uint64_t hi, uint32_t bits) {
+  const uint64_t a = lo * 0x9E3779B97F4A7C15ull, b = hi * 0xC2B2AE3D27D4EB4Full;
   return (uint32_t)(((a ^ ((b << 31) | (b >> 33))) * 0x165667B19E3779F9ull) >> (64 - bits));
 }
-
-__device__ __forceinline__ uint32_t hash4(const uint8_t* p) { return (ld32u(p) * 2654435761u) >> (32 - kHashBits4); }
 
 // Common prefix of a and b (a precedes b), at most limit bytes.
 __device__ __forceinline__ uint32_t common(const uint8_t* a, const uint8_t* b, uint32_t limit) {
@@ -92,7 +86,7 @@ struct EncArgs {
   // the blocks of the current launch: [c0, c1), window start ws (blocks
   // below it, all of level below 3, may be sources)
   uint64_t c0, c1, ws;
-  uint16_t* prev;     // per position of the chunk: distance to the previous one with the same 4-byte hash (0: none)
+  uint32_t* entries;  // per position: the candidate search's links and hashes (64 KiB blocks; smaller ones: shared memory)
   uint2* cand;        // per position: x = in-block candidate length (bits 0..7), external length (8..15), both
                       // capped at kCap, and the in-block source as an offset in the block (16..31); y = the external
                       // source (below kHead blocks, so below 2^24)
@@ -110,37 +104,7 @@ __global__ void table_kernel(EncArgs a) {
   const uint64_t nkeys = a.n >= kKey ? (a.n - kKey) / kStride + 1 : 0;
   for (uint64_t k = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; k < nkeys; k += (uint64_t)gridDim.x * blockDim.x) {
     const uint64_t q = k * kStride;
-    atomicMin(a.table + hash_key(a.in + q, a.bits), (unsigned long long)q);
-  }
-}
-
-// ------------------------------------------------------- in-block chains
-
-// A warp per block: positions in order, 32 at a time; a position's link is
-// the nearest earlier one of the block with the same 4-byte hash (found
-// among the lanes with __match_any_sync, else in the warp's bucket heads).
-__global__ void chain_kernel(EncArgs a) {
-  extern __shared__ uint32_t heads[];  // [warps][4096]
-  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t* head = heads + (wid << kHashBits4);
-  const uint64_t b = a.c0 + blockIdx.x * (blockDim.x >> 5) + wid;
-  if (b >= a.c1) return;
-  for (uint32_t i = lane; i < (1u << kHashBits4); i += 32) head[i] = 0xffffffffu;
-  __syncwarp();
-  const uint64_t B = 1ull << a.log2B, bstart = b << a.log2B, base = a.c0 << a.log2B;
-  const uint32_t blen = (uint32_t)min(B, a.n - bstart);
-  for (uint32_t c = 0; c < blen; c += 32) {
-    const uint32_t p = c + lane;
-    const bool valid = p + 4 <= blen;
-    const uint32_t h = valid ? hash4(a.in + bstart + p) : (1u << kHashBits4) + lane;  // invalid lanes alone
-    const uint32_t grp = __match_any_sync(kFull, h);
-    const uint32_t below = grp & lanemask_lt();
-    uint32_t pp = 0xffffffffu;
-    if (valid) pp = below ? c + (31 - __clz(below)) : head[h];
-    __syncwarp();
-    if (valid && !(grp >> lane >> 1)) head[h] = p;  // the group's last lane is the new head
-    __syncwarp();
-    if (p < blen) a.prev[bstart - base + p] = (valid && pp != 0xffffffffu) ? (uint16_t)(p - pp) : (uint16_t)0;
+    atomicMin(a.table + hash_words(ld64u(a.in + q), ld64u(a.in + q + 8), a.bits), (unsigned long long)q);
   }
 }
 
@@ -161,57 +125,291 @@ __device__ __forceinline__ uint32_t span(const EncArgs& a, uint64_t q, uint64_t 
   return got;
 }
 
-// A thread per position of the launch's blocks: the best in-block candidate
-// (its chain, most recent first, max_chain deep) and the best external one
-// (earliest occurrences of the keys at p .. p + 7, shifted back), each the
-// longest measured up to kCap bytes (ties: the smaller source).
-__global__ void candidate_kernel(EncArgs a) {
-  const uint64_t base = a.c0 << a.log2B, end = min(a.n, a.c1 << a.log2B);
-  for (uint64_t p = base + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < end;
-       p += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t b = p >> a.log2B, bstart = b << a.log2B;
-    const uint64_t bend = min((uint64_t)a.n, (uint64_t)(bstart + (1ull << a.log2B)));
-    const uint32_t room = (uint32_t)(bend - p), lim = min(room, kCap);
-    uint32_t li = 0, le = 0;
-    uint64_t qi = 0, qe = 0;
-    if (room >= a.min_match) {
-      uint32_t d = a.prev[p - base];
-      uint64_t q = p;
-      for (uint32_t depth = 0; d && depth < a.max_chain; depth++) {
-        if (d > q - bstart) break;  // links stay inside the block
-        q -= d;
-        const uint32_t l = common(a.in + q, a.in + p, lim);
-        if (l > li) {
-          li = l;
-          qi = q;
-        }
-        d = a.prev[q - base];
-      }
-      for (uint32_t j = 0; j < kStride; j++) {
-        const uint64_t x = p + j;
-        if (x + kKey > a.n) break;
-        const unsigned long long qq = a.table[hash_key(a.in + x, a.bits)];
-        if (qq == kEmpty || qq < j) continue;
-        q = qq - j;
-        if (q >= p) continue;
-        uint32_t l = common(a.in + q, a.in + p, lim);
-        if (q >= bstart) {  // an earlier occurrence inside the block
-          if (l > li || (l == li && q < qi)) {
-            li = l;
-            qi = q;
-          }
-          continue;
-        }
-        l = span(a, q, b, l);
-        if (l > le || (l == le && q < qe)) {
-          le = l;
-          qe = q;
-        }
+// The 32-bit word at byte o of a staged block (any alignment).
+__device__ __forceinline__ uint32_t word_at(const uint32_t* sb, uint32_t o) {
+  return __funnelshift_r(sb[o >> 2], sb[(o >> 2) + 1], 8 * (o & 3));
+}
+
+// Launch shape of the candidate search for a block size: threads of a CTA,
+// the segments whose links warps build side by side, and whether the entries
+// fit in shared memory beside the block (all but 64 KiB blocks).  16 KiB
+// blocks: 112 KiB, so two CTAs of 16 warps fit an SM.
+struct CandShape {
+  uint32_t threads, segs;
+  bool shared_entries;
+  size_t smem;
+};
+constexpr uint32_t kPadBytes = 64;  // staged past the block: keys and compares read ahead
+
+// One warp's arrays of the candidate walk (over the bucket heads, which are
+// done with by then).
+struct CandWarp {
+  uint32_t key[64];       // the keys of the window's 32 positions and of those after it
+  uint8_t found[64];      // those of them the table holds a usable position for
+  uint32_t ext[32];       // per position, the best external source: length << 24 | (2^24 - 1 - source)
+  uint32_t own[32];       // the best of the keys' sources in the block: length << 16 | (2^16 - 1 - offset)
+};
+
+__host__ __device__ inline CandShape cand_shape(uint32_t log2B) {
+  CandShape c;
+  c.threads = log2B >= 12 ? 512 : log2B >= 10 ? 128 : 64;
+  c.segs = log2B >= 10 ? 4 : 1;
+  c.shared_entries = log2B < 16;
+  const size_t heads = (size_t)c.segs * (2u << kHashBits4), warps = c.threads / 32 * sizeof(CandWarp);
+  c.smem = ((size_t)1 << log2B) + kPadBytes + (c.shared_entries ? (size_t)4 << log2B : 0) +
+           (heads > warps ? heads : warps);
+  return c;
+}
+
+constexpr uint32_t kNoKey = ~0u;
+constexpr uint32_t kCandParts = 4;  // CTAs a block's positions are split over, at most
+
+// A CTA per block, or (gridDim.y > 1) per part of its positions: for every
+// position the best in-block candidate (its chain
+// of earlier positions with the same 4-byte hash, most recent first,
+// max_chain deep) and the best external one (earliest occurrences of the keys
+// at p .. p + 7, shifted back), each the longest measured up to kCap bytes
+// (ties: the more recent in the chain; among keys' sources the smaller one).
+//
+// The block is staged in shared memory, where every link and every in-block
+// compare then reads.  Links: a position's is the nearest earlier one with its
+// hash; warps build them for a segment of the block each (lanes grouped by
+// __match_any_sync, else the segment's bucket heads), and a segment's firsts
+// are looked up in the heads of the segments before.  An entry packs the link
+// with 16 bits of a hash of as many of the position's first bytes as a match
+// must have, so a chain step is one shared load, and a candidate that cannot
+// reach min_match is nearly always dropped there.  Each key is looked up once,
+// by the lane of its position, and shared with the seven positions before;
+// positions a match may not read count as not found, and the pairs of a found
+// key and a position before it are dealt evenly to the lanes.  Bound by issue: about 940 warp instructions
+// per 32 positions of FASTQ.  Byte loads from global memory, a launch for the
+// links and eight lookups a position took 12.4 + 1.5 ms of the 64 MiB FASTQ
+// encode; this takes 2.8 ms.
+template <bool SHARED>
+__global__ void __launch_bounds__(512, 2) candidate_kernel(EncArgs a) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+  const uint32_t B = 1u << a.log2B;
+  const CandShape shape = cand_shape(a.log2B);
+  const uint64_t b = a.c0 + blockIdx.x, bstart = b << a.log2B;
+  const uint32_t blen = (uint32_t)min(a.n - bstart, (uint64_t)B);
+  const uint32_t* sb = reinterpret_cast<const uint32_t*>(smem);
+  uint32_t* ent = SHARED ? reinterpret_cast<uint32_t*>(smem + B + kPadBytes) : a.entries + (blockIdx.x * (uint64_t)gridDim.y + blockIdx.y) * B;
+  uint8_t* after = smem + B + kPadBytes + (SHARED ? 4 * (size_t)B : 0);
+  uint16_t* heads = reinterpret_cast<uint16_t*>(after);  // [segs][2^kHashBits4]
+  CandWarp& w = reinterpret_cast<CandWarp*>(after)[wid];
+  const uint32_t mm = a.min_match;
+
+  // the block and the bytes after it (zero past the input)
+  const uint64_t avail = a.n - bstart;
+  if ((reinterpret_cast<uintptr_t>(a.in) & 15) == 0) {
+    for (uint32_t o = 16 * tid; o < B + kPadBytes; o += 16 * nt) {
+      if (o + 16 <= avail) {
+        *reinterpret_cast<uint4*>(smem + o) = __ldg(reinterpret_cast<const uint4*>(a.in + bstart + o));
+      } else {
+        for (uint32_t k = o; k < o + 16; k++) smem[k] = k < avail ? a.in[bstart + k] : (uint8_t)0;
       }
     }
-    if (li < a.min_match) li = 0;
-    if (le < a.min_match) le = 0;
-    a.cand[p - base] = make_uint2(li | (le << 8) | ((uint32_t)(qi - bstart) << 16), (uint32_t)qe);
+  } else {
+    for (uint32_t k = tid; k < B + kPadBytes; k += nt) smem[k] = k < avail ? a.in[bstart + k] : (uint8_t)0;
+  }
+  for (uint32_t k = tid; k < shape.segs << (kHashBits4 - 1); k += nt) reinterpret_cast<uint32_t*>(heads)[k] = ~0u;
+  __syncthreads();
+
+  // entries: link distance (0: none) in the low half, the hash in the high half
+  uint16_t* ent16 = reinterpret_cast<uint16_t*>(ent);
+  const uint32_t seg = B / shape.segs;
+  auto bucket = [&](uint32_t p) { return (word_at(sb, p) * 2654435761u) >> (32 - kHashBits4); };
+  if (wid < shape.segs) {
+    uint16_t* head = heads + (wid << kHashBits4);
+    const uint32_t end = min((wid + 1) * seg, blen);
+    uint32_t hn = bucket(wid * seg + lane);
+    for (uint32_t c = wid * seg; c < end; c += 32) {
+      const uint32_t p = c + lane;
+      const bool valid = p + 4 <= blen;
+      const uint32_t h = valid ? hn : (1u << kHashBits4) + lane;  // invalid lanes alone
+      hn = bucket(min(p + 32, B));  // the next round's, beside this one's chain
+      const uint32_t grp = __match_any_sync(kFull, h);
+      const uint32_t below = grp & lanemask_lt();
+      uint32_t pp = 0xffffu;  // no position with four bytes left is 0xffff
+      if (valid) pp = below ? c + (31 - __clz(below)) : head[h];
+      __syncwarp();
+      if (valid && !(grp >> lane >> 1)) head[h] = (uint16_t)p;  // the group's last lane is the new head
+      __syncwarp();
+      if (p < blen) ent16[2 * p] = pp != 0xffffu ? (uint16_t)(p - pp) : (uint16_t)0;
+    }
+  }
+  // (a CTA of few warps has the linking ones hash too)
+  const uint32_t hw = nw > shape.segs ? nw - shape.segs : nw, hid = nw > shape.segs ? wid - shape.segs : wid;
+  if (hid < hw)
+    for (uint32_t p = 32 * hid + lane; p < blen; p += 32 * hw) {
+      uint32_t x = word_at(sb, p) * 0x85EBCA6Bu;
+      if (mm >= 8) x = ((x >> 15) ^ x ^ word_at(sb, p + 4)) * 0x85EBCA6Bu;
+      if (mm >= 12) x = ((x >> 15) ^ x ^ word_at(sb, p + 8)) * 0x85EBCA6Bu;
+      if (mm >= 16) x = ((x >> 15) ^ x ^ word_at(sb, p + 12)) * 0x85EBCA6Bu;
+      ent16[2 * p + 1] = (uint16_t)((x ^ (x >> 13)) >> 12);
+    }
+  __syncthreads();
+  for (uint32_t p = seg + tid; p + 4 <= blen; p += nt) {  // the segments' firsts
+    if (ent16[2 * p]) continue;
+    const uint32_t h = bucket(p);
+    for (uint32_t k = p / seg; k-- > 0;) {
+      const uint32_t v = heads[(k << kHashBits4) + h];
+      if (v != 0xffffu) {
+        ent16[2 * p] = (uint16_t)(p - v);
+        break;
+      }
+    }
+  }
+  __syncthreads();
+
+  // the table's position for the key at p: in this block as an offset with the
+  // top bit set, in a block that may be a source (or up to 7 bytes past those,
+  // for the shift back) as it is
+  const uint64_t wend = a.ws << a.log2B;
+  auto key_of = [&](uint32_t p) -> uint32_t {
+    if (p + kKey > avail) return kNoKey;
+    const uint32_t* t = sb + (p >> 2);
+    const uint32_t sh = 8 * (p & 3), t1 = t[1], t2 = t[2], t3 = t[3];
+    const uint32_t x0 = __funnelshift_r(t[0], t1, sh), x1 = __funnelshift_r(t1, t2, sh);
+    const uint32_t x2 = __funnelshift_r(t2, t3, sh), x3 = __funnelshift_r(t3, t[4], sh);
+    const unsigned long long q =
+        __ldg(a.table + hash_words((uint64_t)x1 << 32 | x0, (uint64_t)x3 << 32 | x2, a.bits));
+    if (q >= bstart) return q - bstart < 2 * (uint64_t)B ? 0x80000000u | (uint32_t)(q - bstart) : kNoKey;
+    return q < wend + kStride ? (uint32_t)q : kNoKey;
+  };
+  // common prefix of q and p in the block, at most kCap (never past the staged bytes)
+  auto common_in = [&](uint32_t q, uint32_t p) -> uint32_t {
+    const uint32_t *s = sb + (q >> 2), *t = sb + (p >> 2);
+    const uint32_t sh = 8 * (q & 3), th = 8 * (p & 3);
+    uint32_t u = s[0], v = t[0];
+#pragma unroll
+    for (uint32_t k = 0; k < 8; k++) {
+      const uint32_t u2 = s[k + 1], v2 = t[k + 1];
+      const uint32_t x = __funnelshift_r(u, u2, sh) ^ __funnelshift_r(v, v2, th);
+      if (x) return 4 * k + ((__ffs(x) - 1) >> 3);
+      u = u2;
+      v = v2;
+    }
+    return kCap;
+  };
+  // common prefix of the input at q and the block's p, at most kCap
+  auto common_ex = [&](uint32_t q, uint32_t p, uint32_t lim) -> uint32_t {
+    const uintptr_t A = reinterpret_cast<uintptr_t>(a.in + q);
+    // the aligned words around the source, where they lie in the input
+    if (q < 4 || (uint64_t)q + 40 > a.n) return common(a.in + q, a.in + bstart + p, lim);
+    const uint32_t* g = reinterpret_cast<const uint32_t*>(a.in + q - (A & 3));
+    const uint32_t sh = 8 * (uint32_t)(A & 3);
+    const uint32_t g0 = __ldg(g), g1 = __ldg(g + 1), g2 = __ldg(g + 2);
+    const uint32_t x0 = __funnelshift_r(g0, g1, sh) ^ word_at(sb, p);
+    const uint32_t x1 = __funnelshift_r(g1, g2, sh) ^ word_at(sb, p + 4);
+    if (x0 | x1) return x0 ? (__ffs(x0) - 1) >> 3 : 4 + ((__ffs(x1) - 1) >> 3);
+    uint32_t r[7] = {g2}, l = kCap;
+#pragma unroll
+    for (uint32_t i = 1; i < 7; i++) r[i] = __ldg(g + 2 + i);
+#pragma unroll
+    for (uint32_t i = 6; i-- > 0;) {
+      const uint32_t x = __funnelshift_r(r[i], r[i + 1], sh) ^ word_at(sb, p + 8 + 4 * i);
+      if (x) l = 8 + 4 * i + ((__ffs(x) - 1) >> 3);
+    }
+    return l;
+  };
+  // positions of a warp: of the CTA's part of the block, a multiple of 32
+  const uint32_t per = max(B / (nw * gridDim.y), 32u), first = (blockIdx.y * nw + wid) * per;
+  uint2* out = a.cand + (uint64_t)blockIdx.x * B;
+  uint32_t next = first < blen ? key_of(first + lane) : kNoKey;
+  for (uint32_t c = first; c < min(first + per, blen); c += 32) {
+    const uint32_t p = c + lane;
+    __syncwarp();
+    w.key[lane] = next;
+    w.ext[lane] = w.own[lane] = 0;
+    next = key_of(p + 32);  // in flight during the chain walk
+    uint32_t li = 0, qi = 0;
+    const uint32_t lim = p < blen ? min(blen - p, kCap) : 0u;
+    // one chain step for the whole warp at a time, so its lanes stay together
+    uint32_t e = lim >= mm ? ent[p] : 0u, q = p;
+    const uint32_t mine = e >> 16;
+    uint32_t tail = 0;  // the position's bytes li - 3 .. li: a longer candidate has them too
+    uint32_t P[kCap / 4];
+    {
+      const uint32_t* t = sb + (min(p, B - 1) >> 2);
+      uint32_t v = t[0];
+#pragma unroll
+      for (uint32_t k = 0; k < kCap / 4; k++) {
+        const uint32_t v2 = t[k + 1];
+        P[k] = __funnelshift_r(v, v2, 8 * (p & 3));
+        v = v2;
+      }
+    }
+    for (uint32_t depth = 0; depth < a.max_chain && __any_sync(kFull, e & 0xffffu); depth++) {
+      if (!(e & 0xffffu)) continue;
+      q -= e & 0xffffu;
+      e = ent[q];
+      if (e >> 16 != mine || (li && word_at(sb, q + li - 3) != tail)) continue;
+      // common prefix with p: eight bytes, then word by word
+      const uint32_t* t = sb + (q >> 2);
+      const uint32_t sh = 8 * (q & 3);
+      uint32_t v = t[2], l = kCap;
+      const uint32_t x0 = __funnelshift_r(t[0], t[1], sh) ^ P[0], x1 = __funnelshift_r(t[1], v, sh) ^ P[1];
+      if (x0 | x1) {
+        l = x0 ? (__ffs(x0) - 1) >> 3 : 4 + ((__ffs(x1) - 1) >> 3);
+      } else {
+#pragma unroll
+        for (uint32_t k = 2; k < kCap / 4; k++) {
+          const uint32_t v2 = t[k + 1], x = __funnelshift_r(v, v2, sh) ^ P[k];
+          if (x) {
+            l = 4 * k + ((__ffs(x) - 1) >> 3);
+            break;
+          }
+          v = v2;
+        }
+      }
+      l = min(l, lim);
+      if (l >= mm && l > li) {
+        li = l;
+        qi = q;
+        if (l == lim) e = 0;  // none is longer
+        else tail = word_at(sb, p + l - 3);
+      }
+    }
+    if (lane < kStride - 1) w.key[32 + lane] = next;
+    __syncwarp();
+    // the keys' sources: every key found serves the eight positions up to its
+    // own, (key, shift) pairs dealt to the lanes 32 at a time
+    const uint32_t f0 = __ballot_sync(kFull, w.key[lane] != kNoKey);
+    const uint32_t f1 = __ballot_sync(kFull, lane < kStride - 1 && next != kNoKey);
+    const uint32_t n = __popc(f0) + __popc(f1);
+    if (f0 >> lane & 1) w.found[__popc(f0 & lanemask_lt())] = (uint8_t)lane;
+    if (f1 >> lane & 1) w.found[__popc(f0) + __popc(f1 & lanemask_lt())] = (uint8_t)(32 + lane);
+    __syncwarp();
+    for (uint32_t it = lane; it < kStride * n; it += 32) {
+      const uint32_t k = w.found[it / kStride], j = it % kStride, at = k - j, pq = c + at;
+      if (at >= 32 || pq >= blen) continue;  // (k < j too)
+      const uint32_t room = min(blen - pq, kCap);
+      const uint32_t t = w.key[k], q0 = t & 0x7fffffffu;
+      if (room < mm) continue;
+      if (t >> 31 && q0 >= j) {  // an earlier occurrence inside the block
+        const uint32_t s = q0 - j;
+        if (s >= pq || (ent[s] ^ ent[pq]) >> 16) continue;
+        const uint32_t l = min(common_in(s, pq), room);
+        if (l >= mm) atomicMax(&w.own[at], l << 16 | (0xffffu - s));
+      } else {
+        const uint64_t q64 = (t >> 31 ? bstart : 0) + q0;
+        // in a block that may be a source (its length beyond it: span)
+        if (q64 < j || q64 - j >= wend || __ldg(a.level + ((q64 - j) >> a.log2B)) >= 3) continue;
+        const uint32_t s = (uint32_t)(q64 - j);
+        uint32_t l = min(common_ex(s, pq, room), room);
+        if (l >= mm) l = span(a, s, b, l);
+        if (l >= mm) atomicMax(&w.ext[at], l << 24 | (0xffffffu - s));
+      }
+    }
+    __syncwarp();
+    const uint32_t o = w.own[lane], x = w.ext[lane];
+    if (o >> 16 > li || (li && o >> 16 == li && 0xffffu - (o & 0xffffu) < qi)) {
+      li = o >> 16;
+      qi = 0xffffu - (o & 0xffffu);
+    }
+    if (p < blen) out[p] = make_uint2(li | (x >> 24 << 8) | (qi << 16), 0xffffffu - (x & 0xffffffu));
   }
 }
 
@@ -864,9 +1062,9 @@ __global__ void deps_write_kernel(AsmArgs a, const ace_block_dir* dir, uint8_t* 
 namespace {
 
 struct EncLayout {
-  uint64_t table, level, dir, iv, n_iv, dep_ptr, hdr, prev, cand, tok, ntok, syms, tmp, pay,
+  uint64_t table, level, dir, iv, n_iv, dep_ptr, hdr, entries, cand, tok, ntok, syms, tmp, pay,
       pay_bytes, pay_off, total;
-  uint64_t nb, chunk, reserve, arc_bound;
+  uint64_t nb, chunk, reserve, arc_bound, entry_blocks;
   uint32_t bits, tok_cap, sym_cap, tmp_cap, pay_cap;
 };
 
@@ -906,8 +1104,10 @@ ace_status enc_layout(uint64_t n, const ace_encode_params* p, EncLayout* L) {
   o = a256(o + 4 * nb);
   L->dep_ptr = o;
   o = a256(o + 4 * (nb + 1));
-  L->prev = o;
-  o = a256(o + 2 * cb);
+  L->entries = o;
+  // (an array per part where a launch's blocks are split)
+  L->entry_blocks = cand_shape(p->log2_block).shared_entries ? 0 : std::max<uint64_t>(C, 2 * std::min<uint64_t>(C, kWin));
+  o = a256(o + 4 * B * L->entry_blocks);
   L->cand = o;
   o = a256(o + 8 * cb);
   L->tok = o;
@@ -981,7 +1181,7 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   e.bits = L.bits;
   e.table = reinterpret_cast<unsigned long long*>(base + L.table);
   e.level = reinterpret_cast<uint32_t*>(base + L.level);
-  e.prev = reinterpret_cast<uint16_t*>(base + L.prev);
+  e.entries = reinterpret_cast<uint32_t*>(base + L.entries);
   e.cand = reinterpret_cast<uint2*>(base + L.cand);
   e.tok = reinterpret_cast<uint32_t*>(base + L.tok);
   e.tok_cap = L.tok_cap;
@@ -1024,16 +1224,28 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
     for (uint64_t c = w0; c < std::min(head, w0 + kWin); c += L.chunk)
       pieces.push_back({c, std::min({head, w0 + kWin, c + L.chunk}), w0});
   for (uint64_t c = head; c < nb; c += L.chunk) pieces.push_back({c, std::min(nb, c + L.chunk), head});
-  constexpr uint32_t kChainWarps = 2;  // 16 KiB of bucket heads each: within the default shared memory
+  const CandShape shape = cand_shape(params->log2_block);
+  int dev = 0, num_sms = 0;
+  ENC_TRY(cudaGetDevice(&dev));
+  ENC_TRY(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
+  for (auto k : {candidate_kernel<true>, candidate_kernel<false>})  // the most either asks for, whatever the block size
+    ENC_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)std::max(cand_shape(15).smem, cand_shape(16).smem)));
   for (const Piece& pc : pieces) {
     e.c0 = pc.c0;
     e.c1 = pc.c1;
     e.ws = pc.ws;
     const uint64_t cn = pc.c1 - pc.c0;
-    chain_kernel<<<(uint32_t)((cn + kChainWarps - 1) / kChainWarps), 32 * kChainWarps,
-                   kChainWarps * (4u << kHashBits4), s>>>(e);
-    const uint64_t npos = std::min(n, pc.c1 * B) - pc.c0 * B;
-    candidate_kernel<<<(uint32_t)std::min<uint64_t>((npos + 255) / 256, 152ull * 64), 256, 0, s>>>(e);
+    // a launch of few blocks (the first windows) splits each over CTAs until
+    // there are two per SM; every part links the whole block again, so no
+    // further than needed (the candidate launches of 11 MiB of text, three of
+    // their four over 64 blocks: 1.29 ms split, 1.85 unsplit)
+    uint32_t parts = 1;
+    while (parts < kCandParts && cn * parts < 2ull * num_sms && B / shape.threads >= 2 * parts &&
+           (shape.shared_entries || 2 * cn * parts <= L.entry_blocks))
+      parts *= 2;
+    (shape.shared_entries ? candidate_kernel<true> : candidate_kernel<false>)<<<dim3((uint32_t)cn, parts), shape.threads,
+                                                                                shape.smem, s>>>(e);
     parse_kernel<<<(uint32_t)cn, 32, 3 * (B / 8 + 4), s>>>(e);  // at most 24.1 KB of bit maps
     ca.e = e;
     code_kernel<<<(uint32_t)((cn + 7) / 8), 256, 0, s>>>(ca);
