@@ -18,7 +18,7 @@
 // wave k + 1); candidates deeper than wave 3 are refused, and an external
 // candidate nearly as long as the best is preferred.
 // Entropy layer (Section 3): each block's literal, length and offset
-// streams are rANS-coded, a warp per block, with 32 interleaved states,
+// streams are rANS-coded, a warp per stream, with 32 interleaved states,
 // 12-bit frequencies quantised as the host encoder does, byte
 // renormalisation; with the adaptive option a stream rANS would not shrink
 // is stored (Section 6.1).
@@ -617,8 +617,7 @@ struct CodeArgs {
   EncArgs e;
   uint8_t* syms;       // per chunk block: sym_cap bytes, the three streams' symbols one after another
   uint32_t sym_cap;
-  uint32_t* tmp;       // per chunk block: one word per symbol of the longest stream (pushes of the encode)
-  uint32_t tmp_cap;
+  uint8_t* tmp;        // per chunk block: 2 sym_cap bytes, two for each symbol's pushes
   uint8_t* pay;        // per chunk block: pay_cap bytes, the block's payload
   uint32_t pay_cap;
   ace_block_dir* dir;  // per block of the archive (stream offsets relative to the block's payload for now)
@@ -632,10 +631,10 @@ constexpr uint32_t kIvCap = kHead / 2;  // runs of set bits in a kHead-bit map
 // Frequencies of a stream as the host encoder quantises them: f_s =
 // max(1, floor(n_s 4096 / n)); a shortfall goes to the most frequent symbol
 // (lowest on ties), an excess is taken one at a time from the largest
-// frequency above 1 (lowest on ties).  cnt: the histogram in shared memory;
-// leaves f | c << 16 per symbol in fc.  Lane l holds symbols 8l .. 8l + 7.
-__device__ void quantise_warp(const uint32_t* cnt, uint32_t n, uint32_t* fc, uint32_t lane) {
-  uint32_t f[8], sum = 0, best = 0, most = 0;
+// frequency above 1 (lowest on ties).  cnt: the histogram in shared memory.
+// Lane l holds symbols 8l .. 8l + 7: their frequencies in f.
+__device__ void quantise_warp(const uint32_t* cnt, uint32_t n, uint32_t (&f)[8], uint32_t lane) {
+  uint32_t sum = 0, best = 0, most = 0;
 #pragma unroll
   for (int j = 0; j < 8; j++) {
     const uint32_t s = 8 * lane + j, c = cnt[s];
@@ -685,235 +684,300 @@ __device__ void quantise_warp(const uint32_t* cnt, uint32_t n, uint32_t* fc, uin
     }
     sum--;
   }
-  uint32_t tot = 0;
+}
+
+// ceil(2^(31 + l) / f), l = ceil(log2 f), for f = 1 .. 4096: for x < 2^31,
+// floor(x / f) = floor(2 x m / 2^32) >> l (Granlund and Montgomery, "Division
+// by invariant integers using multiplication", 1994: the rounded-up multiplier
+// exceeds 2^(31 + l) / f by less than 2^l / f).
+struct Reciprocals {
+  uint32_t m[ACE_SCALE + 1];
+  constexpr Reciprocals() : m() {
+    for (uint32_t f = 1, l = 0; f <= ACE_SCALE; f++) {
+      while ((1u << l) < f) l++;
+      m[f] = (uint32_t)(((1ull << (31 + l)) + f - 1) / f);
+    }
+  }
+};
+__device__ const Reciprocals kRecip = Reciprocals();
+
+// One symbol as the coder needs it: x the multiplier, y = f | c << 13 | l << 25.
+__device__ __forceinline__ uint2 coder_entry(uint32_t f, uint32_t c) {
+  return f ? make_uint2(kRecip.m[f], f | c << 13 | (32 - __clz(f - 1)) << 25) : make_uint2(0u, 0u);
+}
+
+// n bytes from src (any alignment, with the aligned words around it readable)
+// to dst (16-byte aligned), zeros up to the next multiple of 16; by a warp.
+__device__ __forceinline__ void copy_padded(uint8_t* dst, const uint8_t* src, uint32_t n, uint32_t lane) {
+  const uint32_t off = (uint32_t)(reinterpret_cast<uintptr_t>(src) & 3), sh = 8 * off;
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(src - off);
+  for (uint32_t i = lane; i < ((n + 15) & ~15u) / 4; i += 32) {
+    uint32_t v = 0;
+    if (4 * i < n) {
+      v = __funnelshift_r(w[i], 4 * i + 4 - off < n ? w[i + 1] : 0u, sh);
+      if (4 * i + 4 > n) v &= (1u << 8 * (n - 4 * i)) - 1;
+    }
+    reinterpret_cast<uint32_t*>(dst)[i] = v;
+  }
+}
+
+// A stream between its two halves: coded, not yet placed.
+struct Coded {
+  uint32_t x;        // this lane's final state
+  uint32_t f[8];     // frequencies of symbols 8 lane .. 8 lane + 7
+  uint32_t pushes, present, head, bytes, mode;
+};
+
+// One stream of n symbols, by a warp: frequencies from the histogram, then the
+// encode from the last symbol to the first, symbol i on state i mod 32,
+// pushing a state's low byte while x >= 2^19 f_s, then x <- (x / f_s) 4096 +
+// x mod f_s + c_s.  The pushes go straight to their places before end
+// (backwards: a symbol's bytes before those of later ones, its last push
+// first), which is the byte order the decoder reads.  The chain from round to
+// round is a compare, a shift, a multiply-high and a multiply-add; the
+// symbols and their entries load ahead of it.
+__device__ Coded code_stream_warp(const uint8_t* sym, uint32_t n, uint8_t* end, const uint32_t* cnt, uint2* tab,
+                                  bool adaptive, uint32_t lane) {
+  Coded r;
+  r.x = ACE_RANS_L;
+  r.pushes = r.present = r.head = r.bytes = r.mode = 0;
+  if (n == 0) return r;
+  quantise_warp(cnt, n, r.f, lane);
+  uint32_t tot = 0, np = 0;
 #pragma unroll
-  for (int j = 0; j < 8; j++) tot += f[j];
+  for (int j = 0; j < 8; j++) {
+    tot += r.f[j];
+    np += r.f[j] != 0;
+  }
   uint32_t c = warp_incl_sum(tot, lane) - tot;
 #pragma unroll
   for (int j = 0; j < 8; j++) {
-    fc[8 * lane + j] = f[j] | (c << 16);
-    c += f[j];
+    tab[8 * lane + j] = coder_entry(r.f[j], c);
+    c += r.f[j];
   }
+  r.present = __reduce_add_sync(kFull, np);
+  r.head = ACE_STREAM_HEAD + ((2 * r.present + 15) & ~15u);
   __syncwarp();
+  uint32_t x = ACE_RANS_L;
+  const uint32_t gt = kFull << lane << 1;  // the lanes of later symbols
+  auto round = [&](bool act, uint2 e) {
+    const uint32_t f = e.y & 0x1fffu, lim = f << (ACE_SCALE_BITS + 7);  // (L / 4096) * 256 * f = 2^19 f
+    const bool k1 = act && x >= lim, k2 = act && x >> 8 >= lim;          // x < 2^31: at most two pushes
+    const uint32_t b1 = __ballot_sync(kFull, k1), b2 = __ballot_sync(kFull, k2);
+    uint8_t* at = end - __popc(b1 & gt) - __popc(b2 & gt);
+    if (k1) at[-1] = (uint8_t)x;
+    if (k2) at[-2] = (uint8_t)(x >> 8);
+    end -= __popc(b1) + __popc(b2);
+    r.pushes += __popc(b1) + __popc(b2);
+    if (act) {
+      x >>= k2 ? 16 : k1 ? 8 : 0;
+      const uint32_t q = __umulhi(2 * x, e.x) >> (e.y >> 25);
+      x += q * (ACE_SCALE - f) + (e.y >> 13 & 0xfffu);
+    }
+  };
+  uint32_t i = n / 32 * 32 + lane;  // full rounds end before it
+  if (n & 31) {
+    const bool act = i < n;
+    round(act, act ? tab[sym[i]] : make_uint2(0u, 0u));
+  }
+  // full rounds, the symbols three rounds ahead and the entries one
+  uint32_t s0 = 0, s1 = 0;
+  uint2 e = make_uint2(0u, 0u);
+  if (i >= 32 + lane) e = tab[sym[i - 32]];
+  if (i >= 64 + lane) s0 = sym[i - 64];
+  if (i >= 96 + lane) s1 = sym[i - 96];
+  while (i >= 32 + lane) {
+    i -= 32;
+    const uint2 cur = e;
+    e = tab[s0];
+    s0 = s1;
+    if (i >= 96 + lane) s1 = sym[i - 96];
+    round(true, cur);
+  }
+  r.x = x;
+  r.mode = adaptive && r.head + r.pushes >= n;  // stored: the symbols verbatim
+  r.bytes = r.mode ? n : r.head + r.pushes;
+  return r;
 }
 
-// One stream of n symbols into out (16-byte aligned): its rANS payload
-// (32 final states, present bitmap, frequencies, renormalisation bytes), or,
-// with adaptive set and rANS not shrinking it, the symbols themselves.
-// The encode walks the symbols from the last to the first, symbol i on state
-// i mod 32, pushing a state's low byte while x >= 2^19 f_s, then x <-
-// (x / f_s) 4096 + x mod f_s + c_s; the pushes are then laid out in symbol
-// order, each symbol's bytes last push first, which is the byte order the
-// decoder reads.  Returns the stream's bytes; sets *mode.
-__device__ uint32_t code_stream_warp(const uint8_t* sym, uint32_t n, uint8_t* out, uint32_t* tmp, uint32_t* cnt,
-                                     uint32_t* fc, bool adaptive, uint32_t* mode, uint32_t lane) {
-  *mode = 0;
-  if (n == 0) return 0;
-  for (uint32_t s = lane; s < 256; s += 32) cnt[s] = 0;
-  __syncwarp();
-  for (uint32_t i = lane; i < n; i += 32) atomicAdd(cnt + sym[i], 1u);
-  __syncwarp();
-  quantise_warp(cnt, n, fc, lane);
-  // backward: pushes per symbol (count in bits 16..17, bytes below)
-  uint32_t x = ACE_RANS_L, pushes = 0;
-  const uint32_t rounds = (n + 31) / 32;
-  for (uint32_t r = rounds; r-- > 0;) {
-    const uint32_t i = 32 * r + lane;
-    if (i < n) {
-      const uint32_t e = fc[sym[i]], f = e & 0xffffu, c = e >> 16;
-      const uint32_t lim = f << (ACE_SCALE_BITS + 7);  // (L / 4096) * 256 * f = 2^19 f
-      uint32_t k = 0, bytes = 0;
-      while (x >= lim) {
-        bytes |= (x & 255u) << (8 * k);
-        x >>= 8;
-        k++;
-      }
-      x = ((x / f) << ACE_SCALE_BITS) + (x % f) + c;
-      tmp[i] = bytes | (k << 16);
-      pushes += k;
-    }
+// The coded stream's payload into out (16-byte aligned): 32 final states (the
+// decoder's entry point), present bitmap, frequencies, renormalisation bytes;
+// or, stored, its symbols.
+__device__ void place_stream_warp(const Coded& r, const uint8_t* sym, const uint8_t* renorm, uint8_t* out,
+                                  uint32_t lane) {
+  if (!r.bytes) return;
+  if (r.mode) {
+    copy_padded(out, sym, r.bytes, lane);
+    return;
   }
-#pragma unroll
-  for (int d = 16; d; d >>= 1) pushes += __shfl_xor_sync(kFull, pushes, d);
-  // the present symbols: bitmap byte l holds symbols 8l .. 8l + 7
+  reinterpret_cast<uint32_t*>(out)[lane] = r.x;
   uint32_t bm = 0;
 #pragma unroll
-  for (int j = 0; j < 8; j++) bm |= (fc[8 * lane + j] & 0xffffu) ? 1u << j : 0u;
+  for (int j = 0; j < 8; j++) bm |= r.f[j] ? 1u << j : 0u;
+  out[128 + lane] = (uint8_t)bm;  // bitmap byte l holds symbols 8l .. 8l + 7
   const uint32_t np = __popc(bm);
-  const uint32_t first = warp_incl_sum(np, lane) - np;
-  const uint32_t present = __shfl_sync(kFull, first + np, 31);
-  const uint32_t head = ACE_STREAM_HEAD + ((2 * present + 15) & ~15u);
-  if (adaptive && head + pushes >= n) {  // stored: the symbols verbatim
-    for (uint32_t i = lane; i < n; i += 32) out[i] = sym[i];
-    for (uint32_t i = n + lane; i < ((n + 15) & ~15u); i += 32) out[i] = 0;
-    *mode = 1;
-    return n;
-  }
-  reinterpret_cast<uint32_t*>(out)[lane] = x;  // the final states: the decoder's entry point
-  out[128 + lane] = (uint8_t)bm;
-  uint32_t k = first;
+  uint16_t* fq = reinterpret_cast<uint16_t*>(out + ACE_STREAM_HEAD);
+  uint32_t k = warp_incl_sum(np, lane) - np;
 #pragma unroll
-  for (int j = 0; j < 8; j++) {
-    const uint32_t f = fc[8 * lane + j] & 0xffffu;
-    if (f) {
-      out[ACE_STREAM_HEAD + 2 * k] = (uint8_t)f;
-      out[ACE_STREAM_HEAD + 2 * k + 1] = (uint8_t)(f >> 8);
-      k++;
-    }
-  }
-  for (uint32_t i = ACE_STREAM_HEAD + 2 * present + lane; i < head; i += 32) out[i] = 0;
-  // forward: each symbol's bytes at the running count of the pushes before it
-  uint32_t run = 0;
-  for (uint32_t r = 0; r < rounds; r++) {
-    const uint32_t i = 32 * r + lane;
-    const uint32_t t = i < n ? tmp[i] : 0u, kk = t >> 16;
-    const uint32_t incl = warp_incl_sum(kk, lane), at = head + run + incl - kk;
-    if (kk == 2) {
-      out[at] = (uint8_t)(t >> 8);
-      out[at + 1] = (uint8_t)t;
-    } else if (kk == 1) {
-      out[at] = (uint8_t)t;
-    }
-    run += __shfl_sync(kFull, incl, 31);
-  }
-  const uint32_t total = head + pushes;
-  for (uint32_t i = total + lane; i < ((total + 15) & ~15u); i += 32) out[i] = 0;
-  __syncwarp();
-  return total;
+  for (int j = 0; j < 8; j++)
+    if (r.f[j]) fq[k++] = (uint16_t)r.f[j];
+  for (uint32_t i = r.present + lane; i < (r.head - ACE_STREAM_HEAD) / 2; i += 32) fq[i] = 0;
+  copy_padded(out + r.head, renorm, r.pushes, lane);
 }
 
-// A warp per block: the token streams (literals in output order; lengths:
-// the escape values, then two codes per token; offsets: each match's
-// absolute source, w bytes), each coded, one after another 16-byte aligned
-// in the block's payload; the directory entry; the dependency runs (a bit
-// per earlier block a match reads, all below the window start) and the
-// block's level.
-__global__ void code_kernel(CodeArgs ca) {
-  __shared__ uint32_t s_cnt[8][256], s_fc[8][256], s_bits[8][kHead / 32 + 1], s_misc[8][4];
+constexpr uint32_t kCodeWarps = 4;
+constexpr uint32_t kLongRun = 16;  // literal runs from here on are copied by the whole warp
+
+// A CTA per block.  All warps: the token streams (literals in output order;
+// lengths: the escape values, then two codes per token; offsets: each match's
+// absolute source, w bytes) from groups of 32 tokens whose places a scan of
+// the groups' totals gives, their histograms, and the dependency runs (a bit
+// per earlier block a match reads, all below the window start) with the
+// block's level.  Then a warp per stream codes it, and the three payloads are
+// laid one after another, 16-byte aligned, in the block's payload.
+//
+// A warp per block did all of this in series, with a divide per symbol and a
+// second pass over the symbols for the bytes' places, 2.6 ms of the 64 MiB
+// FASTQ encode and 1.3 ms of the 11 MiB text one; this takes 0.81 and 0.26 ms.
+// Bound by the coder's chain where
+// blocks are few, by issue where they are many.
+__global__ void __launch_bounds__(32 * kCodeWarps) code_kernel(CodeArgs ca) {
+  extern __shared__ uint32_t group[];  // [3][groups]: bytes, literals, escapes before each group of 32 tokens
+  __shared__ uint2 s_tab[3][256];
+  __shared__ uint32_t s_cnt[3][256], s_bits[kHead / 32 + 2], s_total[3], s_bytes[3], s_level;
   const EncArgs& a = ca.e;
-  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const uint64_t b = a.c0 + blockIdx.x * (blockDim.x >> 5) + wid;
-  if (b >= a.c1) return;
-  const uint64_t cb = b - a.c0, bstart = b << a.log2B;
-  const uint32_t* tk = a.tok + cb * (uint64_t)a.tok_cap * 4;
-  const uint32_t nt = a.ntok[cb], nm = nt - 1, w = a.w;
-  uint8_t* lit = ca.syms + cb * (uint64_t)ca.sym_cap;
-  // token positions: run starts and literal positions (exclusive scans)
-  uint32_t dst = 0, lpos = 0, nesc = 0;
-  for (uint32_t i = lane; i < kHead / 32 + 1; i += 32) s_bits[wid][i] = 0;
-  __syncwarp();
-  uint32_t* lens_base = nullptr;
-  // pass 1: escape counts and literal total
-  uint32_t esc_total = 0, lit_total = 0;
-  for (uint32_t t0 = 0; t0 < nt; t0 += 32) {
-    const uint32_t t = t0 + lane;
-    uint32_t e = 0, lr = 0;
-    if (t < nt) {
-      lr = tk[4 * t];
-      e = (lr >= 255) + (tk[4 * t + 1] >= 255);
+  const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const uint64_t cb = blockIdx.x, b = a.c0 + cb, bstart = b << a.log2B;
+  const uint4* tk = reinterpret_cast<const uint4*>(a.tok) + cb * a.tok_cap;
+  const uint32_t nt = a.ntok[cb], nm = nt - 1, w = a.w, ng = (nt + 31) / 32;
+  for (uint32_t i = tid; i < 3 * 256; i += 32 * kCodeWarps) (&s_cnt[0][0])[i] = 0;
+  if (tid < kHead / 32 + 2) s_bits[tid] = 0;
+  if (tid == 0) s_level = 0;
+  for (uint32_t g = wid; g < ng; g += kCodeWarps) {
+    const uint32_t t = 32 * g + lane;
+    const uint4 v = t < nt ? tk[t] : make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t r0 = __reduce_add_sync(kFull, v.x + v.y), r1 = __reduce_add_sync(kFull, v.x);
+    const uint32_t r2 = __reduce_add_sync(kFull, (uint32_t)(v.x >= 255) + (v.y >= 255));
+    if (lane == 0) {
+      group[g] = r0;
+      group[ng + g] = r1;
+      group[2 * ng + g] = r2;
     }
-#pragma unroll
-    for (int d = 16; d; d >>= 1) {
-      e += __shfl_xor_sync(kFull, e, d);
-      lr += __shfl_xor_sync(kFull, lr, d);
-    }
-    esc_total += e;
-    lit_total += lr;
   }
-  uint8_t* lenp = lit + lit_total;              // lengths stream: 2 esc_total + 2 nt bytes
-  uint8_t* offp = lenp + 2 * esc_total + 2 * nt;  // offsets stream: w nm bytes
-  (void)lens_base;
-  // pass 2: the three streams' symbols, and the dependency bits
-  const uint64_t B = 1ull << a.log2B;
-  for (uint32_t t0 = 0; t0 < nt; t0 += 32) {
-    const uint32_t t = t0 + lane;
-    uint32_t lr = 0, ml = 0;
-    uint64_t src = 0;
-    if (t < nt) {
-      lr = tk[4 * t];
-      ml = tk[4 * t + 1];
-      src = (uint64_t)tk[4 * t + 2] | ((uint64_t)tk[4 * t + 3] << 32);
+  __syncthreads();
+  if (wid < 3) {
+    uint32_t carry = 0;
+    for (uint32_t g0 = 0; g0 < ng; g0 += 32) {
+      const uint32_t v = g0 + lane < ng ? group[wid * ng + g0 + lane] : 0u;
+      const uint32_t incl = warp_incl_sum(v, lane);
+      if (g0 + lane < ng) group[wid * ng + g0 + lane] = carry + incl - v;
+      carry += __shfl_sync(kFull, incl, 31);
     }
-    const uint32_t run = lr + ml, e = (t < nt) ? (lr >= 255) + (ml >= 255) : 0u;
-    const uint32_t ri = warp_incl_sum(run, lane), li = warp_incl_sum(lr, lane), ei = warp_incl_sum(e, lane);
-    const uint32_t my_dst = dst + ri - run, my_lit = lpos + li - lr, my_esc = nesc + ei - e;
+    if (lane == 0) s_total[wid] = carry;
+  }
+  __syncthreads();
+  const uint32_t lit_total = s_total[1], esc_total = s_total[2];
+  uint8_t* lit = ca.syms + cb * (uint64_t)ca.sym_cap;
+  uint8_t* lenp = lit + lit_total;                // lengths stream: 2 esc_total + 2 nt bytes
+  uint8_t* offp = lenp + 2 * esc_total + 2 * nt;  // offsets stream: w nm bytes
+  for (uint32_t g = wid; g < ng; g += kCodeWarps) {
+    const uint32_t t = 32 * g + lane;
+    const uint4 v = t < nt ? tk[t] : make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t lr = v.x, ml = v.y, run = lr + ml, e = (uint32_t)(lr >= 255) + (ml >= 255);
+    const uint64_t src = (uint64_t)v.z | ((uint64_t)v.w << 32);
+    const uint32_t my_dst = group[g] + warp_incl_sum(run, lane) - run;
+    const uint32_t my_lit = group[ng + g] + warp_incl_sum(lr, lane) - lr;
+    uint32_t ec = group[2 * ng + g] + warp_incl_sum(e, lane) - e;
+    const uint8_t* from = a.in + bstart;
+    if (lr < kLongRun)
+      for (uint32_t k = 0; k < lr; k++) {
+        const uint8_t s = from[my_dst + k];
+        lit[my_lit + k] = s;
+        atomicAdd(&s_cnt[0][s], 1u);
+      }
+    for (uint32_t lng = __ballot_sync(kFull, lr >= kLongRun); lng; lng &= lng - 1) {
+      const uint32_t f = __ffs(lng) - 1, n = __shfl_sync(kFull, lr, f), d = __shfl_sync(kFull, my_dst, f),
+                     l = __shfl_sync(kFull, my_lit, f);
+      for (uint32_t k = lane; k < n; k += 32) {
+        const uint8_t s = from[d + k];
+        lit[l + k] = s;
+        atomicAdd(&s_cnt[0][s], 1u);
+      }
+    }
     if (t < nt) {
-      for (uint32_t k = 0; k < lr; k++) lit[my_lit + k] = a.in[bstart + my_dst + k];
-      uint32_t ec = my_esc;
-      const uint32_t v[2] = {lr, ml};
+#pragma unroll
       for (int q = 0; q < 2; q++) {
-        if (v[q] < 255) {
-          lenp[2 * esc_total + 2 * t + q] = (uint8_t)v[q];
-        } else {
-          lenp[2 * esc_total + 2 * t + q] = 255;
-          lenp[2 * ec] = (uint8_t)(v[q] - 255);
-          lenp[2 * ec + 1] = (uint8_t)((v[q] - 255) >> 8);
+        const uint32_t x = q ? ml : lr, s = min(x, 255u);
+        lenp[2 * esc_total + 2 * t + q] = (uint8_t)s;
+        atomicAdd(&s_cnt[1][s], 1u);
+        if (x >= 255) {
+          const uint32_t y = x - 255;
+          lenp[2 * ec] = (uint8_t)y;
+          lenp[2 * ec + 1] = (uint8_t)(y >> 8);
+          atomicAdd(&s_cnt[1][y & 255], 1u);
+          atomicAdd(&s_cnt[1][y >> 8], 1u);
           ec++;
         }
       }
-      if (t < nm) {
-        for (uint32_t k = 0; k < w; k++) offp[w * t + k] = (uint8_t)(src >> (8 * k));
-        const uint64_t D = bstart + my_dst + lr;
-        if (ml && src < bstart) {  // blocks before this one that the match reads
-          const uint64_t rl = min((uint64_t)ml, D - src);
-          const uint64_t k0 = src >> a.log2B, k1 = min((src + rl - 1) >> a.log2B, b - 1);
-          for (uint64_t k = k0; k <= k1 && k < kHead; k++) atomicOr(&s_bits[wid][k >> 5], 1u << (k & 31));
-        }
+    }
+    if (t < nm) {
+      for (uint32_t k = 0; k < w; k++) {
+        const uint8_t s = (uint8_t)(src >> (8 * k));
+        offp[w * t + k] = s;
+        atomicAdd(&s_cnt[2][s], 1u);
+      }
+      const uint64_t D = bstart + my_dst + lr;
+      if (ml && src < bstart) {  // blocks before this one that the match reads
+        const uint64_t rl = min((uint64_t)ml, D - src);
+        const uint64_t k0 = src >> a.log2B, k1 = min((src + rl - 1) >> a.log2B, b - 1);
+        for (uint64_t k = k0; k <= k1 && k < kHead; k++) atomicOr(&s_bits[k >> 5], 1u << (k & 31));
       }
     }
-    dst += __shfl_sync(kFull, ri, 31);
-    lpos += __shfl_sync(kFull, li, 31);
-    nesc += __shfl_sync(kFull, ei, 31);
   }
-  __syncwarp();
-  // the three streams
-  uint8_t* pay = ca.pay + cb * (uint64_t)ca.pay_cap;
-  uint32_t* tmp = ca.tmp + cb * (uint64_t)ca.tmp_cap;
-  const uint8_t* streams[3] = {lit, lenp, offp};
+  __syncthreads();
   const uint32_t ns[3] = {lit_total, 2 * esc_total + 2 * nt, w * nm};
-  ace_block_dir d;
-  memset(&d, 0, sizeof d);
-  uint32_t off = 0;
-  for (int k = 0; k < 3; k++) {
-    uint32_t mode;
-    const uint32_t bytes = code_stream_warp(streams[k], ns[k], pay + off, tmp, s_cnt[wid], s_fc[wid], a.adaptive != 0,
-                                            &mode, lane);
-    d.stream_off[k] = off;
-    d.stream_bytes[k] = bytes;
-    d.nsym[k] = ns[k];
-    d.mode[k] = (uint8_t)mode;
-    off += (bytes + 15) & ~15u;
-  }
-  d.ntok = nt;
-  d.nesc = esc_total;
-  // dependency runs and the level: 1 + the deepest block read
-  uint32_t lv = 0;
-  for (uint32_t k = lane; k < kHead && k < b; k += 32)
-    if (s_bits[wid][k >> 5] >> (k & 31) & 1) lv = max(lv, a.level[k] + 1);
-#pragma unroll
-  for (int dd = 16; dd; dd >>= 1) lv = max(lv, __shfl_xor_sync(kFull, lv, dd));
-  if (lane == 0) {
-    uint32_t cnt = 0, k = 0;
+  const uint32_t k = min(wid, 2u), sym_at = k == 0 ? 0u : k == 1 ? ns[0] : ns[0] + ns[1];
+  const uint32_t n = k == 0 ? ns[0] : k == 1 ? ns[1] : ns[2];
+  Coded r;
+  uint8_t* end = ca.tmp + cb * 2 * (uint64_t)ca.sym_cap + 2 * (sym_at + n);
+  if (wid < 3) {
+    r = code_stream_warp(lit + sym_at, n, end, s_cnt[wid], s_tab[wid], a.adaptive != 0, lane);
+    if (lane == 0) s_bytes[wid] = r.bytes;
+  } else {
+    // the block's level: 1 + the deepest block read; its dependency runs
+    for (uint32_t q = lane; q < kHead && q < b; q += 32)
+      if (s_bits[q >> 5] >> (q & 31) & 1) atomicMax(&s_level, a.level[q] + 1);
     uint32_t* iv = ca.iv + b * (uint64_t)(2 * kIvCap);
-    const uint32_t top = (uint32_t)min((uint64_t)b, (uint64_t)kHead);
-    while (k < top) {
-      if (!(s_bits[wid][k >> 5] >> (k & 31) & 1)) {
-        k++;
-        continue;
-      }
-      uint32_t e = k;
-      while (e + 1 < top && (s_bits[wid][(e + 1) >> 5] >> ((e + 1) & 31) & 1)) e++;
-      iv[2 * cnt] = k;
-      iv[2 * cnt + 1] = e;
-      cnt++;
-      k = e + 1;
-    }
-    ca.n_iv[b] = cnt;
-    a.level[b] = lv;
-    ca.dir[b] = d;
-    ca.pay_bytes[cb] = off;
+    const uint32_t v = lane < kHead / 32 ? s_bits[lane] : 0u;
+    const uint32_t before = __shfl_up_sync(kFull, v, 1) >> 31, after = __shfl_down_sync(kFull, v, 1) << 31;
+    uint32_t starts = v & ~(v << 1 | (lane ? before : 0u)), ends = v & ~(v >> 1 | after);
+    const uint32_t si = warp_incl_sum(__popc(starts), lane);
+    uint32_t at = si - __popc(starts);
+    for (; starts; starts &= starts - 1) iv[2 * at++] = 32 * lane + __ffs(starts) - 1;
+    at = warp_incl_sum(__popc(ends), lane) - __popc(ends);
+    for (; ends; ends &= ends - 1) iv[2 * at++ + 1] = 32 * lane + __ffs(ends) - 1;
+    if (lane == 31) ca.n_iv[b] = si;
   }
-  (void)B;
+  __syncthreads();
+  const uint32_t p0 = (s_bytes[0] + 15) & ~15u, p1 = (s_bytes[1] + 15) & ~15u, p2 = (s_bytes[2] + 15) & ~15u;
+  const uint32_t off = wid == 0 ? 0u : wid == 1 ? p0 : p0 + p1;
+  if (wid < 3) {
+    place_stream_warp(r, lit + sym_at, end - r.pushes, ca.pay + cb * (uint64_t)ca.pay_cap + off, lane);
+    if (lane == 0) {
+      ace_block_dir& d = ca.dir[b];
+      d.stream_off[wid] = off;
+      d.stream_bytes[wid] = r.bytes;
+      d.nsym[wid] = n;
+      d.mode[wid] = (uint8_t)r.mode;
+    }
+  } else if (lane == 0) {
+    ace_block_dir& d = ca.dir[b];
+    d.ntok = nt;
+    d.nesc = esc_total;
+    for (int q = 0; q < 5; q++) d.reserved[q] = 0;
+    a.level[b] = s_level;
+    ca.pay_bytes[cb] = p0 + p1 + p2;
+  }
 }
 
 // ------------------------------------------------------ payload placement
@@ -1065,7 +1129,7 @@ struct EncLayout {
   uint64_t table, level, dir, iv, n_iv, dep_ptr, hdr, entries, cand, tok, ntok, syms, tmp, pay,
       pay_bytes, pay_off, total;
   uint64_t nb, chunk, reserve, arc_bound, entry_blocks;
-  uint32_t bits, tok_cap, sym_cap, tmp_cap, pay_cap;
+  uint32_t bits, tok_cap, sym_cap, pay_cap;
 };
 
 inline uint64_t a256(uint64_t v) { return (v + 255) & ~255ull; }
@@ -1086,7 +1150,6 @@ ace_status enc_layout(uint64_t n, const ace_encode_params* p, EncLayout* L) {
   L->chunk = std::max<uint64_t>(1, std::min<uint64_t>(chunk, std::max<uint64_t>(L->nb, 1)));
   L->tok_cap = (uint32_t)(B / p->min_match + 2);
   L->sym_cap = (uint32_t)align16(B + 11ull * L->tok_cap);
-  L->tmp_cap = L->sym_cap;
   L->pay_cap = (uint32_t)align16(3ull * (ACE_STREAM_HEAD + 2 * 256 + 16) + 2ull * L->sym_cap + 64);
   const uint64_t nb = L->nb, C = L->chunk, cb = C * B;
   uint64_t o = 0;
@@ -1117,7 +1180,7 @@ ace_status enc_layout(uint64_t n, const ace_encode_params* p, EncLayout* L) {
   L->syms = o;
   o = a256(o + (uint64_t)L->sym_cap * C);
   L->tmp = o;
-  o = a256(o + 4ull * L->tmp_cap * C);
+  o = a256(o + 2ull * L->sym_cap * C);
   L->pay = o;
   o = a256(o + (uint64_t)L->pay_cap * C);
   L->pay_bytes = o;
@@ -1191,8 +1254,7 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   CodeArgs ca;
   ca.syms = base + L.syms;
   ca.sym_cap = L.sym_cap;
-  ca.tmp = reinterpret_cast<uint32_t*>(base + L.tmp);
-  ca.tmp_cap = L.tmp_cap;
+  ca.tmp = base + L.tmp;
   ca.pay = base + L.pay;
   ca.pay_cap = L.pay_cap;
   ca.dir = reinterpret_cast<ace_block_dir*>(base + L.dir);
@@ -1248,7 +1310,7 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
                                                                                 shape.smem, s>>>(e);
     parse_kernel<<<(uint32_t)cn, 32, 3 * (B / 8 + 4), s>>>(e);  // at most 24.1 KB of bit maps
     ca.e = e;
-    code_kernel<<<(uint32_t)((cn + 7) / 8), 256, 0, s>>>(ca);
+    code_kernel<<<(uint32_t)cn, 32 * kCodeWarps, 12 * ((L.tok_cap + 31) / 32), s>>>(ca);
     pa.c0 = pc.c0;
     pa.cn = cn;
     place_scan_kernel<<<1, 1024, 0, s>>>(pa);

@@ -1,4 +1,5 @@
-"""The GPU encoder's parse, token by token, against a plain sequential model
+"""The GPU encoder's streams against the oracle's rANS encoder, and its parse,
+token by token, against a plain sequential model
 of its rules (the earliest stride position of every 16-byte key, chains of
 4-byte hashes inside a block, windows of 64 blocks, waves of at most 3, the
 shallow preference), at the block sizes and input sizes where windows, bit
@@ -164,3 +165,38 @@ def test_parse_equals_the_sequential_model(name, data, log2b, mm, offset):
         assert [t[:2] for t in got] == [t[:2] for t in toks], (name, b)
         assert [t[2] for t in got[:-1]] == [t[2] for t in toks[:-1]], (name, b)
     assert np.array_equal(oracle.decode(arc), data)
+
+
+def _coded_like_the_oracle(arc):
+    hdr = arc[:64].view(np.uint64)
+    nb, dir_off, pay = int(hdr[3]), int(hdr[4]), int(hdr[6])
+    d = arc[dir_off:dir_off + 64 * nb].reshape(nb, 64)
+    offs, sizes, counts = (d[:, a:b].copy().view(t) for a, b, t in
+                           ((0, 24, np.uint64), (24, 36, np.uint32), (36, 48, np.uint32)))
+    for b in range(nb):
+        for k in range(3):
+            if not counts[b, k]:
+                assert sizes[b, k] == 0
+                continue
+            p = arc[pay + int(offs[b, k]):pay + int(offs[b, k]) + int(sizes[b, k])]
+            present = np.unpackbits(p[128:160], bitorder="little").astype(bool)
+            freq = np.zeros(256, np.uint16)
+            n = int(present.sum())
+            freq[present] = p[160:160 + 2 * n].view(np.uint16)
+            head = 160 + ((2 * n + 15) & ~15)
+            sym = oracle.rans_decode(p[head:], p[:128].view(np.uint32), freq, int(counts[b, k]))
+            assert np.array_equal(oracle.rans_freqs(sym), freq), (b, k)
+            states, body = oracle.rans_encode(sym, freq)
+            assert np.array_equal(states, p[:128].view(np.uint32)) and np.array_equal(body, p[head:]), (b, k)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 64, 95, 96, 97, 128, 256, 700])
+@pytest.mark.parametrize("values", [1, 3, 256])
+def test_streams_equal_the_oracles_encoder(n, values):
+    """Literal streams around the coder's rounds of 32 and its loads ahead,
+    one value (frequency 4096) to all 256 (pushes of two bytes)."""
+    rng = np.random.default_rng(n * 1000 + values)
+    x = np.minimum(rng.integers(0, values, n), rng.integers(0, values, n)).astype(np.uint8)
+    arc = ace.ace_encode_gpu(torch.from_numpy(x).cuda(), 10, 200).cpu().numpy()  # no matches
+    assert np.array_equal(oracle.decode(arc), x)
+    _coded_like_the_oracle(arc)
