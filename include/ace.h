@@ -258,7 +258,7 @@ enum { ACE_SCHEDULE_AUTO = 0, ACE_SCHEDULE_PASSES = 1, ACE_SCHEDULE_FUSED = 2 };
 typedef struct {
     uint32_t warps_per_cta;   /* 1..8; 0 = default (4) */
     uint32_t ctas_per_sm;     /* 0 = as many as fit */
-    uint32_t chunk_tokens;    /* tokens staged per step, 32..256, multiple of 32; 0 = 128 */
+    uint32_t chunk_tokens;    /* a step of the literal pass lists two literal runs, and takes up to 32 literals, per token of this, 32..256, multiple of 32; 0 = 128 */
     uint32_t schedule;        /* ACE_SCHEDULE_*; 0 = automatic; others: ACE_E_INVAL */
     uint64_t wait_timeout_ns; /* bound on each device-side wait; 0 = 2 s */
     uint32_t copy_width;      /* match copies: 16 = every non-overlapping match above 32 bytes in aligned

@@ -493,7 +493,8 @@ __device__ __forceinline__ uint32_t table_round(uint32_t& x, uint32_t& pos, cons
   const uint32_t slot = x & (ACE_SCALE - 1);
   const uint32_t s = lut.sym[slot];
   const uint32_t fc = lut.fc[s];
-  const uint32_t xn = (fc >> 16) * (x >> ACE_SCALE_BITS) + slot - (fc & 0xffffu);
+  // f (x >> 12) + slot - c; with fc = f << 16 | c this saves taking c out
+  const uint32_t xn = (fc >> 16) * ((x >> ACE_SCALE_BITS) + 65536u) + (slot - fc);
   const bool p1 = xn < ACE_RANS_L, p2 = xn < (1u << 15);
   const uint32_t b1 = __ballot_sync(kFull, p1);
   if (!__any_sync(kFull, p2)) {  // no state takes two bytes (most rounds): one read per lane
@@ -513,15 +514,17 @@ __device__ __forceinline__ uint32_t table_round(uint32_t& x, uint32_t& pos, cons
 }
 
 // nfull full rounds in slot-table mode from a round boundary (st.next a
-// multiple of 32), handing each round's symbol to emit(s) in order.  The ring
+// multiple of 32), handing each round's symbol to emit(s, u) in order, u its
+// place in its group of U rounds (begin() before each group; the last rounds
+// are groups of one).  The ring
 // is checked once per U rounds (U = 2 or 4): a round reads at most 64 bytes,
 // so U rounds after a check, which leaves the position less than one segment
 // into the ring, stay inside its first 1 + U / 2 segments; the check lets at
 // most RING / 128 - 1 - U / 2 segment fills stay in flight, and runs once
 // more at the end.
-template <uint32_t RING = kRing, uint32_t U = 2, class Emit>
+template <uint32_t RING = kRing, uint32_t U = 2, class Begin, class Emit>
 __device__ __forceinline__ void table_full_rounds(Stream& st, uint8_t* ring, const Lut& lut, uint32_t nfull,
-                                                  uint32_t lane, uint32_t lt, Emit&& emit) {
+                                                  uint32_t lane, uint32_t lt, Begin&& begin, Emit&& emit) {
   static_assert(U == 2 || U == 4, "two or four rounds per ring check");
   uint32_t x = st.x, pos = st.pos, base = st.base;
   auto check = [&]() {
@@ -535,12 +538,14 @@ __device__ __forceinline__ void table_full_rounds(Stream& st, uint8_t* ring, con
   uint32_t r = 0;
   for (; r + U <= nfull; r += U) {
     check();
+    begin(U);
 #pragma unroll
-    for (uint32_t u = 0; u < U; u++) emit(table_round<RING>(x, pos, ring, lut, lt));
+    for (uint32_t u = 0; u < U; u++) emit(table_round<RING>(x, pos, ring, lut, lt), u);
   }
   for (; r < nfull; r++) {
     check();
-    emit(table_round<RING>(x, pos, ring, lut, lt));
+    begin(1u);
+    emit(table_round<RING>(x, pos, ring, lut, lt), 0u);
   }
   check();  // the single-round decoders that follow expect less than one segment consumed
   st.x = x;
