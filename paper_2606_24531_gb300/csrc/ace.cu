@@ -1878,73 +1878,85 @@ struct ClosureArgs {
   uint32_t* lv_done;     // fused seeks: per-level counters, cleared here (null otherwise)
 };
 
+// CTAs of a closure search, one cluster (the largest portable size).
+constexpr uint32_t kClosureCtas = 8;
+
 // The blocks a seek must decode: its target blocks and, transitively, every
 // block their matches read (Section 2).  Breadth first from the targets, a
 // warp per frontier block with its lanes over the block's dependency
 // intervals; then an ordered compaction of the marked blocks gives each its
 // slot, and the work list is ordered by dependency level (blocks of a level
 // in ascending order) with the level ranges in the scratch header -- a valid
-// decode order either way, since sources always precede.  One CTA.
-__global__ void closure_kernel(ClosureArgs a) {
-  __shared__ uint32_t n_next, s_min;
+// decode order either way, since sources always precede.
+//
+// A frontier block is four or five loads that wait for one another, so the
+// search is bound by their latency times the blocks a warp takes in turn: the
+// frontier is spread over the 256 warps of a cluster, with a cluster barrier
+// per step; the rest, short, is the first CTA's.  By one CTA the closure of a
+// 16 MiB range of a genome took 35 to 49 us; this takes 20.
+__global__ void __cluster_dims__(kClosureCtas, 1, 1) __launch_bounds__(1024, 1) closure_kernel(ClosureArgs a) {
   __shared__ uint32_t wsum[32];
   __shared__ uint32_t carry;
   __shared__ uint32_t lcnt[kMaxLevelLaunches + 1];
   const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-  if (tid == 0) {
+  const uint32_t rank = cluster_rank();
+  const uint32_t ntar = (uint32_t)(a.last - a.first + 1);
+  if (rank == 0 && tid == 0) {
     const uint32_t e = (a.sh->epoch + 1) & ~kPendingFlag;  // never 0, never with the pending bit
     a.sh->epoch = e ? e : 1u;
     a.sh->ticket = 0;
     a.sh->ticket2 = 0;
     a.sh->ticket3 = 0;
-    s_min = (uint32_t)a.first;
+    a.sh->min_block = (uint32_t)a.first;
+    a.sh->front[0] = ntar;
+    a.sh->front[1] = 0;
   }
-  if (tid <= kMaxLevelLaunches) {
-    lcnt[tid] = 0;
-    if (a.lv_done) a.lv_done[tid] = 0;
-  }
-  uint32_t ntar = (uint32_t)(a.last - a.first + 1);
-  for (uint32_t i = tid; i < ntar; i += blockDim.x) {
-    uint32_t b = (uint32_t)a.first + i;
+  if (rank == 0 && tid <= kMaxLevelLaunches && a.lv_done) a.lv_done[tid] = 0;
+  for (uint32_t i = rank * blockDim.x + tid; i < ntar; i += kClosureCtas * blockDim.x) {
+    const uint32_t b = (uint32_t)a.first + i;
     atomicOr(&a.marks[b >> 5], 1u << (b & 31));
     a.front0[i] = b;
   }
-  uint32_t n_front = ntar;
+  cluster_sync();
+  // step k: the frontier's blocks in front0/front1 in turn, their count in
+  // front[k mod 3]; the next step's counted in front[k + 1 mod 3], the one
+  // after cleared
   uint32_t* cur = a.front0;
   uint32_t* nxt = a.front1;
-  __syncthreads();
-  while (n_front) {
-    if (tid == 0) n_next = 0;
-    __syncthreads();
-    for (uint32_t f = wid; f < n_front; f += nw) {
-      const uint32_t b = cur[f];
-      const uint32_t e1 = a.dep_ptr[b + 1];
-      for (uint32_t e = a.dep_ptr[b] + lane; e < e1; e += 32) {
-        const uint32_t k0 = a.dep_iv[2 * e], k1 = a.dep_iv[2 * e + 1];
-        for (uint32_t k = k0; k <= k1; k++) {
-          uint32_t old = atomicOr(&a.marks[k >> 5], 1u << (k & 31));
-          if (!(old & (1u << (k & 31)))) {
-            nxt[atomicAdd(&n_next, 1u)] = k;
-            atomicMin(&s_min, k);
+  for (uint32_t k = 0;; k++) {
+    const uint32_t n_front = __ldcg(&a.sh->front[k % 3]);
+    if (!n_front) break;  // the same for every CTA: counted before the last barrier
+    uint32_t* n_next = &a.sh->front[(k + 1) % 3];
+    if (rank == 0 && tid == 0) a.sh->front[(k + 2) % 3] = 0;
+    for (uint32_t f = rank * nw + wid; f < n_front; f += kClosureCtas * nw) {
+      const uint32_t b = __ldcg(cur + f);
+      const uint32_t e1 = __ldg(a.dep_ptr + b + 1);
+      for (uint32_t e = __ldg(a.dep_ptr + b) + lane; e < e1; e += 32) {
+        const uint32_t k0 = __ldg(a.dep_iv + 2 * e), k1 = __ldg(a.dep_iv + 2 * e + 1);
+        for (uint32_t q = k0; q <= k1; q++) {
+          const uint32_t old = atomicOr(&a.marks[q >> 5], 1u << (q & 31));
+          if (!(old & (1u << (q & 31)))) {
+            nxt[atomicAdd(n_next, 1u)] = q;
+            atomicMin(&a.sh->min_block, q);
           }
         }
       }
     }
-    __syncthreads();
-    n_front = n_next;
-    uint32_t* t = cur;
+    cluster_sync();
+    uint32_t* const t = cur;
     cur = nxt;
     nxt = t;
-    __syncthreads();
   }
+  if (rank) return;
+  if (tid <= kMaxLevelLaunches) lcnt[tid] = 0;
   // ordered compaction of the marked blocks into front0, clearing the marks
   // behind it; a block's slot is its place in ascending order
   if (tid == 0) carry = 0;
   __syncthreads();
-  uint32_t w0 = s_min >> 5, w1 = (uint32_t)(a.last >> 5);
+  uint32_t w0 = __ldcg(&a.sh->min_block) >> 5, w1 = (uint32_t)(a.last >> 5);
   for (uint32_t c0 = w0; c0 <= w1; c0 += blockDim.x) {
     uint32_t wi = c0 + tid;
-    uint32_t bits = wi <= w1 ? a.marks[wi] : 0u;
+    uint32_t bits = wi <= w1 ? __ldcg(a.marks + wi) : 0u;
     uint32_t cnt = __popc(bits);
     uint32_t incl = warp_incl_sum(cnt, lane);
     if (lane == 31) wsum[wid] = incl;
@@ -2037,7 +2049,9 @@ struct CacheHdr {
   uint32_t ticket2;    // next work item of the literal pass
   uint32_t ticket3;    // next work item of the match pass
   uint64_t decoded;    // blocks decoded, since creation
-  uint32_t pad[48];
+  uint32_t front[3];   // frontier sizes during the closure search
+  uint32_t overflow;   // a frontier outgrew its room (serial of the batch)
+  uint32_t pad[44];
 };
 static_assert(sizeof(CacheHdr) == 256, "cache header");
 static_assert(offsetof(CacheHdr, ticket2) == offsetof(ScratchHdr, ticket2), "shared header fields");
@@ -2093,89 +2107,92 @@ __device__ __forceinline__ bool cache_visit(const CacheArgs& c, uint32_t a, uint
 // (Section 2), listed archive by archive in ascending block order.  Each
 // gets a slot from a clock over the slots: slots this batch uses are passed
 // over, a slot whose reference bit is set gets a second chance (the bit is
-// cleared), and a slot taken from a cached block evicts it.  One CTA.
-__global__ void cache_closure_kernel(CacheArgs c) {
-  __shared__ uint32_t n_next, carry, overflow, s_serial;
+// cleared), and a slot taken from a cached block evicts it.
+//
+// Bound by latency like the plain seek's closure, and searched by a cluster
+// in the same way (a warp per request for the targets, then per frontier
+// block); the listing and the clock are the first CTA's.  By one CTA, with a
+// thread per request, 128 requests over 1900 blocks took 0.297 ms; this takes
+// 0.069 ms.
+__global__ void __cluster_dims__(kClosureCtas, 1, 1) __launch_bounds__(1024, 1) cache_closure_kernel(CacheArgs c) {
+  __shared__ uint32_t carry;
   __shared__ uint32_t s_taken, s_hand, s_scanned, s_stop;
   __shared__ uint32_t wsum[32];
   const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-  const uint32_t epoch = c.h->epoch;
-  if (tid == 0) {
-    n_next = 0;
-    overflow = 0;
-    s_serial = c.h->serial + 1;
-    c.h->serial = s_serial;
+  const uint32_t rank = cluster_rank();
+  const uint32_t epoch = c.h->epoch, serial = c.h->serial + 1;
+  // front[] and overflow are of no use between batches: cleared here, counted
+  // from the first barrier on
+  if (rank == 0) {
+    if (tid < 3) c.h->front[tid] = 0;
+    if (tid == 3) c.h->overflow = 0;
+    for (uint32_t a = tid; a < c.n_arcs; a += blockDim.x) {
+      c.arc_minmax[2 * a] = 0xffffffffu;
+      c.arc_minmax[2 * a + 1] = 0;
+    }
   }
-  for (uint32_t a = tid; a < c.n_arcs; a += blockDim.x) {
-    c.arc_minmax[2 * a] = 0xffffffffu;
-    c.arc_minmax[2 * a + 1] = 0;
-  }
-  __syncthreads();
-  const uint32_t serial = s_serial;
-  // targets: a thread per request
-  for (uint32_t r = tid; r < c.n_reqs; r += blockDim.x) {
+  cluster_sync();
+  if (rank == 0 && tid == 0) c.h->serial = serial;  // every CTA has read it
+  auto push = [&](uint32_t* front, uint32_t* count, uint32_t a, uint32_t b) {
+    const uint32_t i = atomicAdd(count, 1u);
+    if (i < c.front_cap) {
+      front[2 * i] = a;
+      front[2 * i + 1] = b;
+    } else {
+      c.h->overflow = 1;
+    }
+    atomicMin(&c.arc_minmax[2 * a], b);
+  };
+  // targets: a warp per request, its lanes over the request's blocks
+  const uint32_t gw = rank * nw + wid;
+  for (uint32_t r = gw; r < c.n_reqs; r += kClosureCtas * nw) {
     const ace_seek_req q = c.reqs[r];
-    uint64_t first = q.coord >> c.log2B, last = (q.coord + q.len - 1) >> c.log2B;
-    for (uint64_t b = first; b <= last; b++) {
+    const uint64_t first = q.coord >> c.log2B, last = (q.coord + q.len - 1) >> c.log2B;
+    for (uint64_t b = first + lane; b <= last; b += 32) {
       bool cached;
       if (cache_visit(c, q.archive, (uint32_t)b, epoch, serial, cached)) {
-        uint32_t i = atomicAdd(&n_next, 1u);
-        if (i < c.front_cap) {
-          c.front0[2 * i] = q.archive;
-          c.front0[2 * i + 1] = (uint32_t)b;
-        } else {
-          overflow = 1;
-        }
-        atomicMin(&c.arc_minmax[2 * q.archive], (uint32_t)b);
+        push(c.front0, &c.h->front[0], q.archive, (uint32_t)b);
         atomicMax(&c.arc_minmax[2 * q.archive + 1], (uint32_t)b);
       }
     }
   }
-  __syncthreads();
-  uint32_t n_front = min(n_next, c.front_cap);
+  cluster_sync();
   uint32_t* cur = c.front0;
   uint32_t* nxt = c.front1;
-  __syncthreads();
-  while (n_front && !overflow) {
-    if (tid == 0) n_next = 0;
-    __syncthreads();
-    for (uint32_t i = wid; i < n_front; i += nw) {  // a warp per frontier block, lanes over its intervals
-      uint32_t a = cur[2 * i], b = cur[2 * i + 1];
+  for (uint32_t k = 0;; k++) {  // counts as in the plain seek's closure
+    const uint32_t n_front = min(__ldcg(&c.h->front[k % 3]), c.front_cap);
+    if (!n_front || __ldcg(&c.h->overflow)) break;  // the same for every CTA: written before the last barrier
+    cluster_sync();                                 // ... and this step's overflow after this one
+    uint32_t* n_next = &c.h->front[(k + 1) % 3];
+    if (rank == 0 && tid == 0) c.h->front[(k + 2) % 3] = 0;
+    for (uint32_t i = gw; i < n_front; i += kClosureCtas * nw) {  // a warp per frontier block, lanes over its intervals
+      const uint32_t a = __ldcg(cur + 2 * i), b = __ldcg(cur + 2 * i + 1);
       const CacheArc& ca = c.arcs[a];
-      const uint32_t e1 = ca.dep_ptr[b + 1];
-      for (uint32_t e = ca.dep_ptr[b] + lane; e < e1; e += 32)
-        for (uint32_t k = ca.dep_iv[2 * e]; k <= ca.dep_iv[2 * e + 1]; k++) {
+      const uint32_t e1 = __ldg(ca.dep_ptr + b + 1);
+      for (uint32_t e = __ldg(ca.dep_ptr + b) + lane; e < e1; e += 32)
+        for (uint32_t q = __ldg(ca.dep_iv + 2 * e); q <= __ldg(ca.dep_iv + 2 * e + 1); q++) {
           bool cached;
-          if (cache_visit(c, a, k, epoch, serial, cached)) {
-            uint32_t j = atomicAdd(&n_next, 1u);
-            if (j < c.front_cap) {
-              nxt[2 * j] = a;
-              nxt[2 * j + 1] = k;
-            } else {
-              overflow = 1;
-            }
-            atomicMin(&c.arc_minmax[2 * a], k);
-          }
+          if (cache_visit(c, a, q, epoch, serial, cached)) push(nxt, n_next, a, q);
         }
     }
-    __syncthreads();
-    n_front = min(n_next, c.front_cap);
-    uint32_t* t = cur;
+    cluster_sync();
+    uint32_t* const t = cur;
     cur = nxt;
     nxt = t;
-    __syncthreads();
   }
+  if (rank) return;
+  const bool overflow = __ldcg(&c.h->overflow) != 0;
   // ordered compaction into the work list, archive by archive, clearing the
   // marks behind it
   if (tid == 0) carry = 0;
   __syncthreads();
   for (uint32_t a = 0; a < c.n_arcs; a++) {
-    uint32_t lo = c.arc_minmax[2 * a], hi = c.arc_minmax[2 * a + 1];
+    uint32_t lo = __ldcg(c.arc_minmax + 2 * a), hi = __ldcg(c.arc_minmax + 2 * a + 1);
     if (lo > hi) continue;
     const CacheArc& ca = c.arcs[a];
     for (uint32_t c0 = lo >> 5; c0 <= (hi >> 5); c0 += blockDim.x) {
       uint32_t wi = c0 + tid;
-      uint32_t bits = wi <= (hi >> 5) ? ca.marks[wi] : 0u;
+      uint32_t bits = wi <= (hi >> 5) ? __ldcg(ca.marks + wi) : 0u;
       uint32_t cnt = __popc(bits);
       uint32_t incl = warp_incl_sum(cnt, lane);
       if (lane == 31) wsum[wid] = incl;
@@ -2221,8 +2238,8 @@ __global__ void cache_closure_kernel(CacheArgs c) {
     const uint32_t sl = (uint32_t)(((uint64_t)hand + tid) % c.n_slots);
     bool pinned = false, refd = false, elig = false;
     if (tid < win) {
-      pinned = c.use[sl] == serial;
-      refd = c.ref[sl] != 0;
+      pinned = __ldcg(c.use + sl) == serial;
+      refd = __ldcg(c.ref + sl) != 0;
       elig = !pinned && !refd;
     }
     const uint32_t e = elig ? 1u : 0u;
@@ -3199,7 +3216,7 @@ ace_status ace_seek(const ace_index* idx, uint64_t coord, uint64_t len, void* d_
   // the fused schedule needs the closure's work list in level order
   if (!idx->by_levels) L.schedule = ACE_SCHEDULE_PASSES;
   c.lv_done = L.schedule == ACE_SCHEDULE_FUSED ? reinterpret_cast<uint32_t*>(base + S1.lv_done) : nullptr;
-  closure_kernel<<<1, 1024, 0, s>>>(c);
+  closure_kernel<<<kClosureCtas, 1024, 0, s>>>(c);
   DecodeArgs a{};
   a.arc = idx->d_arc;
   a.dir = reinterpret_cast<const ace_block_dir*>(idx->d_arc + idx->h.dir_off);
@@ -3705,7 +3722,7 @@ ace_status ace_seek_batch(const ace_cache* c, const ace_seek_req* d_reqs, uint32
   CacheArgs a = c->args;
   a.reqs = d_reqs;
   a.n_reqs = n;
-  cache_closure_kernel<<<1, 1024, 0, s>>>(a);
+  cache_closure_kernel<<<kClosureCtas, 1024, 0, s>>>(a);
   CacheDecodeArgs d = c->dargs;
   d.c = a;
   const Launch& L = c->L;
@@ -3874,7 +3891,7 @@ ace_status ace_seek_noalloc(const ace_index* idx, uint64_t coord, uint64_t len, 
   if (rc) return rc;
   if (!idx->by_levels) L.schedule = ACE_SCHEDULE_PASSES;
   c.lv_done = L.schedule == ACE_SCHEDULE_FUSED ? reinterpret_cast<uint32_t*>(base + S.lv_done) : nullptr;
-  closure_kernel<<<1, 1024, 0, s>>>(c);
+  closure_kernel<<<kClosureCtas, 1024, 0, s>>>(c);
   DecodeArgs a{};
   a.arc = idx->d_arc;
   a.dir = reinterpret_cast<const ace_block_dir*>(idx->d_arc + idx->h.dir_off);

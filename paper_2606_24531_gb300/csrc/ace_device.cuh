@@ -19,14 +19,15 @@ struct ScratchHdr {
   uint32_t epoch;      // value a block's ready flag takes when it is published
   uint32_t ticket;     // next work item handed to a persistent warp
   uint32_t n_work;     // seek: blocks in the work list
-  uint32_t n_front;    // seek: frontier size during the closure search
+  uint32_t unused;
   uint32_t min_block;  // seek: smallest block reached by the closure
   uint64_t fnv;        // verify: last FNV-1a 64 computed
   uint64_t guard_bad;  // verify: guard bytes that differ from the canary
   uint32_t ticket2;    // next work item of the literal pass
   uint32_t ticket3;    // next work item of the match pass
   uint32_t lv_start[33];  // seek by levels: the work list's level l is [lv_start[l], lv_start[l + 1])
-  uint32_t pad[17];
+  uint32_t front[3];   // seek: frontier sizes during the closure search
+  uint32_t pad[14];
 };
 static_assert(sizeof(ScratchHdr) == 256, "scratch header");
 
@@ -111,6 +112,18 @@ __device__ __forceinline__ bool wait_flag(const uint32_t* flag, uint32_t want, u
     if (abort && *(volatile const uint32_t*)abort) return false;
     if (ns < 1024) ns <<= 1;
   }
+}
+
+// Thread-block clusters: this CTA's rank, and a barrier over the cluster's
+// threads after which their earlier global writes are seen (L1 aside: read
+// what another CTA wrote with L2 loads).
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
