@@ -261,9 +261,10 @@ typedef struct {
     uint32_t chunk_tokens;    /* a step of the literal pass lists two literal runs, and takes up to 32 literals, per token of this, 32..256, multiple of 32; 0 = 128 */
     uint32_t schedule;        /* ACE_SCHEDULE_*; 0 = automatic; others: ACE_E_INVAL */
     uint64_t wait_timeout_ns; /* bound on each device-side wait; 0 = 2 s */
-    uint32_t copy_width;      /* match copies: 16 = every non-overlapping match above 32 bytes in aligned
-                                 16-byte pieces; 8 = 8-byte words up to 32 bytes, bytewise up to 511,
-                                 16-byte pieces from 512; 0 = the library's choice (16); others: ACE_E_INVAL */
+    uint32_t copy_width;      /* match copies where a warp resolves a block's matches in rounds: 16 = every
+                                 non-overlapping match above 32 bytes in aligned 16-byte pieces; 8 = 16-byte
+                                 pieces from 512 bytes, bytewise below; 0 = the library's choice (16);
+                                 others: ACE_E_INVAL */
     uint32_t reserved;        /* 0 */
 } ace_tune;
 
@@ -276,10 +277,10 @@ typedef struct {
  * read are present (Section 2).  The pass schedule (the default) runs three
  * passes: tokens and literals as persistent launches over the blocks, then
  * the match pass one launch per dependency level (a CTA per block for levels
- * of at most two blocks per SM and blocks of at most 32 KiB, a warp per
- * block otherwise), or, for archives of more than 32 levels, one persistent
- * launch in (level, block) order with bounded waits on source blocks' ready
- * flags.  ACE_SCHEDULE_FUSED does all of it in one persistent launch.
+ * of few blocks and archives of many short matches, a warp per block
+ * otherwise), or, for archives of more than 32 levels, one persistent
+ * launch, a CTA per block, in (level, block) order with bounded waits on
+ * source blocks' ready flags.  ACE_SCHEDULE_FUSED does all of it in one persistent launch.
  * A source block whose level is not below its reader's makes the call
  * report ACE_E_CORRUPT.  tune may be NULL.  Asynchronous; check with
  * ace_sync.

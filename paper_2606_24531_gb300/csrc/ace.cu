@@ -10,6 +10,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "ace.h"
@@ -345,11 +346,13 @@ struct LitMem {
   uint16_t* shift;  // [2 window + 1]
 };
 
-constexpr uint32_t kMatchGroup = 32;  // matches whose records sit in shared memory at a time
+constexpr uint32_t kMatchGroup = 32;  // matches resolved together, one per lane
 // Groups of match records in flight to shared memory (a ring after the
-// group's arrays of sources, destinations, lengths and copy starts).
+// group's own arrays).
 constexpr uint32_t kRecDepth = 4;
-constexpr uint32_t kRecRingOff = 20 * kMatchGroup + 16;
+constexpr uint32_t kRowMax = 64;  // longest match of a group resolved in rows
+constexpr uint32_t kRecRingOff = 16 * kMatchGroup + kMatchGroup * kRowMax / 8;
+static_assert(kRecRingOff >= 20 * kMatchGroup + 16, "room for the rounds' arrays too");
 // The match pass keeps only its match-record area in shared memory.
 constexpr uint32_t kMatchSmem = kRecRingOff + 16 * kMatchGroup * kRecDepth;
 
@@ -425,12 +428,6 @@ __device__ __forceinline__ void fail(const DecodeArgs& a, bool& ok, ace_status c
 // every byte read precedes D and is final when the copy starts.
 __device__ __forceinline__ uint64_t src_index(uint64_t S, uint64_t d, uint32_t len, uint32_t i) {
   return d >= len ? S + i : S + (i % (uint32_t)d);
-}
-
-__device__ __forceinline__ uint64_t read_src(const uint8_t* q, uint32_t w) {
-  uint64_t S = (uint64_t)q[0] | ((uint64_t)q[1] << 8) | ((uint64_t)q[2] << 16) | ((uint64_t)q[3] << 24);
-  if (w == 5) S |= (uint64_t)q[4] << 32;
-  return S;
 }
 
 // The records of block b: whole decodes by the index's prefix count of
@@ -606,7 +603,7 @@ __device__ bool token_block(const DecodeArgs& a, const TokMem& m, uint32_t b, ui
   }
   __syncwarp();
   // a source at or after its destination is caught where sources are read:
-  // match_block and match_small_kernel check every record
+  // match_block and match_cta check every record
   if (ok) {
     bool fin = stream_finished(sn) && stream_finished(so);
     if (!__all_sync(kFull, fin)) fail(a, ok, ACE_E_CORRUPT, b, 40, lane);
@@ -760,21 +757,19 @@ __device__ bool literal_block(const DecodeArgs& a, const LitMem& m, uint32_t b, 
   return ok;
 }
 
-// Matches per lane in a group: match j of the group is on lane j mod 32.
-constexpr uint32_t kLaneMatches = kMatchGroup / 32;
+// Rows of 32 bytes in flight in the copy of a group by rows.
+constexpr uint32_t kRowUnroll = 8;
 // Bytes in flight per lane in the bytewise copy of a round's matches.
 constexpr uint32_t kCopyUnroll = 8;
 // 16-byte pieces in flight per lane in the copy of a round's long matches.
 constexpr uint32_t kLongUnroll = 2;
-// Copy classes: a non-overlapping match of at most kShortMax bytes is copied
-// by one lane in aligned 8-byte words, one of at least the call's long_min
-// bytes by the whole warp in aligned 16-byte pieces, every other one
-// bytewise with the round's other such matches.  long_min is the copy-width
-// knob: kLongMinWide (16-byte pieces for everything above the short class)
-// or kLongMinNarrow (bytewise up to 511 bytes).
-constexpr uint32_t kShortMax = 32;
+// Copy classes of a group resolved in rounds: a non-overlapping match of at
+// least the call's long_min bytes is copied by the whole warp in aligned
+// 16-byte pieces, every other one bytewise with the round's other such
+// matches.  long_min is the copy-width knob: kLongMinWide (16-byte pieces for
+// everything above 32 bytes) or kLongMinNarrow (bytewise up to 511 bytes).
 constexpr uint32_t kLongMinNarrow = 512;
-constexpr uint32_t kLongMinWide = kShortMax + 1;
+constexpr uint32_t kLongMinWide = 33;
 
 // A load of match source bytes.  L1: through the SM's L1 cache, for a pass
 // whose sources were all written by earlier launches or by this warp (one
@@ -783,74 +778,6 @@ constexpr uint32_t kLongMinWide = kShortMax + 1;
 template <bool L1, class T>
 __device__ __forceinline__ T ld_src(const T* p) {
   return L1 ? __ldca(p) : __ldcg(p);
-}
-
-// Source of a short match: the aligned 8-byte words covering [S, S + len).
-template <bool SEEK, bool L1>
-__device__ __forceinline__ void short_load(const DecodeArgs& a, uint64_t S, uint32_t len, uint64_t (&w)[5], uint64_t b,
-                                           const uint8_t* obase) {
-  const uint64_t a0 = S & ~7ull;
-  const uint32_t off = (uint32_t)(S & 7);
-#pragma unroll
-  for (uint32_t k = 0; k < 5; k++) {
-    const uint64_t q = a0 + 8ull * k;
-    w[k] = 0;
-    if (8 * k < off + len) {
-      if (q + 8 <= a.total) {
-        w[k] = ld_src<L1>(reinterpret_cast<const unsigned long long*>(Addr<SEEK>::at(a, q, b, obase)));
-      } else {
-        for (uint32_t t = 0; t < 8 && q + t < a.total; t++)
-          w[k] |= (uint64_t)ld_src<L1>(Addr<SEEK>::at(a, q + t, b, obase)) << (8 * t);
-      }
-    }
-  }
-}
-
-// Bytes sh .. sh + 7 of hi:lo (sh < 8).
-__device__ __forceinline__ uint64_t funnel64(uint64_t lo, uint64_t hi, uint32_t sh) {
-  return sh ? (lo >> (8 * sh)) | (hi << (64 - 8 * sh)) : lo;
-}
-
-// Bytes [lo, hi) of w to the 8-byte aligned p, in the widest aligned stores
-// that fit.  The lanes of a round store to different lines, so every store
-// a lane saves is an L1 and L2 transaction saved.
-__device__ __forceinline__ void store_bytes8(uint8_t* p, uint64_t w, uint32_t lo, uint32_t hi) {
-  uint32_t k = lo;
-  while (k < hi) {
-    if (!(k & 3) && k + 4 <= hi) {
-      *reinterpret_cast<uint32_t*>(p + k) = (uint32_t)(w >> (8 * k));
-      k += 4;
-    } else if (!(k & 1) && k + 2 <= hi) {
-      *reinterpret_cast<uint16_t*>(p + k) = (uint16_t)(w >> (8 * k));
-      k += 2;
-    } else {
-      p[k] = (uint8_t)(w >> (8 * k));
-      k++;
-    }
-  }
-}
-
-// Destination of a short match: aligned 8-byte words where the match covers
-// them, the widest aligned stores that fit at its two ends.  Source byte off + i (off = S mod 8,
-// counted from the first source word) lands at dp[i].
-__device__ __forceinline__ void short_store(uint8_t* dp, uint32_t off, uint32_t len, const uint64_t (&w)[5]) {
-  const uint32_t hd = (uint32_t)(reinterpret_cast<uintptr_t>(dp) & 7);
-  uint8_t* dal = dp - hd;
-  const bool same = off >= hd;  // destination word i starts in source word i, else in word i - 1
-  const uint32_t sh = (off - hd) & 7;
-#pragma unroll
-  for (uint32_t i = 0; i < 5; i++) {
-    const int first = 8 * (int)i - (int)hd;  // match byte held by the word's first byte
-    if (first >= (int)len) break;
-    const uint64_t lo = same ? w[i] : (i ? w[i - 1] : 0ull);
-    const uint64_t hi = same ? (i + 1 < 5 ? w[i + 1] : 0ull) : w[i];
-    const uint64_t word = funnel64(lo, hi, sh);
-    if (first >= 0 && first + 8 <= (int)len) {
-      *reinterpret_cast<uint64_t*>(dal + 8 * i) = word;
-    } else {
-      store_bytes8(dal + 8 * i, word, (uint32_t)max(0, -first), (uint32_t)min(8, (int)len - first));
-    }
-  }
 }
 
 // The 16 bytes at absolute output position q (a multiple of 16, possibly
@@ -903,23 +830,6 @@ __device__ __forceinline__ uint4 shfl_down16(uint4 v, uint32_t d) {
 }
 
 
-// Whether a bit of the 128-bit mask (P0, P1, P2, P3) is set in [lo, hi].
-__device__ __forceinline__ bool any_in(uint32_t P0, uint32_t P1, uint32_t P2, uint32_t P3, uint32_t lo,
-                                       uint32_t hi) {
-  bool any = false;
-#pragma unroll
-  for (uint32_t w = 0; w < 4; w++) {
-    const uint32_t P = w == 0 ? P0 : w == 1 ? P1 : w == 2 ? P2 : P3;
-    const uint32_t wlo = 32 * w, whi = wlo + 31;
-    if (lo > hi || hi < wlo || lo > whi) continue;
-    uint32_t m = P;
-    if (lo > wlo) m &= ~0u << (lo - wlo);
-    if (hi < whi) m &= (2u << (hi - wlo)) - 1u;
-    any |= m != 0;
-  }
-  return any;
-}
-
 // First index i in [0, n) with key(i) > x, for keys that never decrease.
 template <class Key>
 __device__ __forceinline__ uint32_t upper_bound(uint32_t n, uint32_t x, Key key) {
@@ -937,18 +847,30 @@ __device__ __forceinline__ uint32_t upper_bound(uint32_t n, uint32_t x, Key key)
 }
 
 // Match pass of one block (Section 2: a block decodes once the blocks holding
-// its sources are present).  Groups of up to 32 matches: their records are
-// loaded together; with WAIT the source blocks before this one are checked
+// its sources are present).  Groups of 32 matches, a lane each: their records
+// are loaded together; with WAIT the source blocks before this one are checked
 // with overlapping relaxed loads (a bounded wait only for one not yet
 // published); without it (one launch per dependency level) each source
 // block's level must be below this launch's level, else the archive's
-// dependency lists disagree with its matches.  Then the group resolves in
-// rounds.  A match is ready in a round when no
-// pending match of its block writes a byte its source reads; literal bytes
-// are final after the literal pass.  The first pending match is always ready,
-// so every round makes progress, and a round's ready matches read no byte
-// another one writes.  Returns false if a record is corrupt or a wait gave up.
-template <bool SEEK, bool WAIT, bool L1 = !WAIT>
+// dependency lists disagree with its matches.  Returns false if a record is
+// corrupt or a wait gave up.
+//
+// A group whose matches are all short (at most kRowMax bytes) and do not
+// overlap their sources -- text, FASTQ and mixed data are almost only such --
+// is copied in rows: its match bytes laid end to end, 32 consecutive ones per
+// row, a lane's match found by counting start bits in a bit map of the group,
+// so that loads and stores of a row touch the few lines its two or three
+// matches lie in.  Rows go in output order, so a source byte is final unless
+// it lies at or after the first byte of the rows in flight; such bytes wait
+// until those before them are stored.  Any other group is copied in rounds of
+// matches none of which reads bytes another pending one of the group writes
+// (literal bytes are final after the literal pass; the first pending match is
+// always ready, so every round makes progress).
+//
+// Every group went through the rounds, short matches one per lane in 8-byte
+// words whose loads and stores touch 32 lines each (FASTQ 256 MiB: 0.145 ms);
+// by rows 0.106 ms, bound by the latency of a group after another.
+template <bool SEEK, bool WAIT, bool L1 = !WAIT, bool ROWS = true>
 __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint32_t lane, uint32_t epoch,
                             uint32_t nm, uint32_t lvl = 0) {
   // L1: every source was written before the launch or by this warp (one
@@ -956,88 +878,51 @@ __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint3
   // SMs wrote them during the launch and loads go to L2.  Without WAIT, lvl
   // is the block's level: its sources must lie in lower ones.
   constexpr bool kL1 = L1;
+  static_assert(kMatchGroup == 32, "one match per lane");
   bool ok = true, bad = false;
   const uint64_t B = (uint64_t)1 << a.log2B, bstart = (uint64_t)b << a.log2B;
   const uint32_t blen = (uint32_t)min(B, a.total - bstart);
+  const uint32_t lt = lanemask_lt(), le = lt | 1u << lane;
   uint8_t* obase = SEEK ? a.out + slot_base(a, b) : a.out + bstart;
   const uint4* rec = reinterpret_cast<const uint4*>(recs_of<SEEK>(a, b));
-  uint64_t* gS = reinterpret_cast<uint64_t*>(gm);                 // [kMatchGroup] sources
-  uint32_t* gD = reinterpret_cast<uint32_t*>(gS + kMatchGroup);   // [kMatchGroup] destinations in the block
-  uint32_t* gL = gD + kMatchGroup;                                // [kMatchGroup] lengths
-  uint32_t* gX = gL + kMatchGroup;                                // [kMatchGroup + 1] starts in a round's copy
   // records reach a ring of kRecDepth groups by cp.async, kRecDepth - 1
   // groups ahead of the one resolving; lane j copies and later reads record
   // j of each group, so no lane reads another's copy
   uint4* const rring = reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(gm) + kRecRingOff);
   auto issue = [&](uint32_t g) {  // one commit group per call, empty past the last record
-    const uint32_t t = g * kMatchGroup;
-#pragma unroll
-    for (uint32_t q = 0; q < kLaneMatches; q++) {
-      const uint32_t j = lane + 32 * q;
-      if (t < nm && j < min(kMatchGroup, nm - t)) cp_async16(rring + (g % kRecDepth) * kMatchGroup + j, rec + t + j);
-    }
+    const uint32_t t = g * kMatchGroup + lane;
+    if (t < nm) cp_async16(rring + (g % kRecDepth) * kMatchGroup + lane, rec + t);
     cp_async_commit();
   };
 #pragma unroll
   for (uint32_t g = 0; g + 1 < kRecDepth; g++) issue(g);
   for (uint32_t t0 = 0, g = 0; ok && t0 < nm; t0 += kMatchGroup, g++) {
-    const uint32_t gn = min(kMatchGroup, nm - t0);
     issue(g + kRecDepth - 1);
     cp_async_wait<kRecDepth - 1>();  // group g has landed
-    uint4 r[kLaneMatches];
-#pragma unroll
-    for (uint32_t q = 0; q < kLaneMatches; q++) {
-      const uint32_t j = lane + 32 * q;
-      r[q] = j < gn ? rring[(g % kRecDepth) * kMatchGroup + j] : make_uint4(0, 0, 0, 0);
-    }
-    uint32_t pend = 0;
-#pragma unroll
-    for (uint32_t q = 0; q < kLaneMatches; q++) {
-      const uint32_t j = lane + 32 * q;
-      if (j >= gn) continue;
-      const uint64_t S = (uint64_t)r[q].x | ((uint64_t)r[q].y << 32);
-      uint32_t ml = r[q].w;
-      if (ml && (S >= bstart + r[q].z || (uint64_t)r[q].z + ml > blen)) {  // checked again: the token pass may have failed
-        bad = true;
-        ml = 0;
-      }
-      gS[j] = S;
-      gD[j] = r[q].z;
-      gL[j] = ml;
-      if (ml) pend |= 1u << q;
+    uint4 r = make_uint4(0, 0, 0, 0);
+    if (t0 + lane < nm) r = rring[(g % kRecDepth) * kMatchGroup + lane];
+    const uint64_t S = (uint64_t)r.x | ((uint64_t)r.y << 32);
+    const uint32_t D = r.z;
+    uint32_t L = r.w;
+    if (L && (S >= bstart + D || (uint64_t)D + L > blen)) {  // checked again: the token pass may have failed
+      bad = true;
+      L = 0;
     }
     if (__any_sync(kFull, bad)) fail(a, ok, ACE_E_CORRUPT, b, 37, lane);
     if (!ok) break;
-    __syncwarp();
 
     // source blocks before this one: all flags loaded, then compared
-    uint32_t f0[kLaneMatches], f1[kLaneMatches], rng[kLaneMatches];
-    uint32_t ext = 0;
-#pragma unroll
-    for (uint32_t q = 0; q < kLaneMatches; q++) {
-      f0[q] = f1[q] = epoch;
-      rng[q] = 1;  // lo = 1 > hi = 0: no match of the group feeds this one
-      if (!(pend >> q & 1)) continue;
-      const uint32_t j = lane + 32 * q;
-      const uint64_t S = gS[j], D = bstart + gD[j];
-      const uint64_t rend = S + min((uint64_t)gL[j], D - S);
-      const uint64_t k0 = S >> a.log2B;
-      if (k0 < b) {  // blocks k0 .. k1 hold the bytes before this block
-        const uint64_t k1 = min((rend - 1) >> a.log2B, (uint64_t)b - 1);
-        ext |= 1u << q;
-        if (WAIT) {  // flags that other warps publish during the launch
-          f0[q] = ld_relaxed(a.ready + k0);
-          f1[q] = k1 != k0 ? ld_relaxed(a.ready + k1) : f0[q];
-        } else {  // levels, fixed for the launch: through the read-only cache
-          f0[q] = __ldg(a.level + k0);
-          f1[q] = k1 != k0 ? __ldg(a.level + k1) : f0[q];
-        }
-      }
-      if (rend > bstart) {  // bytes of this block: the group's matches writing them
-        const uint32_t s_rel = S > bstart ? (uint32_t)(S - bstart) : 0u, e_rel = (uint32_t)(rend - bstart);
-        const uint32_t lo = upper_bound(j, s_rel, [&](uint32_t i) { return gD[i] + gL[i]; });
-        const uint32_t hi = upper_bound(j, e_rel - 1, [&](uint32_t i) { return gD[i]; });  // first with gD >= e_rel
-        rng[q] = hi > lo ? (lo | ((hi - 1) << 8)) : 1u;
+    const uint64_t dist = bstart + D - S, rend = S + min((uint64_t)L, dist), k0 = S >> a.log2B;
+    const uint64_t k1 = min((rend - 1) >> a.log2B, (uint64_t)b - 1);  // blocks k0 .. k1 hold the bytes before this block
+    const bool ext = L && k0 < b;
+    uint32_t f0 = epoch, f1 = epoch;
+    if (ext) {
+      if (WAIT) {  // flags that other warps publish during the launch
+        f0 = ld_relaxed(a.ready + k0);
+        f1 = k1 != k0 ? ld_relaxed(a.ready + k1) : f0;
+      } else {  // levels, fixed for the launch: through the read-only cache
+        f0 = __ldg(a.level + k0);
+        f1 = k1 != k0 ? __ldg(a.level + k1) : f0;
       }
     }
     if (WAIT) {
@@ -1045,205 +930,516 @@ __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint3
       // a source block must sit at a lower dependency level (work lists are
       // in level order, so it was handed out before this block and the wait
       // ends); the block cache keeps no levels and skips this check
-      const uint32_t my_level = a.level ? __ldg(a.level + b) : 0u;
-#pragma unroll
-      for (uint32_t q = 0; q < kLaneMatches; q++) {
-        if (!(ext >> q & 1)) continue;
-        const uint32_t j = lane + 32 * q;
-        const uint64_t S = gS[j], D = bstart + gD[j];
-        const uint64_t rend = S + min((uint64_t)gL[j], D - S);
-        const uint64_t k0 = S >> a.log2B, k1 = min((rend - 1) >> a.log2B, (uint64_t)b - 1);
+      if (ext) {
+        bool low = true;
         if (a.level) {
-          bool low = true;
+          const uint32_t my_level = __ldg(a.level + b);
           for (uint64_t k = k0; k <= k1; k++) low &= __ldg(a.level + k) < my_level;
-          if (!low) {
-            bad = true;  // the dependency table disagrees with the matches
-            continue;
-          }
         }
         if (SEEK && a.closure_flags) {
           // every source block must be a member of this seek's closure: its
           // flag carries the call's epoch (pending or published).  Anything
           // else means the dependency table disagrees with the matches.
-          bool member = (f0[q] & ~kPendingFlag) == epoch && (f1[q] & ~kPendingFlag) == epoch;
-          for (uint64_t k = k0 + 1; member && k < k1; k++)
-            member = (ld_relaxed(a.ready + k) & ~kPendingFlag) == epoch;
-          if (!member) {
-            bad = true;
-            continue;
-          }
+          low &= (f0 & ~kPendingFlag) == epoch && (f1 & ~kPendingFlag) == epoch;
+          for (uint64_t k = k0 + 1; low && k < k1; k++) low = (ld_relaxed(a.ready + k) & ~kPendingFlag) == epoch;
         }
-        if (f0[q] == epoch && f1[q] == epoch && k1 <= k0 + 1) continue;  // blocks between them: the bounded wait
-        for (uint64_t k = k0; k <= k1 && !timeout; k++)
-          if (!wait_flag(a.ready + k, epoch, a.timeout_ns, &a.sh->status)) timeout = true;
+        if (!low) bad = true;  // the dependency table disagrees with the matches
+        else if (f0 != epoch || f1 != epoch || k1 > k0 + 1)  // blocks between them: the bounded wait
+          for (uint64_t k = k0; k <= k1 && !timeout; k++)
+            if (!wait_flag(a.ready + k, epoch, a.timeout_ns, &a.sh->status)) timeout = true;
       }
       if (__any_sync(kFull, bad)) fail(a, ok, ACE_E_CORRUPT, b, 39, lane);
       if (__any_sync(kFull, timeout)) fail(a, ok, ACE_E_TIMEOUT, b, 38, lane);
       if (!ok) break;
-      if (__any_sync(kFull, ext != 0)) fence_acquire();
+      if (__any_sync(kFull, ext)) fence_acquire();
       __syncwarp();  // any lane may copy a match whose flags another lane checked
     }
     // without WAIT the level check below need not hold up the copies: a
     // corrupt archive fails the call whatever bytes they wrote
-    uint32_t chk = ext;
 
-    while (__any_sync(kFull, pend != 0)) {
-      // pending matches of the group, one bit each (words past the group's size are zero)
-      const uint32_t P0 = __ballot_sync(kFull, pend & 1u);
-      const uint32_t P1 = kLaneMatches > 1 ? __ballot_sync(kFull, pend & 2u) : 0u;
-      const uint32_t P2 = kLaneMatches > 2 ? __ballot_sync(kFull, pend & 4u) : 0u;
-      const uint32_t P3 = kLaneMatches > 3 ? __ballot_sync(kFull, pend & 8u) : 0u;
-      uint32_t go = 0;
+    if (ROWS && __all_sync(kFull, L <= kRowMax && (!L || (dist >= L && (!SEEK || k0 == (S + L - 1) >> a.log2B))))) {
+      // rows.  Per match: where byte c of the group's bytes comes from (address
+      // of the source less the match's start among them) and goes to, and the
+      // source's place in the block (below 0: an earlier block, always final).
+      uint4* const row = reinterpret_cast<uint4*>(gm);
+      uint32_t* const bits = reinterpret_cast<uint32_t*>(row + kMatchGroup);
 #pragma unroll
-      for (uint32_t q = 0; q < kLaneMatches; q++)
-        if ((pend >> q & 1) && !any_in(P0, P1, P2, P3, rng[q] & 0xffu, rng[q] >> 8)) go |= 1u << q;
-      // classes: short (one lane), long (the warp), the rest bytewise
-      uint32_t sgo = 0, lgo = 0;
-#pragma unroll
-      for (uint32_t q = 0; q < kLaneMatches; q++) {
-        if (!(go >> q & 1)) continue;
-        const uint32_t j = lane + 32 * q, ml = gL[j];
-        if (bstart + gD[j] - gS[j] < ml) continue;  // overlapping: bytewise
-        if (ml <= kShortMax) sgo |= 1u << q;
-        else if (ml >= a.long_min) lgo |= 1u << q;
+      for (uint32_t k = 0; k < kRowMax / 32; k++) bits[32 * k + lane] = 0;
+      const uint32_t incl = warp_incl_sum(L, lane), X = incl - L, T = __shfl_sync(kFull, incl, 31);
+      const uint32_t have = __ballot_sync(kFull, L != 0);
+      if (L) {
+        const uint64_t from = reinterpret_cast<uintptr_t>(Addr<SEEK>::at(a, S, b, obase)) - X;
+        const int32_t rel = (int32_t)max((int64_t)(S - bstart), -(int64_t)(1 << 30));
+        row[__popc(have & lt)] = make_uint4((uint32_t)from, (uint32_t)(from >> 32), D - X, (uint32_t)(rel - (int32_t)X));
       }
-      if (sgo) {  // short: the next match's loads go out before the previous one's stores
-        uint64_t cur[5], nxt[5];
-        uint32_t jc = lane + 32 * (__ffs(sgo) - 1), rest = sgo & (sgo - 1);
-        short_load<SEEK, kL1>(a, gS[jc], gL[jc], cur, b, obase);
-        while (true) {
-          const uint32_t jn = rest ? lane + 32 * (__ffs(rest) - 1) : 0u;
-          if (rest) short_load<SEEK, kL1>(a, gS[jn], gL[jn], nxt, b, obase);
-          short_store(obase + gD[jc], (uint32_t)(gS[jc] & 7), gL[jc], cur);
-          if (!rest) break;
-          rest &= rest - 1;
-          jc = jn;
+      __syncwarp();
+      if (L) atomicOr(bits + (X >> 5), 1u << (X & 31));
+      __syncwarp();
+      uint32_t rank = ~0u;  // the match before the row's first start
+      for (uint32_t c0 = 0; c0 < T; c0 += 32 * kRowUnroll) {
+        uint32_t v[kRowUnroll], dst[kRowUnroll], pend = 0;
+        const uint32_t rank0 = rank;
+        // bytes at or after F are written by the rows in flight
+        const int32_t F = (int32_t)(row[rank + (bits[c0 >> 5] & 1)].z + c0);
 #pragma unroll
-          for (uint32_t k = 0; k < 5; k++) cur[k] = nxt[k];
+        for (uint32_t u = 0; u < kRowUnroll; u++) {
+          if (c0 + 32 * u >= T) break;
+          const uint32_t c = c0 + 32 * u + lane, w = bits[(c0 >> 5) + u];
+          const uint4 m = row[rank + __popc(w & le)];
+          rank += __popc(w);
+          dst[u] = m.z + c;
+          if (c < T) {
+            if ((int32_t)(m.w + c) < F)
+              v[u] = ld_src<kL1>(reinterpret_cast<const uint8_t*>(((uint64_t)m.y << 32 | m.x) + c));
+            else
+              pend |= 1u << u;
+          }
         }
-      }
-      if (__any_sync(kFull, lgo != 0)) {
-        // long: the round's long matches at once, laid end to end as the
-        // aligned 16-byte source pieces each one needs (its destination
-        // pieces plus one); piece c and piece c + 1 build destination piece
-        // c.  A window gives lane l pieces c0 + 32 u + l, kLongUnroll in
-        // flight; piece c + 1 is the next lane's, or for lane 31 the next
-        // u's lane 0; the window's very last piece only serves as that
-        // source, and the next window starts on it.  Each lane finds its
-        // pieces' match by walking forward (pieces only grow).
-        static_assert(kLaneMatches == 1, "one match per lane");
-        const bool mine = lgo & 1;
-        const uint32_t hd0 = gD[lane] & 15;  // block bases are 16-byte aligned
-        const uint32_t np = mine ? ((hd0 + gL[lane] + 15) >> 4) + 1 : 0u;
-        const uint32_t incl = warp_incl_sum(np, lane);
-        gX[lane] = incl - np;
-        if (lane == 31) gX[32] = incl;
-        const uint32_t T = __shfl_sync(kFull, incl, 31);
-        __syncwarp();
-        uint32_t jc = 0;
-        for (uint32_t c0 = 0; c0 < T; c0 += 32 * kLongUnroll - 1) {
-          uint4 A[kLongUnroll];
-          uint32_t jp[kLongUnroll];
 #pragma unroll
-          for (uint32_t u = 0; u < kLongUnroll; u++) {
-            const uint32_t c = c0 + 32 * u + lane;
-            jp[u] = 0xffffffffu;
-            A[u] = make_uint4(0, 0, 0, 0);
-            if (c < T) {
-              while (gX[jc + 1] <= c) jc++;
-              const uint32_t pc = c - gX[jc];
-              jp[u] = jc | (pc << 5);
-              const int64_t s0 = (int64_t)gS[jc] - (int64_t)(gD[jc] & 15);
-              A[u] = ld16_abs<SEEK, kL1>(a, (s0 & ~(int64_t)15) + 16 * (int64_t)pc, b, obase);
+        for (uint32_t u = 0; u < kRowUnroll; u++)
+          if (c0 + 32 * u + lane < T && !(pend >> u & 1)) obase[dst[u]] = (uint8_t)v[u];
+        __syncwarp();
+        const uint32_t rows = __reduce_or_sync(kFull, pend);
+        if (!rows) continue;
+        uint32_t k = rank0;  // the rows that wait, one after another
+        for (uint32_t u = 0; rows >> u; u++) {
+          const uint32_t c = c0 + 32 * u + lane, w = bits[(c0 >> 5) + u];
+          if (rows >> u & 1) {
+            const uint4 m = row[k + __popc(w & le)];
+            bool p = pend >> u & 1;
+            while (__any_sync(kFull, p)) {
+              const uint32_t first = __reduce_min_sync(kFull, p ? m.z + c : ~0u);  // not yet written
+              if (p && (int32_t)(m.w + c) < (int32_t)first) {
+                obase[m.z + c] = ld_src<kL1>(reinterpret_cast<const uint8_t*>(((uint64_t)m.y << 32 | m.x) + c));
+                p = false;
+              }
+              __syncwarp();
             }
           }
+          k += __popc(w);
+        }
+      }
+    } else {
+      uint64_t* gS = reinterpret_cast<uint64_t*>(gm);                 // sources
+      uint32_t* gD = reinterpret_cast<uint32_t*>(gS + kMatchGroup);   // destinations in the block
+      uint32_t* gL = gD + kMatchGroup;                                // lengths
+      uint32_t* gX = gL + kMatchGroup;                                // [kMatchGroup + 1] starts in a round's copy
+      gS[lane] = S;
+      gD[lane] = D;
+      gL[lane] = L;
+      __syncwarp();
+      uint32_t feeds = 0;  // the group's matches that write bytes this one's source reads
+      if (L && rend > bstart) {
+        const uint32_t s_rel = S > bstart ? (uint32_t)(S - bstart) : 0u, e_rel = (uint32_t)(rend - bstart);
+        const uint32_t lo = upper_bound(lane, s_rel, [&](uint32_t i) { return gD[i] + gL[i]; });
+        const uint32_t hi = upper_bound(lane, e_rel - 1, [&](uint32_t i) { return gD[i]; });  // first with gD >= e_rel
+        if (hi > lo) feeds = ((1u << hi) - 1) & ~((1u << lo) - 1);  // hi <= lane <= 31
+      }
+      uint32_t pend = __ballot_sync(kFull, L != 0);
+      while (pend) {
+        const bool go = (pend >> lane & 1) && !(pend & feeds);
+        const bool lgo = go && L >= a.long_min && dist >= L;
+        if (__any_sync(kFull, lgo)) {
+          // long: the round's long matches at once, laid end to end as the
+          // aligned 16-byte source pieces each one needs (its destination
+          // pieces plus one); piece c and piece c + 1 build destination piece
+          // c.  A window gives lane l pieces c0 + 32 u + l, kLongUnroll in
+          // flight; piece c + 1 is the next lane's, or for lane 31 the next
+          // u's lane 0; the window's very last piece only serves as that
+          // source, and the next window starts on it.  Each lane finds its
+          // pieces' match by walking forward (pieces only grow).
+          const uint32_t hd0 = D & 15;  // block bases are 16-byte aligned
+          const uint32_t np = lgo ? ((hd0 + L + 15) >> 4) + 1 : 0u;
+          const uint32_t incl = warp_incl_sum(np, lane);
+          gX[lane] = incl - np;
+          if (lane == 31) gX[32] = incl;
+          const uint32_t T = __shfl_sync(kFull, incl, 31);
+          __syncwarp();
+          uint32_t jc = 0;
+          for (uint32_t c0 = 0; c0 < T; c0 += 32 * kLongUnroll - 1) {
+            uint4 A[kLongUnroll];
+            uint32_t jp[kLongUnroll];
 #pragma unroll
-          for (uint32_t u = 0; u < kLongUnroll; u++) {
-            const uint4 nb = shfl_down16(A[u], 1);
-            const uint32_t un = u + 1 < kLongUnroll ? u + 1 : u;
-            const uint4 n0 = make_uint4(__shfl_sync(kFull, A[un].x, 0), __shfl_sync(kFull, A[un].y, 0),
-                                        __shfl_sync(kFull, A[un].z, 0), __shfl_sync(kFull, A[un].w, 0));
-            const uint4 B = lane == 31 ? n0 : nb;
-            if (jp[u] == 0xffffffffu || (u + 1 == kLongUnroll && lane == 31)) continue;
-            const uint32_t j = jp[u] & 31, pc = jp[u] >> 5, ml = gL[j];
-            const uint32_t hd = gD[j] & 15;
-            if (pc >= ((hd + ml + 15) >> 4)) continue;  // the trailing source piece stores nothing
-            const uint4 v = funnel128(A[u], B, (uint32_t)(((int64_t)gS[j] - (int64_t)hd) & 15));
-            uint8_t* dp = obase + gD[j] - hd + 16ull * pc;
-            const int first = 16 * (int)pc - (int)hd;  // match byte held by the piece's first byte
-            if (first >= 0 && first + 16 <= (int)ml)
-              *reinterpret_cast<uint4*>(dp) = v;
-            else
-              store_bytes16(dp, v, (uint32_t)max(0, -first), (uint32_t)min(16, (int)ml - first));
+            for (uint32_t u = 0; u < kLongUnroll; u++) {
+              const uint32_t c = c0 + 32 * u + lane;
+              jp[u] = 0xffffffffu;
+              A[u] = make_uint4(0, 0, 0, 0);
+              if (c < T) {
+                while (gX[jc + 1] <= c) jc++;
+                const uint32_t pc = c - gX[jc];
+                jp[u] = jc | (pc << 5);
+                const int64_t s0 = (int64_t)gS[jc] - (int64_t)(gD[jc] & 15);
+                A[u] = ld16_abs<SEEK, kL1>(a, (s0 & ~(int64_t)15) + 16 * (int64_t)pc, b, obase);
+              }
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < kLongUnroll; u++) {
+              const uint4 nb = shfl_down16(A[u], 1);
+              const uint32_t un = u + 1 < kLongUnroll ? u + 1 : u;
+              const uint4 n0 = make_uint4(__shfl_sync(kFull, A[un].x, 0), __shfl_sync(kFull, A[un].y, 0),
+                                          __shfl_sync(kFull, A[un].z, 0), __shfl_sync(kFull, A[un].w, 0));
+              const uint4 B = lane == 31 ? n0 : nb;
+              if (jp[u] == 0xffffffffu || (u + 1 == kLongUnroll && lane == 31)) continue;
+              const uint32_t j = jp[u] & 31, pc = jp[u] >> 5, ml = gL[j];
+              const uint32_t hd = gD[j] & 15;
+              if (pc >= ((hd + ml + 15) >> 4)) continue;  // the trailing source piece stores nothing
+              const uint4 v = funnel128(A[u], B, (uint32_t)(((int64_t)gS[j] - (int64_t)hd) & 15));
+              uint8_t* dp = obase + gD[j] - hd + 16ull * pc;
+              const int first = 16 * (int)pc - (int)hd;  // match byte held by the piece's first byte
+              if (first >= 0 && first + 16 <= (int)ml)
+                *reinterpret_cast<uint4*>(dp) = v;
+              else
+                store_bytes16(dp, v, (uint32_t)max(0, -first), (uint32_t)min(16, (int)ml - first));
+            }
+          }
+          __syncwarp();
+        }
+        // the rest laid end to end in group order: gX[j] is where match j
+        // starts, gX[kMatchGroup] the total
+        const bool bgo = go && !lgo;
+        if (__any_sync(kFull, bgo)) {
+          const uint32_t len = bgo ? L : 0u;
+          const uint32_t incl = warp_incl_sum(len, lane), total = __shfl_sync(kFull, incl, 31);
+          gX[lane] = incl - len;
+          if (lane == 0) gX[kMatchGroup] = total;
+          __syncwarp();
+          // lane l copies bytes c + 32 u + l: consecutive lanes read and write
+          // consecutive bytes of a match, kCopyUnroll loads in flight before
+          // their stores (a round's ready matches read no byte it writes); the
+          // lane's match index only moves forward
+          uint32_t jc = 0;
+          for (uint32_t c = 0; c < total; c += 32 * kCopyUnroll) {
+            uint8_t v[kCopyUnroll];
+            uint32_t dp[kCopyUnroll];
+#pragma unroll
+            for (uint32_t u = 0; u < kCopyUnroll; u++) {
+              const uint32_t p = c + 32 * u + lane;
+              dp[u] = ~0u;
+              if (p < total) {
+                while (gX[jc + 1] <= p) jc++;
+                const uint32_t i = p - gX[jc], ml = gL[jc];
+                const uint64_t Sj = gS[jc], d = bstart + gD[jc] - Sj;
+                v[u] = ld_src<kL1>(Addr<SEEK>::at(a, src_index(Sj, d, ml, i), b, obase));
+                dp[u] = gD[jc] + i;
+              }
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < kCopyUnroll; u++)
+              if (dp[u] != ~0u) obase[dp[u]] = v[u];
           }
         }
-        __syncwarp();
-      }
-      // the rest laid end to end in group order: gX[j] is where match j
-      // starts, gX[kMatchGroup] the total
-      const uint32_t bgo = go & ~sgo & ~lgo;
-      if (!__any_sync(kFull, bgo != 0)) {  // none this round
-        pend &= ~go;
+        pend &= ~__ballot_sync(kFull, go);
         __syncwarp();  // the round's copies are seen by the next round's loads
-        continue;
       }
-      uint32_t carry = 0;
-#pragma unroll
-      for (uint32_t q = 0; q < kLaneMatches; q++) {
-        const uint32_t j = lane + 32 * q;
-        const uint32_t len = (bgo >> q & 1) ? gL[j] : 0u;
-        const uint32_t incl = warp_incl_sum(len, lane);
-        gX[j] = carry + incl - len;
-        carry += __shfl_sync(kFull, incl, 31);
-      }
-      if (lane == 0) gX[kMatchGroup] = carry;
-      __syncwarp();
-      // lane l copies bytes c + 32 u + l: consecutive lanes read and write
-      // consecutive bytes of a match, kCopyUnroll loads in flight before
-      // their stores (a round's ready matches read no byte it writes); the
-      // lane's match index only moves forward
-      uint32_t jc = 0;
-      for (uint32_t c = 0; c < carry; c += 32 * kCopyUnroll) {
-        uint8_t v[kCopyUnroll];
-        uint8_t* dp[kCopyUnroll];
-#pragma unroll
-        for (uint32_t u = 0; u < kCopyUnroll; u++) {
-          const uint32_t p = c + 32 * u + lane;
-          dp[u] = nullptr;
-          if (p < carry) {
-            while (gX[jc + 1] <= p) jc++;
-            const uint32_t i = p - gX[jc], ml = gL[jc];
-            const uint64_t S = gS[jc], d = bstart + gD[jc] - S;
-            v[u] = ld_src<kL1>(Addr<SEEK>::at(a, src_index(S, d, ml, i), b, obase));
-            dp[u] = obase + gD[jc] + i;
-          }
-        }
-#pragma unroll
-        for (uint32_t u = 0; u < kCopyUnroll; u++)
-          if (dp[u]) *dp[u] = v[u];
-      }
-      pend &= ~go;
-      __syncwarp();
     }
     if (!WAIT) {
-#pragma unroll
-      for (uint32_t q = 0; q < kLaneMatches; q++) {
-        if (!(chk >> q & 1)) continue;
-        if (f0[q] >= lvl || f1[q] >= lvl) bad = true;
-        const uint32_t j = lane + 32 * q;
-        const uint64_t S = gS[j], D = bstart + gD[j];
-        const uint64_t rend = S + min((uint64_t)gL[j], D - S);
-        const uint64_t k0 = S >> a.log2B, k1 = min((rend - 1) >> a.log2B, (uint64_t)b - 1);
+      if (ext) {
+        if (f0 >= lvl || f1 >= lvl) bad = true;
         for (uint64_t k = k0 + 1; k < k1; k++)  // a source spanning more than two earlier blocks
           if (__ldg(a.level + k) >= lvl) bad = true;
       }
       if (__any_sync(kFull, bad)) fail(a, ok, ACE_E_CORRUPT, b, 39, lane);
-      __syncwarp();
     }
+    __syncwarp();  // the next group reuses the arrays
   }
   cp_async_wait<0>();  // no record copy may land after the caller reuses the area
   __syncwarp();
   return ok;
+}
+
+// The match pass of one block by a CTA, in windows of kCtaWindow bytes (one for
+// blocks of at most that).  Every byte of the window gets a 16-bit entry in
+// shared memory: 0x8000 | its value where that is known (a literal, or a match
+// byte whose source lies before the window, which is final), else the address
+// of the entry of the byte it copies (twice its place in the window).  A match byte equals the byte one distance
+// before it (Section 2, the sequential LZ77 copy; overlapping matches too), so
+// entries form chains that end at known ones.  The warps set the entries a
+// group of 32 matches each, in rows of 32 match bytes (as match_block, but in
+// any order: an entry waits for nothing), then every thread follows the chains
+// of its 16 bytes and stores them.  Chains longer than kHops (matches of one
+// match after another, runs) are shortened by pointer jumping first: every
+// entry takes its target's, which ends all of them in log2 of the length.
+//
+// No match waits for another, so a block is a few thousand cycles of
+// independent loads over 8 or 16 warps where the warp-per-block pass is a
+// chain of its groups, and whole sectors are written.  It pays for blocks of
+// many short matches (text 128 MiB: 0.25 ms, 0.38 by warps in rounds, 0.33 in
+// rows; bound by issue, about 26,000 warp instructions a 16 KiB block) and
+// wherever blocks are few: levels of 64 blocks 6 to 18 us (9 to 25 by 512
+// threads a block with a sweep of pointer jumping per step), a FASTQ seek's
+// match pass 0.040 ms (0.094 by a warp per block), 1900 blocks of a cached
+// batch 0.11 (0.21), 192 uneven objects 0.49 (0.79).
+// With WAIT a source block before this one may not be published yet: a bounded
+// wait; without it its level must be below lvl.  Returns false, for the whole
+// CTA, if a record is corrupt or a wait gave up (recorded).
+constexpr uint32_t kCtaWindow = 16384;
+constexpr uint32_t kCtaThreads = 512;                       // at most
+constexpr uint32_t kCtaRowBytes = 2048;                     // match bytes whose starts the bit map holds
+constexpr uint32_t kCtaWarpSmem = 16 * 32 + kCtaRowBytes / 8;
+constexpr uint32_t kCtaUnroll = 4;                          // rows in flight per warp (a vector of the map's words)
+constexpr uint32_t kHops = 6;
+
+// Threads of a CTA: 256, or 512 where blocks are few and each one's time
+// counts; less for small blocks.
+__host__ __device__ inline uint32_t cta_threads(uint32_t log2B, bool few) {
+  return log2B >= 12 ? few ? 512 : 256 : log2B >= 10 ? 128 : 64;
+}
+// (enough for smaller blocks of the same launch too)
+__host__ __device__ inline uint32_t cta_smem_bytes(uint32_t log2B, uint32_t threads) {
+  return 2 * (log2B >= 14 ? kCtaWindow : 1u << log2B) + threads / 32 * kCtaWarpSmem;
+}
+
+template <bool SEEK, bool WAIT>
+__device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32_t nm, uint32_t epoch, uint32_t lvl) {
+  __shared__ uint32_t s_group;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+  const uint32_t lt = lanemask_lt(), le = lt | 1u << lane;
+  const uint64_t B = 1ull << a.log2B, bstart = (uint64_t)b << a.log2B;
+  const uint32_t blen = (uint32_t)min(B, a.total - bstart);
+  uint8_t* obase = SEEK ? a.out + slot_base(a, b) : a.out + bstart;
+  const uint4* rec = reinterpret_cast<const uint4*>(recs_of<SEEK>(a, b));
+  uint16_t* e = reinterpret_cast<uint16_t*>(smem);
+  const uint32_t ebase = (uint32_t)__cvta_generic_to_shared(e);
+  // groups of 32 matches, a warp each; with fewer groups than warps, several
+  // warps each, sharing the group's bytes
+  const uint32_t ng = (nm + 31) / 32, split = ng ? max(1u, nw / ng) : 1u;
+  const uint32_t part = wid % split, step = nw / split;
+  uint4* row = reinterpret_cast<uint4*>(smem + 2 * min((uint32_t)B, kCtaWindow) + wid * kCtaWarpSmem);
+  uint32_t* bits = reinterpret_cast<uint32_t*>(row + 32);
+  uint32_t first = 0;  // the group that reaches the window
+  for (uint32_t w0 = 0; w0 < blen; w0 += kCtaWindow) {
+    const uint32_t wn = min(kCtaWindow, blen - w0);
+    uint32_t g = first + wid / split;
+    if (wid >= step * split) g = ng;  // a warp left over
+    uint4 rn;  // records one group ahead
+    auto fetch = [&](uint32_t q) {
+      return 32 * q + lane < nm ? __ldcg(rec + 32 * q + lane) : make_uint4(0, 0, 0, 0);
+    };
+    rn = fetch(g);
+    // every byte known as the literal pass left it; match bytes are set next
+    const uint8_t* wbase = obase + w0;
+    for (uint32_t j0 = 16 * tid; j0 < wn; j0 += 16 * nt * 4) {
+      uint4 v[4];
+#pragma unroll
+      for (uint32_t u = 0; u < 4; u++) {
+        const uint32_t j = j0 + 16 * nt * u;
+        v[u] = make_uint4(0, 0, 0, 0);
+        if (j + 16 <= wn) {
+          v[u] = __ldcg(reinterpret_cast<const uint4*>(wbase + j));
+        } else if (j < wn) {
+          uint32_t x[4] = {0, 0, 0, 0};
+#pragma unroll
+          for (uint32_t k = 0; k < 16; k++)
+            if (j + k < wn) x[k >> 2] |= (uint32_t)__ldcg(wbase + j + k) << (8 * (k & 3));
+          v[u] = make_uint4(x[0], x[1], x[2], x[3]);
+        }
+      }
+#pragma unroll
+      for (uint32_t u = 0; u < 4; u++) {
+        const uint32_t j = j0 + 16 * nt * u;
+        if (j >= wn) continue;
+        uint4* e4 = reinterpret_cast<uint4*>(e + j);
+        e4[0] = make_uint4(__byte_perm(v[u].x, 0x80u, 0x4140), __byte_perm(v[u].x, 0x80u, 0x4342),
+                           __byte_perm(v[u].y, 0x80u, 0x4140), __byte_perm(v[u].y, 0x80u, 0x4342));
+        e4[1] = make_uint4(__byte_perm(v[u].z, 0x80u, 0x4140), __byte_perm(v[u].z, 0x80u, 0x4342),
+                           __byte_perm(v[u].w, 0x80u, 0x4140), __byte_perm(v[u].w, 0x80u, 0x4342));
+      }
+    }
+    if (tid == 0) s_group = first;
+    __syncthreads();
+
+    bool bad = false, timeout = false;
+    uint32_t last = first;
+    for (; g < ng; g += step) {
+      const uint4 r = rn;
+      rn = fetch(g + step);
+      const uint64_t S = (uint64_t)r.x | ((uint64_t)r.y << 32);
+      const uint32_t D = r.z;
+      uint32_t L = r.w;
+      if (L && (S >= bstart + D || (uint64_t)D + L > blen)) {  // a source precedes its match, which stays in the block
+        bad = true;
+        L = 0;
+      }
+      if (__shfl_sync(kFull, D, 0) >= w0 + wn) break;  // (destinations ascend) past the window
+      last = g;
+      const uint64_t dist = bstart + D - S;
+      if (L && S < bstart) {  // the blocks before this one that it reads
+        const uint32_t k0 = (uint32_t)(S >> a.log2B);
+        const uint32_t k1 = (uint32_t)((min(S + min((uint64_t)L, dist), bstart) - 1) >> a.log2B);
+        for (uint32_t k = k0; k <= k1; k++) {
+          if (!WAIT) {
+            bad |= __ldg(a.level + k) >= lvl;
+            continue;
+          }
+          // at a lower level (work lists are in level order, so the wait ends;
+          // the block cache keeps no levels), and a member of a seek's closure
+          // (its flag carries the call's epoch, pending or published)
+          if (a.level && __ldg(a.level + k) >= __ldg(a.level + b)) bad = true;
+          const uint32_t f = ld_relaxed(a.ready + k);
+          if (SEEK && a.closure_flags && (f & ~kPendingFlag) != epoch) bad = true;
+          if (!bad && !timeout && f != epoch && !wait_flag(a.ready + k, epoch, a.timeout_ns, &a.sh->status)) timeout = true;
+        }
+        if (bad || timeout) L = 0;
+      }
+      if (WAIT && __any_sync(kFull, L && S < bstart)) {
+        fence_acquire();
+        __syncwarp();  // any lane may read a source whose flags another lane checked
+      }
+      // the part inside the window, laid end to end with the group's others
+      const uint32_t d0 = max(D, w0), d1 = min(D + L, w0 + wn), n = L && d0 < d1 ? d1 - d0 : 0u;
+      const uint32_t incl = warp_incl_sum(n, lane), X = incl - n, T = __shfl_sync(kFull, incl, 31);
+      const uint32_t have = __ballot_sync(kFull, n != 0);
+      bool odd = false;
+      if (n) {
+        // byte c of the group's bytes: its entry's address, twice its source's
+        // place in the window (below 0: before it) and its source's address.  Marked in the
+        // address's top bits: a seek's source in more than one slot (the
+        // position instead), and a match overlapping its source (distance and
+        // start instead: its bytes repeat the first distance's, not one another
+        // down a long chain)
+        const uint64_t s0 = bstart + d0 - dist;
+        const int32_t rel = (int32_t)max((int64_t)(s0 - bstart) - (int64_t)w0, -(int64_t)(1 << 29));
+        uint64_t from;
+        if (SEEK && rel < 0 && s0 >> a.log2B != min(s0 + n - 1, bstart + w0 - 1) >> a.log2B) {
+          from = (s0 - X) | 1ull << 63;
+          odd = true;
+        } else {
+          from = reinterpret_cast<uintptr_t>(Addr<SEEK>::at(a, s0, b, obase)) - X;
+        }
+        uint32_t w = (uint32_t)(2 * (rel - (int32_t)X));
+        if (dist < L) {
+          from = (uint64_t)(0x40000000u | (D + 0x10000u - w0)) << 32 | dist;
+          w = 0xC0000000u;
+          odd = true;
+        }
+        row[__popc(have & lt)] = make_uint4((uint32_t)from, (uint32_t)(from >> 32), ebase + 2 * (d0 - w0 - X), w);
+      }
+      odd = __any_sync(kFull, odd);
+      constexpr uint32_t kBatch = 32 * kCtaUnroll;
+      const uint32_t share = ((T + split - 1) / split + kBatch - 1) & ~(kBatch - 1);
+      const uint32_t te = min(T, (part + 1) * share);
+      for (uint32_t cb = part * share; cb < te; cb += kCtaRowBytes) {  // one turn but for long matches
+#pragma unroll
+        for (uint32_t k = 0; k < kCtaRowBytes / 32; k += 32) bits[k + lane] = 0;
+        __syncwarp();
+        if (n && X - cb < kCtaRowBytes) atomicOr(bits + ((X - cb) >> 5), 1u << (X & 31));
+        uint32_t rank = __popc(__ballot_sync(kFull, n && X < cb)) - 1;  // the match before the row's first start
+        __syncwarp();
+        const uint32_t ce = min(te, cb + kCtaRowBytes);
+        auto rows = [&](auto marked) {
+          constexpr bool special = decltype(marked)::value;
+          const uint4* words = reinterpret_cast<const uint4*>(bits);
+          for (uint32_t c = cb + lane; c < ce + lane; c += 32 * kCtaUnroll) {
+            const uint4 w4 = *words++;
+            const uint32_t w[kCtaUnroll] = {w4.x, w4.y, w4.z, w4.w};
+            uint32_t v[kCtaUnroll], at[kCtaUnroll];
+#pragma unroll
+            for (uint32_t u = 0; u < kCtaUnroll; u++) {
+              const uint4 m = row[rank + __popc(w[u] & le)];
+              rank += __popc(w[u]);
+              const uint32_t q = c + 32 * u;
+              at[u] = m.z + 2 * q;
+              v[u] = m.w + 2 * q;
+              if ((int32_t)v[u] < 0 && q < ce) {
+                const uint64_t from = ((uint64_t)m.y << 32 | m.x) + q;
+                if (special && m.y >> 30 == 1) {  // overlapping: byte (place - start) mod distance of the source
+                  const int32_t start = (int32_t)(m.y & 0x3ffffu) - 0x10000;
+                  const int32_t s = start - (int32_t)m.x + (int32_t)(((at[u] - ebase) / 2 - (uint32_t)start) % m.x);
+                  v[u] = s >= 0 ? 2 * (uint32_t)s
+                                : 0x8000u | ld_src<!WAIT>(Addr<SEEK>::at(a, bstart + w0 + (int64_t)s, b, obase));
+                } else if (special && SEEK && m.y >> 31) {
+                  v[u] = 0x8000u | ld_src<!WAIT>(Addr<SEEK>::at(a, from & ~(1ull << 63), b, obase));
+                } else {
+                  v[u] = 0x8000u | ld_src<!WAIT>(reinterpret_cast<const uint8_t*>(from));
+                }
+              }
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < kCtaUnroll; u++)
+              if (c + 32 * u < ce) asm volatile("st.shared.u16 [%0], %1;" ::"r"(at[u]), "h"((uint16_t)v[u]) : "memory");
+          }
+        };
+        if (odd) rows(std::true_type());
+        else rows(std::false_type());
+        __syncwarp();  // the next bytes reuse the map
+      }
+      __syncwarp();
+    }
+    if (lane == 0) atomicMax(&s_group, last);
+    const bool any_bad = __syncthreads_or(bad), any_late = __syncthreads_or(timeout);
+    if (any_bad || any_late) {
+      if (tid == 0)
+        record_error(&a.sh->status, &a.sh->err_block, &a.sh->err_where, any_bad ? ACE_E_CORRUPT : ACE_E_TIMEOUT, b,
+                     any_bad ? 39 : 38);
+      return false;
+    }
+    first = s_group;
+
+    // each thread's bytes: their chains followed to known entries
+    bool deep = false;
+    auto settle = [&]() {
+      for (uint32_t j = 16 * tid; j < wn; j += 16 * nt) {
+        const uint4 lo = *reinterpret_cast<const uint4*>(e + j), hi = *reinterpret_cast<const uint4*>(e + j + 8);
+        const uint32_t q[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+        uint32_t x[16], all = ~0u;
+#pragma unroll
+        for (uint32_t k = 0; k < 16; k++) x[k] = k & 1 ? q[k >> 1] >> 16 : q[k >> 1] & 0xffffu;
+#pragma unroll
+        for (uint32_t k = 0; k < 8; k++) all &= q[k];
+        bool open = (all & 0x80008000u) != 0x80008000u;
+        for (uint32_t h = 0; open && h < kHops; h++) {
+          all = ~0u;
+#pragma unroll
+          for (uint32_t k = 0; k < 16; k++) {
+            asm volatile(
+                "{\n.reg .pred p;\n.reg .u32 t, c;\nand.b32 t, %0, 0x8000;\nsetp.eq.u32 p, t, 0;\nadd.u32 c, %0, %1;\n"
+                "@p ld.shared.u16 %0, [c];\n}"
+                : "+r"(x[k])
+                : "r"(ebase)
+                : "memory");
+            all &= x[k];
+          }
+          open = !(all & 0x8000u);
+        }
+        deep |= open;
+        uint4 v;
+        uint32_t* const y = &v.x;
+#pragma unroll
+        for (uint32_t k = 0; k < 4; k++)
+          y[k] = __byte_perm(__byte_perm(x[4 * k], x[4 * k + 1], 0x0040), __byte_perm(x[4 * k + 2], x[4 * k + 3], 0x0040),
+                             0x5410);
+        if (j + 16 <= wn) {
+          *reinterpret_cast<uint4*>(obase + w0 + j) = v;
+        } else {
+          for (uint32_t k = 0; j + k < wn; k++) {
+            const uint32_t z = k < 4 ? v.x : k < 8 ? v.y : k < 12 ? v.z : v.w;
+            obase[w0 + j + k] = (uint8_t)(z >> (8 * (k & 3)));
+          }
+        }
+      }
+    };
+    settle();
+    if (__syncthreads_or(deep)) {
+      // Entries change while others read them: each read sees an entry of the
+      // same chain, old or new, and 16-bit shared stores do not tear.
+      volatile uint16_t* ev = e;
+      while (true) {
+        int pending = 0;
+        for (uint32_t j = tid; j < wn; j += nt) {
+          const uint32_t x = ev[j];
+          if (!(x & 0x8000u)) {
+            const uint32_t y = ev[x >> 1];
+            ev[j] = (uint16_t)y;
+            pending |= !(y & 0x8000u);
+          }
+        }
+        if (!__syncthreads_or(pending)) break;  // every target precedes its entry: at most log2(kCtaWindow) + 1 turns
+      }
+      settle();
+      __syncthreads();
+    }
+  }
+  return true;
 }
 
 // The three passes of a decode, each a persistent launch over the blocks:
@@ -1258,16 +1454,45 @@ __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint3
 // latency-bound match copies of others on the same SM.
 enum { PASS_TOKENS = 0, PASS_LITERALS = 1, PASS_MATCH = 2, PASS_FUSED = 3 };
 
-// Registers per thread allowed by each pass's launch bounds (256 threads).
-#define ACE_PASS_MIN_CTAS(P) ((P) == PASS_TOKENS ? 4 : (P) == PASS_LITERALS ? 4 : (P) == PASS_FUSED ? 4 : 2)
-
-
+// Every pass is held to 64 registers a thread: 256 threads, or the match
+// pass's CTAs of up to 512.
+#define ACE_PASS_BOUNDS(P) __launch_bounds__((P) == PASS_MATCH ? kCtaThreads : 256, (P) == PASS_MATCH ? 2 : 4)
 
 // Publishes block b (its writes visible device-wide before the flag).
 __device__ __forceinline__ void publish(uint32_t* ready, uint32_t b, uint32_t epoch, uint32_t lane) {
   __threadfence();
   __syncwarp();
   if (lane == 0) st_release(ready + b, epoch);
+}
+
+// Publishes a block that the CTA wrote together.
+__device__ __forceinline__ void publish_cta(uint32_t* ready, uint32_t b, uint32_t epoch) {
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) st_release(ready + b, epoch);
+}
+
+// Work items one after another from a ticket, each for the whole CTA.
+template <class F>
+__device__ __forceinline__ void cta_blocks(uint32_t n_items, uint32_t* ticket, F&& block) {
+  __shared__ uint32_t drawn;
+  while (true) {
+    __syncthreads();  // every thread is done with the block before, and has read its number
+    if (threadIdx.x == 0) drawn = atomicAdd(ticket, 1u);
+    __syncthreads();
+    const uint32_t it = drawn;
+    if (it >= n_items) return;
+    block(it);
+  }
+}
+
+// Whether the call recorded an error before this pass: the same answer for a
+// whole CTA in the match pass, whose threads meet at barriers (other CTAs may
+// be recording one now).
+template <int PASS>
+__device__ __forceinline__ bool stop_early(const uint32_t* status) {
+  const bool set = *(const volatile uint32_t*)status != 0;
+  return PASS == PASS_MATCH ? __syncthreads_or(set) : set;
 }
 
 // Blocks level l of a fused call holds (whole decode: the index's level
@@ -1412,19 +1637,41 @@ __device__ void fused_loop(const Jobs& jobs, ScratchHdr* sh, uint32_t n_items, u
 // match pass, launched after them, resolves every block's matches in (level,
 // block) order, waiting on source blocks' flags, and publishes the block.
 template <bool SEEK, int PASS>
-__global__ void __launch_bounds__(256, ACE_PASS_MIN_CTAS(PASS)) decode_kernel(DecodeArgs a) {
+__global__ void ACE_PASS_BOUNDS(PASS) decode_kernel(DecodeArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t epoch = *(volatile uint32_t*)&a.sh->epoch;
   const uint32_t n_items = SEEK ? *(volatile uint32_t*)&a.sh->n_work : a.n_items;
   // the literal and match passes run only after every block's tokens decoded
-  if (PASS != PASS_TOKENS && *(volatile uint32_t*)&a.sh->status) return;
+  if (PASS != PASS_TOKENS && stop_early<PASS>(&a.sh->status)) return;
   uint8_t* wsm = smem + (size_t)wid * a.warp_smem;
   if (PASS == PASS_FUSED) {
     fused_loop<SEEK>(ArchiveJobs<SEEK>{a}, a.sh, n_items, a.timeout_ns, wsm, lane, epoch, a.window);
     return;
   }
-  uint32_t* ticket = PASS == PASS_TOKENS ? &a.sh->ticket : PASS == PASS_LITERALS ? &a.sh->ticket2 : &a.sh->ticket3;
+  if (PASS == PASS_MATCH) {
+    cta_blocks(n_items, &a.sh->ticket3, [&](uint32_t it) {
+      const uint32_t b = __ldg(a.items + it);
+      const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
+      const bool ok = match_cta<SEEK, true>(a, smem, b, ntok ? ntok - 1 : 0, epoch, 0);
+      publish_cta(a.ready, b, epoch);
+      if (SEEK && ok && a.slice) {
+        // the part of this block inside [coord, coord + len) to the caller, a share per warp
+        uint64_t bs = (uint64_t)b << a.log2B, be = min(bs + ((uint64_t)1 << a.log2B), a.total);
+        uint64_t lo = max(bs, a.coord), hi = min(be, a.coord + a.len);
+        if (hi > lo) {
+          const uint32_t nw = blockDim.x >> 5;
+          const uint64_t part = ((hi - lo + nw - 1) / nw + 15) & ~15ull;
+          const uint8_t* src = a.out + slot_base(a, b) - bs;
+          lo += wid * part;
+          hi = min(hi, lo + part);
+          if (hi > lo) warp_copy(a.slice + (lo - a.coord), src + lo, hi - lo, lane);
+        }
+      }
+    });
+    return;
+  }
+  uint32_t* ticket = PASS == PASS_TOKENS ? &a.sh->ticket : &a.sh->ticket2;
   while (true) {
     uint32_t it = 0;
     if (lane == 0) it = atomicAdd(ticket, 1u);
@@ -1435,21 +1682,8 @@ __global__ void __launch_bounds__(256, ACE_PASS_MIN_CTAS(PASS)) decode_kernel(De
       token_block<SEEK>(a, carve_tok(wsm), b, lane);
       continue;
     }
-    if (PASS == PASS_LITERALS) {
-      constexpr uint32_t ring = SEEK ? kSeekRing : kRing;
-      literal_block<SEEK, ring>(a, carve_lit(wsm, a.window, ring), b, lane);
-      continue;
-    }
-    const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
-    bool ok = match_block<SEEK, true>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch, ntok ? ntok - 1 : 0);
-    if (SEEK && ok && a.slice) {
-      // copy the part of this block inside [coord, coord + len) to the caller
-      uint64_t bs = (uint64_t)b << a.log2B, be = min(bs + ((uint64_t)1 << a.log2B), a.total);
-      uint64_t lo = max(bs, a.coord), hi = min(be, a.coord + a.len);
-      const uint8_t* src = a.out + slot_base(a, b) - bs;
-      if (hi > lo) warp_copy(a.slice + (lo - a.coord), src + lo, hi - lo, lane);
-    }
-    publish(a.ready, b, epoch, lane);
+    constexpr uint32_t ring = SEEK ? kSeekRing : kRing;
+    literal_block<SEEK, ring>(a, carve_lit(wsm, a.window, ring), b, lane);
   }
 }
 
@@ -1458,7 +1692,11 @@ __global__ void __launch_bounds__(256, ACE_PASS_MIN_CTAS(PASS)) decode_kernel(De
 // waits.  Blocks are dealt out statically (block k of the level to warp
 // k mod the warps in the grid), and each warp fetches its next block's
 // number and record range while it resolves the current one.
-__global__ void __launch_bounds__(256, 3) match_level_kernel(DecodeArgs a) {
+// ROWS: the archive's matches are mostly short; without it every group goes by
+// rounds.  72 registers: 7 CTAs of 4 warps per SM (genome 1 GiB, long matches:
+// 0.458 ms against 0.493 at 75 to 80 registers, 6 CTAs).
+template <bool ROWS>
+__global__ void __maxnreg__(72) match_level_kernel(DecodeArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t nw = gridDim.x * (blockDim.x >> 5);
@@ -1478,7 +1716,7 @@ __global__ void __launch_bounds__(256, 3) match_level_kernel(DecodeArgs a) {
       bn = __ldg(a.items + nx);
       nmn = n_matches(bn);
     }
-    match_block<false, false>(a, gm, b, lane, 0, nm, a.cur_level);
+    match_block<false, false, true, ROWS>(a, gm, b, lane, 0, nm, a.cur_level);
     if (nx >= a.n_items) break;
     it = nx;
     b = bn;
@@ -1486,260 +1724,15 @@ __global__ void __launch_bounds__(256, 3) match_level_kernel(DecodeArgs a) {
   }
 }
 
-// The match pass of a dependency level with few blocks, a CTA per block: a
-// warp per block would leave most of the GPU idle while each block's matches
-// resolve one round after another.  Every byte of the block gets a 16-bit
-// entry in shared memory: 0x8000 | its value once final (a literal, or a
-// match byte whose source lies in an earlier block, which the launches
-// before finished), else the in-block position it copies.  A match byte
-// equals the byte at its source, which precedes it (Section 2, the
-// sequential LZ77 copy), so the entries form chains that each end at a final
-// one; pointer jumping (every pending entry takes its target's entry) ends
-// all of them in at most log2(B) + 1 sweeps.  The block is then written back
-// with 16-byte stores.
-constexpr uint32_t kSmallThreads = 512;
-constexpr uint32_t kSmallMaxLog2B = 15;               // positions fit the entries' low 15 bits
-constexpr uint32_t kSmallSweeps = kSmallMaxLog2B + 2;  // log2(B) + 1, and one that sees no pending entry
-constexpr uint32_t kSmallUnroll = 8;                   // match bytes per lane with their loads in flight
-constexpr uint32_t kSmallLoads = 4;                    // 16-byte block loads per thread in flight
-
-// The CTA's current kSmallThreads matches (one record per thread), laid end
-// to end: match j's bytes start at X[j], X[kSmallThreads] is their total.
-struct __align__(16) SmallChunk {
-  uint64_t S[kSmallThreads];
-  uint32_t D[kSmallThreads], L[kSmallThreads], X[kSmallThreads + 1];
-  uint32_t wsum[kSmallThreads / 32];
-};
-
-// One warp's current 32 matches, laid end to end (blocks of many matches).
-struct __align__(16) SmallWarp {
-  uint64_t S[32];
-  uint32_t D[32], L[32], X[33];
-};
-// The entries, then the chunk's or the warps' arrays (one or the other per
-// block): 43 KB for 16 KiB blocks, within the default shared-memory limit.
-constexpr size_t kSmallArrays = sizeof(SmallChunk) > kSmallThreads / 32 * sizeof(SmallWarp)
-                                    ? sizeof(SmallChunk)
-                                    : kSmallThreads / 32 * sizeof(SmallWarp);
-__host__ __device__ constexpr size_t small_smem_bytes(uint32_t log2B) {
-  return ((size_t)2 << log2B) + kSmallArrays;
-}
-
-__global__ void __launch_bounds__(kSmallThreads, 1) match_small_kernel(DecodeArgs a) {
+// The same with a CTA per block.
+template <uint32_t THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 4) match_cta_kernel(DecodeArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
-  const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (__syncthreads_or(*(volatile uint32_t*)&a.sh->status != 0)) return;  // the same answer for the whole CTA
-  const uint32_t b = __ldg(a.items + blockIdx.x);
-  const uint64_t B = 1ull << a.log2B, bstart = (uint64_t)b << a.log2B;
-  const uint32_t blen = (uint32_t)min(B, a.total - bstart);
-  uint8_t* obase = a.out + bstart;
-  uint16_t* e = reinterpret_cast<uint16_t*>(smem);
-  SmallChunk* const chunks = reinterpret_cast<SmallChunk*>(smem + (2ull << a.log2B));
-  static_assert(sizeof(SmallChunk) % 16 == 0, "chunk arrays stay 16-byte aligned");
-  const uint64_t m0 = __ldg(a.match_ptr + b), nm = __ldg(a.match_ptr + b + 1) - m0;
-  const uint4* rec = reinterpret_cast<const uint4*>(a.recs + m0);
-  bool bad = false;
-  // the first chunk's match records load with the block
-  uint4 rn = make_uint4(0, 0, 0, 0);
-  if (tid < nm) rn = __ldg(rec + tid);
-
-  // every byte final with what the literal pass left; match bytes are
-  // overwritten next.  16-byte loads, kSmallLoads per thread in flight
-  // (obase is block-aligned, and B is a multiple of 256).
-  for (uint32_t j0 = 16 * tid; j0 < blen; j0 += 16 * kSmallThreads * kSmallLoads) {
-    uint4 v[kSmallLoads];
-#pragma unroll
-    for (uint32_t u = 0; u < kSmallLoads; u++) {
-      const uint32_t j = j0 + 16 * kSmallThreads * u;
-      v[u] = make_uint4(0, 0, 0, 0);
-      if (j + 16 <= blen) {
-        v[u] = *reinterpret_cast<const uint4*>(obase + j);
-      } else if (j < blen) {
-        uint32_t x[4];
-#pragma unroll
-        for (uint32_t q = 0; q < 4; q++) {
-          x[q] = 0;
-#pragma unroll
-          for (uint32_t k = 0; k < 4; k++)
-            if (j + 4 * q + k < blen) x[q] |= (uint32_t)obase[j + 4 * q + k] << (8 * k);
-        }
-        v[u] = make_uint4(x[0], x[1], x[2], x[3]);
-      }
-    }
-#pragma unroll
-    for (uint32_t u = 0; u < kSmallLoads; u++) {
-      const uint32_t j = j0 + 16 * kSmallThreads * u;
-      if (j >= blen) continue;
-      uint4* e4 = reinterpret_cast<uint4*>(e + j);
-      e4[0] = make_uint4(__byte_perm(v[u].x, 0x80u, 0x4140), __byte_perm(v[u].x, 0x80u, 0x4342),
-                         __byte_perm(v[u].y, 0x80u, 0x4140), __byte_perm(v[u].y, 0x80u, 0x4342));
-      e4[1] = make_uint4(__byte_perm(v[u].z, 0x80u, 0x4140), __byte_perm(v[u].z, 0x80u, 0x4342),
-                         __byte_perm(v[u].w, 0x80u, 0x4140), __byte_perm(v[u].w, 0x80u, 0x4342));
-    }
-  }
-  __syncthreads();
-
-  // match bytes: a byte whose source is in an earlier block reads it
-  // (final), one whose source is in this block points there.  Blocks of at
-  // most kSmallThreads matches lay them end to end over the whole CTA (every
-  // thread on bytes tid, tid + kSmallThreads, ...); with more, each warp
-  // takes 32 at a time on its own, without CTA barriers between them.
-  if (nm > kSmallThreads) {
-    SmallWarp& ww = reinterpret_cast<SmallWarp*>(chunks)[wid];
-    for (uint64_t t0 = 32ull * wid; t0 < nm; t0 += kSmallThreads) {
-      const uint64_t t = t0 + lane;
-      const uint4 r = rn;
-      if (t + kSmallThreads < nm) rn = __ldg(rec + t + kSmallThreads);  // the warp's next 32
-      uint32_t len = 0;
-      if (t < nm) {
-        const uint64_t S = (uint64_t)r.x | ((uint64_t)r.y << 32);
-        const uint32_t D = r.z, ml = r.w;
-        if (ml && (S >= bstart + D || (uint64_t)D + ml > blen)) {
-          bad = true;
-        } else {
-          len = ml;
-        }
-        ww.S[lane] = S;
-        ww.D[lane] = D;
-      }
-      ww.L[lane] = len;
-      const uint32_t incl = warp_incl_sum(len, lane);
-      ww.X[lane] = incl - len;
-      if (lane == 31) ww.X[32] = incl;
-      const uint32_t total = __shfl_sync(kFull, incl, 31);
-      __syncwarp();
-      uint32_t jc = 0;  // the match of the lane's byte only moves forward
-      for (uint32_t c = 0; c < total; c += 32 * kSmallUnroll) {
-        uint32_t val[kSmallUnroll], dst[kSmallUnroll];
-#pragma unroll
-        for (uint32_t u = 0; u < kSmallUnroll; u++) {
-          const uint32_t p = c + 32 * u + lane;
-          dst[u] = ~0u;
-          val[u] = 0;
-          if (p < total) {
-            while (ww.X[jc + 1] <= p) jc++;
-            const uint32_t i = p - ww.X[jc], ml = ww.L[jc], D = ww.D[jc];
-            const uint64_t S = ww.S[jc];
-            const uint64_t src = src_index(S, bstart + D - S, ml, i);
-            dst[u] = D + i;
-            val[u] = src < bstart ? 0x8000u | ld_src<true>(a.out + src) : (uint32_t)(src - bstart);
-          }
-        }
-#pragma unroll
-        for (uint32_t u = 0; u < kSmallUnroll; u++)
-          if (dst[u] != ~0u) e[dst[u]] = (uint16_t)val[u];
-      }
-      __syncwarp();  // the warp's next 32 reuse its arrays
-    }
-  }
-  if (nm <= kSmallThreads && nm) {  // one chunk
-    SmallChunk& w = chunks[0];
-    const uint64_t t = tid;
-    const uint4 r = rn;
-    uint32_t len = 0;
-    if (t < nm) {
-      const uint64_t S = (uint64_t)r.x | ((uint64_t)r.y << 32);
-      const uint32_t D = r.z, ml = r.w;
-      if (ml && (S >= bstart + D || (uint64_t)D + ml > blen)) {
-        bad = true;  // a source must precede its destination, which stays in the block
-      } else {
-        len = ml;
-      }
-      w.S[tid] = S;
-      w.D[tid] = D;
-    }
-    w.L[tid] = len;
-    // exclusive scan of the lengths over the CTA
-    const uint32_t incl = warp_incl_sum(len, lane);
-    if (lane == 31) w.wsum[wid] = incl;
-    __syncthreads();
-    uint32_t before = 0, total = 0;
-#pragma unroll
-    for (uint32_t k = 0; k < kSmallThreads / 32; k++) {
-      const uint32_t x = w.wsum[k];
-      before += k < wid ? x : 0u;
-      total += x;
-    }
-    w.X[tid] = before + incl - len;
-    if (tid == 0) w.X[kSmallThreads] = total;
-    __syncthreads();
-    for (uint32_t c = 0; c < total; c += kSmallThreads * kSmallUnroll) {
-      uint32_t val[kSmallUnroll], dst[kSmallUnroll];
-#pragma unroll
-      for (uint32_t u = 0; u < kSmallUnroll; u++) {
-        const uint32_t p = c + kSmallThreads * u + tid;
-        dst[u] = ~0u;
-        val[u] = 0;
-        if (p < total) {
-          const uint32_t jc = upper_bound(kSmallThreads + 1, p, [&](uint32_t i) { return w.X[i]; }) - 1;
-          const uint32_t i = p - w.X[jc], ml = w.L[jc], D = w.D[jc];
-          const uint64_t S = w.S[jc];
-          const uint64_t src = src_index(S, bstart + D - S, ml, i);
-          dst[u] = D + i;
-          val[u] = src < bstart ? 0x8000u | ld_src<true>(a.out + src) : (uint32_t)(src - bstart);
-        }
-      }
-#pragma unroll
-      for (uint32_t u = 0; u < kSmallUnroll; u++)
-        if (dst[u] != ~0u) e[dst[u]] = (uint16_t)val[u];
-    }
-  }
-  if (__syncthreads_or(bad)) {
-    if (tid == 0) record_error(&a.sh->status, &a.sh->err_block, &a.sh->err_where, ACE_E_CORRUPT, b, 39);
-    return;
-  }
-
-  // pointer jumping; every target precedes its entry, so the sweeps end.
-  // Entries change while others read them: each read sees an entry of the
-  // same chain, old or new, and 16-bit shared stores do not tear.
-  volatile uint16_t* ev = e;
-  uint32_t sweep = 0;
-  for (; sweep < kSmallSweeps; sweep++) {
-    int pending = 0;
-    for (uint32_t j = tid; j < blen; j += kSmallThreads) {
-      const uint32_t x = ev[j];
-      if (!(x & 0x8000u)) {
-        const uint32_t y = ev[x];
-        ev[j] = (uint16_t)y;
-        pending |= !(y & 0x8000u);
-      }
-    }
-    if (!__syncthreads_or(pending)) break;
-  }
-  if (sweep == kSmallSweeps) {  // cannot happen for the chains above
-    if (tid == 0) record_error(&a.sh->status, &a.sh->err_block, &a.sh->err_where, ACE_E_CORRUPT, b, 42);
-    return;
-  }
-
-  // the block's bytes: the low byte of each entry
-  for (uint32_t j = 16 * tid; j < blen; j += 16 * kSmallThreads) {
-    const uint4 lo = *reinterpret_cast<const uint4*>(e + j), hi = *reinterpret_cast<const uint4*>(e + j + 8);
-    const uint4 v = make_uint4(__byte_perm(lo.x, lo.y, 0x6420), __byte_perm(lo.z, lo.w, 0x6420),
-                               __byte_perm(hi.x, hi.y, 0x6420), __byte_perm(hi.z, hi.w, 0x6420));
-    if (j + 16 <= blen) {
-      *reinterpret_cast<uint4*>(obase + j) = v;
-    } else {
-      for (uint32_t k = 0; j + k < blen; k++) {
-        const uint32_t x = k < 4 ? v.x : k < 8 ? v.y : k < 12 ? v.z : v.w;
-        obase[j + k] = (uint8_t)(x >> (8 * (k & 3)));
-      }
-    }
-  }
-
-  // the earlier blocks a match reads (at most two) belong to lower levels:
-  // checked last, since a corrupt archive fails the call whatever was written
-  for (uint64_t t = tid; t < nm; t += kSmallThreads) {
-    const uint4 r = __ldg(rec + t);
-    const uint64_t S = (uint64_t)r.x | ((uint64_t)r.y << 32);
-    const uint32_t D = r.z, ml = r.w;
-    if (!ml || (S >> a.log2B) >= b) continue;
-    const uint64_t rend = S + min((uint64_t)ml, bstart + D - S);
-    const uint64_t k1 = min((rend - 1) >> a.log2B, (uint64_t)b - 1);
-    for (uint64_t k = S >> a.log2B; k <= k1; k++)
-      if (__ldg(a.level + k) >= a.cur_level) {
-        record_error(&a.sh->status, &a.sh->err_block, &a.sh->err_where, ACE_E_CORRUPT, b, 39);
-        return;
-      }
+  for (uint32_t it = blockIdx.x; it < a.n_items; it += gridDim.x) {
+    const uint32_t b = __ldg(a.items + it);
+    const uint64_t m0 = __ldg(a.match_ptr + b);
+    if (!match_cta<false, false>(a, smem, b, (uint32_t)(__ldg(a.match_ptr + b + 1) - m0), 0, a.cur_level)) return;
   }
 }
 
@@ -1827,18 +1820,28 @@ __device__ DecodeArgs BatchJobs::job(uint32_t v, uint32_t& b) const {
 }
 
 template <int PASS>
-__global__ void __launch_bounds__(256, ACE_PASS_MIN_CTAS(PASS)) batch_decode_kernel(BatchArgs ba) {
+__global__ void ACE_PASS_BOUNDS(PASS) batch_decode_kernel(BatchArgs ba) {
   extern __shared__ __align__(16) uint8_t smem[];
   const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (PASS != PASS_TOKENS && PASS != PASS_FUSED && *(volatile uint32_t*)&ba.sh->status) return;
+  if (PASS != PASS_TOKENS && PASS != PASS_FUSED && stop_early<PASS>(&ba.sh->status)) return;
   uint8_t* wsm = smem + (size_t)wid * ba.warp_smem;
   const uint32_t epoch = *(volatile uint32_t*)&ba.sh->epoch;
   if (PASS == PASS_FUSED) {
     fused_loop<false>(BatchJobs{ba}, ba.sh, ba.n_items, ba.timeout_ns, wsm, lane, epoch, ba.window);
     return;
   }
-  uint32_t* ticket = PASS == PASS_TOKENS ? &ba.sh->ticket : PASS == PASS_LITERALS ? &ba.sh->ticket2 : &ba.sh->ticket3;
   const BatchJobs jobs{ba};
+  if (PASS == PASS_MATCH) {
+    cta_blocks(ba.n_items, &ba.sh->ticket3, [&](uint32_t it) {
+      uint32_t b;
+      const DecodeArgs a = jobs.job(it, b);
+      const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
+      match_cta<false, true>(a, smem, b, ntok ? ntok - 1 : 0, epoch, 0);
+      publish_cta(a.ready, b, epoch);
+    });
+    return;
+  }
+  uint32_t* ticket = PASS == PASS_TOKENS ? &ba.sh->ticket : &ba.sh->ticket2;
   while (true) {
     uint32_t it = 0;
     if (lane == 0) it = atomicAdd(ticket, 1u);
@@ -1846,15 +1849,8 @@ __global__ void __launch_bounds__(256, ACE_PASS_MIN_CTAS(PASS)) batch_decode_ker
     if (it >= ba.n_items) break;
     uint32_t b;
     const DecodeArgs a = jobs.job(it, b);
-    if (PASS == PASS_TOKENS) {
-      token_block<false>(a, carve_tok(wsm), b, lane);
-    } else if (PASS == PASS_LITERALS) {
-      literal_block<false, kRing>(a, carve_lit(wsm, ba.window, kRing), b, lane);
-    } else {
-      const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
-      match_block<false, true>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch, ntok ? ntok - 1 : 0);
-      publish(a.ready, b, epoch, lane);
-    }
+    if (PASS == PASS_TOKENS) token_block<false>(a, carve_tok(wsm), b, lane);
+    else literal_block<false, kRing>(a, carve_lit(wsm, ba.window, kRing), b, lane);
   }
 }
 
@@ -2014,7 +2010,9 @@ __global__ void __cluster_dims__(kClosureCtas, 1, 1) __launch_bounds__(1024, 1) 
   __syncthreads();
   for (uint32_t i = tid; i < n; i += blockDim.x) {
     const uint32_t b = a.front0[i];
-    a.work[atomicAdd(&lcnt[a.level ? a.level[b] : 0], 1u)] = b;
+    // (any order inside a level; without levels the ascending order is the
+    // decode order, and blocks must not be handed out before their sources)
+    a.work[a.level ? atomicAdd(&lcnt[a.level[b]], 1u) : i] = b;
   }
 }
 
@@ -2329,21 +2327,17 @@ struct CacheDecodeArgs {
 // Decodes a batch's work list into cache slots: the same three passes as a
 // seek, archive by archive.
 template <int PASS>
-__global__ void __launch_bounds__(256, ACE_PASS_MIN_CTAS(PASS)) cache_decode_kernel(CacheDecodeArgs ca) {
+__global__ void ACE_PASS_BOUNDS(PASS) cache_decode_kernel(CacheDecodeArgs ca) {
   extern __shared__ __align__(16) uint8_t smem[];
   const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   uint8_t* wsm = smem + (size_t)wid * ca.warp_smem;
   const CacheArgs& c = ca.c;
-  if (PASS != PASS_TOKENS && *(volatile uint32_t*)&c.h->status) return;
+  if (PASS != PASS_TOKENS && stop_early<PASS>(&c.h->status)) return;
   const uint32_t epoch = *(volatile uint32_t*)&c.h->epoch;
   const uint32_t n_items = *(volatile uint32_t*)&c.h->n_work;
-  uint32_t* ticket = PASS == PASS_TOKENS ? &c.h->ticket : PASS == PASS_LITERALS ? &c.h->ticket2 : &c.h->ticket3;
-  while (true) {
-    uint32_t it = 0;
-    if (lane == 0) it = atomicAdd(ticket, 1u);
-    it = __shfl_sync(kFull, it, 0);
-    if (it >= n_items) break;
-    const uint32_t ai = __ldg(c.work + 2 * it), b = __ldg(c.work + 2 * it + 1);
+  auto job = [&](uint32_t it, uint32_t& b) {
+    const uint32_t ai = __ldg(c.work + 2 * it);
+    b = __ldg(c.work + 2 * it + 1);
     const CacheArc& arc = c.arcs[ai];
     DecodeArgs a{};
     a.arc = arc.arc;
@@ -2368,15 +2362,28 @@ __global__ void __launch_bounds__(256, ACE_PASS_MIN_CTAS(PASS)) cache_decode_ker
     a.timeout_ns = ca.timeout_ns;
     a.recs = c.recs;
     a.match_ptr = nullptr;
-    if (PASS == PASS_TOKENS) {
-      token_block<true>(a, carve_tok(wsm), b, lane);
-    } else if (PASS == PASS_LITERALS) {
-      literal_block<true, kSeekRing>(a, carve_lit(wsm, ca.window, kSeekRing), b, lane);
-    } else {
+    return a;
+  };
+  if (PASS == PASS_MATCH) {
+    cta_blocks(n_items, &c.h->ticket3, [&](uint32_t it) {
+      uint32_t b;
+      const DecodeArgs a = job(it, b);
       const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
-      match_block<true, true>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch, ntok ? ntok - 1 : 0);
-      publish(arc.ready, b, epoch, lane);
-    }
+      match_cta<true, true>(a, smem, b, ntok ? ntok - 1 : 0, epoch, 0);
+      publish_cta(a.ready, b, epoch);
+    });
+    return;
+  }
+  uint32_t* ticket = PASS == PASS_TOKENS ? &c.h->ticket : &c.h->ticket2;
+  while (true) {
+    uint32_t it = 0;
+    if (lane == 0) it = atomicAdd(ticket, 1u);
+    it = __shfl_sync(kFull, it, 0);
+    if (it >= n_items) break;
+    uint32_t b;
+    const DecodeArgs a = job(it, b);
+    if (PASS == PASS_TOKENS) token_block<true>(a, carve_tok(wsm), b, lane);
+    else literal_block<true, kSeekRing>(a, carve_lit(wsm, ca.window, kSeekRing), b, lane);
   }
 }
 
@@ -2507,8 +2514,7 @@ struct ace_index {
   ace_tune tune;
   // occupancy of the decode kernels, per (seek?, pass, warps per CTA, window)
   mutable int occ_cache[2][4][9][9];  // [3]: the fused pass
-  mutable int occ_level[9][9];  // the per-level match kernel
-  mutable bool small_attr = false;  // match_small_kernel allowed its shared memory
+  mutable int occ_level[9];  // the per-level match kernels: a warp per block by warps per CTA; [0] a CTA per block
   // whole decodes resolve matches with one launch per level when there are
   // at most kMaxLevelLaunches levels: level L's blocks are
   // order[level_start[L] .. level_start[L + 1])
@@ -2660,8 +2666,13 @@ struct Launch {
   uint32_t grid[4];
   uint64_t timeout;
   uint32_t schedule;
-  uint32_t long_min;  // the copy-width knob as the long class's shortest match
+  uint32_t long_min;       // the copy-width knob as the long class's shortest match
+  uint32_t match_threads;  // threads of the match pass's CTAs, a block each
 };
+
+constexpr double kCtaMatches = 400;
+constexpr double kRowMatches = 48;
+constexpr uint32_t kCtaLevel = 4;
 
 template <class K>
 ace_status occupancy(K kernel, int device, uint32_t warps, size_t smem, int* occ) {
@@ -2687,8 +2698,7 @@ ace_status occupancy(K kernel, int device, uint32_t warps, size_t smem, int* occ
 // k3 is the fused pass
 template <class K0, class K1, class K2, class K3>
 ace_status plan_launch(const ace_index* idx, const ace_tune* tune, uint32_t log2B, uint64_t max_items,
-                       K0 k0, K1 k1, K2 k2, K3 k3, int* occ_cache, Launch* L,
-                       uint32_t lit_ring = kRing) {
+                       K0 k0, K1 k1, K2 k2, K3 k3, int* occ_cache, Launch* L, uint32_t lit_ring, bool few) {
   ace_tune t = tune ? *tune : idx->tune;
   L->warps = t.warps_per_cta ? t.warps_per_cta : 4;
   L->chunk = t.chunk_tokens ? t.chunk_tokens : 128;
@@ -2705,8 +2715,9 @@ ace_status plan_launch(const ace_index* idx, const ace_tune* tune, uint32_t log2
   if (L->schedule == ACE_SCHEDULE_AUTO) L->schedule = ACE_SCHEDULE_PASSES;
   L->smem[PASS_TOKENS] = tok_smem_bytes(esc_cap(log2B));
   L->smem[PASS_LITERALS] = lit_smem_bytes(L->chunk, lit_ring);
-  L->smem[PASS_MATCH] = kMatchSmem;
-  L->smem[PASS_FUSED] = std::max(std::max(L->smem[PASS_TOKENS], L->smem[PASS_LITERALS]), L->smem[PASS_MATCH]);
+  L->match_threads = cta_threads(log2B, few);
+  L->smem[PASS_MATCH] = cta_smem_bytes(log2B, L->match_threads);  // per CTA; the other passes': per warp
+  L->smem[PASS_FUSED] = std::max(std::max(L->smem[PASS_TOKENS], L->smem[PASS_LITERALS]), kMatchSmem);
   int per[4];
   for (int p = 0; p < 4; p++) {
     int& c = occ_cache[(p * 9 + L->warps) * 9 + L->chunk / 32];
@@ -2714,7 +2725,7 @@ ace_status plan_launch(const ace_index* idx, const ace_tune* tune, uint32_t log2
       const size_t smem = (size_t)L->warps * L->smem[p];
       ace_status rc = p == 0   ? occupancy(k0, idx->device, L->warps, smem, &c)
                       : p == 1 ? occupancy(k1, idx->device, L->warps, smem, &c)
-                      : p == 2 ? occupancy(k2, idx->device, L->warps, smem, &c)
+                      : p == 2 ? occupancy(k2, idx->device, L->match_threads / 32, L->smem[PASS_MATCH], &c)
                                : occupancy(k3, idx->device, L->warps, smem, &c);
       if (rc) return rc;
     }
@@ -2724,6 +2735,8 @@ ace_status plan_launch(const ace_index* idx, const ace_tune* tune, uint32_t log2
   }
   uint64_t need = std::max<uint64_t>(1, (max_items + L->warps - 1) / L->warps);
   for (int p = 0; p < 4; p++) L->grid[p] = (uint32_t)std::min<uint64_t>((uint64_t)idx->num_sms * per[p], need);
+  L->grid[PASS_MATCH] =
+      (uint32_t)std::min<uint64_t>((uint64_t)idx->num_sms * per[PASS_MATCH], std::max<uint64_t>(1, max_items));
   return ACE_OK;
 }
 
@@ -2731,8 +2744,7 @@ template <bool SEEK>
 ace_status plan_index_launch(const ace_index* idx, const ace_tune* tune, uint64_t max_items, Launch* L) {
   return plan_launch(idx, tune, idx->h.log2_block, max_items, decode_kernel<SEEK, PASS_TOKENS>,
                      decode_kernel<SEEK, PASS_LITERALS>, decode_kernel<SEEK, PASS_MATCH>,
-                     decode_kernel<SEEK, PASS_FUSED>, &idx->occ_cache[SEEK][0][0][0], L,
-                     SEEK ? kSeekRing : kRing);
+                     decode_kernel<SEEK, PASS_FUSED>, &idx->occ_cache[SEEK][0][0][0], L, SEEK ? kSeekRing : kRing, SEEK);
 }
 
 // Launches the passes in the mask (bit p: pass p) in order on s, each with
@@ -2749,8 +2761,7 @@ void launch_passes(const Launch& L, uint32_t passes, K0 k0, K1 k1, K2 k2, Args a
     k1<<<L.grid[1], th, (size_t)L.warps * L.smem[1], s>>>(a);
   }
   if (passes & 4) {
-    a.warp_smem = L.smem[2];
-    k2<<<L.grid[2], th, (size_t)L.warps * L.smem[2], s>>>(a);
+    k2<<<L.grid[2], L.match_threads, L.smem[2], s>>>(a);
   }
 }
 
@@ -3127,36 +3138,45 @@ ace_status decode_all_passes(const ace_index* idx, uint32_t passes, void* d_out,
   launch_passes(L, passes & (idx->by_levels ? 3u : 7u), decode_kernel<false, PASS_TOKENS>,
                 decode_kernel<false, PASS_LITERALS>, decode_kernel<false, PASS_MATCH>, a, s);
   if ((passes & 4) && idx->by_levels) {
-    a.warp_smem = L.smem[PASS_MATCH];
-    int& occ = idx->occ_level[L.warps][L.chunk / 32];
+    const ace_tune t = tune ? *tune : idx->tune;
+    int &occ = idx->occ_level[L.warps], &occ_cta = idx->occ_level[0];
+    const uint32_t log2B = idx->h.log2_block, few = cta_threads(log2B, true), many = cta_threads(log2B, false);
+    // a warp per block by rounds, a warp per block by rows, a CTA per block:
+    // by the archive's matches per 16 KiB
+    const double per16k = (double)idx->n_matches * 16384 / (double)idx->h.total_size;
+    const bool dense = per16k >= kCtaMatches, rows = per16k >= kRowMatches;
+    const auto level_kernel = rows ? match_level_kernel<true> : match_level_kernel<false>;
     if (occ == 0) {
-      rc = occupancy(match_level_kernel, idx->device, L.warps, (size_t)L.warps * L.smem[PASS_MATCH], &occ);
+      rc = occupancy(level_kernel, idx->device, L.warps, (size_t)L.warps * kMatchSmem, &occ);
       if (rc) return rc;
     }
-    if (occ < 0) return ACE_E_INVAL;
-    uint32_t per_sm = (uint32_t)occ;
-    const ace_tune t = tune ? *tune : idx->tune;
-    if (t.ctas_per_sm && t.ctas_per_sm < per_sm) per_sm = t.ctas_per_sm;
-    // levels of at most two blocks per SM: a CTA per block (match_small_kernel)
-    const bool small_ok = idx->h.log2_block <= kSmallMaxLog2B;
-    const size_t small_smem = small_smem_bytes(idx->h.log2_block);
-    if (small_ok && small_smem > 48 * 1024 && !idx->small_attr) {  // one value for every block size
-      CUDA_TRY(cudaFuncSetAttribute(match_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)small_smem_bytes(kSmallMaxLog2B)));
-      idx->small_attr = true;
+    if (occ_cta == 0) {
+      int o = 0;  // (levels of few blocks need no count: a CTA each)
+      rc = occupancy(match_cta_kernel<512>, idx->device, few / 32, cta_smem_bytes(log2B, few), &o);
+      if (rc == ACE_OK && o > 0)
+        rc = occupancy(match_cta_kernel<256>, idx->device, many / 32, cta_smem_bytes(log2B, many), &occ_cta);
+      if (rc) return rc;
     }
+    if (occ < 0 || occ_cta <= 0) return ACE_E_INVAL;
+    auto sms = [&](int per) {
+      return (uint64_t)idx->num_sms * (t.ctas_per_sm && (int)t.ctas_per_sm < per ? t.ctas_per_sm : (uint32_t)per);
+    };
     for (uint32_t l = 0; l < idx->n_levels; l++) {
       const uint32_t n = idx->level_start[l + 1] - idx->level_start[l];
       if (!n) continue;
       a.items = idx->d_order + idx->level_start[l];
       a.n_items = n;
       a.cur_level = l;
-      if (small_ok && n <= 2 * idx->num_sms) {
-        match_small_kernel<<<n, kSmallThreads, small_smem, s>>>(a);
+      if (n <= kCtaLevel * idx->num_sms) {
+        match_cta_kernel<512><<<n, few, cta_smem_bytes(log2B, few), s>>>(a);
         continue;
       }
-      const uint32_t grid = (uint32_t)std::min<uint64_t>((uint64_t)idx->num_sms * per_sm, (n + L.warps - 1) / L.warps);
-      match_level_kernel<<<grid, 32 * L.warps, (size_t)L.warps * L.smem[PASS_MATCH], s>>>(a);
+      if (dense) {
+        match_cta_kernel<256><<<(uint32_t)std::min<uint64_t>(sms(occ_cta), n), many, cta_smem_bytes(log2B, many), s>>>(a);
+        continue;
+      }
+      const uint32_t grid = (uint32_t)std::min<uint64_t>(sms(occ), (n + L.warps - 1) / L.warps);
+      level_kernel<<<grid, 32 * L.warps, (size_t)L.warps * kMatchSmem, s>>>(a);
     }
   }
   CUDA_TRY(cudaGetLastError());
@@ -3456,7 +3476,7 @@ ace_status ace_batch_create(const ace_index* const* idx, uint32_t n, void* const
   // the launch shape uses the largest block size's escape table
   rc = plan_launch(idx[0], tune, B.max_log2B, B.items, batch_decode_kernel<PASS_TOKENS>,
                    batch_decode_kernel<PASS_LITERALS>, batch_decode_kernel<PASS_MATCH>,
-                   batch_decode_kernel<PASS_FUSED>, &b->occ[0][0][0], &b->L);
+                   batch_decode_kernel<PASS_FUSED>, &b->occ[0][0][0], &b->L, kRing, false);
   if (rc == ACE_OK &&
       (cudaMemsetAsync(base, 0, B.recs, s) != cudaSuccess ||
        cudaMemcpyAsync(base + B.objs, od.data(), n * sizeof(ObjDesc), cudaMemcpyHostToDevice, s) != cudaSuccess ||
@@ -3667,7 +3687,7 @@ ace_status ace_cache_create(const ace_index* const* idx, uint32_t n, void* const
   // not level order); the fused entry only sizes like the match pass
   rc = plan_launch(idx[0], tune, log2B, C.max_work, cache_decode_kernel<PASS_TOKENS>,
                    cache_decode_kernel<PASS_LITERALS>, cache_decode_kernel<PASS_MATCH>,
-                   cache_decode_kernel<PASS_MATCH>, &c->occ[0][0][0], &c->L, kSeekRing);
+                   cache_decode_kernel<PASS_MATCH>, &c->occ[0][0][0], &c->L, kSeekRing, true);
   // header (epoch 1: no block is cached, since every ready flag starts at 0)
   CacheHdr h{};
   h.epoch = 1;

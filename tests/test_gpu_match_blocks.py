@@ -1,0 +1,107 @@
+"""The match pass's three ways through a block -- a CTA, a warp by rows, a warp
+by rounds -- on matches where they can go wrong: lengths around the rows' limit
+and the bit map's, every overlap, long runs (deep chains of copies), sources in
+the same rows, sources across block and window boundaries, few and many
+matches per block; the original bytes are the one correct answer."""
+import numpy as np
+import pytest
+
+import oracle
+import __graft_entry__
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2606_24531_gb300 import ace  # noqa: E402
+from paper_2606_24531_gb300.archive import DeviceArchive  # noqa: E402
+from paper_2606_24531_gb300.batch import DeviceBatch  # noqa: E402
+from paper_2606_24531_gb300.serve import SeekCache  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    __graft_entry__.build()
+    torch.cuda.set_device(0)
+
+
+def _copies(lengths, back, lit, total, seed):
+    """lit random bytes, then a copy of the given length from at most back
+    bytes earlier, in turn."""
+    rng = np.random.default_rng(seed)
+    out = bytearray(rng.integers(0, 256, 300).astype(np.uint8).tobytes())
+    k = 0
+    while len(out) < total:
+        out += rng.integers(0, 256, int(rng.integers(0, lit + 1))).astype(np.uint8).tobytes()
+        n = lengths[k % len(lengths)]
+        d = int(rng.integers(1, min(back, len(out)) + 1))
+        for _ in range(n):  # overlapping copies repeat
+            out.append(out[-d])
+        k += 1
+    return np.frombuffer(bytes(out[:total]), np.uint8)
+
+
+SHAPES = {
+    "short, recent sources": ((5, 6, 9, 13), 60, 3),
+    "around the rows' limit": ((31, 32, 33, 63, 64, 65), 4000, 40),
+    "every overlap": (tuple(range(4, 70)), 70, 2),
+    "runs": ((700, 3000), 9, 20),
+    "a run of one value": ((40000,), 1, 1),
+    "long": ((900, 2047, 2048, 2049, 5000), 30000, 300),
+    "few": ((20, 40), 8000, 1500),
+}
+
+
+def _check(da, data):
+    out = da.decode_all()
+    assert da.sync() == ace.ACE_OK
+    assert np.array_equal(out.cpu().numpy()[:data.size], data)
+
+
+@pytest.mark.parametrize("log2b", [8, 10, 12, 14, 16])
+@pytest.mark.parametrize("shape", sorted(SHAPES))
+def test_levels_seeks_batches_and_caches(shape, log2b):
+    lengths, back, lit = SHAPES[shape]
+    data = _copies(lengths, back, lit, 150_001, log2b)
+    # the encoders' archives (few levels) and the oracle's (deep chains of blocks)
+    arcs = [ace.ace_encode(data, log2b, 4), oracle.encode(data[:60_001], log2b, 4, 16)]
+    datas = [data, data[:60_001]]
+    for arc, d in zip(arcs, datas):
+        da = DeviceArchive(arc, max_seek_blocks=700)
+        _check(da, d)
+        for coord, n in ((0, 1), (d.size - 5001, 5001), (d.size // 3, 20_000)):
+            s = da.seek(coord, n)
+            assert da.sync() == ace.ACE_OK
+            assert np.array_equal(s.cpu().numpy(), d[coord:coord + n]), (coord, n)
+        if log2b >= 10:
+            cache = SeekCache([da], 800, 8, 1 << 17)
+            for got, (coord, n) in zip(cache.seek_many([(0, 100, 30_000), (0, 40_000, 9_999)]), ((100, 30_000), (40_000, 9_999))):
+                assert np.array_equal(got.cpu().numpy(), d[coord:coord + n])
+            cache.close()
+        da.close()
+    db = DeviceBatch(arcs)
+    db.decode()
+    assert db.sync() == ace.ACE_OK
+    for i, d in enumerate(datas):
+        assert np.array_equal(db.output(i).cpu().numpy(), d)
+    db.close()
+
+
+@pytest.mark.parametrize("shape", ["short, recent sources", "around the rows' limit", "long", "every overlap"])
+def test_levels_of_many_blocks(shape):
+    """More blocks in a level than get a CTA each: the warp-per-block kernels
+    (rows or rounds by the archive's matches) and the dense CTA kernel."""
+    lengths, back, lit = SHAPES[shape]
+    piece = _copies(lengths, back, lit, 1 << 20, 5)
+    for thin in (0, 1, 2):  # fewer matches per 16 KiB each time
+        rng = np.random.default_rng(thin)
+        rows = [piece]
+        for k in range(6):
+            if thin:
+                noise = rng.integers(0, 256, (1 << 20) * thin * 3).astype(np.uint8)
+                rows.append(noise)
+            rows.append(np.roll(piece, 4096 * k + k))
+        data = np.concatenate(rows)
+        arc = ace.ace_encode_gpu(torch.from_numpy(data).cuda(), 12, 4).cpu().numpy()
+        da = DeviceArchive(arc)
+        _check(da, data)
+        da.close()
