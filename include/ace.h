@@ -280,7 +280,9 @@ typedef struct {
  * of few blocks and archives of many short matches, a warp per block
  * otherwise), or, for archives of more than 32 levels, one persistent
  * launch, a CTA per block, in (level, block) order with bounded waits on
- * source blocks' ready flags.  ACE_SCHEDULE_FUSED does all of it in one persistent launch.
+ * source blocks' ready flags.  Decodes of few blocks take the token and
+ * literal passes as one launch, a warp per stream, and the match pass places
+ * the literals too.  ACE_SCHEDULE_FUSED does all of it in one persistent launch.
  * A source block whose level is not below its reader's makes the call
  * report ACE_E_CORRUPT.  tune may be NULL.  Asynchronous; check with
  * ace_sync.

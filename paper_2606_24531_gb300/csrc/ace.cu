@@ -496,67 +496,59 @@ __device__ __forceinline__ void warp_copy(uint8_t* dst, const uint8_t* src, uint
   if (lane < tail) dst[16 * nv + lane] = __ldcg(src + 16 * nv + lane);
 }
 
-// Token pass of one block (Section 3: the block boundary is the entry point
-// of the entropy layer): the length stream parsed into token positions, the
-// offset stream, and one record per match -- absolute source, destination in
-// the block, length -- for the match pass; the literal pass rebuilds the
-// token positions from these records.  Returns false if the block is corrupt
-// (the error is recorded).
-template <bool SEEK>
-__device__ bool token_block(const DecodeArgs& a, const TokMem& m, uint32_t b, uint32_t lane) {
+// A block's directory entry, a word per lane, and what follows from it.
+struct BlockHead {
+  uint32_t dv, blen, ntok, nesc, nlit;
+  __device__ BlockHead(const DecodeArgs& a, uint32_t b, uint32_t lane) {
+    const uint32_t* dw = reinterpret_cast<const uint32_t*>(a.dir + b);
+    dv = lane < 16 ? __ldg(dw + lane) : 0u;
+    blen = (uint32_t)min((uint64_t)1 << a.log2B, a.total - ((uint64_t)b << a.log2B));
+    ntok = __shfl_sync(kFull, dv, 12);
+    nesc = __shfl_sync(kFull, dv, 13);
+    nlit = __shfl_sync(kFull, dv, 9 + ACE_S_LIT);
+  }
+  // opens stream k: entry states, first renormalisation bytes
+  template <uint32_t RING>
+  __device__ bool open(const DecodeArgs& a, uint32_t k, uint8_t* ring, Stream& st, uint32_t lane) const {
+    const uint64_t soff =
+        (uint64_t)__shfl_sync(kFull, dv, 2 * k) | ((uint64_t)__shfl_sync(kFull, dv, 2 * k + 1) << 32);
+    const uint32_t sbytes = __shfl_sync(kFull, dv, 6 + k), nsym = __shfl_sync(kFull, dv, 9 + k);
+    const uint32_t mode = (__shfl_sync(kFull, dv, 14) >> (8 * k)) & 0xffu;  // mode[k] in byte k
+    return stream_open<RING>(a.arc + a.payload_off + soff, sbytes, nsym, ring, st, lane, mode);
+  }
+};
+
+// A block's opened length stream: the escape values, then two codes per token,
+// into the destination and length of every match's record.  Match t ends
+// token t (t < ntok - 1); its destination is the token's start plus its run.
+// SPLIT: the offset stream is decoded by another warp, which fills the
+// source's w bytes (the rest of them are set here), and the destination's word
+// holds above its 16 bits the literals before the match (blocks of at most
+// 32 KiB).  Returns false if
+// the stream is corrupt (recorded).
+template <bool SEEK, uint32_t RING, bool SPLIT>
+__device__ bool length_stream(const DecodeArgs& a, const BlockHead& h, Stream& sn, Lut& lut, uint8_t* ring,
+                              uint16_t* esc, uint32_t b, uint32_t lane) {
   bool ok = true;
-  const uint32_t* dw = reinterpret_cast<const uint32_t*>(a.dir + b);
-  uint32_t dv = lane < 16 ? __ldg(dw + lane) : 0u;
-  const uint64_t B = (uint64_t)1 << a.log2B, bstart = (uint64_t)b << a.log2B;
-  const uint32_t blen = (uint32_t)min(B, a.total - bstart);
-  const uint32_t w = a.w;
-  const uint32_t ntok = __shfl_sync(kFull, dv, 12), nesc = __shfl_sync(kFull, dv, 13);
-  const uint32_t nlit = __shfl_sync(kFull, dv, 9 + ACE_S_LIT);
-  const uint32_t modes = __shfl_sync(kFull, dv, 14);  // mode[k] in byte k
-  const uint32_t lt = lanemask_lt();
-
-  Stream sn, so;
-#pragma unroll
-  for (int k = ACE_S_LEN; k <= ACE_S_OFF; k++) {
-    uint64_t soff = (uint64_t)__shfl_sync(kFull, dv, 2 * k) | ((uint64_t)__shfl_sync(kFull, dv, 2 * k + 1) << 32);
-    uint32_t sbytes = __shfl_sync(kFull, dv, 6 + k), nsym = __shfl_sync(kFull, dv, 9 + k);
-    if (!stream_open(a.arc + a.payload_off + soff, sbytes, nsym, m.ring + (k - ACE_S_LEN) * kRing,
-                     k == ACE_S_LEN ? sn : so, lane, (modes >> (8 * k)) & 0xffu))
-      fail(a, ok, ACE_E_CORRUPT, b, 20 + k, lane);
-  }
-  if (!ok || ntok > a.max_ntok) {
-    fail(a, ok, ACE_E_CORRUPT, b, 23, lane);
-    cp_async_wait<0>();
-    __syncwarp();
-    return false;
-  }
-  cp_async_wait<2>();
-  __syncwarp();
-  uint8_t* rn = m.ring;
-  uint8_t* ro = m.ring + kRing;
-
-  // ---- lengths: escape values, then two codes per token
-  if (!lut_build(sn, *m.lut, lane)) fail(a, ok, ACE_E_CORRUPT, b, 30, lane);
-  uint8_t* escb = reinterpret_cast<uint8_t*>(m.esc);
+  const uint32_t lt = lanemask_lt(), ntok = h.ntok, nesc = h.nesc;
+  if (!lut_build(sn, lut, lane, SPLIT ? kSplitSearch : kSearchMaxSymbols)) fail(a, ok, ACE_E_CORRUPT, b, 30, lane);
+  uint8_t* escb = reinterpret_cast<uint8_t*>(esc);
   if (ok)
-    rans_run(sn, rn, *m.lut, 2 * nesc, lane, lt, [&](bool act, uint32_t i, uint32_t s) {
+    rans_run<RING>(sn, ring, lut, 2 * nesc, lane, lt, [&](bool act, uint32_t i, uint32_t s) {
       if (act) escb[i] = (uint8_t)s;
     });
   __syncwarp();
   uint32_t out_pos = 0, lit_pos = 0, esc_rank = 0;
   bool bad = false;
   const uint32_t cbase = 2 * nesc, cend = cbase + 2 * ntok;
-  // match t's record is written whole here (destination and length; the
-  // source's bytes follow from the offset stream); a match ends token t
-  // (t < ntok - 1), its destination is the token's start plus its run
   uint4* const rec4 = reinterpret_cast<uint4*>(recs_of<SEEK>(a, b));
-  if (ok) rans_run(sn, rn, *m.lut, cend, lane, lt, [&](bool act, uint32_t i, uint32_t s) {
+  if (ok) rans_run<RING>(sn, ring, lut, cend, lane, lt, [&](bool act, uint32_t i, uint32_t s) {
     bool e = act && s == 255;
     uint32_t eb = __ballot_sync(kFull, e);
     uint32_t r = esc_rank + __popc(eb & lt);
     uint32_t v = s;
     if (e) {
-      if (r < nesc) v = 255u + m.esc[r];
+      if (r < nesc) v = 255u + esc[r];
       else bad = true;
     }
     esc_rank += __popc(eb);
@@ -566,25 +558,46 @@ __device__ bool token_block(const DecodeArgs& a, const TokMem& m, uint32_t b, ui
     uint32_t io = warp_incl_sum(to, lane), il = warp_incl_sum(tl, lane);
     if (own) {
       uint32_t t = (i - cbase) >> 1;
-      if (t + 1 < ntok) rec4[t] = make_uint4(0u, 0u, out_pos + io - to + lr, ml);
-      else if (ml) bad = true;  // the block's last token carries no match
+      const uint32_t D = out_pos + io - to + lr;
+      if (t + 1 >= ntok) {
+        if (ml) bad = true;  // the block's last token carries no match
+      } else if (SPLIT) {
+        uint8_t* const r8 = reinterpret_cast<uint8_t*>(rec4 + t);
+        if (a.w == 4) {
+          *reinterpret_cast<uint32_t*>(r8 + 4) = 0;
+        } else {
+          r8[5] = 0;
+          *reinterpret_cast<uint16_t*>(r8 + 6) = 0;
+        }
+        *reinterpret_cast<uint2*>(r8 + 8) = make_uint2(D | (lit_pos + il) << 16, ml);
+      } else {
+        rec4[t] = make_uint4(0u, 0u, D, ml);
+      }
     }
     out_pos += __shfl_sync(kFull, io, 31);
     lit_pos += __shfl_sync(kFull, il, 31);
-    if (out_pos > blen) bad = true;
+    if (out_pos > h.blen) bad = true;
   });
-  bad |= out_pos != blen || lit_pos != nlit || esc_rank != nesc;
+  bad |= out_pos != h.blen || lit_pos != h.nlit || esc_rank != nesc;
   if (__any_sync(kFull, bad)) fail(a, ok, ACE_E_CORRUPT, b, 32, lane);
+  if (ok && !stream_finished(sn)) fail(a, ok, ACE_E_CORRUPT, b, 40, lane);
+  return ok;
+}
 
-  // ---- absolute offsets: off_width bytes for every token but the last
-  const uint32_t nm = ntok - 1;
-  if (ok && nm) {
-    __syncwarp();  // the records' zero source bytes are written before any lane fills them
-    if (!lut_build(so, *m.lut, lane)) fail(a, ok, ACE_E_CORRUPT, b, 33, lane);
+// A block's opened offset stream: off_width bytes for every token but the
+// last, the match's absolute source (little endian), written straight into
+// its record.  A source at or after its destination is caught where sources
+// are read: match_block and match_cta check every record.
+template <bool SEEK, uint32_t RING>
+__device__ bool offset_stream(const DecodeArgs& a, const BlockHead& h, Stream& so, Lut& lut, uint8_t* ring, uint32_t b,
+                              uint32_t lane, uint32_t search) {
+  bool ok = true;
+  const uint32_t lt = lanemask_lt(), w = a.w, nm = h.ntok - 1;
+  if (nm) {
+    if (!lut_build(so, lut, lane, search)) fail(a, ok, ACE_E_CORRUPT, b, 33, lane);
     const uint32_t oend = w * nm;
-    // offset byte i is byte i mod w of match i / w's absolute source (little
-    // endian, w = 4 or 5), written straight into its record
-    uint8_t* const rb = reinterpret_cast<uint8_t*>(rec4);
+    // offset byte i is byte i mod w of match i / w's source
+    uint8_t* const rb = reinterpret_cast<uint8_t*>(recs_of<SEEK>(a, b));
     auto at = [&](uint32_t i) -> uint8_t* {
       const uint32_t t = w == 4 ? i >> 2 : __umulhi(i, 0xCCCCCCCDu) >> 2;  // floor(i / 5) for every 32-bit i
       return rb + 16 * (size_t)t + (i - w * t);
@@ -594,24 +607,89 @@ __device__ bool token_block(const DecodeArgs& a, const TokMem& m, uint32_t b, ui
     };
     if (ok && !so.stored && so.k == 0 && oend >= 64) {  // slot-table streams: full rounds in the fast loop
       uint32_t i = lane;
-      table_full_rounds(so, ro, *m.lut, oend >> 5, lane, lt, [](uint32_t) {}, [&](uint32_t s, uint32_t) {
+      table_full_rounds<RING>(so, ring, lut, oend >> 5, lane, lt, [](uint32_t) {}, [&](uint32_t s, uint32_t) {
         *at(i) = (uint8_t)s;
         i += 32;
       });
     }
-    if (ok) rans_run(so, ro, *m.lut, oend, lane, lt, put);
+    if (ok) rans_run<RING>(so, ring, lut, oend, lane, lt, put);
   }
+  if (ok && !stream_finished(so)) fail(a, ok, ACE_E_CORRUPT, b, 40, lane);
+  return ok;
+}
+
+// Token pass of one block (Section 3: the block boundary is the entry point
+// of the entropy layer): the length stream parsed into token positions, the
+// offset stream, and one record per match -- absolute source, destination in
+// the block, length -- for the match pass; the literal pass rebuilds the
+// token positions from these records.  Returns false if the block is corrupt
+// (the error is recorded).
+template <bool SEEK>
+__device__ bool token_block(const DecodeArgs& a, const TokMem& m, uint32_t b, uint32_t lane) {
+  bool ok = true;
+  const BlockHead h(a, b, lane);
+  Stream sn, so;
+  if (!h.open<kRing>(a, ACE_S_LEN, m.ring, sn, lane)) fail(a, ok, ACE_E_CORRUPT, b, 21, lane);
+  if (!h.open<kRing>(a, ACE_S_OFF, m.ring + kRing, so, lane)) fail(a, ok, ACE_E_CORRUPT, b, 22, lane);
+  if (!ok || h.ntok > a.max_ntok) {
+    fail(a, ok, ACE_E_CORRUPT, b, 23, lane);
+    cp_async_wait<0>();
+    __syncwarp();
+    return false;
+  }
+  cp_async_wait<2>();
   __syncwarp();
-  // a source at or after its destination is caught where sources are read:
-  // match_block and match_cta check every record
-  if (ok) {
-    bool fin = stream_finished(sn) && stream_finished(so);
-    if (!__all_sync(kFull, fin)) fail(a, ok, ACE_E_CORRUPT, b, 40, lane);
-  }
+  ok = length_stream<SEEK, kRing, false>(a, h, sn, *m.lut, m.ring, m.esc, b, lane);
+  __syncwarp();  // the records' zero source bytes are written before any lane fills them
+  if (ok) ok = offset_stream<SEEK, kRing>(a, h, so, *m.lut, m.ring + kRing, b, lane, kSearchMaxSymbols);
   cp_async_wait<0>();  // no ring fill may land after the next block reuses the rings
   __syncwarp();
   return ok;
 }
+
+// One stream of a block by a warp of its own, for calls of few blocks
+// (entropy_kernel): lengths and offsets into the match records as the token
+// pass does, literals in order to the end of the block's place in the output,
+// from where match_cta places them (a literal's final position is never after
+// this one, so placing in ascending windows never overwrites one still to be
+// read).
+template <bool SEEK>
+__device__ void stream_job(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32_t k, uint32_t lane) {
+  bool ok = true;
+  Lut& lut = *reinterpret_cast<Lut*>(smem);
+  uint8_t* ring = smem + sizeof(Lut);
+  uint16_t* esc = reinterpret_cast<uint16_t*>(ring + kSeekRing);
+  const BlockHead h(a, b, lane);
+  Stream st;
+  if (!h.open<kSeekRing>(a, k, ring, st, lane)) fail(a, ok, ACE_E_CORRUPT, b, 20 + k, lane);
+  if (h.ntok > a.max_ntok) fail(a, ok, ACE_E_CORRUPT, b, 23, lane);
+  cp_async_wait<kSeekRing / kSeg - 2>();
+  __syncwarp();
+  if (ok && k == ACE_S_LEN) length_stream<SEEK, kSeekRing, true>(a, h, st, lut, ring, esc, b, lane);
+  if (ok && k == ACE_S_OFF) offset_stream<SEEK, kSeekRing>(a, h, st, lut, ring, b, lane, kSplitSearch);
+  if (ok && k == ACE_S_LIT && st.nsym) {
+    if (!lut_build(st, lut, lane, kSplitSearch)) fail(a, ok, ACE_E_CORRUPT, b, 35, lane);
+    const uint32_t lt = lanemask_lt();
+    uint8_t* const to =
+        (SEEK ? a.out + slot_base(a, b) : a.out + ((uint64_t)b << a.log2B)) + (h.blen - h.nlit);  // nlit <= blen: the index
+    if (ok && !st.stored && st.k == 0 && st.nsym >= 64) {
+      uint8_t* op = to + lane;
+      table_full_rounds<kSeekRing, 4>(st, ring, lut, st.nsym >> 5, lane, lt, [](uint32_t) {}, [&](uint32_t s, uint32_t) {
+        *op = (uint8_t)s;
+        op += 32;
+      });
+    }
+    if (ok)
+      rans_run<kSeekRing>(st, ring, lut, st.nsym, lane, lt, [&](bool act, uint32_t i, uint32_t s) {
+        if (act) to[i] = (uint8_t)s;
+      });
+    if (ok && !stream_finished(st)) fail(a, ok, ACE_E_CORRUPT, b, 41, lane);
+  }
+  cp_async_wait<0>();
+  __syncwarp();
+}
+
+__host__ __device__ inline uint32_t job_smem_bytes(uint32_t escn) { return (sizeof(Lut) + kSeekRing + 2 * escn + 15) & ~15u; }
 
 // Literal pass of one block, after the token pass of every block succeeded:
 // literal i lands at i plus the shift of its run.  Token t's run starts where
@@ -1189,7 +1267,12 @@ __host__ __device__ inline uint32_t cta_smem_bytes(uint32_t log2B, uint32_t thre
   return 2 * (log2B >= 14 ? kCtaWindow : 1u << log2B) + threads / 32 * kCtaWarpSmem;
 }
 
-template <bool SEEK, bool WAIT>
+//
+// LITS: after stream jobs.  The literals are still in order at the end of the
+// block's place (a record's destination word holds above it the literals
+// before the match), so literal runs are laid in rows too, the last one as
+// token nm, and every byte of the window gets its entry from a row.
+template <bool SEEK, bool WAIT, bool LITS>
 __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32_t nm, uint32_t epoch, uint32_t lvl) {
   __shared__ uint32_t s_group;
   const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nt = blockDim.x, nw = nt >> 5;
@@ -1202,7 +1285,12 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
   const uint32_t ebase = (uint32_t)__cvta_generic_to_shared(e);
   // groups of 32 matches, a warp each; with fewer groups than warps, several
   // warps each, sharing the group's bytes
-  const uint32_t ng = (nm + 31) / 32, split = ng ? max(1u, nw / ng) : 1u;
+  const uint32_t nt32 = nm + (LITS ? 1 : 0), ng = (nt32 + 31) / 32, split = ng ? max(1u, nw / ng) : 1u;
+  uint32_t nlit = 0;
+  if (LITS) {  // the block's literals: those before its last match, and what follows it
+    const uint4 r = nm ? __ldcg(rec + nm - 1) : make_uint4(0, 0, 0, 0);
+    nlit = (r.z >> 16) + blen - (r.z & 0xffffu) - r.w;
+  }
   const uint32_t part = wid % split, step = nw / split;
   uint4* row = reinterpret_cast<uint4*>(smem + 2 * min((uint32_t)B, kCtaWindow) + wid * kCtaWarpSmem);
   uint32_t* bits = reinterpret_cast<uint32_t*>(row + 32);
@@ -1218,7 +1306,7 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
     rn = fetch(g);
     // every byte known as the literal pass left it; match bytes are set next
     const uint8_t* wbase = obase + w0;
-    for (uint32_t j0 = 16 * tid; j0 < wn; j0 += 16 * nt * 4) {
+    for (uint32_t j0 = 16 * tid; !LITS && j0 < wn; j0 += 16 * nt * 4) {
       uint4 v[4];
 #pragma unroll
       for (uint32_t u = 0; u < 4; u++) {
@@ -1245,125 +1333,159 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
                            __byte_perm(v[u].w, 0x80u, 0x4140), __byte_perm(v[u].w, 0x80u, 0x4342));
       }
     }
+    if (LITS && tid < 16 && wn + tid < ((wn + 15) & ~15u)) e[wn + tid] = 0x8000;  // the last vector's rest
     if (tid == 0) s_group = first;
     __syncthreads();
 
     bool bad = false, timeout = false;
     uint32_t last = first;
-    for (; g < ng; g += step) {
-      const uint4 r = rn;
-      rn = fetch(g + step);
-      const uint64_t S = (uint64_t)r.x | ((uint64_t)r.y << 32);
-      const uint32_t D = r.z;
-      uint32_t L = r.w;
-      if (L && (S >= bstart + D || (uint64_t)D + L > blen)) {  // a source precedes its match, which stays in the block
-        bad = true;
-        L = 0;
+    // with waits, the literals of every group first: they wait for nothing
+    constexpr uint32_t kPhases = LITS && WAIT ? 2 : 1;
+#pragma unroll
+    for (uint32_t phase = 0; phase < kPhases; phase++) {
+      const bool place = LITS && phase == 0, copy = phase + 1 == kPhases;
+      if (phase) {
+        g = wid >= step * split ? ng : first + wid / split;
+        rn = fetch(g);
       }
-      if (__shfl_sync(kFull, D, 0) >= w0 + wn) break;  // (destinations ascend) past the window
-      last = g;
-      const uint64_t dist = bstart + D - S;
-      if (L && S < bstart) {  // the blocks before this one that it reads
-        const uint32_t k0 = (uint32_t)(S >> a.log2B);
-        const uint32_t k1 = (uint32_t)((min(S + min((uint64_t)L, dist), bstart) - 1) >> a.log2B);
-        for (uint32_t k = k0; k <= k1; k++) {
-          if (!WAIT) {
-            bad |= __ldg(a.level + k) >= lvl;
-            continue;
+      for (; g < ng; g += step) {
+        const uint4 r = rn;
+        rn = fetch(g + step);
+        const uint64_t S = (uint64_t)r.x | ((uint64_t)r.y << 32);
+        uint32_t D = LITS ? r.z & 0xffffu : r.z, lits = 0, lr = 0;
+        uint32_t L = r.w;
+        if (LITS) {  // lits: literals before the match; lr: those of its token's run
+          lits = r.z >> 16;
+          if (32 * g + lane >= nm) {
+            D = blen;
+            lits = nlit;
           }
-          // at a lower level (work lists are in level order, so the wait ends;
-          // the block cache keeps no levels), and a member of a seek's closure
-          // (its flag carries the call's epoch, pending or published)
-          if (a.level && __ldg(a.level + k) >= __ldg(a.level + b)) bad = true;
-          const uint32_t f = ld_relaxed(a.ready + k);
-          if (SEEK && a.closure_flags && (f & ~kPendingFlag) != epoch) bad = true;
-          if (!bad && !timeout && f != epoch && !wait_flag(a.ready + k, epoch, a.timeout_ns, &a.sh->status)) timeout = true;
+          uint32_t before = __shfl_up_sync(kFull, lits, 1);
+          if (lane == 0) before = g ? __ldcg(&rec[32 * g - 1].z) >> 16 : 0u;
+          lr = lits - before;  // (0 past token nm)
         }
-        if (bad || timeout) L = 0;
-      }
-      if (WAIT && __any_sync(kFull, L && S < bstart)) {
-        fence_acquire();
-        __syncwarp();  // any lane may read a source whose flags another lane checked
-      }
-      // the part inside the window, laid end to end with the group's others
-      const uint32_t d0 = max(D, w0), d1 = min(D + L, w0 + wn), n = L && d0 < d1 ? d1 - d0 : 0u;
-      const uint32_t incl = warp_incl_sum(n, lane), X = incl - n, T = __shfl_sync(kFull, incl, 31);
-      const uint32_t have = __ballot_sync(kFull, n != 0);
-      bool odd = false;
-      if (n) {
-        // byte c of the group's bytes: its entry's address, twice its source's
-        // place in the window (below 0: before it) and its source's address.  Marked in the
-        // address's top bits: a seek's source in more than one slot (the
-        // position instead), and a match overlapping its source (distance and
-        // start instead: its bytes repeat the first distance's, not one another
-        // down a long chain)
-        const uint64_t s0 = bstart + d0 - dist;
-        const int32_t rel = (int32_t)max((int64_t)(s0 - bstart) - (int64_t)w0, -(int64_t)(1 << 29));
-        uint64_t from;
-        if (SEEK && rel < 0 && s0 >> a.log2B != min(s0 + n - 1, bstart + w0 - 1) >> a.log2B) {
-          from = (s0 - X) | 1ull << 63;
-          odd = true;
-        } else {
-          from = reinterpret_cast<uintptr_t>(Addr<SEEK>::at(a, s0, b, obase)) - X;
+        if (L && (S >= bstart + D || (uint64_t)D + L > blen)) {  // a source precedes its match, which stays in the block
+          bad = true;
+          L = 0;
         }
-        uint32_t w = (uint32_t)(2 * (rel - (int32_t)X));
-        if (dist < L) {
-          from = (uint64_t)(0x40000000u | (D + 0x10000u - w0)) << 32 | dist;
-          w = 0xC0000000u;
-          odd = true;
-        }
-        row[__popc(have & lt)] = make_uint4((uint32_t)from, (uint32_t)(from >> 32), ebase + 2 * (d0 - w0 - X), w);
-      }
-      odd = __any_sync(kFull, odd);
-      constexpr uint32_t kBatch = 32 * kCtaUnroll;
-      const uint32_t share = ((T + split - 1) / split + kBatch - 1) & ~(kBatch - 1);
-      const uint32_t te = min(T, (part + 1) * share);
-      for (uint32_t cb = part * share; cb < te; cb += kCtaRowBytes) {  // one turn but for long matches
-#pragma unroll
-        for (uint32_t k = 0; k < kCtaRowBytes / 32; k += 32) bits[k + lane] = 0;
-        __syncwarp();
-        if (n && X - cb < kCtaRowBytes) atomicOr(bits + ((X - cb) >> 5), 1u << (X & 31));
-        uint32_t rank = __popc(__ballot_sync(kFull, n && X < cb)) - 1;  // the match before the row's first start
-        __syncwarp();
-        const uint32_t ce = min(te, cb + kCtaRowBytes);
-        auto rows = [&](auto marked) {
-          constexpr bool special = decltype(marked)::value;
-          const uint4* words = reinterpret_cast<const uint4*>(bits);
-          for (uint32_t c = cb + lane; c < ce + lane; c += 32 * kCtaUnroll) {
-            const uint4 w4 = *words++;
-            const uint32_t w[kCtaUnroll] = {w4.x, w4.y, w4.z, w4.w};
-            uint32_t v[kCtaUnroll], at[kCtaUnroll];
-#pragma unroll
-            for (uint32_t u = 0; u < kCtaUnroll; u++) {
-              const uint4 m = row[rank + __popc(w[u] & le)];
-              rank += __popc(w[u]);
-              const uint32_t q = c + 32 * u;
-              at[u] = m.z + 2 * q;
-              v[u] = m.w + 2 * q;
-              if ((int32_t)v[u] < 0 && q < ce) {
-                const uint64_t from = ((uint64_t)m.y << 32 | m.x) + q;
-                if (special && m.y >> 30 == 1) {  // overlapping: byte (place - start) mod distance of the source
-                  const int32_t start = (int32_t)(m.y & 0x3ffffu) - 0x10000;
-                  const int32_t s = start - (int32_t)m.x + (int32_t)(((at[u] - ebase) / 2 - (uint32_t)start) % m.x);
-                  v[u] = s >= 0 ? 2 * (uint32_t)s
-                                : 0x8000u | ld_src<!WAIT>(Addr<SEEK>::at(a, bstart + w0 + (int64_t)s, b, obase));
-                } else if (special && SEEK && m.y >> 31) {
-                  v[u] = 0x8000u | ld_src<!WAIT>(Addr<SEEK>::at(a, from & ~(1ull << 63), b, obase));
-                } else {
-                  v[u] = 0x8000u | ld_src<!WAIT>(reinterpret_cast<const uint8_t*>(from));
-                }
-              }
+        if (lr > D) bad = true, lr = 0;  // the length stream's own checks hold: only a changed archive gets here
+        if (__shfl_sync(kFull, D - lr, 0) >= w0 + wn) break;  // (destinations ascend) past the window
+        last = g;
+        const uint64_t dist = bstart + D - S;
+        if (copy && L && S < bstart) {  // the blocks before this one that it reads
+          const uint32_t k0 = (uint32_t)(S >> a.log2B);
+          const uint32_t k1 = (uint32_t)((min(S + min((uint64_t)L, dist), bstart) - 1) >> a.log2B);
+          for (uint32_t k = k0; k <= k1; k++) {
+            if (!WAIT) {
+              bad |= __ldg(a.level + k) >= lvl;
+              continue;
             }
-#pragma unroll
-            for (uint32_t u = 0; u < kCtaUnroll; u++)
-              if (c + 32 * u < ce) asm volatile("st.shared.u16 [%0], %1;" ::"r"(at[u]), "h"((uint16_t)v[u]) : "memory");
+            // at a lower level (work lists are in level order, so the wait ends;
+            // the block cache keeps no levels), and a member of a seek's closure
+            // (its flag carries the call's epoch, pending or published)
+            if (a.level && __ldg(a.level + k) >= __ldg(a.level + b)) bad = true;
+            const uint32_t f = ld_relaxed(a.ready + k);
+            if (SEEK && a.closure_flags && (f & ~kPendingFlag) != epoch) bad = true;
+            if (!bad && !timeout && f != epoch && !wait_flag(a.ready + k, epoch, a.timeout_ns, &a.sh->status)) timeout = true;
           }
+          if (bad || timeout) L = 0;
+        }
+        if (WAIT && copy && __any_sync(kFull, L && S < bstart)) {
+          fence_acquire();
+          __syncwarp();  // any lane may read a source whose flags another lane checked
+        }
+        // The warp's share of n bytes per lane laid end to end, in rows.  Byte c
+        // of them: its entry's address, twice its source's place in the window
+        // (below 0: before it, or marked) and its source's address, each less
+        // c's share.  Marked in the address's top bits: a seek's source in more
+        // than one slot (the position instead), and a match overlapping its
+        // source (distance and start instead: its bytes repeat the first
+        // distance's, not one another down a long chain).
+        auto lay = [&](uint32_t n, uint32_t dst, int32_t rel, uint64_t from, bool marked) {
+          const uint32_t incl = warp_incl_sum(n, lane), X = incl - n, T = __shfl_sync(kFull, incl, 31);
+          const uint32_t have = __ballot_sync(kFull, n != 0);
+          if (n)
+            row[__popc(have & lt)] =
+                marked && (from >> 62 & 1)
+                    ? make_uint4((uint32_t)from, (uint32_t)(from >> 32), ebase + 2 * (dst - X), 0xC0000000u)
+                    : make_uint4((uint32_t)(from - X), (uint32_t)((from - X) >> 32) | (marked ? 0x80000000u : 0u),
+                                 ebase + 2 * (dst - X), (uint32_t)(2 * (rel - (int32_t)X)));
+          const bool odd = __any_sync(kFull, marked);
+          constexpr uint32_t kBatch = 32 * kCtaUnroll;
+          const uint32_t share = ((T + split - 1) / split + kBatch - 1) & ~(kBatch - 1);
+          const uint32_t te = min(T, (part + 1) * share);
+          for (uint32_t cb = part * share; cb < te; cb += kCtaRowBytes) {  // one turn but for long matches
+  #pragma unroll
+            for (uint32_t k = 0; k < kCtaRowBytes / 32; k += 32) bits[k + lane] = 0;
+            __syncwarp();
+            if (n && X - cb < kCtaRowBytes) atomicOr(bits + ((X - cb) >> 5), 1u << (X & 31));
+            uint32_t rank = __popc(__ballot_sync(kFull, n && X < cb)) - 1;  // the one before the row's first start
+            __syncwarp();
+            const uint32_t ce = min(te, cb + kCtaRowBytes);
+            auto rows = [&](auto kind) {
+              constexpr bool special = decltype(kind)::value;
+              const uint4* words = reinterpret_cast<const uint4*>(bits);
+              for (uint32_t c = cb + lane; c < ce + lane; c += kBatch) {
+                const uint4 w4 = *words++;
+                const uint32_t w[kCtaUnroll] = {w4.x, w4.y, w4.z, w4.w};
+                uint32_t v[kCtaUnroll], at[kCtaUnroll];
+  #pragma unroll
+                for (uint32_t u = 0; u < kCtaUnroll; u++) {
+                  const uint4 m = row[rank + __popc(w[u] & le)];
+                  rank += __popc(w[u]);
+                  const uint32_t q = c + 32 * u;
+                  at[u] = m.z + 2 * q;
+                  v[u] = m.w + 2 * q;
+                  if ((int32_t)v[u] < 0 && q < ce) {
+                    const uint64_t src = ((uint64_t)m.y << 32 | m.x) + q;
+                    if (special && m.y >> 30 == 1) {  // overlapping: byte (place - start) mod distance of the source
+                      const int32_t start = (int32_t)(m.y & 0x3ffffu) - 0x10000;
+                      const int32_t s = start - (int32_t)m.x + (int32_t)(((at[u] - ebase) / 2 - (uint32_t)start) % m.x);
+                      v[u] = s >= 0 ? 2 * (uint32_t)s
+                                    : 0x8000u | ld_src<!WAIT>(Addr<SEEK>::at(a, bstart + w0 + (int64_t)s, b, obase));
+                    } else if (special && SEEK && m.y >> 31) {
+                      v[u] = 0x8000u | ld_src<!WAIT>(Addr<SEEK>::at(a, src & ~(1ull << 63), b, obase));
+                    } else {
+                      v[u] = 0x8000u | ld_src<!WAIT>(reinterpret_cast<const uint8_t*>(src));
+                    }
+                  }
+                }
+  #pragma unroll
+                for (uint32_t u = 0; u < kCtaUnroll; u++)
+                  if (c + 32 * u < ce) asm volatile("st.shared.u16 [%0], %1;" ::"r"(at[u]), "h"((uint16_t)v[u]) : "memory");
+              }
+            };
+            if (odd) rows(std::true_type());
+            else rows(std::false_type());
+            __syncwarp();  // the next bytes reuse the map
+          }
+          __syncwarp();
         };
-        if (odd) rows(std::true_type());
-        else rows(std::false_type());
-        __syncwarp();  // the next bytes reuse the map
+        if (place) {  // the literal run before the match, as far as it lies in the window
+          const uint32_t d0 = max(D - lr, w0), d1 = min(D, w0 + wn), n = d0 < d1 && lr ? d1 - d0 : 0u;
+          const uint8_t* from = obase + (blen - nlit) + (lits - (D - d0));
+          lay(n, d0 - w0, -(1 << 29), reinterpret_cast<uintptr_t>(from), false);
+        }
+        if (!copy) continue;
+        // the match, as far as it lies in the window
+        const uint32_t d0 = max(D, w0), d1 = min(D + L, w0 + wn), n = L && d0 < d1 ? d1 - d0 : 0u;
+        const uint64_t s0 = bstart + d0 - dist;
+        const int32_t rel = n ? (int32_t)max((int64_t)(s0 - bstart) - (int64_t)w0, -(int64_t)(1 << 29)) : 0;
+        uint64_t from = 0;
+        bool marked = false;
+        if (n) {
+          if (dist < L) {
+            from = (uint64_t)(0x40000000u | (D + 0x10000u - w0)) << 32 | dist;
+            marked = true;
+          } else if (SEEK && rel < 0 && s0 >> a.log2B != min(s0 + n - 1, bstart + w0 - 1) >> a.log2B) {
+            from = s0;
+            marked = true;
+          } else {
+            from = reinterpret_cast<uintptr_t>(Addr<SEEK>::at(a, s0, b, obase));
+          }
+        }
+        lay(n, d0 - w0, rel, from, marked);
       }
-      __syncwarp();
     }
     if (lane == 0) atomicMax(&s_group, last);
     const bool any_bad = __syncthreads_or(bad), any_late = __syncthreads_or(timeout);
@@ -1452,11 +1574,13 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
 // blocks' flags, then the block's publication.  One launch covers the whole
 // decode, so the issue-bound entropy decode of some warps overlaps the
 // latency-bound match copies of others on the same SM.
-enum { PASS_TOKENS = 0, PASS_LITERALS = 1, PASS_MATCH = 2, PASS_FUSED = 3 };
+// PASS_PLACE is PASS_MATCH after stream jobs, which leave the literals to it.
+enum { PASS_TOKENS = 0, PASS_LITERALS = 1, PASS_MATCH = 2, PASS_FUSED = 3, PASS_PLACE = 4 };
 
 // Every pass is held to 64 registers a thread: 256 threads, or the match
 // pass's CTAs of up to 512.
-#define ACE_PASS_BOUNDS(P) __launch_bounds__((P) == PASS_MATCH ? kCtaThreads : 256, (P) == PASS_MATCH ? 2 : 4)
+#define ACE_PASS_CTA(P) ((P) == PASS_MATCH || (P) == PASS_PLACE)
+#define ACE_PASS_BOUNDS(P) __launch_bounds__(ACE_PASS_CTA(P) ? kCtaThreads : 256, ACE_PASS_CTA(P) ? 2 : 4)
 
 // Publishes block b (its writes visible device-wide before the flag).
 __device__ __forceinline__ void publish(uint32_t* ready, uint32_t b, uint32_t epoch, uint32_t lane) {
@@ -1492,7 +1616,7 @@ __device__ __forceinline__ void cta_blocks(uint32_t n_items, uint32_t* ticket, F
 template <int PASS>
 __device__ __forceinline__ bool stop_early(const uint32_t* status) {
   const bool set = *(const volatile uint32_t*)status != 0;
-  return PASS == PASS_MATCH ? __syncthreads_or(set) : set;
+  return ACE_PASS_CTA(PASS) ? __syncthreads_or(set) : set;
 }
 
 // Blocks level l of a fused call holds (whole decode: the index's level
@@ -1649,11 +1773,11 @@ __global__ void ACE_PASS_BOUNDS(PASS) decode_kernel(DecodeArgs a) {
     fused_loop<SEEK>(ArchiveJobs<SEEK>{a}, a.sh, n_items, a.timeout_ns, wsm, lane, epoch, a.window);
     return;
   }
-  if (PASS == PASS_MATCH) {
+  if (ACE_PASS_CTA(PASS)) {
     cta_blocks(n_items, &a.sh->ticket3, [&](uint32_t it) {
       const uint32_t b = __ldg(a.items + it);
       const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
-      const bool ok = match_cta<SEEK, true>(a, smem, b, ntok ? ntok - 1 : 0, epoch, 0);
+      const bool ok = match_cta<SEEK, true, PASS == PASS_PLACE>(a, smem, b, ntok ? ntok - 1 : 0, epoch, 0);
       publish_cta(a.ready, b, epoch);
       if (SEEK && ok && a.slice) {
         // the part of this block inside [coord, coord + len) to the caller, a share per warp
@@ -1685,6 +1809,18 @@ __global__ void ACE_PASS_BOUNDS(PASS) decode_kernel(DecodeArgs a) {
     constexpr uint32_t ring = SEEK ? kSeekRing : kRing;
     literal_block<SEEK, ring>(a, carve_lit(wsm, a.window, ring), b, lane);
   }
+}
+
+// The entropy layer of few blocks: a warp per stream (a block's three streams
+// are independent entry points, Section 3), each a CTA of its own so that they
+// spread over the SMs.  A block's time is then its longest stream's, where the
+// token and literal passes add the three up.
+template <bool SEEK>
+__global__ void __launch_bounds__(32) entropy_kernel(DecodeArgs a) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const uint32_t lane = threadIdx.x;
+  const uint32_t n_jobs = 3 * (SEEK ? *(volatile uint32_t*)&a.sh->n_work : a.n_items);
+  for (uint32_t j = blockIdx.x; j < n_jobs; j += gridDim.x) stream_job<SEEK>(a, smem, __ldg(a.items + j / 3), j % 3, lane);
 }
 
 // The match pass of one dependency level of a whole decode: every lower
@@ -1725,14 +1861,14 @@ __global__ void __maxnreg__(72) match_level_kernel(DecodeArgs a) {
 }
 
 // The same with a CTA per block.
-template <uint32_t THREADS>
+template <uint32_t THREADS, bool LITS>
 __global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 4) match_cta_kernel(DecodeArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   if (__syncthreads_or(*(volatile uint32_t*)&a.sh->status != 0)) return;  // the same answer for the whole CTA
   for (uint32_t it = blockIdx.x; it < a.n_items; it += gridDim.x) {
     const uint32_t b = __ldg(a.items + it);
     const uint64_t m0 = __ldg(a.match_ptr + b);
-    if (!match_cta<false, false>(a, smem, b, (uint32_t)(__ldg(a.match_ptr + b + 1) - m0), 0, a.cur_level)) return;
+    if (!match_cta<false, false, LITS>(a, smem, b, (uint32_t)(__ldg(a.match_ptr + b + 1) - m0), 0, a.cur_level)) return;
   }
 }
 
@@ -1836,7 +1972,7 @@ __global__ void ACE_PASS_BOUNDS(PASS) batch_decode_kernel(BatchArgs ba) {
       uint32_t b;
       const DecodeArgs a = jobs.job(it, b);
       const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
-      match_cta<false, true>(a, smem, b, ntok ? ntok - 1 : 0, epoch, 0);
+      match_cta<false, true, false>(a, smem, b, ntok ? ntok - 1 : 0, epoch, 0);
       publish_cta(a.ready, b, epoch);
     });
     return;
@@ -2324,6 +2460,38 @@ struct CacheDecodeArgs {
   uint32_t long_min;
 };
 
+// The decode arguments of a batch's work item, and its block.
+__device__ __forceinline__ DecodeArgs cache_job(const CacheDecodeArgs& ca, uint32_t it, uint32_t& b) {
+  const CacheArgs& c = ca.c;
+  const uint32_t ai = __ldg(c.work + 2 * it);
+  b = __ldg(c.work + 2 * it + 1);
+  const CacheArc& arc = c.arcs[ai];
+  DecodeArgs a{};
+  a.arc = arc.arc;
+  a.dir = arc.dir;
+  a.payload_off = arc.payload_off;
+  a.total = arc.total;
+  a.nb = arc.nb;
+  a.log2B = c.log2B;
+  a.w = arc.w;
+  a.window = ca.window;
+  a.esc_cap = ca.esc_cap;
+  a.warp_smem = ca.warp_smem;
+  a.max_ntok = ca.max_ntok;
+  a.out = c.slots;
+  a.sh = reinterpret_cast<ScratchHdr*>(c.h);
+  a.ready = arc.ready;
+  a.slot_of = arc.slot_of;
+  a.n_slots = c.n_slots;
+  a.rec_index = arc.wpos;
+  a.n_rec_slots = c.front_cap;
+  a.long_min = ca.long_min;
+  a.timeout_ns = ca.timeout_ns;
+  a.recs = c.recs;
+  a.match_ptr = nullptr;
+  return a;
+}
+
 // Decodes a batch's work list into cache slots: the same three passes as a
 // seek, archive by archive.
 template <int PASS>
@@ -2335,41 +2503,12 @@ __global__ void ACE_PASS_BOUNDS(PASS) cache_decode_kernel(CacheDecodeArgs ca) {
   if (PASS != PASS_TOKENS && stop_early<PASS>(&c.h->status)) return;
   const uint32_t epoch = *(volatile uint32_t*)&c.h->epoch;
   const uint32_t n_items = *(volatile uint32_t*)&c.h->n_work;
-  auto job = [&](uint32_t it, uint32_t& b) {
-    const uint32_t ai = __ldg(c.work + 2 * it);
-    b = __ldg(c.work + 2 * it + 1);
-    const CacheArc& arc = c.arcs[ai];
-    DecodeArgs a{};
-    a.arc = arc.arc;
-    a.dir = arc.dir;
-    a.payload_off = arc.payload_off;
-    a.total = arc.total;
-    a.nb = arc.nb;
-    a.log2B = c.log2B;
-    a.w = arc.w;
-    a.window = ca.window;
-    a.esc_cap = ca.esc_cap;
-    a.warp_smem = ca.warp_smem;
-    a.max_ntok = ca.max_ntok;
-    a.out = c.slots;
-    a.sh = reinterpret_cast<ScratchHdr*>(c.h);
-    a.ready = arc.ready;
-    a.slot_of = arc.slot_of;
-    a.n_slots = c.n_slots;
-    a.rec_index = arc.wpos;
-    a.n_rec_slots = c.front_cap;
-    a.long_min = ca.long_min;
-    a.timeout_ns = ca.timeout_ns;
-    a.recs = c.recs;
-    a.match_ptr = nullptr;
-    return a;
-  };
-  if (PASS == PASS_MATCH) {
+  if (ACE_PASS_CTA(PASS)) {
     cta_blocks(n_items, &c.h->ticket3, [&](uint32_t it) {
       uint32_t b;
-      const DecodeArgs a = job(it, b);
+      const DecodeArgs a = cache_job(ca, it, b);
       const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
-      match_cta<true, true>(a, smem, b, ntok ? ntok - 1 : 0, epoch, 0);
+      match_cta<true, true, PASS == PASS_PLACE>(a, smem, b, ntok ? ntok - 1 : 0, epoch, 0);
       publish_cta(a.ready, b, epoch);
     });
     return;
@@ -2381,9 +2520,20 @@ __global__ void ACE_PASS_BOUNDS(PASS) cache_decode_kernel(CacheDecodeArgs ca) {
     it = __shfl_sync(kFull, it, 0);
     if (it >= n_items) break;
     uint32_t b;
-    const DecodeArgs a = job(it, b);
+    const DecodeArgs a = cache_job(ca, it, b);
     if (PASS == PASS_TOKENS) token_block<true>(a, carve_tok(wsm), b, lane);
     else literal_block<true, kSeekRing>(a, carve_lit(wsm, ca.window, kSeekRing), b, lane);
+  }
+}
+
+// The entropy layer of a batch's work list, a warp per stream (entropy_kernel).
+__global__ void __launch_bounds__(32) cache_entropy_kernel(CacheDecodeArgs ca) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const uint32_t lane = threadIdx.x, n_jobs = 3 * *(volatile uint32_t*)&ca.c.h->n_work;
+  for (uint32_t j = blockIdx.x; j < n_jobs; j += gridDim.x) {
+    uint32_t b;
+    const DecodeArgs a = cache_job(ca, j / 3, b);
+    stream_job<true>(a, smem, b, j % 3, lane);
   }
 }
 
@@ -2673,6 +2823,24 @@ struct Launch {
 constexpr double kCtaMatches = 400;
 constexpr double kRowMatches = 48;
 constexpr uint32_t kCtaLevel = 4;
+// Calls of few blocks decode a stream per warp (entropy_kernel) and leave the
+// literals to the match pass, whose CTAs place them.  That shortens a block's
+// chain and spreads it wider, and costs more instructions per literal, so the
+// limit depends on the literals.  Against the token and literal passes, us:
+// FASTQ 2 MiB 99 (109), 4 MiB 132 (128), 16 MiB 161 (150); text 2 MiB 81
+// (158), 16 MiB 177 (224), 32 MiB 270 (271); genome 2 MiB 95 (105), 16 MiB 139
+// (158), 32 MiB 167 (163).
+constexpr uint32_t kSplitMaxLog2B = 15;  // places and literal counts of a record in 16 bits each
+constexpr uint32_t kSplitBlocks = 1;       // whole decodes, blocks per SM
+constexpr uint32_t kSplitBlocksLight = 8;  // ... of archives with many matches or few compressed bytes (few literals)
+// Seeks, by target blocks: FASTQ 1 block 154 (179), 1024 259 (275), 2048 366
+// (350); text 239 (326), 402 (476), 591 (639), 4096 1048 (986); genome 119
+// (122), 195 (203), 272 (272).
+constexpr uint64_t kSplitSeek = 1024;
+// Seek batches, by target blocks (1900 over four profiles: 301 us against 371)
+// where the host has the requests, else by their number.
+constexpr uint64_t kSplitBatch = 3072;
+constexpr uint32_t kSplitReqs = 64;
 
 template <class K>
 ace_status occupancy(K kernel, int device, uint32_t warps, size_t smem, int* occ) {
@@ -2784,10 +2952,16 @@ void launch_three_pass(const Launch& L, const DecodeArgs& a, cudaStream_t s) {
 // schedule, tokens and literals over the list, then one match launch that
 // waits the same way.  (One launch per level, as whole decodes by passes do,
 // is slower for a seek's hundred-odd blocks.)
-ace_status launch_seek(const ace_index* idx, const Launch& L, const DecodeArgs& a, cudaStream_t s) {
-  (void)idx;
-  if (L.schedule == ACE_SCHEDULE_FUSED) launch_fused(L, decode_kernel<true, PASS_FUSED>, a, s);
-  else launch_three_pass<true>(L, a, s);
+ace_status launch_seek(const ace_index* idx, const Launch& L, const DecodeArgs& a, uint64_t targets, cudaStream_t s) {
+  if (L.schedule == ACE_SCHEDULE_FUSED) {
+    launch_fused(L, decode_kernel<true, PASS_FUSED>, a, s);
+  } else if (targets <= kSplitSeek && a.log2B <= kSplitMaxLog2B) {
+    const uint32_t grid = (uint32_t)std::min<uint64_t>(3ull * a.n_slots, 16ull * idx->num_sms);
+    entropy_kernel<true><<<grid, 32, job_smem_bytes(a.esc_cap), s>>>(a);
+    decode_kernel<true, PASS_PLACE><<<L.grid[PASS_MATCH], L.match_threads, L.smem[PASS_MATCH], s>>>(a);
+  } else {
+    launch_three_pass<true>(L, a, s);
+  }
   return ACE_OK;
 }
 
@@ -3134,17 +3308,21 @@ ace_status decode_all_passes(const ace_index* idx, uint32_t passes, void* d_out,
     CUDA_TRY(cudaGetLastError());
     return ACE_OK;
   }
-  if (passes & 1) begin_call_kernel<<<1, 1, 0, s>>>(sh);
-  launch_passes(L, passes & (idx->by_levels ? 3u : 7u), decode_kernel<false, PASS_TOKENS>,
+  // a warp per block by rounds, a warp per block by rows, a CTA per block:
+  // by the archive's matches per 16 KiB
+  const double per16k = (double)idx->n_matches * 16384 / (double)idx->h.total_size;
+  const bool dense = per16k >= kCtaMatches, rows = per16k >= kRowMatches;
+  const bool light = dense || idx->h.archive_bytes < idx->h.total_size / 4;
+  const bool split = passes == 7 && idx->by_levels && idx->h.log2_block <= kSplitMaxLog2B &&
+                     idx->h.n_blocks <= (uint64_t)(light ? kSplitBlocksLight : kSplitBlocks) * idx->num_sms;
+  if (split) entropy_kernel<false><<<3 * a.n_items, 32, job_smem_bytes(a.esc_cap), s>>>(a);  // (needs no ticket or epoch)
+  else if (passes & 1) begin_call_kernel<<<1, 1, 0, s>>>(sh);
+  launch_passes(L, split ? 0u : passes & (idx->by_levels ? 3u : 7u), decode_kernel<false, PASS_TOKENS>,
                 decode_kernel<false, PASS_LITERALS>, decode_kernel<false, PASS_MATCH>, a, s);
   if ((passes & 4) && idx->by_levels) {
     const ace_tune t = tune ? *tune : idx->tune;
     int &occ = idx->occ_level[L.warps], &occ_cta = idx->occ_level[0];
     const uint32_t log2B = idx->h.log2_block, few = cta_threads(log2B, true), many = cta_threads(log2B, false);
-    // a warp per block by rounds, a warp per block by rows, a CTA per block:
-    // by the archive's matches per 16 KiB
-    const double per16k = (double)idx->n_matches * 16384 / (double)idx->h.total_size;
-    const bool dense = per16k >= kCtaMatches, rows = per16k >= kRowMatches;
     const auto level_kernel = rows ? match_level_kernel<true> : match_level_kernel<false>;
     if (occ == 0) {
       rc = occupancy(level_kernel, idx->device, L.warps, (size_t)L.warps * kMatchSmem, &occ);
@@ -3152,9 +3330,9 @@ ace_status decode_all_passes(const ace_index* idx, uint32_t passes, void* d_out,
     }
     if (occ_cta == 0) {
       int o = 0;  // (levels of few blocks need no count: a CTA each)
-      rc = occupancy(match_cta_kernel<512>, idx->device, few / 32, cta_smem_bytes(log2B, few), &o);
+      rc = occupancy(match_cta_kernel<512, false>, idx->device, few / 32, cta_smem_bytes(log2B, few), &o);
       if (rc == ACE_OK && o > 0)
-        rc = occupancy(match_cta_kernel<256>, idx->device, many / 32, cta_smem_bytes(log2B, many), &occ_cta);
+        rc = occupancy(match_cta_kernel<256, false>, idx->device, many / 32, cta_smem_bytes(log2B, many), &occ_cta);
       if (rc) return rc;
     }
     if (occ < 0 || occ_cta <= 0) return ACE_E_INVAL;
@@ -3167,12 +3345,12 @@ ace_status decode_all_passes(const ace_index* idx, uint32_t passes, void* d_out,
       a.items = idx->d_order + idx->level_start[l];
       a.n_items = n;
       a.cur_level = l;
-      if (n <= kCtaLevel * idx->num_sms) {
-        match_cta_kernel<512><<<n, few, cta_smem_bytes(log2B, few), s>>>(a);
+      if (split || n <= kCtaLevel * idx->num_sms) {  // (a split decode's levels: every block by a CTA)
+        (split ? match_cta_kernel<512, true> : match_cta_kernel<512, false>)<<<n, few, cta_smem_bytes(log2B, few), s>>>(a);
         continue;
       }
       if (dense) {
-        match_cta_kernel<256><<<(uint32_t)std::min<uint64_t>(sms(occ_cta), n), many, cta_smem_bytes(log2B, many), s>>>(a);
+        match_cta_kernel<256, false><<<(uint32_t)std::min<uint64_t>(sms(occ_cta), n), many, cta_smem_bytes(log2B, many), s>>>(a);
         continue;
       }
       const uint32_t grid = (uint32_t)std::min<uint64_t>(sms(occ), (n + L.warps - 1) / L.warps);
@@ -3265,7 +3443,7 @@ ace_status ace_seek(const ace_index* idx, uint64_t coord, uint64_t len, void* d_
   a.closure_flags = true;
   a.long_min = L.long_min;
   a.lv_done = c.lv_done;
-  rc = launch_seek(idx, L, a, s);
+  rc = launch_seek(idx, L, a, last - first + 1, s);
   if (rc) return rc;
   CUDA_TRY(cudaGetLastError());
   return ACE_OK;
@@ -3549,6 +3727,7 @@ ace_status ace_batch_free(ace_batch* b) {
 struct ace_cache {
   int device;
   uint32_t n_arcs, log2B, n_slots, front_cap, max_reqs;
+  int num_sms;
   uint8_t* mem;
   uint64_t bytes;
   CacheArgs args;
@@ -3679,6 +3858,7 @@ ace_status ace_cache_create(const ace_index* const* idx, uint32_t n, void* const
   c->n_slots = (uint32_t)n_slots;
   c->front_cap = (uint32_t)C.max_work;
   c->max_reqs = max_reqs;
+  c->num_sms = idx[0]->num_sms;
   c->mem = base;
   c->bytes = bytes;
   c->req_off = C.reqs;
@@ -3734,11 +3914,13 @@ ace_status ace_cache_create(const ace_index* const* idx, uint32_t n, void* const
   return ACE_OK;
 }
 
-ace_status ace_seek_batch(const ace_cache* c, const ace_seek_req* d_reqs, uint32_t n, void* d_pool, uint64_t pool_bytes,
-                          cudaStream_t s) {
-  if (!c || (!d_reqs && n) || (!d_pool && n)) return ACE_E_INVAL;
-  if (n == 0) return ACE_OK;
-  (void)pool_bytes;  // request ranges are validated on the host by ace_seek_batch_host
+}  // extern "C"
+
+namespace {
+
+// split: decode the batch's blocks a stream per warp
+ace_status seek_batch(const ace_cache* c, const ace_seek_req* d_reqs, uint32_t n, void* d_pool, bool split,
+                      cudaStream_t s) {
   CacheArgs a = c->args;
   a.reqs = d_reqs;
   a.n_reqs = n;
@@ -3746,8 +3928,14 @@ ace_status ace_seek_batch(const ace_cache* c, const ace_seek_req* d_reqs, uint32
   CacheDecodeArgs d = c->dargs;
   d.c = a;
   const Launch& L = c->L;
-  launch_passes(L, 7, cache_decode_kernel<PASS_TOKENS>, cache_decode_kernel<PASS_LITERALS>,
-                cache_decode_kernel<PASS_MATCH>, d, s);
+  if (split && c->log2B <= kSplitMaxLog2B) {
+    const uint32_t grid = std::min(3 * c->front_cap, 16 * (uint32_t)c->num_sms);
+    cache_entropy_kernel<<<grid, 32, job_smem_bytes(d.esc_cap), s>>>(d);
+    cache_decode_kernel<PASS_PLACE><<<L.grid[PASS_MATCH], L.match_threads, L.smem[PASS_MATCH], s>>>(d);
+  } else {
+    launch_passes(L, 7, cache_decode_kernel<PASS_TOKENS>, cache_decode_kernel<PASS_LITERALS>,
+                  cache_decode_kernel<PASS_MATCH>, d, s);
+  }
   // CTAs of 8 warps per request until there are about 8 per SM's worth
   const uint32_t per = std::max(1u, std::min(8u, 1024 / n));
   cache_copy_kernel<<<dim3(std::min<uint32_t>(n, 1024), per), 256, 0, s>>>(a, static_cast<uint8_t*>(d_pool));
@@ -3755,20 +3943,36 @@ ace_status ace_seek_batch(const ace_cache* c, const ace_seek_req* d_reqs, uint32
   return ACE_OK;
 }
 
+}  // namespace
+
+extern "C" {
+
+ace_status ace_seek_batch(const ace_cache* c, const ace_seek_req* d_reqs, uint32_t n, void* d_pool, uint64_t pool_bytes,
+                          cudaStream_t s) {
+  if (!c || (!d_reqs && n) || (!d_pool && n)) return ACE_E_INVAL;
+  if (n == 0) return ACE_OK;
+  (void)pool_bytes;  // request ranges are validated on the host by ace_seek_batch_host
+  return seek_batch(c, d_reqs, n, d_pool, n <= kSplitReqs, s);
+}
+
 ace_status ace_seek_batch_host(const ace_cache* c, const ace_seek_req* h_reqs, const uint64_t* h_totals, uint32_t n,
                                void* d_pool, uint64_t pool_bytes, cudaStream_t s) {
   if (!c || (!h_reqs && n)) return ACE_E_INVAL;
   if (n > c->max_reqs) return ACE_E_NOMEM;
+  uint64_t blocks = 0;
   for (uint32_t i = 0; i < n; i++) {
     const ace_seek_req& q = h_reqs[i];
     if (q.archive >= c->n_arcs) return ACE_E_INVAL;
     if (q.len == 0 || (h_totals && (q.coord >= h_totals[q.archive] || q.len > h_totals[q.archive] - q.coord)))
       return ACE_E_RANGE;
     if (q.out_off + q.len > pool_bytes) return ACE_E_NOMEM;
+    blocks += (q.len >> c->log2B) + 1;
   }
   ace_seek_req* d = reinterpret_cast<ace_seek_req*>(c->mem + c->req_off);
   if (n) CUDA_TRY(cudaMemcpyAsync(d, h_reqs, n * sizeof(ace_seek_req), cudaMemcpyHostToDevice, s));
-  return ace_seek_batch(c, d, n, d_pool, pool_bytes, s);
+  if (n == 0) return ACE_OK;
+  if (!d_pool) return ACE_E_INVAL;
+  return seek_batch(c, d, n, d_pool, blocks <= kSplitBatch, s);
 }
 
 ace_status ace_cache_sync(const ace_cache* c, cudaStream_t s) {
@@ -3940,7 +4144,7 @@ ace_status ace_seek_noalloc(const ace_index* idx, uint64_t coord, uint64_t len, 
   a.closure_flags = true;
   a.long_min = L.long_min;
   a.lv_done = c.lv_done;
-  rc = launch_seek(idx, L, a, s);
+  rc = launch_seek(idx, L, a, last - first + 1, s);
   if (rc) return rc;
   CUDA_TRY(cudaGetLastError());
   // the status lives in the shared array, so the call waits for it

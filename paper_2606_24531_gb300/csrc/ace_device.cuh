@@ -265,6 +265,7 @@ __device__ __forceinline__ bool stream_open(const uint8_t* pay, uint32_t sbytes,
 // build costs more than such a stream's rounds save (measured on the FASTQ,
 // genome and text token streams and on batches of 4-64 KiB blocks).
 constexpr uint32_t kSearchMaxSymbols = 2048;
+constexpr uint32_t kSplitSearch = 512;  // the same for a warp that decodes only this stream, on its own time
 constexpr uint32_t kCoarseOff = 1024;  // search mode: the coarse table after the (at most 256) packed words
 
 // Builds the stream's decode tables.  Slot table mode: fc[s] = f_s << 16 |
@@ -273,7 +274,8 @@ constexpr uint32_t kCoarseOff = 1024;  // search mode: the coarse table after th
 // (short streams): one sorted word per present symbol, c << 20 | (f - 1) << 8
 // | s, searched per symbol.  Returns false (all lanes) if the frequencies do
 // not sum to 4096.
-__device__ __forceinline__ bool lut_build(Stream& st, Lut& lut, uint32_t lane) {
+__device__ __forceinline__ bool lut_build(Stream& st, Lut& lut, uint32_t lane,
+                                          uint32_t search = kSearchMaxSymbols) {
   if (st.nsym == 0 || st.stored) return true;
   const uint8_t* sp = st.g - st.head;
   uint32_t bm = sp[128 + lane];
@@ -297,7 +299,7 @@ __device__ __forceinline__ bool lut_build(Stream& st, Lut& lut, uint32_t lane) {
   bad |= __shfl_sync(kFull, cincl, 31) != ACE_SCALE;
   if (__any_sync(kFull, bad)) return false;
   const uint32_t present = __shfl_sync(kFull, first + cnt, 31);  // present symbols
-  if (st.nsym <= kSearchMaxSymbols) {
+  if (st.nsym <= search) {
     // the packed words, and beside them the coarse table: entry b is the
     // index of the symbol owning slot 16 b.  Each symbol marks the first
     // bucket start in its range; a prefix maximum carries the mark over the
