@@ -839,8 +839,6 @@ __device__ bool literal_block(const DecodeArgs& a, const LitMem& m, uint32_t b, 
 constexpr uint32_t kRowUnroll = 8;
 // Bytes in flight per lane in the bytewise copy of a round's matches.
 constexpr uint32_t kCopyUnroll = 8;
-// 16-byte pieces in flight per lane in the copy of a round's long matches.
-constexpr uint32_t kLongUnroll = 2;
 // Copy classes of a group resolved in rounds: a non-overlapping match of at
 // least the call's long_min bytes is copied by the whole warp in aligned
 // 16-byte pieces, every other one bytewise with the round's other such
@@ -857,56 +855,6 @@ template <bool L1, class T>
 __device__ __forceinline__ T ld_src(const T* p) {
   return L1 ? __ldca(p) : __ldcg(p);
 }
-
-// The 16 bytes at absolute output position q (a multiple of 16, possibly
-// negative), bytes outside [0, total) read as zero.  An aligned piece never
-// straddles a block (blocks are multiples of 256 bytes), so a seek finds it
-// in one slot.
-template <bool SEEK, bool L1>
-__device__ __forceinline__ uint4 ld16_abs(const DecodeArgs& a, int64_t q, uint64_t b, const uint8_t* obase) {
-  if (q >= 0 && (uint64_t)q + 16 <= a.total)
-    return ld_src<L1>(reinterpret_cast<const uint4*>(Addr<SEEK>::at(a, (uint64_t)q, b, obase)));
-  uint4 v = make_uint4(0, 0, 0, 0);
-#pragma unroll 1
-  for (uint32_t k = 0; k < 16; k++) {
-    const int64_t p = q + k;
-    if (p < 0 || (uint64_t)p >= a.total) continue;
-    const uint32_t x = (uint32_t)ld_src<L1>(Addr<SEEK>::at(a, (uint64_t)p, b, obase)) << (8 * (k & 3));
-    if (k < 4) v.x |= x;
-    else if (k < 8) v.y |= x;
-    else if (k < 12) v.z |= x;
-    else v.w |= x;
-  }
-  return v;
-}
-
-// Bytes [lo, hi) of v to the 16-byte aligned p, in the widest aligned
-// stores that fit (a piece at either end of a match).
-__device__ __forceinline__ void store_bytes16(uint8_t* p, uint4 v, uint32_t lo, uint32_t hi) {
-  auto word = [&](uint32_t k) { return k < 4 ? v.x : k < 8 ? v.y : k < 12 ? v.z : v.w; };
-  uint32_t k = lo;
-  while (k < hi) {
-    if (!(k & 7) && k + 8 <= hi) {
-      *reinterpret_cast<uint2*>(p + k) = make_uint2(word(k), word(k + 4));
-      k += 8;
-    } else if (!(k & 3) && k + 4 <= hi) {
-      *reinterpret_cast<uint32_t*>(p + k) = word(k);
-      k += 4;
-    } else if (!(k & 1) && k + 2 <= hi) {
-      *reinterpret_cast<uint16_t*>(p + k) = (uint16_t)(word(k) >> (8 * (k & 3)));
-      k += 2;
-    } else {
-      p[k] = (uint8_t)(word(k) >> (8 * (k & 3)));
-      k++;
-    }
-  }
-}
-
-__device__ __forceinline__ uint4 shfl_down16(uint4 v, uint32_t d) {
-  return make_uint4(__shfl_down_sync(kFull, v.x, d), __shfl_down_sync(kFull, v.y, d), __shfl_down_sync(kFull, v.z, d),
-                    __shfl_down_sync(kFull, v.w, d));
-}
-
 
 // First index i in [0, n) with key(i) > x, for keys that never decrease.
 template <class Key>
@@ -1117,60 +1065,28 @@ __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint3
       while (pend) {
         const bool go = (pend >> lane & 1) && !(pend & feeds);
         const bool lgo = go && L >= a.long_min && dist >= L;
-        if (__any_sync(kFull, lgo)) {
-          // long: the round's long matches at once, laid end to end as the
-          // aligned 16-byte source pieces each one needs (its destination
-          // pieces plus one); piece c and piece c + 1 build destination piece
-          // c.  A window gives lane l pieces c0 + 32 u + l, kLongUnroll in
-          // flight; piece c + 1 is the next lane's, or for lane 31 the next
-          // u's lane 0; the window's very last piece only serves as that
-          // source, and the next window starts on it.  Each lane finds its
-          // pieces' match by walking forward (pieces only grow).
-          const uint32_t hd0 = D & 15;  // block bases are 16-byte aligned
-          const uint32_t np = lgo ? ((hd0 + L + 15) >> 4) + 1 : 0u;
-          const uint32_t incl = warp_incl_sum(np, lane);
-          gX[lane] = incl - np;
-          if (lane == 31) gX[32] = incl;
-          const uint32_t T = __shfl_sync(kFull, incl, 31);
-          __syncwarp();
-          uint32_t jc = 0;
-          for (uint32_t c0 = 0; c0 < T; c0 += 32 * kLongUnroll - 1) {
-            uint4 A[kLongUnroll];
-            uint32_t jp[kLongUnroll];
-#pragma unroll
-            for (uint32_t u = 0; u < kLongUnroll; u++) {
-              const uint32_t c = c0 + 32 * u + lane;
-              jp[u] = 0xffffffffu;
-              A[u] = make_uint4(0, 0, 0, 0);
-              if (c < T) {
-                while (gX[jc + 1] <= c) jc++;
-                const uint32_t pc = c - gX[jc];
-                jp[u] = jc | (pc << 5);
-                const int64_t s0 = (int64_t)gS[jc] - (int64_t)(gD[jc] & 15);
-                A[u] = ld16_abs<SEEK, kL1>(a, (s0 & ~(int64_t)15) + 16 * (int64_t)pc, b, obase);
-              }
-            }
-#pragma unroll
-            for (uint32_t u = 0; u < kLongUnroll; u++) {
-              const uint4 nb = shfl_down16(A[u], 1);
-              const uint32_t un = u + 1 < kLongUnroll ? u + 1 : u;
-              const uint4 n0 = make_uint4(__shfl_sync(kFull, A[un].x, 0), __shfl_sync(kFull, A[un].y, 0),
-                                          __shfl_sync(kFull, A[un].z, 0), __shfl_sync(kFull, A[un].w, 0));
-              const uint4 B = lane == 31 ? n0 : nb;
-              if (jp[u] == 0xffffffffu || (u + 1 == kLongUnroll && lane == 31)) continue;
-              const uint32_t j = jp[u] & 31, pc = jp[u] >> 5, ml = gL[j];
-              const uint32_t hd = gD[j] & 15;
-              if (pc >= ((hd + ml + 15) >> 4)) continue;  // the trailing source piece stores nothing
-              const uint4 v = funnel128(A[u], B, (uint32_t)(((int64_t)gS[j] - (int64_t)hd) & 15));
-              uint8_t* dp = obase + gD[j] - hd + 16ull * pc;
-              const int first = 16 * (int)pc - (int)hd;  // match byte held by the piece's first byte
-              if (first >= 0 && first + 16 <= (int)ml)
-                *reinterpret_cast<uint4*>(dp) = v;
-              else
-                store_bytes16(dp, v, (uint32_t)max(0, -first), (uint32_t)min(16, (int)ml - first));
-            }
+        // long: one match after another by the whole warp, in aligned 16-byte
+        // stores, each from the two aligned vectors of the source that hold its
+        // bytes (which end before the match does: it does not overlap its
+        // source); the ragged ends a byte per lane
+        for (uint32_t todo = __ballot_sync(kFull, lgo); todo; todo &= todo - 1) {
+          const uint32_t j = __ffs(todo) - 1, Dj = __shfl_sync(kFull, D, j), Lj = __shfl_sync(kFull, L, j);
+          const uint64_t Sj = (uint64_t)__shfl_sync(kFull, r.x, j) | (uint64_t)__shfl_sync(kFull, r.y, j) << 32;
+          const uint32_t head = (0u - Dj) & 15, tail = (Dj + Lj) & 15, n = (Lj - head) >> 4;
+          const bool ragged = lane < 16 ? lane < head : lane - 16 < tail;
+          const uint32_t i = lane < 16 ? lane : Lj - tail + (lane - 16);
+          uint8_t end = 0;
+          if (ragged) end = ld_src<kL1>(Addr<SEEK>::at(a, Sj + i, b, obase));
+          const uint32_t off = (uint32_t)(Sj + head) & 15;
+          const uint64_t q0 = Sj + head - off;
+          uint4* const dp = reinterpret_cast<uint4*>(obase + Dj + head);
+          for (uint32_t c = lane; c < n; c += 32) {
+            const uint64_t q = q0 + 16ull * c;
+            uint4 v = ld_src<kL1>(reinterpret_cast<const uint4*>(Addr<SEEK>::at(a, q, b, obase)));
+            if (off) v = funnel128(v, ld_src<kL1>(reinterpret_cast<const uint4*>(Addr<SEEK>::at(a, q + 16, b, obase))), off);
+            dp[c] = v;
           }
-          __syncwarp();
+          if (ragged) obase[Dj + i] = end;
         }
         // the rest laid end to end in group order: gX[j] is where match j
         // starts, gX[kMatchGroup] the total
@@ -1225,6 +1141,14 @@ __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint3
   return ok;
 }
 
+// Sixteen known bytes as entries of match_cta.
+__device__ __forceinline__ void known16(uint4* e, uint4 v) {
+  e[0] = make_uint4(__byte_perm(v.x, 0x80u, 0x4140), __byte_perm(v.x, 0x80u, 0x4342), __byte_perm(v.y, 0x80u, 0x4140),
+                    __byte_perm(v.y, 0x80u, 0x4342));
+  e[1] = make_uint4(__byte_perm(v.z, 0x80u, 0x4140), __byte_perm(v.z, 0x80u, 0x4342), __byte_perm(v.w, 0x80u, 0x4140),
+                    __byte_perm(v.w, 0x80u, 0x4342));
+}
+
 // The match pass of one block by a CTA, in windows of kCtaWindow bytes (one for
 // blocks of at most that).  Every byte of the window gets a 16-bit entry in
 // shared memory: 0x8000 | its value where that is known (a literal, or a match
@@ -1256,6 +1180,7 @@ constexpr uint32_t kCtaRowBytes = 2048;                     // match bytes whose
 constexpr uint32_t kCtaWarpSmem = 16 * 32 + kCtaRowBytes / 8;
 constexpr uint32_t kCtaUnroll = 4;                          // rows in flight per warp (a vector of the map's words)
 constexpr uint32_t kHops = 6;
+constexpr uint32_t kCtaLong = 256;                          // shortest run of known bytes set 16 at a time
 
 // Threads of a CTA: 256, or 512 where blocks are few and each one's time
 // counts; less for small blocks.
@@ -1326,11 +1251,7 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
       for (uint32_t u = 0; u < 4; u++) {
         const uint32_t j = j0 + 16 * nt * u;
         if (j >= wn) continue;
-        uint4* e4 = reinterpret_cast<uint4*>(e + j);
-        e4[0] = make_uint4(__byte_perm(v[u].x, 0x80u, 0x4140), __byte_perm(v[u].x, 0x80u, 0x4342),
-                           __byte_perm(v[u].y, 0x80u, 0x4140), __byte_perm(v[u].y, 0x80u, 0x4342));
-        e4[1] = make_uint4(__byte_perm(v[u].z, 0x80u, 0x4140), __byte_perm(v[u].z, 0x80u, 0x4342),
-                           __byte_perm(v[u].w, 0x80u, 0x4140), __byte_perm(v[u].w, 0x80u, 0x4342));
+        known16(reinterpret_cast<uint4*>(e + j), v[u]);
       }
     }
     if (LITS && tid < 16 && wn + tid < ((wn + 15) & ~15u)) e[wn + tid] = 0x8000;  // the last vector's rest
@@ -1394,6 +1315,30 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
           fence_acquire();
           __syncwarp();  // any lane may read a source whose flags another lane checked
         }
+        // Long runs of bytes from before the window (big, per lane), one after
+        // another by the whole warp (the group's warps in turn): 16 entries per
+        // lane from the one or two aligned vectors that hold them, the ragged
+        // ends a byte per lane.
+        auto copy_long = [&](bool big, uint32_t n, uint32_t dst, uint64_t from) {
+          uint32_t todo = __ballot_sync(kFull, big);
+          for (uint32_t q = 0; todo; todo &= todo - 1, q++) {
+            if (q % split != part) continue;
+            const uint32_t j = __ffs(todo) - 1, nj = __shfl_sync(kFull, n, j), dj = __shfl_sync(kFull, dst, j);
+            const uint8_t* const src = reinterpret_cast<const uint8_t*>(
+                (uint64_t)__shfl_sync(kFull, (uint32_t)from, j) | (uint64_t)__shfl_sync(kFull, (uint32_t)(from >> 32), j) << 32);
+            const uint32_t head = (0u - dj) & 15, tail = (dj + nj) & 15, nv = (nj - head) >> 4;
+            const uint32_t i = lane < 16 ? lane : nj - tail + (lane - 16);
+            if (lane < 16 ? lane < head : lane - 16 < tail) e[dj + i] = (uint16_t)(0x8000u | ld_src<!WAIT>(src + i));
+            const uint32_t off = (uint32_t)(reinterpret_cast<uintptr_t>(src + head) & 15);
+            const uint4* const sv = reinterpret_cast<const uint4*>(src + head - off);
+            uint4* const ev = reinterpret_cast<uint4*>(e + dj + head);
+            for (uint32_t c = lane; c < nv; c += 32) {
+              uint4 v = ld_src<!WAIT>(sv + c);
+              if (off) v = funnel128(v, ld_src<!WAIT>(sv + c + 1), off);
+              known16(ev + 2 * c, v);
+            }
+          }
+        };
         // The warp's share of n bytes per lane laid end to end, in rows.  Byte c
         // of them: its entry's address, twice its source's place in the window
         // (below 0: before it, or marked) and its source's address, each less
@@ -1484,7 +1429,9 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
             from = reinterpret_cast<uintptr_t>(Addr<SEEK>::at(a, s0, b, obase));
           }
         }
-        lay(n, d0 - w0, rel, from, marked);
+        const bool big = n >= kCtaLong && !marked && rel + (int32_t)n <= 0;
+        copy_long(big, n, d0 - w0, from);
+        lay(big ? 0u : n, d0 - w0, rel, from, marked);
       }
     }
     if (lane == 0) atomicMax(&s_group, last);
@@ -1829,10 +1776,13 @@ __global__ void __launch_bounds__(32) entropy_kernel(DecodeArgs a) {
 // k mod the warps in the grid), and each warp fetches its next block's
 // number and record range while it resolves the current one.
 // ROWS: the archive's matches are mostly short; without it every group goes by
-// rounds.  72 registers: 7 CTAs of 4 warps per SM (genome 1 GiB, long matches:
-// 0.458 ms against 0.493 at 75 to 80 registers, 6 CTAs).
+// rounds, in fewer registers (genome 1 GiB, the match pass: 342 us at 56
+// registers, 360 at 72; the rows' kernel spills below 72: FASTQ 129 us, 147 at
+// 56).  A long match by the whole warp, not the round's long matches laid end
+// to end in pieces with the next lane's vector shuffled in, took the genome's
+// from 518 us.
 template <bool ROWS>
-__global__ void __maxnreg__(72) match_level_kernel(DecodeArgs a) {
+__global__ void __maxnreg__(ROWS ? 72 : 56) match_level_kernel(DecodeArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t nw = gridDim.x * (blockDim.x >> 5);
