@@ -329,8 +329,9 @@ ace_status ace_sync(const ace_index *idx, void *d_scratch, cudaStream_t s);
 /*
  * Many independent archives decoded in one persistent launch (the batching
  * pattern: thousands of uneven objects with mixed block sizes).  Each
- * archive's blocks keep their own (level, block) order; warps take
- * (archive, block) items from one ticket, so a warp only waits on blocks of
+ * archive's blocks keep their own (level, block) order; warps and CTAs take
+ * (archive, block) items from one ticket, lower levels of every archive first
+ * in the match pass, so a block only waits on blocks of
  * its own archive handed out before it (Section 2's dependency rule).
  *
  * ace_batch_scratch_size sizes the batch scratch (256-byte aligned).
