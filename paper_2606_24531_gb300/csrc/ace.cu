@@ -522,9 +522,8 @@ struct BlockHead {
 // into the destination and length of every match's record.  Match t ends
 // token t (t < ntok - 1); its destination is the token's start plus its run.
 // SPLIT: the offset stream is decoded by another warp, which fills the
-// source's w bytes (the rest of them are set here), and the destination's word
-// holds above its 16 bits the literals before the match (blocks of at most
-// 32 KiB).  Returns false if
+// source's w bytes, and the rest of the source's eight are set here: above the
+// fifth, the literals before the match.  Returns false if
 // the stream is corrupt (recorded).
 template <bool SEEK, uint32_t RING, bool SPLIT>
 __device__ bool length_stream(const DecodeArgs& a, const BlockHead& h, Stream& sn, Lut& lut, uint8_t* ring,
@@ -563,13 +562,14 @@ __device__ bool length_stream(const DecodeArgs& a, const BlockHead& h, Stream& s
         if (ml) bad = true;  // the block's last token carries no match
       } else if (SPLIT) {
         uint8_t* const r8 = reinterpret_cast<uint8_t*>(rec4 + t);
+        const uint32_t lits = lit_pos + il;
         if (a.w == 4) {
-          *reinterpret_cast<uint32_t*>(r8 + 4) = 0;
+          *reinterpret_cast<uint32_t*>(r8 + 4) = lits << 8;
         } else {
-          r8[5] = 0;
-          *reinterpret_cast<uint16_t*>(r8 + 6) = 0;
+          r8[5] = (uint8_t)lits;
+          *reinterpret_cast<uint16_t*>(r8 + 6) = (uint16_t)(lits >> 8);
         }
-        *reinterpret_cast<uint2*>(r8 + 8) = make_uint2(D | (lit_pos + il) << 16, ml);
+        *reinterpret_cast<uint2*>(r8 + 8) = make_uint2(D, ml);
       } else {
         rec4[t] = make_uint4(0u, 0u, D, ml);
       }
@@ -653,20 +653,20 @@ __device__ bool token_block(const DecodeArgs& a, const TokMem& m, uint32_t b, ui
 // from where match_cta places them (a literal's final position is never after
 // this one, so placing in ascending windows never overwrites one still to be
 // read).
-template <bool SEEK>
+template <bool SEEK, uint32_t RING>
 __device__ void stream_job(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32_t k, uint32_t lane) {
   bool ok = true;
   Lut& lut = *reinterpret_cast<Lut*>(smem);
   uint8_t* ring = smem + sizeof(Lut);
-  uint16_t* esc = reinterpret_cast<uint16_t*>(ring + kSeekRing);
+  uint16_t* esc = reinterpret_cast<uint16_t*>(ring + RING);
   const BlockHead h(a, b, lane);
   Stream st;
-  if (!h.open<kSeekRing>(a, k, ring, st, lane)) fail(a, ok, ACE_E_CORRUPT, b, 20 + k, lane);
+  if (!h.open<RING>(a, k, ring, st, lane)) fail(a, ok, ACE_E_CORRUPT, b, 20 + k, lane);
   if (h.ntok > a.max_ntok) fail(a, ok, ACE_E_CORRUPT, b, 23, lane);
-  cp_async_wait<kSeekRing / kSeg - 2>();
+  cp_async_wait<RING / kSeg - 2>();
   __syncwarp();
-  if (ok && k == ACE_S_LEN) length_stream<SEEK, kSeekRing, true>(a, h, st, lut, ring, esc, b, lane);
-  if (ok && k == ACE_S_OFF) offset_stream<SEEK, kSeekRing>(a, h, st, lut, ring, b, lane, kSplitSearch);
+  if (ok && k == ACE_S_LEN) length_stream<SEEK, RING, true>(a, h, st, lut, ring, esc, b, lane);
+  if (ok && k == ACE_S_OFF) offset_stream<SEEK, RING>(a, h, st, lut, ring, b, lane, kSplitSearch);
   if (ok && k == ACE_S_LIT && st.nsym) {
     if (!lut_build(st, lut, lane, kSplitSearch)) fail(a, ok, ACE_E_CORRUPT, b, 35, lane);
     const uint32_t lt = lanemask_lt();
@@ -674,13 +674,13 @@ __device__ void stream_job(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint3
         (SEEK ? a.out + slot_base(a, b) : a.out + ((uint64_t)b << a.log2B)) + (h.blen - h.nlit);  // nlit <= blen: the index
     if (ok && !st.stored && st.k == 0 && st.nsym >= 64) {
       uint8_t* op = to + lane;
-      table_full_rounds<kSeekRing, 4>(st, ring, lut, st.nsym >> 5, lane, lt, [](uint32_t) {}, [&](uint32_t s, uint32_t) {
+      table_full_rounds<RING, 4>(st, ring, lut, st.nsym >> 5, lane, lt, [](uint32_t) {}, [&](uint32_t s, uint32_t) {
         *op = (uint8_t)s;
         op += 32;
       });
     }
     if (ok)
-      rans_run<kSeekRing>(st, ring, lut, st.nsym, lane, lt, [&](bool act, uint32_t i, uint32_t s) {
+      rans_run<RING>(st, ring, lut, st.nsym, lane, lt, [&](bool act, uint32_t i, uint32_t s) {
         if (act) to[i] = (uint8_t)s;
       });
     if (ok && !stream_finished(st)) fail(a, ok, ACE_E_CORRUPT, b, 41, lane);
@@ -689,7 +689,9 @@ __device__ void stream_job(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint3
   __syncwarp();
 }
 
-__host__ __device__ inline uint32_t job_smem_bytes(uint32_t escn) { return (sizeof(Lut) + kSeekRing + 2 * escn + 15) & ~15u; }
+__host__ __device__ inline uint32_t job_smem_bytes(uint32_t escn, uint32_t ring) {
+  return (sizeof(Lut) + ring + 2 * escn + 15) & ~15u;
+}
 
 // Literal pass of one block, after the token pass of every block succeeded:
 // literal i lands at i plus the shift of its run.  Token t's run starts where
@@ -1194,7 +1196,7 @@ __host__ __device__ inline uint32_t cta_smem_bytes(uint32_t log2B, uint32_t thre
 
 //
 // LITS: after stream jobs.  The literals are still in order at the end of the
-// block's place (a record's destination word holds above it the literals
+// block's place (a record's source holds above its five bytes the literals
 // before the match), so literal runs are laid in rows too, the last one as
 // token nm, and every byte of the window gets its entry from a row.
 template <bool SEEK, bool WAIT, bool LITS>
@@ -1214,7 +1216,7 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
   uint32_t nlit = 0;
   if (LITS) {  // the block's literals: those before its last match, and what follows it
     const uint4 r = nm ? __ldcg(rec + nm - 1) : make_uint4(0, 0, 0, 0);
-    nlit = (r.z >> 16) + blen - (r.z & 0xffffu) - r.w;
+    nlit = (r.y >> 8) + blen - r.z - r.w;
   }
   const uint32_t part = wid % split, step = nw / split;
   uint4* row = reinterpret_cast<uint4*>(smem + 2 * min((uint32_t)B, kCtaWindow) + wid * kCtaWarpSmem);
@@ -1272,17 +1274,17 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
       for (; g < ng; g += step) {
         const uint4 r = rn;
         rn = fetch(g + step);
-        const uint64_t S = (uint64_t)r.x | ((uint64_t)r.y << 32);
-        uint32_t D = LITS ? r.z & 0xffffu : r.z, lits = 0, lr = 0;
+        const uint64_t S = (uint64_t)r.x | ((uint64_t)(LITS ? r.y & 0xffu : r.y) << 32);
+        uint32_t D = r.z, lits = 0, lr = 0;
         uint32_t L = r.w;
         if (LITS) {  // lits: literals before the match; lr: those of its token's run
-          lits = r.z >> 16;
+          lits = r.y >> 8;
           if (32 * g + lane >= nm) {
             D = blen;
             lits = nlit;
           }
           uint32_t before = __shfl_up_sync(kFull, lits, 1);
-          if (lane == 0) before = g ? __ldcg(&rec[32 * g - 1].z) >> 16 : 0u;
+          if (lane == 0) before = g ? __ldcg(&rec[32 * g - 1].y) >> 8 : 0u;
           lr = lits - before;  // (0 past token nm)
         }
         if (L && (S >= bstart + D || (uint64_t)D + L > blen)) {  // a source precedes its match, which stays in the block
@@ -1767,7 +1769,7 @@ __global__ void __launch_bounds__(32) entropy_kernel(DecodeArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   const uint32_t lane = threadIdx.x;
   const uint32_t n_jobs = 3 * (SEEK ? *(volatile uint32_t*)&a.sh->n_work : a.n_items);
-  for (uint32_t j = blockIdx.x; j < n_jobs; j += gridDim.x) stream_job<SEEK>(a, smem, __ldg(a.items + j / 3), j % 3, lane);
+  for (uint32_t j = blockIdx.x; j < n_jobs; j += gridDim.x) stream_job<SEEK, kSeekRing>(a, smem, __ldg(a.items + j / 3), j % 3, lane);
 }
 
 // The match pass of one dependency level of a whole decode: every lower
@@ -1930,13 +1932,13 @@ __global__ void ACE_PASS_BOUNDS(PASS) batch_decode_kernel(BatchArgs ba) {
     fused_loop<false>(BatchJobs{ba, ba.by_level, ba.n_level}, ba.sh, ba.n_items, ba.timeout_ns, wsm, lane, epoch, ba.window);
     return;
   }
-  const BatchJobs jobs = PASS == PASS_MATCH ? BatchJobs{ba, ba.by_level, ba.n_level} : BatchJobs{ba, ba.by_size, ba.n_size};
-  if (PASS == PASS_MATCH) {
+  const BatchJobs jobs = ACE_PASS_CTA(PASS) ? BatchJobs{ba, ba.by_level, ba.n_level} : BatchJobs{ba, ba.by_size, ba.n_size};
+  if (ACE_PASS_CTA(PASS)) {
     cta_blocks(ba.n_items, &ba.sh->ticket3, [&](uint32_t it) {
       uint32_t b;
       const DecodeArgs a = jobs.job(it, b);
       const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
-      match_cta<false, true, false>(a, smem, b, ntok ? ntok - 1 : 0, epoch, 0);
+      match_cta<false, true, PASS == PASS_PLACE>(a, smem, b, ntok ? ntok - 1 : 0, epoch, 0);
       publish_cta(a.ready, b, epoch);
     });
     return;
@@ -1951,6 +1953,25 @@ __global__ void ACE_PASS_BOUNDS(PASS) batch_decode_kernel(BatchArgs ba) {
     const DecodeArgs a = jobs.job(it, b);
     if (PASS == PASS_TOKENS) token_block<false>(a, carve_tok(wsm), b, lane);
     else literal_block<false, kRing>(a, carve_lit(wsm, ba.window, kRing), b, lane);
+  }
+}
+
+// The entropy layer of a batch, a warp per stream, largest blocks first: one
+// launch whose time is its longest stream's, where the token and literal
+// passes each had that tail.
+__global__ void __launch_bounds__(128, 8) batch_entropy_kernel(BatchArgs ba) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const BatchJobs jobs{ba, ba.by_size, ba.n_size};
+  uint8_t* wsm = smem + wid * job_smem_bytes(ba.esc_cap, kRing);
+  while (true) {
+    uint32_t it = 0;
+    if (lane == 0) it = atomicAdd(&ba.sh->ticket, 1u);
+    it = __shfl_sync(kFull, it, 0);
+    if (it / 3 >= ba.n_items) break;
+    uint32_t b;
+    const DecodeArgs a = jobs.job(it / 3, b);
+    stream_job<false, kRing>(a, wsm, b, it % 3, lane);
   }
 }
 
@@ -2497,7 +2518,7 @@ __global__ void __launch_bounds__(32) cache_entropy_kernel(CacheDecodeArgs ca) {
   for (uint32_t j = blockIdx.x; j < n_jobs; j += gridDim.x) {
     uint32_t b;
     const DecodeArgs a = cache_job(ca, j / 3, b);
-    stream_job<true>(a, smem, b, j % 3, lane);
+    stream_job<true, kSeekRing>(a, smem, b, j % 3, lane);
   }
 }
 
@@ -2793,8 +2814,8 @@ constexpr uint32_t kCtaLevel = 4;
 // limit depends on the literals.  Against the token and literal passes, us:
 // FASTQ 2 MiB 99 (109), 4 MiB 132 (128), 16 MiB 161 (150); text 2 MiB 81
 // (158), 16 MiB 177 (224), 32 MiB 270 (271); genome 2 MiB 95 (105), 16 MiB 139
-// (158), 32 MiB 167 (163).
-constexpr uint32_t kSplitMaxLog2B = 15;  // places and literal counts of a record in 16 bits each
+// (158), 32 MiB 167 (163).  Word text in 64 KiB blocks: 1 MiB 152 (361), 16
+// MiB 304 (496).
 constexpr uint32_t kSplitBlocks = 1;       // whole decodes, blocks per SM
 constexpr uint32_t kSplitBlocksLight = 8;  // ... of archives with many matches or few compressed bytes (few literals)
 // Seeks, by target blocks: FASTQ 1 block 154 (179), 1024 259 (275), 2048 366
@@ -2805,6 +2826,10 @@ constexpr uint64_t kSplitSeek = 1024;
 // where the host has the requests, else by their number.
 constexpr uint64_t kSplitBatch = 3072;
 constexpr uint32_t kSplitReqs = 64;
+// Archive batches, by the bytes they give: uneven objects of 16 MB 391 us (576
+// in three passes), 57 MB 503 (781), 118 MB 804 (900), 124 MB 912 (929), 183
+// MB 1157 (1122), 364 MB 2312 (1676).
+constexpr uint64_t kSplitBatchBytes = 128ull << 20;
 
 template <class K>
 ace_status occupancy(K kernel, int device, uint32_t warps, size_t smem, int* occ) {
@@ -2919,9 +2944,9 @@ void launch_three_pass(const Launch& L, const DecodeArgs& a, cudaStream_t s) {
 ace_status launch_seek(const ace_index* idx, const Launch& L, const DecodeArgs& a, uint64_t targets, cudaStream_t s) {
   if (L.schedule == ACE_SCHEDULE_FUSED) {
     launch_fused(L, decode_kernel<true, PASS_FUSED>, a, s);
-  } else if (targets <= kSplitSeek && a.log2B <= kSplitMaxLog2B) {
+  } else if (targets <= kSplitSeek) {
     const uint32_t grid = (uint32_t)std::min<uint64_t>(3ull * a.n_slots, 16ull * idx->num_sms);
-    entropy_kernel<true><<<grid, 32, job_smem_bytes(a.esc_cap), s>>>(a);
+    entropy_kernel<true><<<grid, 32, job_smem_bytes(a.esc_cap, kSeekRing), s>>>(a);
     decode_kernel<true, PASS_PLACE><<<L.grid[PASS_MATCH], L.match_threads, L.smem[PASS_MATCH], s>>>(a);
   } else {
     launch_three_pass<true>(L, a, s);
@@ -3277,9 +3302,9 @@ ace_status decode_all_passes(const ace_index* idx, uint32_t passes, void* d_out,
   const double per16k = (double)idx->n_matches * 16384 / (double)idx->h.total_size;
   const bool dense = per16k >= kCtaMatches, rows = per16k >= kRowMatches;
   const bool light = dense || idx->h.archive_bytes < idx->h.total_size / 4;
-  const bool split = passes == 7 && idx->by_levels && idx->h.log2_block <= kSplitMaxLog2B &&
+  const bool split = passes == 7 && idx->by_levels &&
                      idx->h.n_blocks <= (uint64_t)(light ? kSplitBlocksLight : kSplitBlocks) * idx->num_sms;
-  if (split) entropy_kernel<false><<<3 * a.n_items, 32, job_smem_bytes(a.esc_cap), s>>>(a);  // (needs no ticket or epoch)
+  if (split) entropy_kernel<false><<<3 * a.n_items, 32, job_smem_bytes(a.esc_cap, kSeekRing), s>>>(a);  // (needs no ticket or epoch)
   else if (passes & 1) begin_call_kernel<<<1, 1, 0, s>>>(sh);
   launch_passes(L, split ? 0u : passes & (idx->by_levels ? 3u : 7u), decode_kernel<false, PASS_TOKENS>,
                 decode_kernel<false, PASS_LITERALS>, decode_kernel<false, PASS_MATCH>, a, s);
@@ -3512,24 +3537,27 @@ struct ace_batch {
   uint64_t lv_done_off, lv_done_bytes;  // the fused schedule's level counters
   BatchArgs args;
   Launch L;
+  bool split;             // the entropy layer a stream per warp
+  uint32_t entropy_grid;
   int occ[4][9][9];
 };
 
 namespace {
 
 struct BatchLayout {
-  uint64_t objs, by_size, by_level, segs, ready, lv_done, lv_done_bytes, recs, total, max_ntok, items, n_matches;
+  uint64_t objs, by_size, by_level, ready, lv_done, lv_done_bytes, recs, total, max_ntok, items, n_matches, bytes;
   uint32_t max_log2B;
 };
 
 ace_status batch_layout(const ace_index* const* idx, uint32_t n, BatchLayout* B) {
   if (!idx || n == 0) return ACE_E_INVAL;
-  uint64_t ready = 0, items = 0, max_ntok = 0, matches = 0, levels = 0, segs = 0;
+  uint64_t ready = 0, items = 0, max_ntok = 0, matches = 0, levels = 0, segs = 0, bytes = 0;
   uint32_t max_log2B = 0;
   int dev = idx[0] ? idx[0]->device : -1;
   for (uint32_t i = 0; i < n; i++) {
     if (!idx[i] || idx[i]->device != dev) return ACE_E_INVAL;
     items += idx[i]->h.n_blocks;
+    bytes += idx[i]->h.total_size;
     ready += align256(4 * idx[i]->h.n_blocks);
     matches += idx[i]->n_matches;
     levels += idx[i]->n_levels;
@@ -3554,6 +3582,7 @@ ace_status batch_layout(const ace_index* const* idx, uint32_t n, BatchLayout* B)
   o = align256(o + 16 * matches);
   B->total = o;
   B->n_matches = matches;
+  B->bytes = bytes;
   B->max_ntok = max_ntok;
   B->items = items;
   B->max_log2B = max_log2B;
@@ -3656,6 +3685,8 @@ ace_status ace_batch_create(const ace_index* const* idx, uint32_t n, void* const
   }
   BatchArgs& a = b->args;
   a.objs = reinterpret_cast<const ObjDesc*>(base + B.objs);
+  b->split = B.bytes <= kSplitBatchBytes;
+  b->entropy_grid = (uint32_t)std::min<uint64_t>((3 * B.items + 3) / 4, 8ull * idx[0]->num_sms);
   a.by_size = reinterpret_cast<const BatchSeg*>(base + B.by_size);
   a.by_level = reinterpret_cast<const BatchSeg*>(base + B.by_level);
   a.n_size = (uint32_t)by_size.size();
@@ -3681,7 +3712,10 @@ ace_status ace_decode_batch(const ace_batch* b, cudaStream_t s) {
   begin_call_kernel<<<1, 1, 0, s>>>(b->args.sh);
   if (L.schedule == ACE_SCHEDULE_FUSED)
     launch_fused(L, batch_decode_kernel<PASS_FUSED>, b->args, s);
-  else
+  else if (b->split) {
+    batch_entropy_kernel<<<b->entropy_grid, 128, 4 * job_smem_bytes(b->args.esc_cap, kRing), s>>>(b->args);
+    batch_decode_kernel<PASS_PLACE><<<L.grid[PASS_MATCH], L.match_threads, L.smem[PASS_MATCH], s>>>(b->args);
+  } else
     launch_passes(L, 7, batch_decode_kernel<PASS_TOKENS>, batch_decode_kernel<PASS_LITERALS>,
                   batch_decode_kernel<PASS_MATCH>, b->args, s);
   CUDA_TRY(cudaGetLastError());
@@ -3919,9 +3953,9 @@ ace_status seek_batch(const ace_cache* c, const ace_seek_req* d_reqs, uint32_t n
   CacheDecodeArgs d = c->dargs;
   d.c = a;
   const Launch& L = c->L;
-  if (split && c->log2B <= kSplitMaxLog2B) {
+  if (split) {
     const uint32_t grid = std::min(3 * c->front_cap, 16 * (uint32_t)c->num_sms);
-    cache_entropy_kernel<<<grid, 32, job_smem_bytes(d.esc_cap), s>>>(d);
+    cache_entropy_kernel<<<grid, 32, job_smem_bytes(d.esc_cap, kSeekRing), s>>>(d);
     cache_decode_kernel<PASS_PLACE><<<L.grid[PASS_MATCH], L.match_threads, L.smem[PASS_MATCH], s>>>(d);
   } else {
     launch_passes(L, 7, cache_decode_kernel<PASS_TOKENS>, cache_decode_kernel<PASS_LITERALS>,

@@ -105,3 +105,24 @@ def test_levels_of_many_blocks(shape):
         da = DeviceArchive(arc)
         _check(da, data)
         da.close()
+
+
+def test_batches_of_either_size():
+    """A batch that decodes a stream per warp and one, above 128 MiB, in three
+    passes: blocks of every size, objects of a block and of many."""
+    arcs, datas = [], []
+    for k, log2b in enumerate((9, 12, 14, 16)):
+        lengths, back, lit = SHAPES[sorted(SHAPES)[k]]
+        for n in (77, 40_000, 700_001):
+            datas.append(_copies(lengths, back, lit, n, k))
+            arcs.append(ace.ace_encode(datas[-1], log2b, 4))
+    per = sum(d.size for d in datas)
+    for copies in (1, (128 << 20) // per + 2):
+        db = DeviceBatch(arcs * copies)
+        db.decode()
+        assert db.sync() == ace.ACE_OK
+        for k in range(len(datas)):
+            want = torch.from_numpy(datas[k].copy()).cuda()
+            for c in {0, copies // 2, copies - 1}:
+                assert torch.equal(db.output(c * len(datas) + k), want)
+        db.close()
