@@ -114,16 +114,17 @@ ace_status ace_encode_get_stats(const ace_encoder *enc, ace_encode_stats *h_stat
  * memory) to an archive in d_arc (device memory, 256-byte aligned) in the
  * layout of ace_format.h.  Section 2's global match search as a table of
  * the earliest occurrence of every 16-byte key at 8-byte strides (built with
- * atomic minima), in-block repeats through 4-byte hash chains (a warp per
- * block), candidates measured for every position at once (a thread per
- * position), then a greedy walk per block (a thread per block) that takes
- * the longest allowed candidate, refusing in-block resolution waves deeper
- * than 3 and preferring a shallower candidate nearly as long; blocks in
- * windows of 64 that take no sources from each other, the first three
- * windows in order, every later block taking external sources only from
- * them (dependency levels at most 3).  Each block's literal, length and
- * offset streams rANS-coded by a warp (Section 3; the host encoder's
- * frequency quantisation, 32 interleaved states), stored verbatim with
+ * atomic minima), in-block repeats through 4-byte hash chains in shared
+ * memory, candidates measured for every position at once (a CTA per block),
+ * then a greedy walk per block (a warp, 32 positions decided at once) that
+ * takes the longest allowed candidate, refusing in-block resolution waves
+ * deeper than 3 and preferring a shallower candidate nearly as long; windows
+ * of 64 blocks take no sources from each other: one of the first three takes
+ * external sources from the windows before it, every later block from those
+ * three (dependency levels at most 3), so all blocks of a launch are searched
+ * and parsed at once.  Each block's literal, length and offset streams
+ * rANS-coded by a warp each (Section 3; the host encoder's frequency
+ * quantisation, 32 interleaved states), stored verbatim with
  * params->adaptive where rANS would not shrink them (Section 6.1).  The
  * parse differs from the host encoder's; every decoder reads both.
  * params->threads is read as the blocks parsed per launch (0: 64 MiB of

@@ -9,11 +9,11 @@
 // around it (a table over the whole input, built with atomic minima) and
 // the most recent repeats inside its block (hash chains in shared memory)
 // -- then a warp per block walks its positions greedily, taking
-// at each the longest candidate allowed there.  Blocks are parsed in
-// windows of 64 that take no sources from each other; the first three
-// windows are parsed one after another, and every later block takes its
-// external sources only from them, so dependency levels stay at most 3 as
-// with the host encoder.  A match of a block's own earlier bytes resolves
+// at each the longest candidate allowed there.  Windows of 64 blocks take
+// no sources from each other: one of the first three windows takes its
+// external sources from the windows before it, and every later block from
+// those three, so dependency levels stay at most 3 as with the host encoder
+// and no block waits on another's parse.  A match of a block's own earlier bytes resolves
 // in waves (one reading only literals is wave 1, one reading wave-k bytes
 // wave k + 1); candidates deeper than wave 3 are refused, and an external
 // candidate nearly as long as the best is preferred.
@@ -30,7 +30,6 @@
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
-#include <vector>
 
 #include "ace.h"
 #include "ace_device.cuh"
@@ -42,13 +41,19 @@ namespace {
 
 constexpr uint32_t kKey = 16;        // long-key length of the global table
 constexpr uint32_t kStride = 8;      // positions whose keys enter the table
-constexpr uint32_t kWin = 64;        // blocks of a parse window
-constexpr uint32_t kHeadWins = 3;    // windows parsed one after another
+constexpr uint32_t kWin = 64;        // blocks of a window
+constexpr uint32_t kHeadWins = 3;    // windows whose blocks may be sources
 constexpr uint32_t kHead = kWin * kHeadWins;
 constexpr uint32_t kMaxWave = 3;     // deepest in-block resolution wave taken
 constexpr uint32_t kCap = 32;        // match lengths measured by the candidate search (extended later)
 constexpr uint32_t kHashBits4 = 12;  // in-block chains: hash of 4 bytes
 constexpr uint32_t kMaxChain = 64;
+
+// The blocks below which block b takes sources: those of the windows before its
+// own, the first three windows at most.  So a block of window k has level k at
+// most and no block one above 3, whatever is found, and the search and the
+// walk of a block need nothing of any other's.
+__device__ __forceinline__ uint64_t source_end(uint64_t b) { return min(b / kWin * kWin, (uint64_t)kHead); }
 
 __host__ __device__ inline uint64_t align16(uint64_t v) { return (v + 15) & ~15ull; }
 
@@ -82,10 +87,7 @@ struct EncArgs {
   uint64_t n, nb;
   uint32_t log2B, min_match, max_chain, w, adaptive, bits;
   unsigned long long* table;  // 2^bits: the earliest stride position with each key hash
-  uint32_t* level;            // per block
-  // the blocks of the current launch: [c0, c1), window start ws (blocks
-  // below it, all of level below 3, may be sources)
-  uint64_t c0, c1, ws;
+  uint64_t c0;  // the launch's first block
   uint32_t* entries;  // per position: the candidate search's links and hashes (64 KiB blocks; smaller ones: shared memory)
   uint2* cand;        // per position: x = in-block candidate length (bits 0..7), external length (8..15), both
                       // capped at kCap, and the in-block source as an offset in the block (16..31); y = the external
@@ -111,13 +113,12 @@ __global__ void table_kernel(EncArgs a) {
 // ------------------------------------------------------ candidate search
 
 // Bytes from q a match of block b may read without entering a block it may
-// not read (its own block, or blocks below the window start of level below
-// 3), at most want.
+// not read (its own block, or blocks below source_end), at most want.
 __device__ __forceinline__ uint32_t span(const EncArgs& a, uint64_t q, uint64_t b, uint32_t want) {
   uint64_t k = q >> a.log2B;
   uint32_t got = 0;
   while (got < want) {
-    if (k != b && (k >= a.ws || a.level[k] >= 3)) break;
+    if (k != b && k >= source_end(b)) break;
     const uint64_t end = (k + 1) << a.log2B;
     got = (uint32_t)min((uint64_t)want, end - q);
     k++;
@@ -163,6 +164,7 @@ __host__ __device__ inline CandShape cand_shape(uint32_t log2B) {
 
 constexpr uint32_t kNoKey = ~0u;
 constexpr uint32_t kCandParts = 4;  // CTAs a block's positions are split over, at most
+constexpr uint64_t kSplitEntries = 256;  // 64 KiB blocks whose entries fill scratch, where launches split
 
 // A CTA per block, or (gridDim.y > 1) per part of its positions: for every
 // position the best in-block candidate (its chain
@@ -184,7 +186,7 @@ constexpr uint32_t kCandParts = 4;  // CTAs a block's positions are split over, 
 // key and a position before it are dealt evenly to the lanes.  Bound by issue: about 940 warp instructions
 // per 32 positions of FASTQ.  Byte loads from global memory, a launch for the
 // links and eight lookups a position took 12.4 + 1.5 ms of the 64 MiB FASTQ
-// encode; this takes 2.8 ms.
+// encode; this takes 2.5 ms.
 template <bool SHARED>
 __global__ void __launch_bounds__(512, 2) candidate_kernel(EncArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
@@ -266,7 +268,7 @@ __global__ void __launch_bounds__(512, 2) candidate_kernel(EncArgs a) {
   // the table's position for the key at p: in this block as an offset with the
   // top bit set, in a block that may be a source (or up to 7 bytes past those,
   // for the shift back) as it is
-  const uint64_t wend = a.ws << a.log2B;
+  const uint64_t wend = source_end(b) << a.log2B;
   auto key_of = [&](uint32_t p) -> uint32_t {
     if (p + kKey > avail) return kNoKey;
     const uint32_t* t = sb + (p >> 2);
@@ -396,7 +398,7 @@ __global__ void __launch_bounds__(512, 2) candidate_kernel(EncArgs a) {
       } else {
         const uint64_t q64 = (t >> 31 ? bstart : 0) + q0;
         // in a block that may be a source (its length beyond it: span)
-        if (q64 < j || q64 - j >= wend || __ldg(a.level + ((q64 - j) >> a.log2B)) >= 3) continue;
+        if (q64 < j || q64 - j >= wend) continue;
         const uint32_t s = (uint32_t)(q64 - j);
         uint32_t l = min(common_ex(s, pq, room), room);
         if (l >= mm) l = span(a, s, b, l);
@@ -486,7 +488,7 @@ __device__ __forceinline__ bool external_wins(uint32_t li, uint32_t wi, uint32_t
 // (256 bytes compared a round).  The next 32 positions' candidates load ahead.
 // A thread per block with a byte per wave took 14.5 ms of the 64 MiB FASTQ
 // encode and 45.8 ms of the 11 MiB text one; a warp per block that decided one
-// position at a time 4.2 ms of the text one; this takes 0.93 and 2.1 ms.
+// position at a time 4.2 ms of the text one; this takes 0.33 and 0.62 ms.
 __global__ void __launch_bounds__(32) parse_kernel(EncArgs a) {
   extern __shared__ uint32_t planes[];  // [3][B / 32 + 1]
   const uint32_t lane = threadIdx.x;
@@ -838,13 +840,13 @@ constexpr uint32_t kLongRun = 16;  // literal runs from here on are copied by th
 //
 // A warp per block did all of this in series, with a divide per symbol and a
 // second pass over the symbols for the bytes' places, 2.6 ms of the 64 MiB
-// FASTQ encode and 1.3 ms of the 11 MiB text one; this takes 0.81 and 0.26 ms.
+// FASTQ encode and 1.3 ms of the 11 MiB text one; this takes 0.41 and 0.09 ms.
 // Bound by the coder's chain where
 // blocks are few, by issue where they are many.
 __global__ void __launch_bounds__(32 * kCodeWarps) code_kernel(CodeArgs ca) {
   extern __shared__ uint32_t group[];  // [3][groups]: bytes, literals, escapes before each group of 32 tokens
   __shared__ uint2 s_tab[3][256];
-  __shared__ uint32_t s_cnt[3][256], s_bits[kHead / 32 + 2], s_total[3], s_bytes[3], s_level;
+  __shared__ uint32_t s_cnt[3][256], s_bits[kHead / 32 + 2], s_total[3], s_bytes[3];
   const EncArgs& a = ca.e;
   const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const uint64_t cb = blockIdx.x, b = a.c0 + cb, bstart = b << a.log2B;
@@ -852,7 +854,6 @@ __global__ void __launch_bounds__(32 * kCodeWarps) code_kernel(CodeArgs ca) {
   const uint32_t nt = a.ntok[cb], nm = nt - 1, w = a.w, ng = (nt + 31) / 32;
   for (uint32_t i = tid; i < 3 * 256; i += 32 * kCodeWarps) (&s_cnt[0][0])[i] = 0;
   if (tid < kHead / 32 + 2) s_bits[tid] = 0;
-  if (tid == 0) s_level = 0;
   for (uint32_t g = wid; g < ng; g += kCodeWarps) {
     const uint32_t t = 32 * g + lane;
     const uint4 v = t < nt ? tk[t] : make_uint4(0u, 0u, 0u, 0u);
@@ -944,9 +945,7 @@ __global__ void __launch_bounds__(32 * kCodeWarps) code_kernel(CodeArgs ca) {
     r = code_stream_warp(lit + sym_at, n, end, s_cnt[wid], s_tab[wid], a.adaptive != 0, lane);
     if (lane == 0) s_bytes[wid] = r.bytes;
   } else {
-    // the block's level: 1 + the deepest block read; its dependency runs
-    for (uint32_t q = lane; q < kHead && q < b; q += 32)
-      if (s_bits[q >> 5] >> (q & 31) & 1) atomicMax(&s_level, a.level[q] + 1);
+    // the block's dependency runs
     uint32_t* iv = ca.iv + b * (uint64_t)(2 * kIvCap);
     const uint32_t v = lane < kHead / 32 ? s_bits[lane] : 0u;
     const uint32_t before = __shfl_up_sync(kFull, v, 1) >> 31, after = __shfl_down_sync(kFull, v, 1) << 31;
@@ -975,7 +974,6 @@ __global__ void __launch_bounds__(32 * kCodeWarps) code_kernel(CodeArgs ca) {
     d.ntok = nt;
     d.nesc = esc_total;
     for (int q = 0; q < 5; q++) d.reserved[q] = 0;
-    a.level[b] = s_level;
     ca.pay_bytes[cb] = p0 + p1 + p2;
   }
 }
@@ -1065,9 +1063,38 @@ struct AsmArgs {
   const uint32_t* n_iv;   // per block
   const uint32_t* iv;     // per block: kIvCap pairs
   uint32_t* dep_ptr;      // scratch: nb + 1
-  const uint32_t* level;
+  uint32_t* level;        // per block
   uint64_t nb;
 };
+
+// A block's level by the warp: 1 + the deepest block it reads.
+__device__ __forceinline__ void block_level(const AsmArgs& a, uint64_t b, uint32_t lane) {
+  const uint2* runs = reinterpret_cast<const uint2*>(a.iv) + b * kIvCap;
+  const uint32_t n = a.n_iv[b];
+  uint32_t l = 0;
+  for (uint32_t i = lane; i < n; i += 32) {
+    const uint2 r = runs[i];
+    for (uint32_t k = r.x; k <= r.y; k++) l = max(l, a.level[k] + 1);
+  }
+  l = __reduce_max_sync(kFull, l);
+  if (lane == 0) a.level[b] = l;
+}
+
+// The levels: HEAD, one CTA over the windows that may be sources, one after
+// another; without it the blocks after them, a warp per block.
+template <bool HEAD>
+__global__ void level_kernel(AsmArgs a) {
+  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (HEAD) {
+    for (uint32_t w = 0; w < kHead; w += kWin) {
+      for (uint64_t b = w + wid; b < min((uint64_t)w + kWin, a.nb); b += nw) block_level(a, b, lane);
+      __syncthreads();
+    }
+  } else {
+    const uint64_t b = kHead + blockIdx.x * (uint64_t)nw + wid;
+    if (b < a.nb) block_level(a, b, lane);
+  }
+}
 
 // One CTA: the dependency table's pointers (exclusive prefix of the runs),
 // the total, and the deepest level.
@@ -1169,7 +1196,7 @@ ace_status enc_layout(uint64_t n, const ace_encode_params* p, EncLayout* L) {
   o = a256(o + 4 * (nb + 1));
   L->entries = o;
   // (an array per part where a launch's blocks are split)
-  L->entry_blocks = cand_shape(p->log2_block).shared_entries ? 0 : std::max<uint64_t>(C, 2 * std::min<uint64_t>(C, kWin));
+  L->entry_blocks = cand_shape(p->log2_block).shared_entries ? 0 : 2 * C <= kSplitEntries ? 2 * C : C;
   o = a256(o + 4 * B * L->entry_blocks);
   L->cand = o;
   o = a256(o + 8 * cb);
@@ -1231,7 +1258,6 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   EncHdr* hdr = reinterpret_cast<EncHdr*>(base + L.hdr);
   ENC_TRY(cudaMemsetAsync(base + L.hdr, 0, sizeof(EncHdr), s));
   ENC_TRY(cudaMemsetAsync(base + L.table, 0xff, 8ull << L.bits, s));
-  if (nb) ENC_TRY(cudaMemsetAsync(base + L.level, 0, 4 * nb, s));
   EncArgs e{};
   e.in = static_cast<const uint8_t*>(d_in);
   e.n = n;
@@ -1243,7 +1269,6 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   e.adaptive = params->adaptive;
   e.bits = L.bits;
   e.table = reinterpret_cast<unsigned long long*>(base + L.table);
-  e.level = reinterpret_cast<uint32_t*>(base + L.level);
   e.entries = reinterpret_cast<uint32_t*>(base + L.entries);
   e.cand = reinterpret_cast<uint2*>(base + L.cand);
   e.tok = reinterpret_cast<uint32_t*>(base + L.tok);
@@ -1274,18 +1299,6 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
     const uint64_t nkeys = (n - kKey) / kStride + 1;
     table_kernel<<<(uint32_t)std::min<uint64_t>((nkeys + 255) / 256, 65535ull * 8), 256, 0, s>>>(e);
   }
-  // launches: the first three windows one after another (a window takes
-  // sources only from the windows before it), then every later block
-  // taking sources only from the first three windows
-  struct Piece {
-    uint64_t c0, c1, ws;
-  };
-  std::vector<Piece> pieces;
-  const uint64_t head = std::min<uint64_t>(nb, kHead);
-  for (uint64_t w0 = 0; w0 < head; w0 += kWin)
-    for (uint64_t c = w0; c < std::min(head, w0 + kWin); c += L.chunk)
-      pieces.push_back({c, std::min({head, w0 + kWin, c + L.chunk}), w0});
-  for (uint64_t c = head; c < nb; c += L.chunk) pieces.push_back({c, std::min(nb, c + L.chunk), head});
   const CandShape shape = cand_shape(params->log2_block);
   int dev = 0, num_sms = 0;
   ENC_TRY(cudaGetDevice(&dev));
@@ -1293,15 +1306,15 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   for (auto k : {candidate_kernel<true>, candidate_kernel<false>})  // the most either asks for, whatever the block size
     ENC_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)std::max(cand_shape(15).smem, cand_shape(16).smem)));
-  for (const Piece& pc : pieces) {
-    e.c0 = pc.c0;
-    e.c1 = pc.c1;
-    e.ws = pc.ws;
-    const uint64_t cn = pc.c1 - pc.c0;
-    // a launch of few blocks (the first windows) splits each over CTAs until
-    // there are two per SM; every part links the whole block again, so no
-    // further than needed (the candidate launches of 11 MiB of text, three of
-    // their four over 64 blocks: 1.29 ms split, 1.85 unsplit)
+  // As many blocks at once as the scratch holds.  Levels come after all of them,
+  // so the first windows run beside the rest, where they had been four rounds
+  // of launches, each as long as its slowest block: 11 MiB of text 3.75 ms, now 1.90; 64
+  // MiB of FASTQ 5.1 and 3.7 ms.
+  for (e.c0 = 0; e.c0 < nb; e.c0 += L.chunk) {
+    const uint64_t cn = std::min(nb - e.c0, L.chunk);
+    // a launch of few blocks splits each over CTAs until there are two per SM;
+    // every part links the whole block again, so no further than needed (text:
+    // 256 KiB 804 us split, 910 unsplit, 1 MiB 842 and 933, 3 MiB 1151 and 1133)
     uint32_t parts = 1;
     while (parts < kCandParts && cn * parts < 2ull * num_sms && B / shape.threads >= 2 * parts &&
            (shape.shared_entries || 2 * cn * parts <= L.entry_blocks))
@@ -1311,7 +1324,7 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
     parse_kernel<<<(uint32_t)cn, 32, 3 * (B / 8 + 4), s>>>(e);  // at most 24.1 KB of bit maps
     ca.e = e;
     code_kernel<<<(uint32_t)cn, 32 * kCodeWarps, 12 * ((L.tok_cap + 31) / 32), s>>>(ca);
-    pa.c0 = pc.c0;
+    pa.c0 = e.c0;
     pa.cn = cn;
     place_scan_kernel<<<1, 1024, 0, s>>>(pa);
     place_copy_kernel<<<(uint32_t)((cn + 7) / 8), 256, 0, s>>>(pa);
@@ -1321,9 +1334,13 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   aa.n_iv = ca.n_iv;
   aa.iv = ca.iv;
   aa.dep_ptr = reinterpret_cast<uint32_t*>(base + L.dep_ptr);
-  aa.level = e.level;
+  aa.level = reinterpret_cast<uint32_t*>(base + L.level);
   aa.nb = nb;
-  if (nb) deps_scan_kernel<<<1, 1024, 0, s>>>(aa);
+  if (nb) {
+    level_kernel<true><<<1, 1024, 0, s>>>(aa);
+    if (nb > kHead) level_kernel<false><<<(uint32_t)((nb - kHead + 7) / 8), 256, 0, s>>>(aa);
+    deps_scan_kernel<<<1, 1024, 0, s>>>(aa);
+  }
   ENC_TRY(cudaGetLastError());
   EncHdr h;
   ENC_TRY(cudaMemcpyAsync(&h, hdr, sizeof h, cudaMemcpyDeviceToHost, s));
