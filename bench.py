@@ -322,7 +322,7 @@ def roofline_of(alg, ms_pass, ms_whole, peaks, peak_kind, sm_count, clocks, work
     roofline (warp instructions per second against 4 per SM per cycle at the
     sampled SM clock); the summary's limiter names the bound."""
     names = ["decode_kernel<false, PASS_TOKENS>", "decode_kernel<false, PASS_LITERALS>",
-             "match_level_kernel + match_small_kernel"]
+             "match_level_kernel + match_cta_kernel"]
     top = max(range(3), key=lambda p: ms_pass[p])
     hbm_peak = peaks["hbm_gbs"]
     achieved = alg["passes"][top] / (ms_pass[top] / 1e3) / 1e9

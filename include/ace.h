@@ -245,7 +245,9 @@ ace_status ace_scratch_init(const ace_index *idx, void *d_scratch, uint64_t scra
 /* How a decode is laid out in launches.
  * ACE_SCHEDULE_PASSES: three passes -- tokens (length and offset streams
  * into match records) and literals as persistent launches over the blocks,
- * then the match pass, one launch per dependency level.
+ * then the match pass, one launch per dependency level; with little work to
+ * spread (few blocks, small batches) the first two become one launch, a warp
+ * per stream, and the match pass places the literals.
  * ACE_SCHEDULE_FUSED: one persistent launch.  Each warp takes a block in
  * (level, block) order and decodes its entropy layer, then holds the
  * block's matches until every block of the lower levels is resolved,
@@ -328,12 +330,12 @@ ace_status ace_sync(const ace_index *idx, void *d_scratch, cudaStream_t s);
 /* ---------------------------------------------------------------- batches */
 
 /*
- * Many independent archives decoded in one persistent launch (the batching
- * pattern: thousands of uneven objects with mixed block sizes).  Each
- * archive's blocks keep their own (level, block) order; warps and CTAs take
- * (archive, block) items from one ticket, lower levels of every archive first
- * in the match pass, so a block only waits on blocks of
- * its own archive handed out before it (Section 2's dependency rule).
+ * Many independent archives decoded in one persistent launch per pass (the
+ * batching pattern: thousands of uneven objects with mixed block sizes).
+ * Each archive's blocks keep their own (level, block) order; warps and CTAs
+ * take (archive, block) items from one ticket, the lower levels of every
+ * archive first in the match pass, so a block only waits on blocks of its own
+ * archive handed out before it (Section 2's dependency rule).
  *
  * ace_batch_scratch_size sizes the batch scratch (256-byte aligned).
  * ace_batch_create records the archives (all on the current device) and
@@ -342,7 +344,8 @@ ace_status ace_sync(const ace_index *idx, void *d_scratch, cudaStream_t s);
  * plans the launch from tune (NULL = defaults), and synchronises s.  It
  * allocates no device memory.  ace_decode_batch then enqueues, with no host
  * synchronisation, a header reset and the token, literal and match passes
- * (pass schedule) or a memset of the level counters, a header reset and one
+ * (pass schedule; up to 128 MiB of output a launch of a warp per stream, then
+ * the match pass) or a memset of the level counters, a header reset and one
  * fused launch (ACE_SCHEDULE_FUSED), so it can be captured into a CUDA graph
  * and replayed; each replay decodes every archive again.
  * ace_batch_sync synchronises s and returns (then clears) the first device
@@ -387,8 +390,8 @@ ace_status ace_batch_free(ace_batch *batch);
  * All archives of a cache share one device and one block size.  Batches on
  * one cache must be ordered on one stream; separate caches (each with its
  * own per-archive states) may run concurrently on separate streams.
- * ace_seek_batch reads device-resident requests and enqueues three kernels
- * plus the passes; ace_seek_batch_host validates host requests against the
+ * ace_seek_batch reads device-resident requests and enqueues the closure
+ * search, the passes and the slice copies; ace_seek_batch_host validates host requests against the
  * archives' sizes (h_totals, may be NULL) and the pool, stages them in the
  * cache memory (n <= max_reqs) and calls it.  ace_cache_sync returns (then
  * clears) the first device error; ace_cache_usage reports slots holding a

@@ -1868,8 +1868,8 @@ struct BatchArgs {
   uint32_t long_min;
 };
 
-// The work of a batch: (archive, block) items, each archive's blocks in its
-// own level order.
+// The work of a batch: (archive, block) items in one of the two orders, each
+// archive's blocks in its own level order in both.
 struct BatchJobs {
   const BatchArgs& ba;
   const BatchSeg* segs;
@@ -1878,10 +1878,10 @@ struct BatchJobs {
   __device__ uint32_t below(const DecodeArgs& x, uint32_t L) const { return __ldg(x.lv_count + L - 1); }
 };
 
-// Thousands of independent archives in one persistent launch per pass:
-// warps take (archive, block) items from one ticket; each archive's items
-// are in its own (level, block) order, so in the match pass a warp only
-// ever waits on blocks of its archive that were handed out before its own.
+// Thousands of independent archives in one persistent launch per pass: warps
+// (match pass: CTAs) take (archive, block) items from one ticket; each
+// archive's items are in its own (level, block) order, so in the match pass a
+// block only ever waits on blocks of its archive handed out before it.
 __device__ DecodeArgs batch_args(const BatchArgs& ba, const ObjDesc& od) {
   DecodeArgs a{};
   a.arc = od.arc;
