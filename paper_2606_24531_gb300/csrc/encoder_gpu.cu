@@ -1000,6 +1000,8 @@ struct PlaceArgs {
   uint32_t pay_cap;
   uint8_t* dst;               // where the payload is assembled (the archive buffer's tail)
   uint64_t dst_cap;           // bytes available there
+  uint8_t* arc;               // or (not null), once the dependency runs are counted: the archive, whose payload
+  uint64_t fixed;             // starts after these bytes and the runs
 };
 
 // One CTA: the chunk's block payloads laid end to end after the payload so
@@ -1051,7 +1053,8 @@ __global__ void place_copy_kernel(PlaceArgs p) {
   const uint64_t i = blockIdx.x * (uint64_t)(blockDim.x >> 5) + wid;
   if (i >= p.cn || *(volatile uint32_t*)&p.h->status) return;
   const uint4* src = reinterpret_cast<const uint4*>(p.pay + i * (uint64_t)p.pay_cap);
-  uint4* dst = reinterpret_cast<uint4*>(p.dst + p.pay_off[i]);
+  uint8_t* const to = p.arc ? p.arc + align16(p.fixed + 8 * p.h->n_iv) : p.dst;
+  uint4* dst = reinterpret_cast<uint4*>(to + p.pay_off[i]);
   const uint32_t n16 = p.pay_bytes[i] / 16;
   for (uint32_t k = lane; k < n16; k += 32) dst[k] = src[k];
 }
@@ -1131,18 +1134,24 @@ __global__ void deps_scan_kernel(AsmArgs a) {
   }
 }
 
-// The directory and the dependency table into the archive: pointers, then
-// each block's runs at its pointer.
+// The directory and the dependency table into the archive, a warp per block:
+// its directory entry, its pointer, and its runs at that pointer.  (A thread
+// per block took 23 us for the 704 blocks of 11 MiB of text, 33 for the 4096 of
+// 64 MiB of FASTQ; this takes 3 and 5.)
 __global__ void deps_write_kernel(AsmArgs a, const ace_block_dir* dir, uint8_t* arc, uint64_t dir_off,
                                   uint64_t deps_off) {
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i <= a.nb; i += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t* ptr = reinterpret_cast<uint32_t*>(arc + deps_off);
-    ptr[i] = a.dep_ptr[i];
+  const uint32_t lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  uint32_t* const ptr = reinterpret_cast<uint32_t*>(arc + deps_off);
+  for (uint64_t i = blockIdx.x * (uint64_t)nw + (threadIdx.x >> 5); i <= a.nb; i += (uint64_t)gridDim.x * nw) {
+    const uint32_t at = a.dep_ptr[i];
+    if (lane == 0) ptr[i] = at;
     if (i == a.nb) continue;
-    reinterpret_cast<ace_block_dir*>(arc + dir_off)[i] = dir[i];
-    uint32_t* ivs = ptr + a.nb + 1 + 2ull * a.dep_ptr[i];
+    static_assert(sizeof(ace_block_dir) == 64, "directory entry");
+    if (lane < 16)
+      reinterpret_cast<uint32_t*>(arc + dir_off + 64 * i)[lane] = reinterpret_cast<const uint32_t*>(dir + i)[lane];
+    uint32_t* ivs = ptr + a.nb + 1 + 2ull * at;
     const uint32_t* src = a.iv + i * (uint64_t)(2 * kIvCap);
-    for (uint32_t k = 0; k < 2 * a.n_iv[i]; k++) ivs[k] = src[k];
+    for (uint32_t k = lane; k < 2 * a.n_iv[i]; k += 32) ivs[k] = src[k];
   }
 }
 
@@ -1306,6 +1315,25 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   for (auto k : {candidate_kernel<true>, candidate_kernel<false>})  // the most either asks for, whatever the block size
     ENC_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)std::max(cand_shape(15).smem, cand_shape(16).smem)));
+  AsmArgs aa;
+  aa.h = hdr;
+  aa.n_iv = ca.n_iv;
+  aa.iv = ca.iv;
+  aa.dep_ptr = reinterpret_cast<uint32_t*>(base + L.dep_ptr);
+  aa.level = reinterpret_cast<uint32_t*>(base + L.level);
+  aa.nb = nb;
+  auto count_runs = [&] {
+    level_kernel<true><<<1, 1024, 0, s>>>(aa);
+    if (nb > kHead) level_kernel<false><<<(uint32_t)((nb - kHead + 7) / 8), 256, 0, s>>>(aa);
+    deps_scan_kernel<<<1, 1024, 0, s>>>(aa);
+  };
+  // An input of one launch places its payload where it stays: the runs are
+  // counted before.  One of several places it above room for the largest table
+  // and moves it down in the end, in copies no longer than the gap between the
+  // two (22 copies, 127 us, for 64 MiB of FASTQ).
+  const bool whole = nb <= L.chunk;
+  pa.arc = whole ? arc : nullptr;
+  pa.fixed = sizeof(ace_file_header) + 64 * nb + 4 * (nb + 1);
   // As many blocks at once as the scratch holds.  Levels come after all of them,
   // so the first windows run beside the rest, where they had been four rounds
   // of launches, each as long as its slowest block: 11 MiB of text 3.75 ms, now 1.90; 64
@@ -1326,21 +1354,11 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
     code_kernel<<<(uint32_t)cn, 32 * kCodeWarps, 12 * ((L.tok_cap + 31) / 32), s>>>(ca);
     pa.c0 = e.c0;
     pa.cn = cn;
+    if (whole) count_runs();
     place_scan_kernel<<<1, 1024, 0, s>>>(pa);
     place_copy_kernel<<<(uint32_t)((cn + 7) / 8), 256, 0, s>>>(pa);
   }
-  AsmArgs aa;
-  aa.h = hdr;
-  aa.n_iv = ca.n_iv;
-  aa.iv = ca.iv;
-  aa.dep_ptr = reinterpret_cast<uint32_t*>(base + L.dep_ptr);
-  aa.level = reinterpret_cast<uint32_t*>(base + L.level);
-  aa.nb = nb;
-  if (nb) {
-    level_kernel<true><<<1, 1024, 0, s>>>(aa);
-    if (nb > kHead) level_kernel<false><<<(uint32_t)((nb - kHead + 7) / 8), 256, 0, s>>>(aa);
-    deps_scan_kernel<<<1, 1024, 0, s>>>(aa);
-  }
+  if (nb && !whole) count_runs();
   ENC_TRY(cudaGetLastError());
   EncHdr h;
   ENC_TRY(cudaMemcpyAsync(&h, hdr, sizeof h, cudaMemcpyDeviceToHost, s));
@@ -1363,10 +1381,10 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   if (fh.archive_bytes > arc_cap || fh.payload_off > L.reserve) return ACE_E_NOMEM;
   ENC_TRY(cudaMemsetAsync(arc, 0, fh.payload_off, s));
   if (nb) {
-    deps_write_kernel<<<(uint32_t)std::min<uint64_t>((nb + 256) / 256, 65535), 256, 0, s>>>(aa, ca.dir, arc, fh.dir_off,
+    deps_write_kernel<<<(uint32_t)std::min<uint64_t>((nb + 8) / 8, 65535), 256, 0, s>>>(aa, ca.dir, arc, fh.dir_off,
                                                                                            fh.deps_off);
     // the payload down to its place, in pieces no longer than the gap
-    const uint64_t gap = L.reserve - fh.payload_off;
+    const uint64_t gap = whole ? 0 : L.reserve - fh.payload_off;
     for (uint64_t o = 0; o < h.payload;) {
       const uint64_t len = gap ? std::min(gap, h.payload - o) : h.payload;
       if (gap) ENC_TRY(cudaMemcpyAsync(arc + fh.payload_off + o, arc + L.reserve + o, len, cudaMemcpyDeviceToDevice, s));
