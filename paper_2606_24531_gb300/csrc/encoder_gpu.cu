@@ -998,11 +998,16 @@ struct PlaceArgs {
   uint64_t c0, cn;            // the chunk's first block and block count
   const uint8_t* pay;
   uint32_t pay_cap;
-  uint8_t* dst;               // where the payload is assembled (the archive buffer's tail)
-  uint64_t dst_cap;           // bytes available there
-  uint8_t* arc;               // or (not null), once the dependency runs are counted: the archive, whose payload
-  uint64_t fixed;             // starts after these bytes and the runs
+  uint8_t* arc;               // the archive's buffer
+  uint64_t arc_cap;
+  uint64_t reserve;           // where the payload is assembled, or
+  uint64_t fixed;             // (not 0) once the dependency runs are counted: it starts after these bytes and the runs
 };
+
+// Where the payload goes in the archive's buffer.
+__device__ __forceinline__ uint64_t payload_start(const PlaceArgs& p) {
+  return p.fixed ? align16(p.fixed + 8 * p.h->n_iv) : p.reserve;
+}
 
 // One CTA: the chunk's block payloads laid end to end after the payload so
 // far (each a multiple of 16 bytes), their directory offsets made relative
@@ -1042,7 +1047,7 @@ __global__ void place_scan_kernel(PlaceArgs p) {
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    if (carry > p.dst_cap) record_error(&p.h->status, &p.h->status, &p.h->status, ACE_E_NOMEM, 0, 0);
+    if (payload_start(p) + carry > p.arc_cap) p.h->status = ACE_E_NOMEM;  // this chunk and later ones are not copied
     p.h->payload = carry;
   }
 }
@@ -1053,8 +1058,7 @@ __global__ void place_copy_kernel(PlaceArgs p) {
   const uint64_t i = blockIdx.x * (uint64_t)(blockDim.x >> 5) + wid;
   if (i >= p.cn || *(volatile uint32_t*)&p.h->status) return;
   const uint4* src = reinterpret_cast<const uint4*>(p.pay + i * (uint64_t)p.pay_cap);
-  uint8_t* const to = p.arc ? p.arc + align16(p.fixed + 8 * p.h->n_iv) : p.dst;
-  uint4* dst = reinterpret_cast<uint4*>(to + p.pay_off[i]);
+  uint4* dst = reinterpret_cast<uint4*>(p.arc + payload_start(p) + p.pay_off[i]);
   const uint32_t n16 = p.pay_bytes[i] / 16;
   for (uint32_t k = lane; k < n16; k += 32) dst[k] = src[k];
 }
@@ -1302,8 +1306,9 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   pa.dir = ca.dir;
   pa.pay = ca.pay;
   pa.pay_cap = L.pay_cap;
-  pa.dst = arc + L.reserve;
-  pa.dst_cap = arc_cap - L.reserve;
+  pa.arc = arc;
+  pa.arc_cap = arc_cap;
+  pa.reserve = L.reserve;
   if (n >= kKey) {
     const uint64_t nkeys = (n - kKey) / kStride + 1;
     table_kernel<<<(uint32_t)std::min<uint64_t>((nkeys + 255) / 256, 65535ull * 8), 256, 0, s>>>(e);
@@ -1332,8 +1337,7 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   // and moves it down in the end, in copies no longer than the gap between the
   // two (22 copies, 127 us, for 64 MiB of FASTQ).
   const bool whole = nb <= L.chunk;
-  pa.arc = whole ? arc : nullptr;
-  pa.fixed = sizeof(ace_file_header) + 64 * nb + 4 * (nb + 1);
+  pa.fixed = whole ? sizeof(ace_file_header) + 64 * nb + 4 * (nb + 1) : 0;
   // As many blocks at once as the scratch holds.  Levels come after all of them,
   // so the first windows run beside the rest, where they had been four rounds
   // of launches, each as long as its slowest block: 11 MiB of text 3.75 ms, now 1.90; 64

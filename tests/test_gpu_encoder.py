@@ -105,3 +105,33 @@ def test_gpu_encoder_adaptive_offsets_and_edges():
             x = rng.integers(0, alpha, n).astype(np.uint8)
             arc, _ = _encode(x, 8, 4)
             assert np.array_equal(oracle.decode(arc), x), (n, alpha)
+
+
+@pytest.mark.parametrize("chunk", [0, 16])  # one launch: the payload placed where it stays; several: after the reserve
+@pytest.mark.parametrize("log2b", [12, 16])
+def test_archive_buffer_too_small(log2b, chunk):
+    """A buffer one vector short is refused without a byte written past it;
+    one of exactly the needed size holds the same archive as the bound."""
+    import ctypes
+
+    n = 40 << log2b
+    data = torch.from_numpy(np.random.default_rng(5).integers(0, 256, n, dtype=np.uint8)).cuda()
+    full = ace.ace_encode_gpu(data, log2b, 4, chunk_blocks=chunk).cpu().numpy()
+    payload_off = int(full[:64].view(np.uint64)[6])
+    prm = ace.ace_encode_params(log2b, 4, chunk, 16, 0, 0)
+    sb, bound = ctypes.c_uint64(), ctypes.c_uint64()
+    assert ace.lib().ace_encode_gpu_size(n, ctypes.byref(prm), ctypes.byref(sb), ctypes.byref(bound)) == ace.ACE_OK
+    reserve = bound.value - ace._enc_payload_room(40, log2b, 4)
+    need = full.size if chunk == 0 else reserve + full.size - payload_off
+    scratch = torch.empty(sb.value, dtype=torch.uint8, device="cuda")
+    for cap, want in ((need - 16, ace.ACE_E_NOMEM), (need - full.size // 2, ace.ACE_E_NOMEM), (need, ace.ACE_OK)):
+        assert cap >= reserve + 256
+        store = torch.full((bound.value + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+        ln = ctypes.c_uint64()
+        rc = ace.lib().ace_encode_gpu(data.data_ptr(), n, ctypes.byref(prm), scratch.data_ptr(), sb.value,
+                                      store.data_ptr(), cap, ctypes.byref(ln), None,
+                                      torch.cuda.current_stream().cuda_stream)
+        assert rc == want
+        assert bool((store[cap:] == 0xA5).all())
+        if rc == ace.ACE_OK:
+            assert np.array_equal(store[:ln.value].cpu().numpy(), full)
