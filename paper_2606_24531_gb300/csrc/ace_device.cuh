@@ -116,13 +116,15 @@ __device__ __forceinline__ bool wait_flag(const uint32_t* flag, uint32_t want, u
 
 // Thread-block clusters: this CTA's rank, and a barrier over the cluster's
 // threads after which their earlier global writes are seen (L1 aside: read
-// what another CTA wrote with L2 loads).
+// what another CTA wrote with L2 loads).  The aligned barrier wants each warp
+// together, and callers come from loops of uneven lengths.
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %cluster_ctarank;" : "=r"(r));
   return r;
 }
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
