@@ -430,6 +430,12 @@ __device__ __forceinline__ uint64_t src_index(uint64_t S, uint64_t d, uint32_t l
   return d >= len ? S + i : S + (i % (uint32_t)d);
 }
 
+// A record's source: five bytes.  Stream jobs keep the literals before the match
+// in the three above them, where a later call's match pass still finds them.
+__device__ __forceinline__ uint64_t record_source(uint4 r) {
+  return (uint64_t)r.x | (uint64_t)(r.y & 0xffu) << 32;
+}
+
 // The records of block b: whole decodes by the index's prefix count of
 // matches; seeks max_ntok per slot; seek batches max_ntok per work item
 // (rec_index: block -> its place in the batch's work list).
@@ -929,7 +935,7 @@ __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint3
     cp_async_wait<kRecDepth - 1>();  // group g has landed
     uint4 r = make_uint4(0, 0, 0, 0);
     if (t0 + lane < nm) r = rring[(g % kRecDepth) * kMatchGroup + lane];
-    const uint64_t S = (uint64_t)r.x | ((uint64_t)r.y << 32);
+    const uint64_t S = record_source(r);
     const uint32_t D = r.z;
     uint32_t L = r.w;
     if (L && (S >= bstart + D || (uint64_t)D + L > blen)) {  // checked again: the token pass may have failed
@@ -1073,7 +1079,7 @@ __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint3
         // source); the ragged ends a byte per lane
         for (uint32_t todo = __ballot_sync(kFull, lgo); todo; todo &= todo - 1) {
           const uint32_t j = __ffs(todo) - 1, Dj = __shfl_sync(kFull, D, j), Lj = __shfl_sync(kFull, L, j);
-          const uint64_t Sj = (uint64_t)__shfl_sync(kFull, r.x, j) | (uint64_t)__shfl_sync(kFull, r.y, j) << 32;
+          const uint64_t Sj = (uint64_t)__shfl_sync(kFull, (uint32_t)S, j) | (uint64_t)__shfl_sync(kFull, (uint32_t)(S >> 32), j) << 32;
           const uint32_t head = (0u - Dj) & 15, tail = (Dj + Lj) & 15, n = (Lj - head) >> 4;
           const bool ragged = lane < 16 ? lane < head : lane - 16 < tail;
           const uint32_t i = lane < 16 ? lane : Lj - tail + (lane - 16);
@@ -1274,7 +1280,7 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
       for (; g < ng; g += step) {
         const uint4 r = rn;
         rn = fetch(g + step);
-        const uint64_t S = (uint64_t)r.x | ((uint64_t)(LITS ? r.y & 0xffu : r.y) << 32);
+        const uint64_t S = record_source(r);
         uint32_t D = r.z, lits = 0, lr = 0;
         uint32_t L = r.w;
         if (LITS) {  // lits: literals before the match; lr: those of its token's run

@@ -107,6 +107,32 @@ def test_levels_of_many_blocks(shape):
         da.close()
 
 
+@pytest.mark.parametrize("off_width", [4, 5])
+@pytest.mark.parametrize("log2b", [8, 12, 14, 16, "long"])
+def test_match_pass_over_the_records_of_a_whole_decode(log2b, off_width):
+    """A whole decode of few blocks leaves records with the literals before each
+    match beside its source; the match pass by itself reads the same sources, by
+    a CTA per block and (long: 1100 blocks, most of a level) by a warp per block."""
+    if log2b == "long":
+        piece = np.random.default_rng(7).integers(0, 256, 40_000).astype(np.uint8)
+        data = np.concatenate([np.roll(piece, 1500 * k) for k in range(113)])[:1100 << 12]
+        arc = ace.ace_encode_gpu(torch.from_numpy(data).cuda(), 12, 16, off_width=off_width).cpu().numpy()
+    else:
+        lengths, back, lit = SHAPES["every overlap"]
+        data = _copies(lengths, back, lit, 30_001, log2b)
+        arc = ace.ace_encode(data, log2b, 4, off_width=off_width)
+    da = DeviceArchive(arc)
+    out = da.decode_all()
+    ace.ace_decode_pass(da.idx, 2, out, out.numel(), da.d_scratch, da.scratch_bytes, None, da.stream)
+    assert da.sync() == ace.ACE_OK
+    assert np.array_equal(out.cpu().numpy(), data)
+    if log2b == "long":  # the sizes the case is for
+        levels = ace.ace_index_levels(da.idx, da.info["n_levels"])
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        assert max(levels) > 4 * sms and da.info["n_blocks"] <= 8 * sms and arc.size < data.size // 4
+    da.close()
+
+
 def test_batches_of_either_size():
     """A batch that decodes a stream per warp and one, above 128 MiB, in three
     passes: blocks of every size, objects of a block and of many."""
