@@ -849,11 +849,16 @@ constexpr uint32_t kRowUnroll = 8;
 constexpr uint32_t kCopyUnroll = 8;
 // Copy classes of a group resolved in rounds: a non-overlapping match of at
 // least the call's long_min bytes is copied by the whole warp in aligned
-// 16-byte pieces, every other one bytewise with the round's other such
+// 16-byte pieces, one of at most kShortMax bytes (WAY_LANES) by one lane in
+// aligned 8-byte words, every other one bytewise with the round's other such
 // matches.  long_min is the copy-width knob: kLongMinWide (16-byte pieces for
 // everything above 32 bytes) or kLongMinNarrow (bytewise up to 511 bytes).
+constexpr uint32_t kShortMax = 32;
 constexpr uint32_t kLongMinNarrow = 512;
-constexpr uint32_t kLongMinWide = 33;
+constexpr uint32_t kLongMinWide = kShortMax + 1;
+
+// The ways a warp takes through a group of matches (match_block).
+enum { WAY_ROUNDS = 0, WAY_LANES = 1, WAY_ROWS = 2 };
 
 // A load of match source bytes.  L1: through the SM's L1 cache, for a pass
 // whose sources were all written by earlier launches or by this warp (one
@@ -862,6 +867,74 @@ constexpr uint32_t kLongMinWide = 33;
 template <bool L1, class T>
 __device__ __forceinline__ T ld_src(const T* p) {
   return L1 ? __ldca(p) : __ldcg(p);
+}
+
+// Source of a short match: the aligned 8-byte words covering [S, S + len).
+template <bool SEEK, bool L1>
+__device__ __forceinline__ void short_load(const DecodeArgs& a, uint64_t S, uint32_t len, uint64_t (&w)[5], uint64_t b,
+                                           const uint8_t* obase) {
+  const uint64_t a0 = S & ~7ull;
+  const uint32_t off = (uint32_t)(S & 7);
+#pragma unroll
+  for (uint32_t k = 0; k < 5; k++) {
+    const uint64_t q = a0 + 8ull * k;
+    w[k] = 0;
+    if (8 * k < off + len) {
+      if (q + 8 <= a.total) {
+        w[k] = ld_src<L1>(reinterpret_cast<const unsigned long long*>(Addr<SEEK>::at(a, q, b, obase)));
+      } else {
+        for (uint32_t t = 0; t < 8 && q + t < a.total; t++)
+          w[k] |= (uint64_t)ld_src<L1>(Addr<SEEK>::at(a, q + t, b, obase)) << (8 * t);
+      }
+    }
+  }
+}
+
+// Bytes sh .. sh + 7 of hi:lo (sh < 8).
+__device__ __forceinline__ uint64_t funnel64(uint64_t lo, uint64_t hi, uint32_t sh) {
+  return sh ? (lo >> (8 * sh)) | (hi << (64 - 8 * sh)) : lo;
+}
+
+// Bytes [lo, hi) of w to the 8-byte aligned p, in the widest aligned stores
+// that fit.  The lanes of a round store to different lines, so every store
+// a lane saves is an L1 and L2 transaction saved.
+__device__ __forceinline__ void store_bytes8(uint8_t* p, uint64_t w, uint32_t lo, uint32_t hi) {
+  uint32_t k = lo;
+  while (k < hi) {
+    if (!(k & 3) && k + 4 <= hi) {
+      *reinterpret_cast<uint32_t*>(p + k) = (uint32_t)(w >> (8 * k));
+      k += 4;
+    } else if (!(k & 1) && k + 2 <= hi) {
+      *reinterpret_cast<uint16_t*>(p + k) = (uint16_t)(w >> (8 * k));
+      k += 2;
+    } else {
+      p[k] = (uint8_t)(w >> (8 * k));
+      k++;
+    }
+  }
+}
+
+// Destination of a short match: aligned 8-byte words where the match covers
+// them, the widest aligned stores that fit at its two ends.  Source byte off + i (off = S mod 8,
+// counted from the first source word) lands at dp[i].
+__device__ __forceinline__ void short_store(uint8_t* dp, uint32_t off, uint32_t len, const uint64_t (&w)[5]) {
+  const uint32_t hd = (uint32_t)(reinterpret_cast<uintptr_t>(dp) & 7);
+  uint8_t* dal = dp - hd;
+  const bool same = off >= hd;  // destination word i starts in source word i, else in word i - 1
+  const uint32_t sh = (off - hd) & 7;
+#pragma unroll
+  for (uint32_t i = 0; i < 5; i++) {
+    const int first = 8 * (int)i - (int)hd;  // match byte held by the word's first byte
+    if (first >= (int)len) break;
+    const uint64_t lo = same ? w[i] : (i ? w[i - 1] : 0ull);
+    const uint64_t hi = same ? (i + 1 < 5 ? w[i + 1] : 0ull) : w[i];
+    const uint64_t word = funnel64(lo, hi, sh);
+    if (first >= 0 && first + 8 <= (int)len) {
+      *reinterpret_cast<uint64_t*>(dal + 8 * i) = word;
+    } else {
+      store_bytes8(dal + 8 * i, word, (uint32_t)max(0, -first), (uint32_t)min(8, (int)len - first));
+    }
+  }
 }
 
 // First index i in [0, n) with key(i) > x, for keys that never decrease.
@@ -904,7 +977,7 @@ __device__ __forceinline__ uint32_t upper_bound(uint32_t n, uint32_t x, Key key)
 // Every group went through the rounds, short matches one per lane in 8-byte
 // words whose loads and stores touch 32 lines each (FASTQ 256 MiB: 0.145 ms);
 // by rows 0.106 ms, bound by the latency of a group after another.
-template <bool SEEK, bool WAIT, bool L1 = !WAIT, bool ROWS = true>
+template <bool SEEK, bool WAIT, bool L1, int WAY>
 __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint32_t lane, uint32_t epoch,
                             uint32_t nm, uint32_t lvl = 0) {
   // L1: every source was written before the launch or by this warp (one
@@ -991,7 +1064,7 @@ __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint3
     // without WAIT the level check below need not hold up the copies: a
     // corrupt archive fails the call whatever bytes they wrote
 
-    if (ROWS && __all_sync(kFull, L <= kRowMax && (!L || (dist >= L && (!SEEK || k0 == (S + L - 1) >> a.log2B))))) {
+    if (WAY == WAY_ROWS && __all_sync(kFull, L <= kRowMax && (!L || (dist >= L && (!SEEK || k0 == (S + L - 1) >> a.log2B))))) {
       // rows.  Per match: where byte c of the group's bytes comes from (address
       // of the source less the match's start among them) and goes to, and the
       // source's place in the block (below 0: an earlier block, always final).
@@ -1073,6 +1146,12 @@ __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint3
       while (pend) {
         const bool go = (pend >> lane & 1) && !(pend & feeds);
         const bool lgo = go && L >= a.long_min && dist >= L;
+        const bool sgo = WAY == WAY_LANES && go && L <= kShortMax && dist >= L;
+        if (sgo) {
+          uint64_t w[5];
+          short_load<SEEK, kL1>(a, S, L, w, b, obase);
+          short_store(obase + D, (uint32_t)(S & 7), L, w);
+        }
         // long: one match after another by the whole warp, in aligned 16-byte
         // stores, each from the two aligned vectors of the source that hold its
         // bytes (which end before the match does: it does not overlap its
@@ -1098,7 +1177,7 @@ __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint3
         }
         // the rest laid end to end in group order: gX[j] is where match j
         // starts, gX[kMatchGroup] the total
-        const bool bgo = go && !lgo;
+        const bool bgo = go && !lgo && !sgo;
         if (__any_sync(kFull, bgo)) {
           const uint32_t len = bgo ? L : 0u;
           const uint32_t incl = warp_incl_sum(len, lane), total = __shfl_sync(kFull, incl, 31);
@@ -1530,12 +1609,16 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
 // decode, so the issue-bound entropy decode of some warps overlaps the
 // latency-bound match copies of others on the same SM.
 // PASS_PLACE is PASS_MATCH after stream jobs, which leave the literals to it.
-enum { PASS_TOKENS = 0, PASS_LITERALS = 1, PASS_MATCH = 2, PASS_FUSED = 3, PASS_PLACE = 4 };
+// PASS_WARP is PASS_MATCH with a warp per block instead of a CTA: for many
+// blocks of few matches, where a CTA's sweep over all of the block's bytes
+// costs more than the matches do.
+enum { PASS_TOKENS = 0, PASS_LITERALS = 1, PASS_MATCH = 2, PASS_FUSED = 3, PASS_PLACE = 4, PASS_WARP = 5 };
 
-// Every pass is held to 64 registers a thread: 256 threads, or the match
-// pass's CTAs of up to 512.
+// A pass is held to 64 registers a thread: 256 threads, or the match pass's
+// CTAs of up to 512; the match pass by warps to 80.
 #define ACE_PASS_CTA(P) ((P) == PASS_MATCH || (P) == PASS_PLACE)
-#define ACE_PASS_BOUNDS(P) __launch_bounds__(ACE_PASS_CTA(P) ? kCtaThreads : 256, ACE_PASS_CTA(P) ? 2 : 4)
+#define ACE_PASS_BOUNDS(P) \
+  __launch_bounds__(ACE_PASS_CTA(P) ? kCtaThreads : 256, ACE_PASS_CTA(P) ? 2 : (P) == PASS_WARP ? 3 : 4)
 
 // Publishes block b (its writes visible device-wide before the flag).
 __device__ __forceinline__ void publish(uint32_t* ready, uint32_t b, uint32_t epoch, uint32_t lane) {
@@ -1666,7 +1749,7 @@ __device__ void fused_loop(const Jobs& jobs, ScratchHdr* sh, uint32_t n_items, u
           // source blocks must be members of the closure; published ones
           // carry the epoch without the pending bit, so the flag checks do
           // not wait
-          ok = match_block<true, true, true>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch,
+          ok = match_block<true, true, true, WAY_ROWS>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch,
                                              ntok ? ntok - 1 : 0);
           if (ok && a.slice) {
             uint64_t bs = (uint64_t)b << a.log2B, be = min(bs + ((uint64_t)1 << a.log2B), a.total);
@@ -1676,7 +1759,7 @@ __device__ void fused_loop(const Jobs& jobs, ScratchHdr* sh, uint32_t n_items, u
           }
           if (ok) publish(a.ready, b, epoch, lane);
         } else {
-          ok = match_block<false, false, true>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch,
+          ok = match_block<false, false, true, WAY_ROWS>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch,
                                                ntok ? ntok - 1 : 0, L);
         }
         if (!ok) break;  // the error is recorded; every warp stops
@@ -1789,8 +1872,8 @@ __global__ void __launch_bounds__(32) entropy_kernel(DecodeArgs a) {
 // 56).  A long match by the whole warp, not the round's long matches laid end
 // to end in pieces with the next lane's vector shuffled in, took the genome's
 // from 518 us.
-template <bool ROWS>
-__global__ void __maxnreg__(ROWS ? 72 : 56) match_level_kernel(DecodeArgs a) {
+template <int WAY>
+__global__ void __maxnreg__(WAY == WAY_ROUNDS ? 56 : 72) match_level_kernel(DecodeArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t nw = gridDim.x * (blockDim.x >> 5);
@@ -1810,7 +1893,7 @@ __global__ void __maxnreg__(ROWS ? 72 : 56) match_level_kernel(DecodeArgs a) {
       bn = __ldg(a.items + nx);
       nmn = n_matches(bn);
     }
-    match_block<false, false, true, ROWS>(a, gm, b, lane, 0, nm, a.cur_level);
+    match_block<false, false, true, WAY>(a, gm, b, lane, 0, nm, a.cur_level);
     if (nx >= a.n_items) break;
     it = nx;
     b = bn;
@@ -1938,7 +2021,8 @@ __global__ void ACE_PASS_BOUNDS(PASS) batch_decode_kernel(BatchArgs ba) {
     fused_loop<false>(BatchJobs{ba, ba.by_level, ba.n_level}, ba.sh, ba.n_items, ba.timeout_ns, wsm, lane, epoch, ba.window);
     return;
   }
-  const BatchJobs jobs = ACE_PASS_CTA(PASS) ? BatchJobs{ba, ba.by_level, ba.n_level} : BatchJobs{ba, ba.by_size, ba.n_size};
+  const BatchJobs jobs = ACE_PASS_CTA(PASS) || PASS == PASS_WARP ? BatchJobs{ba, ba.by_level, ba.n_level}
+                                                                  : BatchJobs{ba, ba.by_size, ba.n_size};
   if (ACE_PASS_CTA(PASS)) {
     cta_blocks(ba.n_items, &ba.sh->ticket3, [&](uint32_t it) {
       uint32_t b;
@@ -1949,7 +2033,8 @@ __global__ void ACE_PASS_BOUNDS(PASS) batch_decode_kernel(BatchArgs ba) {
     });
     return;
   }
-  uint32_t* ticket = PASS == PASS_TOKENS ? &ba.sh->ticket : &ba.sh->ticket2;
+  uint32_t* ticket =
+      PASS == PASS_TOKENS ? &ba.sh->ticket : PASS == PASS_LITERALS ? &ba.sh->ticket2 : &ba.sh->ticket3;
   while (true) {
     uint32_t it = 0;
     if (lane == 0) it = atomicAdd(ticket, 1u);
@@ -1957,8 +2042,15 @@ __global__ void ACE_PASS_BOUNDS(PASS) batch_decode_kernel(BatchArgs ba) {
     if (it >= ba.n_items) break;
     uint32_t b;
     const DecodeArgs a = jobs.job(it, b);
-    if (PASS == PASS_TOKENS) token_block<false>(a, carve_tok(wsm), b, lane);
-    else literal_block<false, kRing>(a, carve_lit(wsm, ba.window, kRing), b, lane);
+    if (PASS == PASS_TOKENS) {
+      token_block<false>(a, carve_tok(wsm), b, lane);
+    } else if (PASS == PASS_WARP) {
+      const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
+      match_block<false, true, false, WAY_LANES>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch, ntok ? ntok - 1 : 0);
+      publish(a.ready, b, epoch, lane);
+    } else {
+      literal_block<false, kRing>(a, carve_lit(wsm, ba.window, kRing), b, lane);
+    }
   }
 }
 
@@ -2809,10 +2901,16 @@ struct Launch {
   uint32_t schedule;
   uint32_t long_min;       // the copy-width knob as the long class's shortest match
   uint32_t match_threads;  // threads of the match pass's CTAs, a block each
+  bool warp_match;         // ... or a block per warp (PASS_WARP)
 };
 
-constexpr double kCtaMatches = 400;
+// Archives of many matches ("dense"): their match pass goes by a CTA per block
+// wherever there are blocks enough to fill the GPU.
+constexpr double kCtaMatches = 400;  // matches per 16 KiB
 constexpr double kRowMatches = 48;
+inline bool dense_matches(uint64_t matches, uint64_t bytes) {
+  return (double)matches * 16384 >= kCtaMatches * (double)bytes;
+}
 constexpr uint32_t kCtaLevel = 4;
 // Calls of few blocks decode a stream per warp (entropy_kernel) and leave the
 // literals to the match pass, whose CTAs place them.  That shortens a block's
@@ -2832,10 +2930,6 @@ constexpr uint64_t kSplitSeek = 1024;
 // where the host has the requests, else by their number.
 constexpr uint64_t kSplitBatch = 3072;
 constexpr uint32_t kSplitReqs = 64;
-// Archive batches, by the bytes they give: uneven objects of 16 MB 391 us (576
-// in three passes), 57 MB 503 (781), 118 MB 804 (900), 124 MB 912 (929), 183
-// MB 1157 (1122), 364 MB 2312 (1676).
-constexpr uint64_t kSplitBatchBytes = 128ull << 20;
 
 template <class K>
 ace_status occupancy(K kernel, int device, uint32_t warps, size_t smem, int* occ) {
@@ -2861,7 +2955,8 @@ ace_status occupancy(K kernel, int device, uint32_t warps, size_t smem, int* occ
 // k3 is the fused pass
 template <class K0, class K1, class K2, class K3>
 ace_status plan_launch(const ace_index* idx, const ace_tune* tune, uint32_t log2B, uint64_t max_items,
-                       K0 k0, K1 k1, K2 k2, K3 k3, int* occ_cache, Launch* L, uint32_t lit_ring, bool few) {
+                       K0 k0, K1 k1, K2 k2, K3 k3, int* occ_cache, Launch* L, uint32_t lit_ring, bool few,
+                       bool warp_match) {
   ace_tune t = tune ? *tune : idx->tune;
   L->warps = t.warps_per_cta ? t.warps_per_cta : 4;
   L->chunk = t.chunk_tokens ? t.chunk_tokens : 128;
@@ -2878,8 +2973,10 @@ ace_status plan_launch(const ace_index* idx, const ace_tune* tune, uint32_t log2
   if (L->schedule == ACE_SCHEDULE_AUTO) L->schedule = ACE_SCHEDULE_PASSES;
   L->smem[PASS_TOKENS] = tok_smem_bytes(esc_cap(log2B));
   L->smem[PASS_LITERALS] = lit_smem_bytes(L->chunk, lit_ring);
-  L->match_threads = cta_threads(log2B, few);
-  L->smem[PASS_MATCH] = cta_smem_bytes(log2B, L->match_threads);  // per CTA; the other passes': per warp
+  L->warp_match = warp_match;
+  L->match_threads = warp_match ? 32 * L->warps : cta_threads(log2B, few);
+  // per CTA; the other passes': per warp
+  L->smem[PASS_MATCH] = warp_match ? L->warps * kMatchSmem : cta_smem_bytes(log2B, L->match_threads);
   L->smem[PASS_FUSED] = std::max(std::max(L->smem[PASS_TOKENS], L->smem[PASS_LITERALS]), kMatchSmem);
   int per[4];
   for (int p = 0; p < 4; p++) {
@@ -2898,8 +2995,9 @@ ace_status plan_launch(const ace_index* idx, const ace_tune* tune, uint32_t log2
   }
   uint64_t need = std::max<uint64_t>(1, (max_items + L->warps - 1) / L->warps);
   for (int p = 0; p < 4; p++) L->grid[p] = (uint32_t)std::min<uint64_t>((uint64_t)idx->num_sms * per[p], need);
-  L->grid[PASS_MATCH] =
-      (uint32_t)std::min<uint64_t>((uint64_t)idx->num_sms * per[PASS_MATCH], std::max<uint64_t>(1, max_items));
+  if (!warp_match)
+    L->grid[PASS_MATCH] =
+        (uint32_t)std::min<uint64_t>((uint64_t)idx->num_sms * per[PASS_MATCH], std::max<uint64_t>(1, max_items));
   return ACE_OK;
 }
 
@@ -2907,7 +3005,8 @@ template <bool SEEK>
 ace_status plan_index_launch(const ace_index* idx, const ace_tune* tune, uint64_t max_items, Launch* L) {
   return plan_launch(idx, tune, idx->h.log2_block, max_items, decode_kernel<SEEK, PASS_TOKENS>,
                      decode_kernel<SEEK, PASS_LITERALS>, decode_kernel<SEEK, PASS_MATCH>,
-                     decode_kernel<SEEK, PASS_FUSED>, &idx->occ_cache[SEEK][0][0][0], L, SEEK ? kSeekRing : kRing, SEEK);
+                     decode_kernel<SEEK, PASS_FUSED>, &idx->occ_cache[SEEK][0][0][0], L, SEEK ? kSeekRing : kRing, SEEK,
+                     false);
 }
 
 // Launches the passes in the mask (bit p: pass p) in order on s, each with
@@ -2924,6 +3023,7 @@ void launch_passes(const Launch& L, uint32_t passes, K0 k0, K1 k1, K2 k2, Args a
     k1<<<L.grid[1], th, (size_t)L.warps * L.smem[1], s>>>(a);
   }
   if (passes & 4) {
+    a.warp_smem = kMatchSmem;  // (a warp per block)
     k2<<<L.grid[2], L.match_threads, L.smem[2], s>>>(a);
   }
 }
@@ -3305,8 +3405,8 @@ ace_status decode_all_passes(const ace_index* idx, uint32_t passes, void* d_out,
   }
   // a warp per block by rounds, a warp per block by rows, a CTA per block:
   // by the archive's matches per 16 KiB
-  const double per16k = (double)idx->n_matches * 16384 / (double)idx->h.total_size;
-  const bool dense = per16k >= kCtaMatches, rows = per16k >= kRowMatches;
+  const bool dense = dense_matches(idx->n_matches, idx->h.total_size);
+  const bool rows = (double)idx->n_matches * 16384 >= kRowMatches * (double)idx->h.total_size;
   const bool light = dense || idx->h.archive_bytes < idx->h.total_size / 4;
   const bool split = passes == 7 && idx->by_levels &&
                      idx->h.n_blocks <= (uint64_t)(light ? kSplitBlocksLight : kSplitBlocks) * idx->num_sms;
@@ -3318,7 +3418,7 @@ ace_status decode_all_passes(const ace_index* idx, uint32_t passes, void* d_out,
     const ace_tune t = tune ? *tune : idx->tune;
     int &occ = idx->occ_level[L.warps], &occ_cta = idx->occ_level[0];
     const uint32_t log2B = idx->h.log2_block, few = cta_threads(log2B, true), many = cta_threads(log2B, false);
-    const auto level_kernel = rows ? match_level_kernel<true> : match_level_kernel<false>;
+    const auto level_kernel = rows ? match_level_kernel<WAY_ROWS> : match_level_kernel<WAY_ROUNDS>;
     if (occ == 0) {
       rc = occupancy(level_kernel, idx->device, L.warps, (size_t)L.warps * kMatchSmem, &occ);
       if (rc) return rc;
@@ -3543,7 +3643,7 @@ struct ace_batch {
   uint64_t lv_done_off, lv_done_bytes;  // the fused schedule's level counters
   BatchArgs args;
   Launch L;
-  bool split;             // the entropy layer a stream per warp
+  bool split;             // the entropy layer a stream per warp, literals placed by the match CTAs
   uint32_t entropy_grid;
   int occ[4][9][9];
 };
@@ -3551,19 +3651,66 @@ struct ace_batch {
 namespace {
 
 struct BatchLayout {
-  uint64_t objs, by_size, by_level, ready, lv_done, lv_done_bytes, recs, total, max_ntok, items, n_matches, bytes;
+  uint64_t objs, by_size, by_level, ready, lv_done, lv_done_bytes, recs, total, max_ntok, items;
   uint32_t max_log2B;
+  bool split, warp_match;  // the way its passes take (batch_route)
 };
+
+// A batch's entropy layer goes a block per warp (two passes) or a stream per
+// warp (one launch, split), and its match pass a CTA or a warp per block.
+//
+// Match pass.  A CTA sweeps all of its block's bytes, which pays for dense
+// archives alone: 115 MB of text in 16 KiB blocks 0.71 ms by CTAs and 1.02 by
+// warps, in 4 KiB blocks 1.05 and 1.00; FASTQ 0.40 and 0.32, 0.74 and 0.45;
+// genome 0.35 and 0.31, 0.61 and 0.37.  A 64 KiB text block is 1 ms of a warp
+// whatever else there is, so warps take over only where hardly anything is dense
+// (by those costs, a sixth of the bytes) and no dense block is large.
+//
+// Entropy layer.  Split, a block takes as long as its longest stream, where the
+// passes add its streams up; but it costs more per block, in the match CTAs above
+// all, which then place the literals.  For dense archives both are estimated: the
+// longest block's chain (about 8 and 2.3 ns a byte) or the sum of the work (3 us
+// a MB, 2 where matches are few), the larger of the two, plus a second launch or
+// 17 ns a block (6 where matches are few; less in proportion below 2 KiB).  Text,
+// us split (passes): 4 MB in 4 KiB blocks 72 (104), 16 KiB 85 (170), 64 KiB 250
+// (549); 36 MB 500 (360), 269 (279), 348 (622); 115 MB 1670 (1054), 844 (710),
+// 783 (910).  Uneven objects of all profiles: 57 MB 503 (781), 118 MB 804 (900),
+// 183 MB 1157 (1122).  Without dense archives only few blocks are worth it: FASTQ,
+// 4 MB in 8 KiB blocks 70 (79), 16 KiB 101 (116), 64 KiB 380 (342); genome 70
+// (68), 97 (101), 285 (291); 36 MB in 16 KiB blocks 210 (147) and 177 (162).
+constexpr uint32_t kSplitBatchSparse = 4;  // blocks per SM
+constexpr uint32_t kSplitSparseLog2B = 15;
+
+void batch_route(const ace_index* const* idx, uint32_t n, BatchLayout* B) {
+  double bytes = 0, dense_bytes = 0, chain = 0, per_block = 0;
+  for (uint32_t i = 0; i < n; i++) {
+    const ace_index& x = *idx[i];
+    const double total = (double)x.h.total_size, block = std::min(total, (double)(1ull << x.h.log2_block));
+    const bool dense = x.h.total_size && dense_matches(x.n_matches, x.h.total_size);
+    bytes += total;
+    per_block += (double)x.h.n_blocks * std::min(1.0, block / 2048) * (dense ? 17e-3 : 6e-3);
+    if (dense) {
+      dense_bytes += total;
+      chain = std::max(chain, block);
+    }
+  }
+  const double work = (2 * bytes + dense_bytes) * 1e-6;  // us
+  B->warp_match = dense_bytes * 6 <= bytes && chain <= 8192;
+  if (B->warp_match)
+    B->split = B->items <= (uint64_t)kSplitBatchSparse * idx[0]->num_sms && B->max_log2B <= kSplitSparseLog2B;
+  else
+    B->split = std::max(2.3e-3 * chain, work) + per_block < std::max(8e-3 * chain, work) + 25;
+  if (B->split) B->warp_match = false;
+}
 
 ace_status batch_layout(const ace_index* const* idx, uint32_t n, BatchLayout* B) {
   if (!idx || n == 0) return ACE_E_INVAL;
-  uint64_t ready = 0, items = 0, max_ntok = 0, matches = 0, levels = 0, segs = 0, bytes = 0;
+  uint64_t ready = 0, items = 0, max_ntok = 0, matches = 0, levels = 0, segs = 0;
   uint32_t max_log2B = 0;
   int dev = idx[0] ? idx[0]->device : -1;
   for (uint32_t i = 0; i < n; i++) {
     if (!idx[i] || idx[i]->device != dev) return ACE_E_INVAL;
     items += idx[i]->h.n_blocks;
-    bytes += idx[i]->h.total_size;
     ready += align256(4 * idx[i]->h.n_blocks);
     matches += idx[i]->n_matches;
     levels += idx[i]->n_levels;
@@ -3587,11 +3734,10 @@ ace_status batch_layout(const ace_index* const* idx, uint32_t n, BatchLayout* B)
   B->recs = o;
   o = align256(o + 16 * matches);
   B->total = o;
-  B->n_matches = matches;
-  B->bytes = bytes;
   B->max_ntok = max_ntok;
   B->items = items;
   B->max_log2B = max_log2B;
+  batch_route(idx, n, B);
   return ACE_OK;
 }
 
@@ -3674,8 +3820,9 @@ ace_status ace_batch_create(const ace_index* const* idx, uint32_t n, void* const
   b->lv_done_bytes = B.lv_done_bytes;
   // the launch shape uses the largest block size's escape table
   rc = plan_launch(idx[0], tune, B.max_log2B, B.items, batch_decode_kernel<PASS_TOKENS>,
-                   batch_decode_kernel<PASS_LITERALS>, batch_decode_kernel<PASS_MATCH>,
-                   batch_decode_kernel<PASS_FUSED>, &b->occ[0][0][0], &b->L, kRing, false);
+                   batch_decode_kernel<PASS_LITERALS>,
+                   B.warp_match ? batch_decode_kernel<PASS_WARP> : batch_decode_kernel<PASS_MATCH>,
+                   batch_decode_kernel<PASS_FUSED>, &b->occ[0][0][0], &b->L, kRing, false, B.warp_match);
   if (rc == ACE_OK &&
       (cudaMemsetAsync(base, 0, B.recs, s) != cudaSuccess ||
        cudaMemcpyAsync(base + B.objs, od.data(), n * sizeof(ObjDesc), cudaMemcpyHostToDevice, s) != cudaSuccess ||
@@ -3691,7 +3838,7 @@ ace_status ace_batch_create(const ace_index* const* idx, uint32_t n, void* const
   }
   BatchArgs& a = b->args;
   a.objs = reinterpret_cast<const ObjDesc*>(base + B.objs);
-  b->split = B.bytes <= kSplitBatchBytes;
+  b->split = B.split;
   b->entropy_grid = (uint32_t)std::min<uint64_t>((3 * B.items + 3) / 4, 8ull * idx[0]->num_sms);
   a.by_size = reinterpret_cast<const BatchSeg*>(base + B.by_size);
   a.by_level = reinterpret_cast<const BatchSeg*>(base + B.by_level);
@@ -3723,7 +3870,7 @@ ace_status ace_decode_batch(const ace_batch* b, cudaStream_t s) {
     batch_decode_kernel<PASS_PLACE><<<L.grid[PASS_MATCH], L.match_threads, L.smem[PASS_MATCH], s>>>(b->args);
   } else
     launch_passes(L, 7, batch_decode_kernel<PASS_TOKENS>, batch_decode_kernel<PASS_LITERALS>,
-                  batch_decode_kernel<PASS_MATCH>, b->args, s);
+                  L.warp_match ? batch_decode_kernel<PASS_WARP> : batch_decode_kernel<PASS_MATCH>, b->args, s);
   CUDA_TRY(cudaGetLastError());
   return ACE_OK;
 }
@@ -3898,7 +4045,7 @@ ace_status ace_cache_create(const ace_index* const* idx, uint32_t n, void* const
   // not level order); the fused entry only sizes like the match pass
   rc = plan_launch(idx[0], tune, log2B, C.max_work, cache_decode_kernel<PASS_TOKENS>,
                    cache_decode_kernel<PASS_LITERALS>, cache_decode_kernel<PASS_MATCH>,
-                   cache_decode_kernel<PASS_MATCH>, &c->occ[0][0][0], &c->L, kSeekRing, true);
+                   cache_decode_kernel<PASS_MATCH>, &c->occ[0][0][0], &c->L, kSeekRing, true, false);
   // header (epoch 1: no block is cached, since every ready flag starts at 0)
   CacheHdr h{};
   h.epoch = 1;

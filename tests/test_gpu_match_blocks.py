@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 
 import oracle
+import synth
 import __graft_entry__
 
 torch = pytest.importorskip("torch")
@@ -16,6 +17,7 @@ from paper_2606_24531_gb300 import ace  # noqa: E402
 from paper_2606_24531_gb300.archive import DeviceArchive  # noqa: E402
 from paper_2606_24531_gb300.batch import DeviceBatch  # noqa: E402
 from paper_2606_24531_gb300.serve import SeekCache  # noqa: E402
+from conftest import with_dep_removed  # noqa: E402
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -152,3 +154,34 @@ def test_batches_of_either_size():
             for c in {0, copies // 2, copies - 1}:
                 assert torch.equal(db.output(c * len(datas) + k), want)
         db.close()
+
+
+@pytest.mark.parametrize("profile, log2b, size", [
+    ("genome", 8, 300_000), ("fastq", 12, 900_000), ("genome", 16, 3_600_001),  # many blocks, few matches: a warp per block
+    ("fastq", 15, 150_000), ("genome", 9, 20_001),                              # few blocks: a warp per stream
+    ("text", 10, 700_000), ("mixed", 13, 2_400_000),                            # many blocks of many matches: a CTA per block
+    ("text", 16, 900_000), ("mixed", 12, 90_000)])                              # few blocks: a warp per stream
+def test_batch_routes(profile, log2b, size):
+    """Every way a batch's passes take, on objects of one profile, and the same
+    batch again (its epoch moved on)."""
+    datas = [synth.generate(profile, size - 1009 * k, 31 * k + log2b) for k in range(12)]
+    mm = {"genome": 20, "fastq": 16}.get(profile, 4)
+    arcs = [ace.ace_encode_gpu(torch.from_numpy(d).cuda(), log2b, mm).cpu().numpy() for d in datas]
+    db = DeviceBatch(arcs)
+    for _ in range(2):
+        db.out.zero_()
+        db.decode()
+        assert db.sync() == ace.ACE_OK
+        for k, d in enumerate(datas):
+            assert torch.equal(db.output(k), torch.from_numpy(d).cuda())
+    db.close()
+
+
+def test_batch_by_warps_reports_a_source_outside_its_levels():
+    data = synth.generate("genome", 2_500_000, 3)
+    arc = ace.ace_encode(data, 12, 20)
+    bad = with_dep_removed(arc, int(np.nonzero(oracle.levels(arc) == 2)[0][-1]))  # it reads a block of level 1
+    db = DeviceBatch([arc, bad])
+    db.decode()
+    assert db.sync() == ace.ACE_E_CORRUPT
+    db.close()
