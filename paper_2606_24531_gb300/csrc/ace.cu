@@ -1833,7 +1833,7 @@ __global__ void ACE_PASS_BOUNDS(PASS) decode_kernel(DecodeArgs a) {
     });
     return;
   }
-  uint32_t* ticket = PASS == PASS_TOKENS ? &a.sh->ticket : &a.sh->ticket2;
+  uint32_t* ticket = PASS == PASS_TOKENS ? &a.sh->ticket : PASS == PASS_LITERALS ? &a.sh->ticket2 : &a.sh->ticket3;
   while (true) {
     uint32_t it = 0;
     if (lane == 0) it = atomicAdd(ticket, 1u);
@@ -1842,6 +1842,12 @@ __global__ void ACE_PASS_BOUNDS(PASS) decode_kernel(DecodeArgs a) {
     uint32_t b = __ldg(a.items + it);
     if (PASS == PASS_TOKENS) {
       token_block<SEEK>(a, carve_tok(wsm), b, lane);
+      continue;
+    }
+    if (PASS == PASS_WARP) {
+      const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
+      match_block<SEEK, true, false, WAY_ROWS>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch, ntok ? ntok - 1 : 0);
+      publish(a.ready, b, epoch, lane);
       continue;
     }
     constexpr uint32_t ring = SEEK ? kSeekRing : kRing;
@@ -2931,6 +2937,16 @@ constexpr uint64_t kSplitSeek = 1024;
 constexpr uint64_t kSplitBatch = 3072;
 constexpr uint32_t kSplitReqs = 64;
 
+// Archives of more than 32 levels: the match pass by warps, where a block is
+// short or has few matches.  600 KB written with the most recent sources first,
+// us by CTAs (warps by rows): text in 256-byte blocks 4811 (3657), 1 KiB 3669
+// (6201), 16 KiB 1270 (5749); FASTQ in 1 KiB blocks 239 (202), 4 KiB 469 (390), 8
+// KiB 417 (427), 16 KiB 315 (468).
+inline bool deep_by_warps(const ace_index* x) {
+  const bool dense = x->h.total_size && dense_matches(x->n_matches, x->h.total_size);
+  return !x->by_levels && (x->h.log2_block < 9 || (!dense && x->h.log2_block < 13));
+}
+
 template <class K>
 ace_status occupancy(K kernel, int device, uint32_t warps, size_t smem, int* occ) {
   int optin = 0;
@@ -3003,10 +3019,12 @@ ace_status plan_launch(const ace_index* idx, const ace_tune* tune, uint32_t log2
 
 template <bool SEEK>
 ace_status plan_index_launch(const ace_index* idx, const ace_tune* tune, uint64_t max_items, Launch* L) {
+  const bool warps = !SEEK && deep_by_warps(idx);
   return plan_launch(idx, tune, idx->h.log2_block, max_items, decode_kernel<SEEK, PASS_TOKENS>,
-                     decode_kernel<SEEK, PASS_LITERALS>, decode_kernel<SEEK, PASS_MATCH>,
+                     decode_kernel<SEEK, PASS_LITERALS>,
+                     warps ? decode_kernel<false, PASS_WARP> : decode_kernel<SEEK, PASS_MATCH>,
                      decode_kernel<SEEK, PASS_FUSED>, &idx->occ_cache[SEEK][0][0][0], L, SEEK ? kSeekRing : kRing, SEEK,
-                     false);
+                     warps);
 }
 
 // Launches the passes in the mask (bit p: pass p) in order on s, each with
@@ -3413,7 +3431,8 @@ ace_status decode_all_passes(const ace_index* idx, uint32_t passes, void* d_out,
   if (split) entropy_kernel<false><<<3 * a.n_items, 32, job_smem_bytes(a.esc_cap, kSeekRing), s>>>(a);  // (needs no ticket or epoch)
   else if (passes & 1) begin_call_kernel<<<1, 1, 0, s>>>(sh);
   launch_passes(L, split ? 0u : passes & (idx->by_levels ? 3u : 7u), decode_kernel<false, PASS_TOKENS>,
-                decode_kernel<false, PASS_LITERALS>, decode_kernel<false, PASS_MATCH>, a, s);
+                decode_kernel<false, PASS_LITERALS>,
+                L.warp_match ? decode_kernel<false, PASS_WARP> : decode_kernel<false, PASS_MATCH>, a, s);
   if ((passes & 4) && idx->by_levels) {
     const ace_tune t = tune ? *tune : idx->tune;
     int &occ = idx->occ_level[L.warps], &occ_cta = idx->occ_level[0];

@@ -185,3 +185,22 @@ def test_batch_by_warps_reports_a_source_outside_its_levels():
     db.decode()
     assert db.sync() == ace.ACE_E_CORRUPT
     db.close()
+
+
+@pytest.mark.parametrize("profile, log2b, size", [("text", 8, 120_000), ("fastq", 10, 700_000), ("fastq", 13, 500_000),
+                                                  ("fastq", 14, 700_000), ("mixed", 9, 60_000)])
+def test_whole_decodes_of_many_levels(profile, log2b, size):
+    """Archives of more than 32 levels (the oracle takes the most recent
+    sources), by warps and by CTAs waiting on one another's blocks; a block
+    that reads past its levels is reported."""
+    data = synth.generate(profile, size, 17 * log2b)
+    arc = oracle.encode(data, log2b, {"fastq": 16}.get(profile, 4), 16)
+    da = DeviceArchive(arc)
+    assert da.info["n_levels"] > 32
+    for _ in range(2):
+        _check(da, data)
+    bad = DeviceArchive(with_dep_removed(arc, int(np.argmax(oracle.levels(arc)))))
+    bad.decode_all()
+    assert bad.sync() == ace.ACE_E_CORRUPT
+    da.close()
+    bad.close()
