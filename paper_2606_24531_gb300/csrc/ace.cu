@@ -1274,6 +1274,15 @@ constexpr uint32_t kCtaLong = 256;                          // shortest run of k
 __host__ __device__ inline uint32_t cta_threads(uint32_t log2B, bool few) {
   return log2B >= 12 ? few ? 512 : 256 : log2B >= 10 ? 128 : 64;
 }
+// ... where they are many and dense: a thread to 64 bytes.  48 MiB of text (with
+// no match below 12 bytes), match pass, us by 32, 64, 128, 256 threads: 1 KiB
+// blocks 142, 167, 225 (110, 137, 205); 2 KiB 144, 157, 173 (115, 117, 146); 4 KiB
+// 186, 155, 156, 178 (148, 124, 123, 156); 8 KiB 318, 193, 155, 160; 16 KiB 589,
+// 329, 202, 162.  256 threads had been 178 (156) where a warp per block took 176
+// (125).
+__host__ __device__ inline uint32_t dense_threads(uint32_t log2B) {
+  return log2B >= 14 ? 256 : log2B > 11 ? 1u << (log2B - 6) : 32;
+}
 // (enough for smaller blocks of the same launch too)
 __host__ __device__ inline uint32_t cta_smem_bytes(uint32_t log2B, uint32_t threads) {
   return 2 * (log2B >= 14 ? kCtaWindow : 1u << log2B) + threads / 32 * kCtaWarpSmem;
@@ -2910,13 +2919,30 @@ struct Launch {
   bool warp_match;         // ... or a block per warp (PASS_WARP)
 };
 
-// Archives of many matches ("dense"): their match pass goes by a CTA per block
-// wherever there are blocks enough to fill the GPU.
-constexpr double kCtaMatches = 400;  // matches per 16 KiB
+// The match pass of a level of many blocks, by the archive's matches per 16 KiB.
+// Dense archives, in blocks of at least 512 bytes: a CTA per block.  It costs a
+// sweep over the block whatever the matches, a warp's rows cost by the match.
+// Match pass of 48 MiB of text with ever fewer matches, us by CTAs (rows): 4 KiB
+// blocks 155 (245) at 774, 124 (156) at 512, 110 (108) at 349; 1 KiB 142 (185) at
+// 647, 110 (120) at 442, 91 (84) at 293; 512 bytes 147 (180) at 576, 130 (126) at
+// 401; 256 bytes 392 (203) at 505.  In larger blocks CTAs are ahead from fewer on
+// (128 MiB of spread copies, 16 KiB blocks: 210 (261) at 349, 151 (147) at 190);
+// one line for all keeps FASTQ, 100 to 220, with the rows that suit 16 KiB blocks.
+constexpr double kCtaMatches = 400;
+constexpr uint32_t kCtaLog2B = 9;
+// Others go by warps: in rows, unless matches are few and, by the archive's size,
+// long.  128 MiB, us by rows (rounds): genome (18 matches per 16 KiB, of 880 bytes)
+// 126 (109) in 16 KiB blocks, 79 (74) in 4 KiB; copies of 32 bytes at 41 per 16
+// KiB 52 (85) and 36 (48), in 64 KiB blocks 99 (197); of 17 bytes at 20 in 64 KiB
+// blocks 62 (81); of 490 at 16 68 (70), 42 (40); FASTQ 128 (177), 82 (100).
 constexpr double kRowMatches = 48;
 inline bool dense_matches(uint64_t matches, uint64_t bytes) {
   return (double)matches * 16384 >= kCtaMatches * (double)bytes;
 }
+// Levels of at most this many blocks per SM: a CTA per block whatever the archive.
+// Match pass, us by CTAs (warps) at 2, 4, 6 and 12 blocks per SM: genome in 16 KiB
+// blocks 52 (74), 60 (62), 68 (60), 101 (102); FASTQ 40 (52), 46 (53), 53 (52), 70
+// (54); genome in 64 KiB blocks 122 (124), 126 (124), 144 (140), 267 (148).
 constexpr uint32_t kCtaLevel = 4;
 // Calls of few blocks decode a stream per warp (entropy_kernel) and leave the
 // literals to the match pass, whose CTAs place them.  That shortens a block's
@@ -2928,6 +2954,17 @@ constexpr uint32_t kCtaLevel = 4;
 // MiB 304 (496).
 constexpr uint32_t kSplitBlocks = 1;       // whole decodes, blocks per SM
 constexpr uint32_t kSplitBlocksLight = 8;  // ... of archives with many matches or few compressed bytes (few literals)
+// ... in blocks up to this: where literals are many, placing those of a large
+// block takes its CTA longer than the shorter chain saves.  FASTQ in 64 KiB
+// blocks: 1.5 MiB 339 (308), 9 MiB 528 (386), 600 KB in 10 levels 1117 (464); in
+// 32 KiB blocks 1.5 MiB 154 (170), 19 levels 695 (355).
+constexpr uint32_t kSplitLog2B = 14;
+// ... of at most this many levels, unless dense and in blocks of 4 KiB or more:
+// placing the literals is a part of every level's time.  26 blocks written with
+// the most recent sources first, us split (passes): FASTQ in 16 KiB blocks, 26
+// levels, 392 (273), 4 KiB, 21 levels, 201 (175); mixed data in 1 KiB blocks, 27
+// levels, 236 (208), in 4 KiB blocks 249 (279).
+constexpr uint32_t kSplitLevels = 8;
 // Seeks, by target blocks: FASTQ 1 block 154 (179), 1024 259 (275), 2048 366
 // (350); text 239 (326), 402 (476), 591 (639), 4096 1048 (986); genome 119
 // (122), 195 (203), 272 (272).
@@ -3424,9 +3461,12 @@ ace_status decode_all_passes(const ace_index* idx, uint32_t passes, void* d_out,
   // a warp per block by rounds, a warp per block by rows, a CTA per block:
   // by the archive's matches per 16 KiB
   const bool dense = dense_matches(idx->n_matches, idx->h.total_size);
-  const bool rows = (double)idx->n_matches * 16384 >= kRowMatches * (double)idx->h.total_size;
+  const bool by_cta = dense && idx->h.log2_block >= kCtaLog2B;
+  const bool rows = (double)idx->n_matches * 16384 >= kRowMatches * (double)idx->h.total_size ||
+                    idx->h.archive_bytes >= idx->h.total_size / 2;
   const bool light = dense || idx->h.archive_bytes < idx->h.total_size / 4;
-  const bool split = passes == 7 && idx->by_levels &&
+  const bool split = passes == 7 && idx->by_levels && (light || idx->h.log2_block <= kSplitLog2B) &&
+                     (idx->n_levels <= kSplitLevels || (dense && idx->h.log2_block >= 12)) &&
                      idx->h.n_blocks <= (uint64_t)(light ? kSplitBlocksLight : kSplitBlocks) * idx->num_sms;
   if (split) entropy_kernel<false><<<3 * a.n_items, 32, job_smem_bytes(a.esc_cap, kSeekRing), s>>>(a);  // (needs no ticket or epoch)
   else if (passes & 1) begin_call_kernel<<<1, 1, 0, s>>>(sh);
@@ -3436,7 +3476,7 @@ ace_status decode_all_passes(const ace_index* idx, uint32_t passes, void* d_out,
   if ((passes & 4) && idx->by_levels) {
     const ace_tune t = tune ? *tune : idx->tune;
     int &occ = idx->occ_level[L.warps], &occ_cta = idx->occ_level[0];
-    const uint32_t log2B = idx->h.log2_block, few = cta_threads(log2B, true), many = cta_threads(log2B, false);
+    const uint32_t log2B = idx->h.log2_block, few = cta_threads(log2B, true), many = dense_threads(log2B);
     const auto level_kernel = rows ? match_level_kernel<WAY_ROWS> : match_level_kernel<WAY_ROUNDS>;
     if (occ == 0) {
       rc = occupancy(level_kernel, idx->device, L.warps, (size_t)L.warps * kMatchSmem, &occ);
@@ -3463,7 +3503,7 @@ ace_status decode_all_passes(const ace_index* idx, uint32_t passes, void* d_out,
         (split ? match_cta_kernel<512, true> : match_cta_kernel<512, false>)<<<n, few, cta_smem_bytes(log2B, few), s>>>(a);
         continue;
       }
-      if (dense) {
+      if (by_cta) {
         match_cta_kernel<256, false><<<(uint32_t)std::min<uint64_t>(sms(occ_cta), n), many, cta_smem_bytes(log2B, many), s>>>(a);
         continue;
       }

@@ -204,3 +204,21 @@ def test_whole_decodes_of_many_levels(profile, log2b, size):
     assert bad.sync() == ace.ACE_E_CORRUPT
     da.close()
     bad.close()
+
+
+@pytest.mark.parametrize("profile, mm", [("text", 4), ("text", 12), ("fastq", 16), ("genome", 20)])
+@pytest.mark.parametrize("log2b", [8, 9, 10, 11, 12, 13, 14, 15, 16])
+def test_levels_of_many_blocks_at_every_size(profile, mm, log2b):
+    """More than four blocks per SM in a level where the size allows it: a CTA of
+    32 to 256 threads per dense block, rows, rounds; and few blocks, in few levels
+    and in many, with and without a warp per stream."""
+    n = min(5000 << log2b, 24 << 20) - 7
+    data = synth.generate(profile, n, log2b)
+    da = DeviceArchive(ace.ace_encode_gpu(torch.from_numpy(data).cuda(), log2b, mm).cpu().numpy())
+    _check(da, data)
+    da.close()
+    small = data[:26 << log2b]
+    for arc in (ace.ace_encode(small, log2b, mm), oracle.encode(small, log2b, mm, 16)):
+        da = DeviceArchive(arc)
+        _check(da, small)
+        da.close()
