@@ -1674,6 +1674,14 @@ __device__ __forceinline__ uint32_t level_size(const DecodeArgs& a, uint32_t l) 
   return __ldg(a.lv_count + l);
 }
 
+// The part of a seek's block inside [coord, coord + len) to the caller, by a warp.
+__device__ __forceinline__ void slice_part(const DecodeArgs& a, uint32_t b, uint32_t lane) {
+  const uint64_t bs = (uint64_t)b << a.log2B, be = min(bs + ((uint64_t)1 << a.log2B), a.total);
+  const uint64_t lo = max(bs, a.coord), hi = min(be, a.coord + a.len);
+  const uint8_t* src = a.out + slot_base(a, b) - bs;
+  if (hi > lo) warp_copy(a.slice + (lo - a.coord), src + lo, hi - lo, lane);
+}
+
 // The work of one archive (whole decode or seek): its list, in level order.
 template <bool SEEK>
 struct ArchiveJobs {
@@ -1760,12 +1768,7 @@ __device__ void fused_loop(const Jobs& jobs, ScratchHdr* sh, uint32_t n_items, u
           // not wait
           ok = match_block<true, true, true, WAY_ROWS>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch,
                                              ntok ? ntok - 1 : 0);
-          if (ok && a.slice) {
-            uint64_t bs = (uint64_t)b << a.log2B, be = min(bs + ((uint64_t)1 << a.log2B), a.total);
-            uint64_t lo = max(bs, a.coord), hi = min(be, a.coord + a.len);
-            const uint8_t* src = a.out + slot_base(a, b) - bs;
-            if (hi > lo) warp_copy(a.slice + (lo - a.coord), src + lo, hi - lo, lane);
-          }
+          if (ok && a.slice) slice_part(a, b, lane);
           if (ok) publish(a.ready, b, epoch, lane);
         } else {
           ok = match_block<false, false, true, WAY_ROWS>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch,
@@ -1855,7 +1858,9 @@ __global__ void ACE_PASS_BOUNDS(PASS) decode_kernel(DecodeArgs a) {
     }
     if (PASS == PASS_WARP) {
       const uint32_t ntok = __ldg(reinterpret_cast<const uint32_t*>(a.dir + b) + 12);
-      match_block<SEEK, true, false, WAY_ROWS>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch, ntok ? ntok - 1 : 0);
+      const bool ok = match_block<SEEK, true, false, WAY_ROWS>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch,
+                                                               ntok ? ntok - 1 : 0);
+      if (SEEK && ok && a.slice) slice_part(a, b, lane);
       publish(a.ready, b, epoch, lane);
       continue;
     }
@@ -2965,10 +2970,17 @@ constexpr uint32_t kSplitLog2B = 14;
 // levels, 392 (273), 4 KiB, 21 levels, 201 (175); mixed data in 1 KiB blocks, 27
 // levels, 236 (208), in 4 KiB blocks 249 (279).
 constexpr uint32_t kSplitLevels = 8;
-// Seeks, by target blocks: FASTQ 1 block 154 (179), 1024 259 (275), 2048 366
-// (350); text 239 (326), 402 (476), 591 (639), 4096 1048 (986); genome 119
-// (122), 195 (203), 272 (272).
+// Seeks decode a stream per warp too: dense archives, and others in blocks up to
+// kSplitLog2B unless few blocks of few matches are wanted (one long stream each,
+// no shorter alone).  Us (in two passes): FASTQ in 64 KiB blocks 1 byte 375 (312),
+// 7 MiB 515 (400); genome in 4 KiB blocks 1 block 59 (50), 51 blocks 58 (57), 257
+// blocks 76 (79), in 16 KiB blocks 1 block 102 (97), 65 blocks 111 (118), in 1 KiB
+// blocks 1 block 48 (48), 17 blocks 46 (49).  By target blocks: FASTQ 1 block 154
+// (179), 1024 259 (275), 2048 366 (350); text 239 (326), 402 (476), 591 (639),
+// 4096 1048 (986); genome 119 (122), 195 (203), 272 (272).
 constexpr uint64_t kSplitSeek = 1024;
+constexpr uint64_t kSplitFew = 48;
+constexpr uint32_t kSplitFewLog2B = 12;
 // Seek batches, by target blocks (1900 over four profiles: 301 us against 371)
 // where the host has the requests, else by their number.
 constexpr uint64_t kSplitBatch = 3072;
@@ -3056,10 +3068,10 @@ ace_status plan_launch(const ace_index* idx, const ace_tune* tune, uint32_t log2
 
 template <bool SEEK>
 ace_status plan_index_launch(const ace_index* idx, const ace_tune* tune, uint64_t max_items, Launch* L) {
-  const bool warps = !SEEK && deep_by_warps(idx);
+  const bool warps = deep_by_warps(idx);
   return plan_launch(idx, tune, idx->h.log2_block, max_items, decode_kernel<SEEK, PASS_TOKENS>,
                      decode_kernel<SEEK, PASS_LITERALS>,
-                     warps ? decode_kernel<false, PASS_WARP> : decode_kernel<SEEK, PASS_MATCH>,
+                     warps ? decode_kernel<SEEK, PASS_WARP> : decode_kernel<SEEK, PASS_MATCH>,
                      decode_kernel<SEEK, PASS_FUSED>, &idx->occ_cache[SEEK][0][0][0], L, SEEK ? kSeekRing : kRing, SEEK,
                      warps);
 }
@@ -3090,29 +3102,28 @@ void launch_fused(const Launch& L, K3 k3, Args a, cudaStream_t s) {
   k3<<<L.grid[PASS_FUSED], 32 * L.warps, (size_t)L.warps * L.smem[PASS_FUSED], s>>>(a);
 }
 
-template <bool SEEK>
-void launch_three_pass(const Launch& L, const DecodeArgs& a, cudaStream_t s) {
-  launch_passes(L, 7, decode_kernel<SEEK, PASS_TOKENS>, decode_kernel<SEEK, PASS_LITERALS>,
-                decode_kernel<SEEK, PASS_MATCH>, a, s);
-}
-
-// A seek after its closure kernel, over the level-ordered work list: by
-// default one fused launch (each warp decodes a block through both layers,
-// waiting, bounded, only on pending members of the closure); with the pass
-// schedule, tokens and literals over the list, then one match launch that
-// waits the same way.  (One launch per level, as whole decodes by passes do,
-// is slower for a seek's hundred-odd blocks.)
-ace_status launch_seek(const ace_index* idx, const Launch& L, const DecodeArgs& a, uint64_t targets, cudaStream_t s) {
+// A seek after its closure kernel, over the level-ordered work list: by the pass
+// schedule (the automatic choice) the entropy layer a stream per warp or in two
+// passes over the list, then one match launch whose blocks wait, bounded, on
+// pending members of the closure; or one fused launch that waits the same way.
+// (One launch per level, as whole decodes by passes do, is slower for a seek's
+// hundred-odd blocks.)
+void launch_seek(const ace_index* idx, const Launch& L, const DecodeArgs& a, uint64_t targets, cudaStream_t s) {
+  const bool dense = dense_matches(idx->n_matches, idx->h.total_size);
+  const bool few = (double)idx->n_matches * 16384 < kRowMatches * (double)idx->h.total_size;
+  const bool split = targets <= kSplitSeek && !L.warp_match &&
+                     (dense || (idx->h.log2_block <= kSplitLog2B &&
+                                (!few || idx->h.log2_block < kSplitFewLog2B || targets > kSplitFew)));
   if (L.schedule == ACE_SCHEDULE_FUSED) {
     launch_fused(L, decode_kernel<true, PASS_FUSED>, a, s);
-  } else if (targets <= kSplitSeek) {
+  } else if (split) {
     const uint32_t grid = (uint32_t)std::min<uint64_t>(3ull * a.n_slots, 16ull * idx->num_sms);
     entropy_kernel<true><<<grid, 32, job_smem_bytes(a.esc_cap, kSeekRing), s>>>(a);
     decode_kernel<true, PASS_PLACE><<<L.grid[PASS_MATCH], L.match_threads, L.smem[PASS_MATCH], s>>>(a);
   } else {
-    launch_three_pass<true>(L, a, s);
+    launch_passes(L, 7, decode_kernel<true, PASS_TOKENS>, decode_kernel<true, PASS_LITERALS>,
+                  L.warp_match ? decode_kernel<true, PASS_WARP> : decode_kernel<true, PASS_MATCH>, a, s);
   }
-  return ACE_OK;
 }
 
 }  // namespace
@@ -3597,8 +3608,7 @@ ace_status ace_seek(const ace_index* idx, uint64_t coord, uint64_t len, void* d_
   a.closure_flags = true;
   a.long_min = L.long_min;
   a.lv_done = c.lv_done;
-  rc = launch_seek(idx, L, a, last - first + 1, s);
-  if (rc) return rc;
+  launch_seek(idx, L, a, last - first + 1, s);
   CUDA_TRY(cudaGetLastError());
   return ACE_OK;
 }
@@ -4381,8 +4391,7 @@ ace_status ace_seek_noalloc(const ace_index* idx, uint64_t coord, uint64_t len, 
   a.closure_flags = true;
   a.long_min = L.long_min;
   a.lv_done = c.lv_done;
-  rc = launch_seek(idx, L, a, last - first + 1, s);
-  if (rc) return rc;
+  launch_seek(idx, L, a, last - first + 1, s);
   CUDA_TRY(cudaGetLastError());
   // the status lives in the shared array, so the call waits for it
   uint32_t status = 0;
