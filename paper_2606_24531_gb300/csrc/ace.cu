@@ -1624,10 +1624,13 @@ __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32
 enum { PASS_TOKENS = 0, PASS_LITERALS = 1, PASS_MATCH = 2, PASS_FUSED = 3, PASS_PLACE = 4, PASS_WARP = 5 };
 
 // A pass is held to 64 registers a thread: 256 threads, or the match pass's
-// CTAs of up to 512; the match pass by warps to 80.
+// CTAs of up to 512; the match pass by warps and the fused pass to 80.  (Fused, us
+// at 80, at 64 with its spills: FASTQ 256 MiB 766, 806, text 64 MiB 831, 826,
+// mixed data in 4 KiB blocks 264, 297; with rows of match bytes instead of lanes
+// 811, 795, 308 at 80 and 926, 1080, 390 at 64.)
 #define ACE_PASS_CTA(P) ((P) == PASS_MATCH || (P) == PASS_PLACE)
 #define ACE_PASS_BOUNDS(P) \
-  __launch_bounds__(ACE_PASS_CTA(P) ? kCtaThreads : 256, ACE_PASS_CTA(P) ? 2 : (P) == PASS_WARP ? 3 : 4)
+  __launch_bounds__(ACE_PASS_CTA(P) ? kCtaThreads : 256, ACE_PASS_CTA(P) ? 2 : (P) == PASS_WARP || (P) == PASS_FUSED ? 3 : 4)
 
 // Publishes block b (its writes visible device-wide before the flag).
 __device__ __forceinline__ void publish(uint32_t* ready, uint32_t b, uint32_t epoch, uint32_t lane) {
@@ -1766,12 +1769,12 @@ __device__ void fused_loop(const Jobs& jobs, ScratchHdr* sh, uint32_t n_items, u
           // source blocks must be members of the closure; published ones
           // carry the epoch without the pending bit, so the flag checks do
           // not wait
-          ok = match_block<true, true, true, WAY_ROWS>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch,
+          ok = match_block<true, true, true, WAY_LANES>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch,
                                              ntok ? ntok - 1 : 0);
           if (ok && a.slice) slice_part(a, b, lane);
           if (ok) publish(a.ready, b, epoch, lane);
         } else {
-          ok = match_block<false, false, true, WAY_ROWS>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch,
+          ok = match_block<false, false, true, WAY_LANES>(a, reinterpret_cast<MatchRec*>(wsm), b, lane, epoch,
                                                ntok ? ntok - 1 : 0, L);
         }
         if (!ok) break;  // the error is recorded; every warp stops

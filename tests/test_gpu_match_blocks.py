@@ -222,3 +222,29 @@ def test_levels_of_many_blocks_at_every_size(profile, mm, log2b):
         da = DeviceArchive(arc)
         _check(da, small)
         da.close()
+
+
+@pytest.mark.parametrize("log2b", [8, 12, 14, 16])
+@pytest.mark.parametrize("shape", sorted(SHAPES))
+def test_fused_schedule(shape, log2b):
+    """A match of up to 32 bytes by one lane in 8-byte words, at every length,
+    alignment and overlap of the shapes, in whole decodes, seeks and batches."""
+    lengths, back, lit = SHAPES[shape]
+    data = _copies(lengths, back, lit, 90_001, 7 * log2b)
+    arc = ace.ace_encode(data, log2b, 4)
+    fused = ace.make_tune(schedule=ace.ACE_SCHEDULE_FUSED)
+    da = DeviceArchive(arc, max_seek_blocks=400)
+    out = da.decode_all(tune=fused)
+    assert da.sync() == ace.ACE_OK
+    assert np.array_equal(out.cpu().numpy(), data)
+    ace.ace_index_set_tune(da.idx, fused)
+    for coord, n in ((0, 1), (31_007, 20_002), (data.size - 5001, 5001)):
+        s = da.seek(coord, n)
+        assert da.sync() == ace.ACE_OK
+        assert np.array_equal(s.cpu().numpy(), data[coord:coord + n])
+    da.close()
+    db = DeviceBatch([arc, arc], tune=fused)
+    db.decode()
+    assert db.sync() == ace.ACE_OK
+    assert all(np.array_equal(db.output(k).cpu().numpy(), data) for k in range(2))
+    db.close()
