@@ -715,23 +715,12 @@ __host__ __device__ inline uint32_t job_smem_bytes(uint32_t escn, uint32_t ring)
 template <bool SEEK, uint32_t RING>
 __device__ bool literal_block(const DecodeArgs& a, const LitMem& m, uint32_t b, uint32_t lane) {
   bool ok = true;
-  const uint32_t* dw = reinterpret_cast<const uint32_t*>(a.dir + b);
-  uint32_t dv = lane < 16 ? __ldg(dw + lane) : 0u;
-  const uint64_t B = (uint64_t)1 << a.log2B, bstart = (uint64_t)b << a.log2B;
-  const uint32_t blen = (uint32_t)min(B, a.total - bstart);
-  const uint32_t ntok = __shfl_sync(kFull, dv, 12);
-  const uint32_t nm = ntok ? ntok - 1 : 0;
-  uint8_t* obase = SEEK ? a.out + slot_base(a, b) : a.out + bstart;
+  const BlockHead h(a, b, lane);
+  const uint32_t blen = h.blen, ntok = h.ntok, nm = ntok ? ntok - 1 : 0;
+  uint8_t* obase = SEEK ? a.out + slot_base(a, b) : a.out + ((uint64_t)b << a.log2B);
   const uint32_t lt = lanemask_lt();
   Stream sl;
-  {
-    const int k = ACE_S_LIT;
-    uint64_t soff = (uint64_t)__shfl_sync(kFull, dv, 2 * k) | ((uint64_t)__shfl_sync(kFull, dv, 2 * k + 1) << 32);
-    uint32_t sbytes = __shfl_sync(kFull, dv, 6 + k), nsym = __shfl_sync(kFull, dv, 9 + k);
-    const uint32_t mode = __shfl_sync(kFull, dv, 14) & 0xffu;
-    if (!stream_open<RING>(a.arc + a.payload_off + soff, sbytes, nsym, m.ring, sl, lane, mode))
-      fail(a, ok, ACE_E_CORRUPT, b, 20, lane);
-  }
+  if (!h.open<RING>(a, ACE_S_LIT, m.ring, sl, lane)) fail(a, ok, ACE_E_CORRUPT, b, 20, lane);
   cp_async_wait<RING / kSeg - 2>();
   __syncwarp();
   if (ok && sl.nsym) {
@@ -962,21 +951,24 @@ __device__ __forceinline__ uint32_t upper_bound(uint32_t n, uint32_t x, Key key)
 // dependency lists disagree with its matches.  Returns false if a record is
 // corrupt or a wait gave up.
 //
-// A group whose matches are all short (at most kRowMax bytes) and do not
-// overlap their sources -- text, FASTQ and mixed data are almost only such --
+// WAY_ROWS: a group whose matches are all short (at most kRowMax bytes) and do
+// not overlap their sources -- text, FASTQ and mixed data are almost only such --
 // is copied in rows: its match bytes laid end to end, 32 consecutive ones per
 // row, a lane's match found by counting start bits in a bit map of the group,
 // so that loads and stores of a row touch the few lines its two or three
 // matches lie in.  Rows go in output order, so a source byte is final unless
 // it lies at or after the first byte of the rows in flight; such bytes wait
-// until those before them are stored.  Any other group is copied in rounds of
-// matches none of which reads bytes another pending one of the group writes
-// (literal bytes are final after the literal pass; the first pending match is
-// always ready, so every round makes progress).
+// until those before them are stored.  Any other group, and every one of the
+// other ways, is copied in rounds of matches none of which reads bytes another
+// pending one of the group writes (literal bytes are final after the literal
+// pass; the first pending match is always ready, so every round makes progress).
 //
-// Every group went through the rounds, short matches one per lane in 8-byte
-// words whose loads and stores touch 32 lines each (FASTQ 256 MiB: 0.145 ms);
-// by rows 0.106 ms, bound by the latency of a group after another.
+// Short matches by lanes (WAY_LANES) touch 32 lines with every load and store:
+// FASTQ 256 MiB, a launch per level, 0.145 ms, by rows 0.106.  But a group is then
+// two trips to memory where its rows are four, and where waits have already cost
+// one and few warps are resident that decides: 115 MB of FASTQ objects in 64 KiB
+// blocks 411 us by lanes, 447 by rows; in 1 KiB blocks 908 and 909.  Bound by the
+// latency of a group after another.
 template <bool SEEK, bool WAIT, bool L1, int WAY>
 __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint32_t lane, uint32_t epoch,
                             uint32_t nm, uint32_t lvl = 0) {
@@ -1036,13 +1028,11 @@ __device__ bool match_block(const DecodeArgs& a, MatchRec* gm, uint32_t b, uint3
       bool timeout = false;
       // a source block must sit at a lower dependency level (work lists are
       // in level order, so it was handed out before this block and the wait
-      // ends); the block cache keeps no levels and skips this check
+      // ends)
       if (ext) {
         bool low = true;
-        if (a.level) {
-          const uint32_t my_level = __ldg(a.level + b);
-          for (uint64_t k = k0; k <= k1; k++) low &= __ldg(a.level + k) < my_level;
-        }
+        const uint32_t my_level = __ldg(a.level + b);
+        for (uint64_t k = k0; k <= k1; k++) low &= __ldg(a.level + k) < my_level;
         if (SEEK && a.closure_flags) {
           // every source block must be a member of this seek's closure: its
           // flag carries the call's epoch (pending or published).  Anything
@@ -1261,6 +1251,11 @@ __device__ __forceinline__ void known16(uint4* e, uint4 v) {
 // With WAIT a source block before this one may not be published yet: a bounded
 // wait; without it its level must be below lvl.  Returns false, for the whole
 // CTA, if a record is corrupt or a wait gave up (recorded).
+//
+// LITS: after stream jobs.  The literals are still in order at the end of the
+// block's place (a record's source holds above its five bytes the literals
+// before the match), so literal runs are laid in rows too, the last one as
+// token nm, and every byte of the window gets its entry from a row.
 constexpr uint32_t kCtaWindow = 16384;
 constexpr uint32_t kCtaThreads = 512;                       // at most
 constexpr uint32_t kCtaRowBytes = 2048;                     // match bytes whose starts the bit map holds
@@ -1288,11 +1283,6 @@ __host__ __device__ inline uint32_t cta_smem_bytes(uint32_t log2B, uint32_t thre
   return 2 * (log2B >= 14 ? kCtaWindow : 1u << log2B) + threads / 32 * kCtaWarpSmem;
 }
 
-//
-// LITS: after stream jobs.  The literals are still in order at the end of the
-// block's place (a record's source holds above its five bytes the literals
-// before the match), so literal runs are laid in rows too, the last one as
-// token nm, and every byte of the window gets its entry from a row.
 template <bool SEEK, bool WAIT, bool LITS>
 __device__ bool match_cta(const DecodeArgs& a, uint8_t* smem, uint32_t b, uint32_t nm, uint32_t epoch, uint32_t lvl) {
   __shared__ uint32_t s_group;
@@ -2282,7 +2272,7 @@ struct CacheHdr {
   uint32_t ticket;
   uint32_t n_work;
   uint32_t n_cached;   // slots holding a decoded block
-  uint32_t n_front;
+  uint32_t reserved;
   uint32_t hand;       // clock hand: the next slot the allocation looks at
   uint32_t serial;     // batches run: the slots a batch uses carry its serial
   uint64_t evicted;    // cached blocks evicted to make room, since creation
@@ -2984,8 +2974,13 @@ constexpr uint32_t kSplitLevels = 8;
 constexpr uint64_t kSplitSeek = 1024;
 constexpr uint64_t kSplitFew = 48;
 constexpr uint32_t kSplitFewLog2B = 12;
-// Seek batches, by target blocks (1900 over four profiles: 301 us against 371)
-// where the host has the requests, else by their number.
+// Seek batches, by target blocks where the host has the requests, us (in two
+// passes): 1900 blocks over four profiles 301 (371); genome, 1152 blocks of 16 KiB
+// 204 (226), 1040 of 4 KiB 126 (133), 4224 of them 264 (242), 4112 of 1 KiB 159
+// (163), 16512 of them 405 (322); text 361 (428), 185 (218), 400 (395), 215 (213)
+// and 538 (462).  Else by their number, which says less: genome, 64 requests of 16
+// KiB 162 (180) in 16 KiB blocks, 97 (103) in 4 KiB, 128 of them 172 (190) and 107
+// (117), but 128 requests of 128 KiB in 1 KiB blocks 400 (318).
 constexpr uint64_t kSplitBatch = 3072;
 constexpr uint32_t kSplitReqs = 64;
 

@@ -19,7 +19,7 @@ struct ScratchHdr {
   uint32_t epoch;      // value a block's ready flag takes when it is published
   uint32_t ticket;     // next work item handed to a persistent warp
   uint32_t n_work;     // seek: blocks in the work list
-  uint32_t unused;
+  uint32_t reserved;
   uint32_t min_block;  // seek: smallest block reached by the closure
   uint64_t fnv;        // verify: last FNV-1a 64 computed
   uint64_t guard_bad;  // verify: guard bytes that differ from the canary

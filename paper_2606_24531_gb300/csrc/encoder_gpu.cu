@@ -44,7 +44,6 @@ constexpr uint32_t kStride = 8;      // positions whose keys enter the table
 constexpr uint32_t kWin = 64;        // blocks of a window
 constexpr uint32_t kHeadWins = 3;    // windows whose blocks may be sources
 constexpr uint32_t kHead = kWin * kHeadWins;
-constexpr uint32_t kMaxWave = 3;     // deepest in-block resolution wave taken
 constexpr uint32_t kCap = 32;        // match lengths measured by the candidate search (extended later)
 constexpr uint32_t kHashBits4 = 12;  // in-block chains: hash of 4 bytes
 constexpr uint32_t kMaxChain = 64;
@@ -84,7 +83,7 @@ __device__ __forceinline__ uint32_t common(const uint8_t* a, const uint8_t* b, u
 
 struct EncArgs {
   const uint8_t* in;
-  uint64_t n, nb;
+  uint64_t n;
   uint32_t log2B, min_match, max_chain, w, adaptive, bits;
   unsigned long long* table;  // 2^bits: the earliest stride position with each key hash
   uint64_t c0;  // the launch's first block
@@ -95,7 +94,6 @@ struct EncArgs {
   uint32_t* tok;      // per chunk block: tok_cap x (lit_run, match_len, src lo, src hi)
   uint32_t tok_cap;
   uint32_t* ntok;     // per chunk block
-  uint32_t* status;   // first error
   unsigned long long* stats;  // n_tokens, n_matches, literal, match, match_src bytes
 };
 
@@ -476,7 +474,7 @@ __device__ __forceinline__ bool external_wins(uint32_t li, uint32_t wi, uint32_t
 // position with an acceptable candidate a match, literals before it.  A
 // match's resolution wave is 1 + the deepest wave among the bytes of its own
 // block it reads (literals and bytes of earlier blocks are wave 0); deeper
-// than kMaxWave is refused.
+// than 3 is refused.
 //
 // The walk is a serial chain of decisions, so its latency bounds it.  The
 // warp therefore decides 32 positions at once, a lane each, as if every
@@ -1274,7 +1272,6 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   EncArgs e{};
   e.in = static_cast<const uint8_t*>(d_in);
   e.n = n;
-  e.nb = nb;
   e.log2B = params->log2_block;
   e.min_match = params->min_match;
   e.max_chain = params->max_chain ? params->max_chain : 16;
@@ -1287,7 +1284,6 @@ ace_status ace_encode_gpu(const void* d_in, uint64_t n, const ace_encode_params*
   e.tok = reinterpret_cast<uint32_t*>(base + L.tok);
   e.tok_cap = L.tok_cap;
   e.ntok = reinterpret_cast<uint32_t*>(base + L.ntok);
-  e.status = &hdr->status;
   e.stats = hdr->stats;
   CodeArgs ca;
   ca.syms = base + L.syms;
