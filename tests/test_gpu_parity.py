@@ -81,7 +81,7 @@ def test_decode_all_oracle_archives(profile, log2b, schedule):
 
 @pytest.mark.parametrize("schedule", sorted(SCHEDULES))
 def test_seeks_under_both_schedules(schedule):
-    """Seeks through the fused launch and through the three passes, on a
+    """Seeks through the fused launch and through the pass schedule, on a
     library archive and on a deep-chain oracle archive, equal the original."""
     for arc_of, n in ((lambda d: ace.ace_encode(d, 12, 4), 2_000_000), (lambda d: oracle.encode(d, 10, 4, 16), 300_000)):
         data = synth.generate("text", n, 33)
@@ -426,7 +426,8 @@ def test_levels_match_oracle():
 def test_copy_widths_decode_and_seek(copy_width):
     """Both copy widths (16-byte pieces from 33 bytes, or from 512 with
     bytewise copies below) give the original bytes in whole decodes, seeks
-    (which now take the piece copies too) and every overlap distance."""
+    and every overlap distance (of these few blocks the fused whole decodes are
+    those that copy by it; decodes of many blocks: test_gpu_routes)."""
     rng = np.random.default_rng(12)
     parts = []
     for d in range(1, 80, 3):

@@ -13,6 +13,7 @@ pytestmark = pytest.mark.gpu
 
 from paper_2606_24531_gb300 import ace  # noqa: E402
 from paper_2606_24531_gb300.archive import DeviceArchive  # noqa: E402
+from paper_2606_24531_gb300.batch import DeviceBatch  # noqa: E402
 from paper_2606_24531_gb300.serve import SeekCache  # noqa: E402
 
 MM = {"fastq": 16, "genome": 20, "text": 4, "mixed": 4}
@@ -22,6 +23,10 @@ MM = {"fastq": 16, "genome": 20, "text": 4, "mixed": 4}
 def built():
     __graft_entry__.build()
     torch.cuda.set_device(0)
+
+
+def _blocks(size, log2b):
+    return (size + (1 << log2b) - 1) >> log2b
 
 
 def _archive(profile, n, log2b, seed=3, **kw):
@@ -133,3 +138,57 @@ def test_whole_decodes_by_blocks(profile, log2b, per_sm):
         assert da.sync() == ace.ACE_OK
         assert np.array_equal(out.cpu().numpy(), data)
         da.close()
+
+
+@pytest.mark.parametrize("copy_width", [8, 16])
+def test_copy_widths_of_many_blocks(copy_width):
+    """Where a warp resolves a block's matches: levels of more than four blocks
+    per SM by rounds and by rows, fused seeks, batches of few matches."""
+    tune = ace.make_tune(copy_width=copy_width)
+    for profile in ("genome", "fastq"):
+        data, da = _archive(profile, 6_000_001, 12, seed=9, max_seek_blocks=600)
+        out = da.decode_all(tune=tune)
+        assert da.sync() == ace.ACE_OK
+        assert np.array_equal(out.cpu().numpy(), data)
+        ace.ace_index_set_tune(da.idx, ace.make_tune(schedule=ace.ACE_SCHEDULE_FUSED, copy_width=copy_width))
+        s = da.seek(5_000_003, 700_001)
+        assert da.sync() == ace.ACE_OK
+        assert np.array_equal(s.cpu().numpy(), data[5_000_003:5_700_004])
+        db = DeviceBatch([da.d_arc.cpu().numpy()] * 2, tune=tune)
+        db.decode()
+        assert db.sync() == ace.ACE_OK
+        assert np.array_equal(db.output(1).cpu().numpy(), data)
+        db.close()
+        da.close()
+
+
+@pytest.mark.parametrize("profile, log2b, size", [("text", 8, 340_000), ("text", 12, 6_000_000), ("fastq", 12, 4_000_000),
+                                                  ("genome", 12, 6_000_000)])
+def test_corrupt_payloads_in_the_passes(profile, log2b, size):
+    """A flipped payload bit, in decodes, seeks and batches that take the token,
+    literal and match passes: reported, or the bytes the oracle decodes from the
+    same archive."""
+    data = synth.generate(profile, size, 13)
+    arc = ace.ace_encode(data, log2b, MM[profile])
+    payload_off = int(arc[48:56].view(np.uint64)[0])
+    rng = np.random.default_rng(log2b)
+    seen = set()
+    for trial in range(8):
+        bad = arc.copy()
+        bad[int(rng.integers(payload_off, bad.size))] ^= np.uint8(1 << int(rng.integers(0, 8)))
+        ref = None
+        da = DeviceArchive(bad, max_seek_blocks=_blocks(size, log2b))
+        ace.ace_index_set_tune(da.idx, ace.make_tune(wait_timeout_ns=50_000_000))
+        db = DeviceBatch([bad, arc], tune=ace.make_tune(wait_timeout_ns=50_000_000))
+        db.decode()
+        got = [(lambda o: (da.sync(), o))(da.decode_all()), (lambda o: (da.sync(), o))(da.seek(0, size)),
+               (db.sync(), db.output(0))]
+        for st, out in got:
+            assert st in (ace.ACE_OK, ace.ACE_E_CORRUPT), ace.ace_status_str(st)
+            seen.add(st)
+            if st == ace.ACE_OK:
+                ref = oracle.decode(bad) if ref is None else ref
+                assert np.array_equal(out.cpu().numpy()[:size], ref)
+        db.close()
+        da.close()
+    assert ace.ACE_E_CORRUPT in seen
