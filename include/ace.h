@@ -245,9 +245,9 @@ ace_status ace_scratch_init(const ace_index *idx, void *d_scratch, uint64_t scra
 /* How a decode is laid out in launches.
  * ACE_SCHEDULE_PASSES: three passes -- tokens (length and offset streams
  * into match records) and literals as persistent launches over the blocks,
- * then the match pass, one launch per dependency level; with little work to
- * spread (few blocks, small batches) the first two become one launch, a warp
- * per stream, and the match pass places the literals.
+ * then the match pass, one launch per dependency level; with few blocks to
+ * spread the first two become one launch, a warp per stream, and the match pass
+ * places the literals, where that is the shorter way.
  * ACE_SCHEDULE_FUSED: one persistent launch.  Each warp takes a block in
  * (level, block) order and decodes its entropy layer, then holds the
  * block's matches until every block of the lower levels is resolved,
@@ -258,16 +258,20 @@ ace_status ace_scratch_init(const ace_index *idx, void *d_scratch, uint64_t scra
  * take the fused schedule only for archives of at most 32 levels. */
 enum { ACE_SCHEDULE_AUTO = 0, ACE_SCHEDULE_PASSES = 1, ACE_SCHEDULE_FUSED = 2 };
 
+/* What each knob reaches.  Calls of few blocks (ACE_SCHEDULE_PASSES above) have a
+ * launch of their own shape for the entropy layer, and only wait_timeout_ns and
+ * schedule change anything there. */
 typedef struct {
-    uint32_t warps_per_cta;   /* 1..8; 0 = default (4) */
-    uint32_t ctas_per_sm;     /* 0 = as many as fit */
-    uint32_t chunk_tokens;    /* a step of the literal pass lists two literal runs, and takes up to 32 literals, per token of this, 32..256, multiple of 32; 0 = 128 */
+    uint32_t warps_per_cta;   /* 1..8; 0 = default (4).  Passes that take a block per warp, and the fused pass */
+    uint32_t ctas_per_sm;     /* 0 = as many as fit.  Persistent launches of the passes and the fused pass */
+    uint32_t chunk_tokens;    /* the literal pass and the fused pass: a step lists two literal runs, and takes up to
+                                 32 literals, per token of this; 32..256, a multiple of 32; 0 = 128 */
     uint32_t schedule;        /* ACE_SCHEDULE_*; 0 = automatic; others: ACE_E_INVAL */
     uint64_t wait_timeout_ns; /* bound on each device-side wait; 0 = 2 s */
-    uint32_t copy_width;      /* match copies where a warp resolves a block's matches in rounds: 16 = every
-                                 non-overlapping match above 32 bytes in aligned 16-byte pieces; 8 = 16-byte
-                                 pieces from 512 bytes, bytewise below; 0 = the library's choice (16);
-                                 others: ACE_E_INVAL */
+    uint32_t copy_width;      /* match copies where a warp resolves a block's matches in rounds (levels of many
+                                 blocks, batches of few matches, the fused pass): 16 = every non-overlapping match
+                                 above 32 bytes in aligned 16-byte pieces; 8 = 16-byte pieces from 512 bytes,
+                                 shorter ones bytewise; 0 = the library's choice (16); others: ACE_E_INVAL */
     uint32_t reserved;        /* 0 */
 } ace_tune;
 
@@ -282,8 +286,10 @@ typedef struct {
  * the match pass one launch per dependency level (a CTA per block for levels
  * of few blocks and archives of many short matches, a warp per block
  * otherwise), or, for archives of more than 32 levels, one persistent
- * launch, a CTA per block, in (level, block) order with bounded waits on
- * source blocks' ready flags.  Decodes of few blocks take the token and
+ * launch, a CTA or, for short blocks or few matches, a warp per block, in
+ * (level, block) order with bounded waits on source blocks' ready flags.
+ * Decodes of few blocks (not of large ones with many literals, nor of many
+ * levels with few matches) take the token and
  * literal passes as one launch, a warp per stream, and the match pass places
  * the literals too.  ACE_SCHEDULE_FUSED does all of it in one persistent launch.
  * A source block whose level is not below its reader's makes the call
@@ -296,9 +302,10 @@ ace_status ace_decode_all(const ace_index *idx, void *d_out, uint64_t out_bytes,
 /*
  * The passes of ace_decode_all's pass schedule as separate calls, so that a
  * caller can time each one with events on s: ACE_PASS_TOKENS (which also
- * resets the call's status), ACE_PASS_LITERALS, then ACE_PASS_MATCH, same
- * arguments, same stream; together they are exactly ace_decode_all with
- * ACE_SCHEDULE_PASSES.  Any other pass value: ACE_E_INVAL.
+ * resets the call's work counters), ACE_PASS_LITERALS, then ACE_PASS_MATCH, same
+ * arguments, same stream.  Together they give what ace_decode_all gives, by the
+ * kernels it takes for many blocks; for few it has others (above).  Any other
+ * pass value: ACE_E_INVAL.
  */
 enum { ACE_PASS_TOKENS = 0, ACE_PASS_LITERALS = 1, ACE_PASS_MATCH = 2 };
 ace_status ace_decode_pass(const ace_index *idx, int pass, void *d_out, uint64_t out_bytes, void *d_scratch,
@@ -344,13 +351,14 @@ ace_status ace_sync(const ace_index *idx, void *d_scratch, cudaStream_t s);
  * plans the launch from tune (NULL = defaults), and synchronises s.  It
  * allocates no device memory.  ace_decode_batch then enqueues, with no host
  * synchronisation, a header reset and the token, literal and match passes
- * (pass schedule; up to 128 MiB of output a launch of a warp per stream, then
- * the match pass) or a memset of the level counters, a header reset and one
+ * (pass schedule; where few or long blocks of many matches would be the passes'
+ * tail, a launch of a warp per stream and the match pass) or a memset of the level counters, a header reset and one
  * fused launch (ACE_SCHEDULE_FUSED), so it can be captured into a CUDA graph
  * and replayed; each replay decodes every archive again.
  * ace_batch_sync synchronises s and returns (then clears) the first device
- * error.  ace_batch_launch_shape reports the planned grid, warps per CTA and
- * token window.
+ * error.  ace_batch_launch_shape reports the grid, warps per CTA and token window
+ * of the entropy layer's (or the fused) launch; the window is 0 where a warp takes
+ * a stream, which has none.
  */
 typedef struct ace_batch ace_batch;
 ace_status ace_batch_scratch_size(const ace_index *const *idx, uint32_t n, uint64_t *bytes);
@@ -391,9 +399,11 @@ ace_status ace_batch_free(ace_batch *batch);
  * one cache must be ordered on one stream; separate caches (each with its
  * own per-archive states) may run concurrently on separate streams.
  * ace_seek_batch reads device-resident requests and enqueues the closure
- * search, the passes and the slice copies; ace_seek_batch_host validates host requests against the
- * archives' sizes (h_totals, may be NULL) and the pool, stages them in the
- * cache memory (n <= max_reqs) and calls it.  ace_cache_sync returns (then
+ * search, the passes and the slice copies; ace_seek_batch_host validates host
+ * requests against the archives' sizes (h_totals, may be NULL) and the pool,
+ * stages them in the cache memory (n <= max_reqs) and enqueues the same.  Whether
+ * the passes take a block or a stream per warp follows from the blocks the host
+ * requests cover, and from the number of device requests.  ace_cache_sync returns (then
  * clears) the first device error; ace_cache_usage reports slots holding a
  * block; ace_cache_counters the blocks evicted and decoded since creation;
  * ace_cache_limits the slots, the blocks one batch may decode and the

@@ -73,7 +73,9 @@ TUNE_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "ace_gb300", "tune.
 def autotune(db, candidates=None, reps=3, cache_key=None, cache_path=TUNE_CACHE):
     """Times each (warps per CTA, token window, schedule, copy width)
     candidate on the batch and keeps the fastest; results are cached by
-    cache_key in a JSON file."""
+    cache_key in a JSON file.  Candidates that come to a launch already timed
+    (a batch decoded a stream per warp has one, whatever the knobs) are
+    passed over."""
     def tune_of(c):
         return ace.make_tune(c["warps_per_cta"], 0, c["window"], schedule=c.get("schedule", 0),
                              copy_width=c.get("copy_width", 0))
@@ -92,14 +94,19 @@ def autotune(db, candidates=None, reps=3, cache_key=None, cache_path=TUNE_CACHE)
                       for w in (1, 2, 4, 8) for c in (64, 128, 256) for cw in (8, 16)]
     best = None
     results = []
+    timed = set()
     for cand in candidates:
         w, c = cand[0], cand[1]
         sch = cand[2] if len(cand) > 2 else ace.ACE_SCHEDULE_PASSES
         cw = cand[3] if len(cand) > 3 else 0
         try:
-            db.retune(ace.make_tune(w, 0, c, schedule=sch, copy_width=cw))
+            shape = db.retune(ace.make_tune(w, 0, c, schedule=sch, copy_width=cw))
         except ace.AceError:
             continue
+        launch = (*shape.values(), sch, cw if shape["window"] else 0)
+        if launch in timed:
+            continue
+        timed.add(launch)
         db.decode()
         if db.sync() != ace.ACE_OK:
             continue

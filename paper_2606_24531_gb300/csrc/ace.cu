@@ -2070,7 +2070,8 @@ __global__ void ACE_PASS_BOUNDS(PASS) batch_decode_kernel(BatchArgs ba) {
 // The entropy layer of a batch, a warp per stream, largest blocks first: one
 // launch whose time is its longest stream's, where the token and literal
 // passes each had that tail.
-__global__ void __launch_bounds__(128, 8) batch_entropy_kernel(BatchArgs ba) {
+constexpr uint32_t kBatchEntropyWarps = 4;
+__global__ void __launch_bounds__(32 * kBatchEntropyWarps, 8) batch_entropy_kernel(BatchArgs ba) {
   extern __shared__ __align__(16) uint8_t smem[];
   const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const BatchJobs jobs{ba, ba.by_size, ba.n_size};
@@ -3906,7 +3907,7 @@ ace_status ace_batch_create(const ace_index* const* idx, uint32_t n, void* const
   BatchArgs& a = b->args;
   a.objs = reinterpret_cast<const ObjDesc*>(base + B.objs);
   b->split = B.split;
-  b->entropy_grid = (uint32_t)std::min<uint64_t>((3 * B.items + 3) / 4, 8ull * idx[0]->num_sms);
+  b->entropy_grid = (uint32_t)std::min<uint64_t>((3 * B.items + kBatchEntropyWarps - 1) / kBatchEntropyWarps, 8ull * idx[0]->num_sms);
   a.by_size = reinterpret_cast<const BatchSeg*>(base + B.by_size);
   a.by_level = reinterpret_cast<const BatchSeg*>(base + B.by_level);
   a.n_size = (uint32_t)by_size.size();
@@ -3933,7 +3934,8 @@ ace_status ace_decode_batch(const ace_batch* b, cudaStream_t s) {
   if (L.schedule == ACE_SCHEDULE_FUSED)
     launch_fused(L, batch_decode_kernel<PASS_FUSED>, b->args, s);
   else if (b->split) {
-    batch_entropy_kernel<<<b->entropy_grid, 128, 4 * job_smem_bytes(b->args.esc_cap, kRing), s>>>(b->args);
+    batch_entropy_kernel<<<b->entropy_grid, 32 * kBatchEntropyWarps,
+                           kBatchEntropyWarps * job_smem_bytes(b->args.esc_cap, kRing), s>>>(b->args);
     batch_decode_kernel<PASS_PLACE><<<L.grid[PASS_MATCH], L.match_threads, L.smem[PASS_MATCH], s>>>(b->args);
   } else
     launch_passes(L, 7, batch_decode_kernel<PASS_TOKENS>, batch_decode_kernel<PASS_LITERALS>,
@@ -3956,9 +3958,10 @@ ace_status ace_batch_sync(const ace_batch* b, cudaStream_t s) {
 
 ace_status ace_batch_launch_shape(const ace_batch* b, uint32_t* grid, uint32_t* warps_per_cta, uint32_t* window) {
   if (!b) return ACE_E_INVAL;
-  if (grid) *grid = b->L.grid[PASS_TOKENS];
-  if (warps_per_cta) *warps_per_cta = b->L.warps;
-  if (window) *window = b->L.chunk;
+  const bool fused = b->L.schedule == ACE_SCHEDULE_FUSED, split = b->split && !fused;
+  if (grid) *grid = split ? b->entropy_grid : b->L.grid[fused ? PASS_FUSED : PASS_TOKENS];
+  if (warps_per_cta) *warps_per_cta = split ? kBatchEntropyWarps : b->L.warps;
+  if (window) *window = split ? 0 : b->L.chunk;
   return ACE_OK;
 }
 

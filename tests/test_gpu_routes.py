@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 from paper_2606_24531_gb300 import ace  # noqa: E402
 from paper_2606_24531_gb300.archive import DeviceArchive  # noqa: E402
-from paper_2606_24531_gb300.batch import DeviceBatch  # noqa: E402
+from paper_2606_24531_gb300.batch import DeviceBatch, autotune  # noqa: E402
 from paper_2606_24531_gb300.serve import SeekCache  # noqa: E402
 
 MM = {"fastq": 16, "genome": 20, "text": 4, "mixed": 4}
@@ -192,3 +192,24 @@ def test_corrupt_payloads_in_the_passes(profile, log2b, size):
         db.close()
         da.close()
     assert ace.ACE_E_CORRUPT in seen
+
+
+def test_autotune_times_each_launch_once():
+    """A batch decoded a stream per warp has one launch under the pass schedule,
+    and reports it; one of many blocks has the candidates' own."""
+    for size, one in ((60_000, True), (9_000_000, False)):
+        data = synth.generate("text", size, 2)
+        arc = ace.ace_encode(data, 12, 4)
+        db = DeviceBatch([arc, arc])
+        shape = db.retune()
+        assert (shape["window"] == 0) == one
+        if one:
+            assert (shape["grid"], shape["warps_per_cta"]) == ((2 * 3 * 15 + 3) // 4, 4)
+        best = autotune(db, reps=1, cache_key=None)
+        rows = [r for r in best["sweep"] if r["schedule"] == ace.ACE_SCHEDULE_PASSES]
+        assert len(rows) == (1 if one else 24)
+        db.out.zero_()
+        db.decode()
+        assert db.sync() == ace.ACE_OK
+        assert np.array_equal(db.output(1).cpu().numpy(), data)
+        db.close()
