@@ -1230,9 +1230,9 @@ __device__ __forceinline__ void known16(uint4* e, uint4 v) {
 // blocks of at most that).  Every byte of the window gets a 16-bit entry in
 // shared memory: 0x8000 | its value where that is known (a literal, or a match
 // byte whose source lies before the window, which is final), else the address
-// of the entry of the byte it copies (twice its place in the window).  A match byte equals the byte one distance
-// before it (Section 2, the sequential LZ77 copy; overlapping matches too), so
-// entries form chains that end at known ones.  The warps set the entries a
+// of the entry of the byte it copies (twice its place in the window).  A match
+// byte equals the byte one distance before it (Section 2, the sequential LZ77
+// copy; overlapping matches too), so entries form chains that end at known ones.  The warps set the entries a
 // group of 32 matches each, in rows of 32 match bytes (as match_block, but in
 // any order: an entry waits for nothing), then every thread follows the chains
 // of its 16 bytes and stores them.  Chains longer than kHops (matches of one
@@ -1879,10 +1879,9 @@ __global__ void __launch_bounds__(32) entropy_kernel(DecodeArgs a) {
 // waits.  Blocks are dealt out statically (block k of the level to warp
 // k mod the warps in the grid), and each warp fetches its next block's
 // number and record range while it resolves the current one.
-// ROWS: the archive's matches are mostly short; without it every group goes by
-// rounds, in fewer registers (genome 1 GiB, the match pass: 342 us at 56
-// registers, 360 at 72; the rows' kernel spills below 72: FASTQ 129 us, 147 at
-// 56).  A long match by the whole warp, not the round's long matches laid end
+// WAY_ROWS for matches mostly short, WAY_ROUNDS, in fewer registers, for few long
+// ones (genome 1 GiB, the match pass: 342 us at 56 registers, 360 at 72; the rows
+// spill below 72: FASTQ 129 us, 147 at 56).  A long match by the whole warp, not the round's long matches laid end
 // to end in pieces with the next lane's vector shuffled in, took the genome's
 // from 518 us.
 template <int WAY>
