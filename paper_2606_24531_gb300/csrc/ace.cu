@@ -3738,9 +3738,9 @@ struct BatchLayout {
 // all, which then place the literals.  For dense archives both are estimated: the
 // longest block's chain (about 8 and 2.3 ns a byte) or the sum of the work (3 us
 // a MB, 2 where matches are few), the larger of the two, plus a second launch or
-// 17 ns a block (6 where matches are few; less in proportion below 2 KiB).  Text,
-// us split (passes): 4 MB in 4 KiB blocks 72 (104), 16 KiB 85 (170), 64 KiB 250
-// (549); 36 MB 500 (360), 269 (279), 348 (622); 115 MB 1670 (1054), 844 (710),
+// 17 ns a block (6 where matches are few; less in proportion below 4 KiB, at least
+// 2).  Text, us split (passes): 4 MB in 256-byte blocks 179 (158), 1 KiB 109 (104),
+// 2 KiB 83 (93), 4 KiB 72 (104), 16 KiB 85 (170), 64 KiB 250 (549); 36 MB 500 (360), 269 (279), 348 (622); 115 MB 1670 (1054), 844 (710),
 // 783 (910).  Uneven objects of all profiles: 57 MB 503 (781), 118 MB 804 (900),
 // 183 MB 1157 (1122).  Without dense archives only few blocks are worth it: FASTQ,
 // 4 MB in 8 KiB blocks 70 (79), 16 KiB 101 (116), 64 KiB 380 (342); genome 70
@@ -3755,7 +3755,7 @@ void batch_route(const ace_index* const* idx, uint32_t n, BatchLayout* B) {
     const double total = (double)x.h.total_size, block = std::min(total, (double)(1ull << x.h.log2_block));
     const bool dense = x.h.total_size && dense_matches(x.n_matches, x.h.total_size);
     bytes += total;
-    per_block += (double)x.h.n_blocks * std::min(1.0, block / 2048) * (dense ? 17e-3 : 6e-3);
+    per_block += (double)x.h.n_blocks * std::max(0.12, std::min(1.0, block / 4096)) * (dense ? 17e-3 : 6e-3);
     if (dense) {
       dense_bytes += total;
       chain = std::max(chain, block);
