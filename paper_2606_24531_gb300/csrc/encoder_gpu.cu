@@ -181,10 +181,11 @@ constexpr uint64_t kSplitEntries = 256;  // 64 KiB blocks whose entries fill scr
 // reach min_match is nearly always dropped there.  Each key is looked up once,
 // by the lane of its position, and shared with the seven positions before;
 // positions a match may not read count as not found, and the pairs of a found
-// key and a position before it are dealt evenly to the lanes.  Bound by issue: about 940 warp instructions
-// per 32 positions of FASTQ.  Byte loads from global memory, a launch for the
-// links and eight lookups a position took 12.4 + 1.5 ms of the 64 MiB FASTQ
-// encode; this takes 2.5 ms.
+// key and a position before it are dealt evenly to the lanes.  Bound by issue and
+// the chains' dependent steps: about 860 warp instructions per 32 positions of
+// FASTQ, 1,940 of text, issued on 57% and 64% of cycles.  Byte loads from global
+// memory, a launch for the links and eight lookups a position took 12.4 + 1.5 ms
+// of the 64 MiB FASTQ encode; this takes 2.5 ms.
 template <bool SHARED>
 __global__ void __launch_bounds__(512, 2) candidate_kernel(EncArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
